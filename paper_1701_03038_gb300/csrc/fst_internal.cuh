@@ -42,6 +42,22 @@ struct __align__(16) WinMeta {
   uint32_t mask[4];
 };
 
+// A slot of the (symbol, state) table: key = symbol << 32 | state (~0:
+// empty), the segment's length << 32 | first position, and its first arc's
+// record.  Two slots make a bucket, 64 aligned bytes that a lookup reads at
+// once: one memory latency, which for the segments of one arc (most of them)
+// brings the arc too.  A key that finds its bucket full goes to the next
+// ones, and marks its own as spilled (SPILLED in the first slot's `at`), so
+// that a lookup that misses reads on only past a spilled bucket; with three
+// slots a segment about 3% of the buckets are.  (One slot after another at
+// up to half load, a warp's 32 lookups waited for the longest of their probe
+// sequences: 7,000 cycles in the readout of a large position.)
+struct alignas(32) SegSlot {
+  unsigned long long key, at;
+  int4 arc;
+};
+constexpr unsigned long long SPILLED = 1ull << 63;
+
 struct Layout {
   int64_t P = 0;         // padded arcs = nwin * WIN
   int64_t nwin = 0;
@@ -54,14 +70,14 @@ struct Layout {
   int32_t* seg_state = nullptr;  // [nseg] dst (forward) / src (backward)
   int32_t* seg_pos = nullptr;    // [nseg] padded start position
   int32_t* seg_len = nullptr;    // [nseg] arcs in the segment
-  // (symbol, state) -> arcs of the segment, open addressing: slot = {key,
-  // len << 32 | first position}; key = symbol << 32 | state, empty slots
-  // hold ~0 (source-segmented layout only)
-  ulonglong2* seg_hash = nullptr;
+  // (symbol, state) -> arcs of the segment, open addressing by buckets of
+  // two slots (source-segmented layout only)
+  SegSlot* seg_hash = nullptr;
+  uint32_t* seg_slot = nullptr;  // [nseg] the slot of each segment
   // [P] the arcs packed for one 16-byte load each: {other, theta bits,
   // caller id, 0} (source-segmented layout only)
   int4* arcs = nullptr;
-  int64_t hash_mask = 0;
+  int64_t buckets = 0;
   int64_t* sym_win = nullptr;    // [m+1]
   int64_t* sym_seg = nullptr;    // [m+1]
   int64_t* sym_lseg = nullptr;   // [m+1] long segments
@@ -238,9 +254,12 @@ int radix_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaSt
 int exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total, cudaStream_t s);
 int exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, cudaStream_t s);
 
-// Slot of key k in a power-of-two table (Fibonacci hashing).
-__host__ __device__ __forceinline__ uint64_t seg_hash_slot(uint64_t k, int64_t mask) {
-  return (k * 0x9E3779B97F4A7C15ull >> 17) & (uint64_t)mask;
+// Bucket of key k among n (Fibonacci hashing; the product's high bits scaled
+// to the range).
+__device__ __forceinline__ uint64_t seg_bucket(uint64_t k, int64_t n) {
+  uint64_t x = k * 0x9E3779B97F4A7C15ull;
+  x ^= x >> 32;
+  return __umul64hi(x * 0x9E3779B97F4A7C15ull, (uint64_t)n);
 }
 __host__ __device__ __forceinline__ uint64_t seg_hash_key(int32_t sym, int32_t state) {
   return ((uint64_t)(uint32_t)sym << 32) | (uint64_t)(uint32_t)state;

@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <cstdlib>
 
+#include "frontier.cuh"
 #include "kernels.cuh"
 
 namespace fstgpu {
@@ -45,40 +46,6 @@ namespace {
 
 constexpr int KT = 256;  // threads per block of the step kernels
 constexpr int FT = 256;  // threads per block of the final reductions
-
-// Error bits of a run (FrontierState::flags[1]): the live pool overflowed,
-// or a grid barrier of a persistent pass gave up waiting.
-constexpr uint32_t ERR_POOL = 1u;
-constexpr uint32_t ERR_TIMEOUT = 2u;
-__device__ __forceinline__ int32_t run_error(uint32_t err) {
-  return (err & ERR_TIMEOUT) ? FST_ERR_TIMEOUT : FST_ERR_OOM;
-}
-
-__device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
-
-// Bounds-checked build (FST_DEBUG): in_bounds(code, i, n) checks 0 <= i < n,
-// and on a violation counts it, records the first (code, index, bound) and
-// returns false so that the caller skips the access.  A normal build
-// compiles every check away.
-enum : int { CHK_STAGE = 1, CHK_POOL_WRITE = 2, CHK_POOL_READ = 3, CHK_ACC = 4, CHK_ARC = 5, CHK_TOKEN = 6 };
-#ifdef FST_DEBUG
-__device__ unsigned long long g_dbg[4];  // violations, code, index, bound
-__device__ __noinline__ bool in_bounds_slow(int code, long long i, long long n) {
-  if (atomicAdd(&g_dbg[0], 1ull) == 0ull) {
-    g_dbg[1] = (unsigned long long)code;
-    g_dbg[2] = (unsigned long long)i;
-    g_dbg[3] = (unsigned long long)n;
-  }
-  return false;
-}
-__device__ __forceinline__ bool in_bounds(int code, long long i, long long n) {
-  return (i >= 0 && i < n) ? true : in_bounds_slow(code, i, n);
-}
-#else
-__device__ __forceinline__ bool in_bounds(int, long long, long long) { return true; }
-#endif
-
-__device__ __forceinline__ float decode_max(uint32_t k) { return k ? fkey_inv(k) : neg_inf(); }
 
 // Owner of flat entry j among the n slots whose first entries base[0..n)
 // are nondecreasing with base[0] <= j: the last slot with base <= j.  The
@@ -131,28 +98,6 @@ __device__ __forceinline__ Owner flat_owner(const int64_t* __restrict__ base, in
     }
   }
   return o;
-}
-
-// The arcs out of state q on symbol a: a lookup in the open-addressing
-// table of the source-segmented layout (load factor <= 1/2, one 16-byte
-// probe on average) giving their first position and count (0 when none).
-struct Arcs {
-  int32_t pos, len;
-};
-__device__ __forceinline__ Arcs find_arcs(const LayoutView& L, int32_t a, int32_t q) {
-  const uint64_t k = seg_hash_key(a, q);
-  uint64_t h = seg_hash_slot(k, L.hash_mask);
-  for (int64_t probe = 0; probe <= L.hash_mask; ++probe) {
-    const ulonglong2 e = __ldg(L.seg_hash + h);
-    if (e.x == k) {
-      const Arcs r{(int32_t)(uint32_t)e.y, (int32_t)(e.y >> 32)};
-      if (r.len > 0 && !in_bounds(CHK_ARC, (long long)r.pos + r.len - 1, L.P)) return Arcs{0, 0};
-      return r;
-    }
-    if (e.x == ~0ull) break;
-    h = (h + 1) & (uint64_t)L.hash_mask;
-  }
-  return Arcs{0, 0};
 }
 
 // Staging buffer of forward position t (two, by parity: a step reads
@@ -398,9 +343,6 @@ __device__ __forceinline__ int32_t block_stage(BlockScratch<Ctx>& sh, int32_t e0
   __syncthreads();
   return total;
 }
-
-// Order key of a float64 value rounded to float32 (0 = -inf, nothing).
-__device__ __forceinline__ uint32_t fkey64(double v) { return v == -INFINITY ? 0u : fkey((float)v); }
 
 // Reductions over each thread's segment: Op maps a value to a 64-bit key,
 // combines keys atomically and maps the result back.
@@ -1048,21 +990,6 @@ __global__ void __launch_bounds__(KT) k_fwd_sum(LayoutView L, TokenView T, StepV
 // live in the forward pass are never visited: their posteriors are zero and
 // no backward value of theirs is read.
 // ======================================================================
-__device__ __forceinline__ void add_count(const CountView& C, int32_t id, float g) {
-  if (C.batched) {
-    atomicAdd(C.cnt64 + id, (double)g);
-  } else {
-    // compensated float32 summation (one string: one writer per arc and
-    // step; read through L2, as a persistent pass meets the same arc at
-    // later positions in other blocks)
-    const float s0 = __ldcg(C.cnt + id), cmp = __ldcg(C.comp + id);
-    const float y = __fsub_rn(g, cmp);
-    const float s1 = __fadd_rn(s0, y);
-    C.comp[id] = __fsub_rn(__fsub_rn(s1, s0), y);
-    C.cnt[id] = s1;
-  }
-}
-
 struct BwdCtx {
   int32_t b, n;
   float et;     // e_t (0 at the string's last position)
@@ -1753,6 +1680,13 @@ int debug_read(int64_t* violations, int32_t* code, int64_t* index, int64_t* boun
   FST_CUDA(cudaMemcpyFromSymbol(h, g_dbg, sizeof(h)));
   const unsigned long long z[4] = {0, 0, 0, 0};
   FST_CUDA(cudaMemcpyToSymbol(g_dbg, z, sizeof(z)));
+  unsigned long long g[4] = {0, 0, 0, 0};
+  const int rc = string_debug_read(g);
+  if (rc) return rc;
+  g[0] += h[0];
+  if (h[0])
+    for (int i = 1; i < 4; ++i) g[i] = h[i];
+  for (int i = 0; i < 4; ++i) h[i] = g[i];
   if (violations) *violations = (int64_t)h[0];
   if (code) *code = (int32_t)h[1];
   if (index) *index = (int64_t)h[2];

@@ -11,12 +11,12 @@ namespace fstgpu {
 // on symbol a are consecutive, found through a (symbol, state) hash.
 struct LayoutView {
   const int4* arcs;            // [P] {destination, theta bits, caller id, 0}
-  const ulonglong2* seg_hash;  // (symbol, state) -> len << 32 | first position
-  int64_t hash_mask;
+  const SegSlot* seg_hash;     // (symbol, state) -> arcs
+  int64_t buckets;
   int64_t P;                   // arc records (the bounds-checked build checks against it)
 };
 
-inline LayoutView view_of(const Layout& L) { return LayoutView{L.arcs, L.seg_hash, L.hash_mask, L.P}; }
+inline LayoutView view_of(const Layout& L) { return LayoutView{L.arcs, L.seg_hash, L.buckets, L.P}; }
 
 // The tokens of one input position t: slots slot0 .. slot0+n-1 of the
 // step list T.step_tok (tokens of a wave in step order).  Token p is
@@ -232,6 +232,94 @@ int launch_final_posteriors(const FrontierState& S, int32_t Bw, const CountView&
 int launch_fill_neg_inf(double* p, int64_t n, cudaStream_t s);
 // out[i] = (float)in[i], i < n.
 int launch_to_float(const double* in, int64_t n, float* out, cudaStream_t s);
+// The string kernels (strings.cu): a warp or block runs one string over all
+// of its positions.  Control words of a wave's run: error flags, pool top,
+// live entries and arcs; then, cleared before each pass, the strings started
+// and finished, a counter of progress, the open jobs, the heads and tails of
+// the two queues, the blocks that have begun, the light warps at work and the
+// open jobs of many chunks.
+// Each on a cache line of its own: they are polled.
+enum : int {
+  CTL_FLAGS = 0, CTL_TOP = 2, CTL_LIVE = 4, CTL_TAKE = 32, CTL_FINISHED = 64, CTL_PROGRESS = 96, CTL_OPEN = 128,
+  CTL_BIG = 129, CTL_HEAD = 160, CTL_TAIL = 224, CTL_BEGUN = 288, CTL_ALIVE = 289, CTL_WORDS = 320,
+  CTL_LINE = 32
+};
+// Where a string was left when it changed hands (t = 0: not started), and
+// what its backward pass has so far.
+struct StringPark {
+  int32_t t;
+  uint32_t ek;
+  double tE;
+};
+// A position that a heavy block shares out in chunks (strings.cu).
+struct alignas(128) StringJob {
+  unsigned long long word;  // phase number, chunks, next chunk
+  uint32_t done;            // chunks finished
+  uint32_t staged;          // destinations staged (forward, phase 0)
+  uint32_t tot, mk;         // arcs of the new entries; order key of the largest value
+  int32_t phase, owner;
+  int32_t t, a, an;         // position, its symbol, the next symbol (-1: none)
+  int32_t cnt, per;         // entries of t-1, entries a chunk
+  int32_t nb;               // entries of t
+  long long base, nbase;    // their pool ranges
+  double K;                 // backward: C_{t-1} + E_t - log Z - m_{t-1}
+  float shift, gw;          // m_{t-1} (forward) or e_t (backward); the string's weight
+  int32_t single, last;     // every destination has one arc; t is the last position
+  int32_t cur_big, next_big;  // backward: the values of t and t-1 are in the dense arrays
+  int32_t shared;           // its chunks are open to other blocks
+};
+// Device storage of the string kernels.
+struct StringWork {
+  int32_t Bw;
+  uint32_t* ctl;              // [string_ctl_words] control words, jobs, queues and places of the strings
+  uint32_t* dirty;            // [groups2] the block's dense accumulators were left unclean
+  double* kept;               // [Bw][string_kept_values()] backward values of a string that changes hands
+  unsigned long long* dense;  // [groups2][Q] (Viterbi) or [groups2][Q][2] accumulators, zero between runs
+  double* dval;               // [groups2][2][Q] backward values
+  int32_t* dstage;            // [groups2][Q] staged states
+  int2* fe;                   // arcs of the last position's entries (Viterbi): [groups2][Q], then the light warps'
+  int64_t fe_light;           // where the light warps' begin
+  int32_t groups2;            // heavy blocks that run strings
+  int32_t chunk;              // pool entries a group reserves at a time (0: each range by itself)
+};
+// What a launch sees of it.
+struct StringQueue {
+  int32_t strings, heavy_blocks, owners;
+  uint32_t* ctl;
+  StringJob* jobs;
+  uint32_t* ring;
+  uint32_t ring_mask;
+  StringPark* park;
+  uint32_t* dirty;
+  double* kept;
+  unsigned long long* dense;
+  double* dval;
+  int32_t* dstage;
+  int2* fe;
+  int64_t fe_light;
+  int32_t chunk;
+};
+int64_t string_ctl_words(int32_t Bw, int32_t groups2);
+int64_t string_light_entries(int num_sms);
+int32_t string_kept_values();
+// The forward recursion of every string: S.flags and S.pool_top point into
+// W.ctl, which is cleared first.  Fills the pool and the per-token ranges
+// (Viterbi: each entry's best arc and predecessor entry, -2 where it has to
+// be looked up; forward: the arcs on the next symbol and the step maxima).
+int launch_string_forward(bool viterbi, const LayoutView& L, const int32_t* sym, const FrontierState& S,
+                          const StringWork& W, int num_sms, cudaStream_t s);
+// The backward recursion and the posteriors, after launch_string_forward
+// and launch_fb_final.
+int launch_string_backward(const LayoutView& L, const int32_t* sym, const FrontierState& S, const CountView& C,
+                           const StringWork& W, int num_sms, cudaStream_t s);
+// The best path of each string after launch_string_forward and
+// launch_vit_final.
+int launch_string_trace(const FrontierState& S, const int32_t* olabel_by_id, int32_t Bw, const int32_t* jfinal,
+                        int32_t* paths, int32_t* olabels, cudaStream_t s);
+#ifdef FST_DEBUG
+int string_debug_read(unsigned long long* h);  // as debug_read, of strings.cu
+#endif
+
 // Bounds-checked build (compiled with FST_DEBUG): the kernels check every
 // computed index into the staging buffers, the live pool, the dense
 // accumulators and the arc records against its buffer's size, count the

@@ -70,14 +70,13 @@ struct Wave {
   std::vector<int32_t> step0;  // [tmax + 2]: tokens of position t are step_tok[step0[t] .. step0[t+1])
   int32_t* d_step0 = nullptr;  // the same on the device (persistent passes)
   int32_t grid_est = 1;        // blocks of the busiest position (about 64 live states per token)
-  // the device arrays above point into the plan's token arena
-  void release() {}
+  // the device arrays above point into the plan's arenas
 };
 
-// Host copies of a wave's token tables, uploaded into the token arena.
+// Host copies of a wave's step lists, uploaded into the step arena.
 struct HostWave {
-  std::vector<int32_t> sym, tb, step_tok, bn;
-  std::vector<int64_t> stf, boff;
+  std::vector<int32_t> tb, step_tok;
+  std::vector<int64_t> stf;
 };
 
 }  // namespace
@@ -99,11 +98,16 @@ int64_t dense_bytes_per_string(const fst_s* f, bool fb, bool vit) {
   return (int64_t)f->Q * ((fb ? 48 : 16) + (vit ? 8 : 0));
 }
 
-// The device storage of a plan (everything but the per-wave token tables).
-#define PLAN_STORAGE(X)                                                                                          \
-  X(acc) X(beta) X(vmap) X(stage) X(stage_b) X(scnt) X(pool_q) X(pool_x) X(pool_n) X(pool_v) X(pool_base)          \
-  X(pool_cnt) X(slot_base) X(step_rng) X(pool_top) X(flags_d) X(mkey) X(ekey) X(csum) X(esum) X(jfinal) X(logz) \
-  X(cnt64) X(start64) X(final64) X(gbar) X(htab) X(bslot) X(tok_arena) X(dvec) X(dslot) X(dlist) X(dcnt)
+// The device storage of a plan: what every run needs, and what only the
+// per-position kernels need (allocated by plan_steps when a setting first
+// asks for them).
+#define PLAN_STORAGE(X)                                                                                       \
+  X(pool_q) X(pool_x) X(pool_n) X(pool_v) X(pool_base) X(pool_cnt) X(mkey) X(ekey) X(csum) X(jfinal) X(logz) \
+  X(cnt64) X(start64) X(final64) X(tok_arena) X(str_ctl) X(str_kept) X(str_dense_v)  \
+  X(str_dense_f) X(str_dval) X(str_stage) X(str_fe) X(str_dirty)
+#define PLAN_STEPS(X)                                                                                        \
+  X(acc) X(beta) X(vmap) X(stage) X(stage_b) X(scnt) X(slot_base) X(step_rng) X(pool_top) X(flags_d) X(esum) \
+  X(gbar) X(htab) X(bslot) X(step_arena) X(dvec) X(dslot) X(dlist) X(dcnt)
 
 struct fst_plan_s {
   fst_t* fst = nullptr;
@@ -125,9 +129,12 @@ struct fst_plan_s {
   int64_t table_limit = 0;             // fst_plan_limit_table: slots a run may use (0 = cap_hslots)
   unsigned long long* htab = nullptr;
   int32_t* bslot = nullptr;            // [pool_cap]
-  // every wave's token tables, one allocation (cap_tok bytes)
+  // every wave's symbols, string lengths and offsets, one allocation
+  // (cap_tok bytes); the step lists of the per-position kernels, another
   unsigned char* tok_arena = nullptr;
   int64_t cap_tok = 0;
+  unsigned char* step_arena = nullptr;
+  bool steps = false;  // the per-position kernels' storage is there (plan_steps)
   // direction switch of the forward pass (dense accumulators, launch
   // driver): dense value vectors and the dense tokens of each position
   double* dvec = nullptr;      // [DENSE_SLOTS][2][Q], -inf between uses
@@ -155,7 +162,18 @@ struct fst_plan_s {
   int64_t max_bw = 0, max_ntok = 0, max_stage = 0;
   // capacities of the device storage below: this plan's needs, or more when
   // the storage was taken over from an earlier plan of the same handle
-  int64_t cap_bw = 0, cap_nt = 0, cap_stage = 0, cap_len = 0, cap_B = 0, store_bytes = 0, cap_hslots = 0;
+  int64_t cap_bw = 0, cap_nt = 0, cap_stage = 0, cap_B = 0, store_bytes = 0, cap_hslots = 0;
+  // the string kernels (strings.cu): queues, and the last level's dense
+  // accumulators (str_groups2 blocks)
+  uint32_t *str_ctl = nullptr, *str_dirty = nullptr;
+  double* str_kept = nullptr;
+  unsigned long long *str_dense_v = nullptr, *str_dense_f = nullptr;
+  double* str_dval = nullptr;
+  int32_t* str_stage = nullptr;
+  int2* str_fe = nullptr;
+  int32_t str_groups2 = 0;
+  int64_t cap_fe = 0;
+  bool str_last = false;  // the last forward (or Viterbi) run took the string kernels
   bool forward_done = false;
   // optional per-launch CUDA events (fst_plan_profile)
   LaunchProfile prof;
@@ -187,9 +205,9 @@ struct fst_plan_s {
     for (cudaEvent_t e : part_event) cudaEventDestroy(e);
     if (run_event) cudaEventDestroy(run_event);
     if (borrowed_counts) cnt64 = start64 = final64 = nullptr;
-    for (Wave& w : waves) w.release();
 #define PLAN_FREE(x) dfree(x);
     PLAN_STORAGE(PLAN_FREE)
+    PLAN_STEPS(PLAN_FREE)
 #undef PLAN_FREE
   }
 };
@@ -222,30 +240,52 @@ int alloc_store(fst_plan_s* P, T** p, int64_t n) {
   return rc;
 }
 
-// Token tables of one wave, built on the host from the offsets and symbols.
+// Per string: the arcs its symbols' slices hold and the destinations they
+// can reach, its symbols copied into the plan; *bad is set where a symbol is
+// outside [0, m).  A warp per string.
+__global__ void k_string_stats(const int32_t* __restrict__ ids, const int64_t* __restrict__ off, int32_t B, int32_t m,
+                               const int64_t* __restrict__ sym_arc, const int64_t* __restrict__ sym_seg,
+                               int32_t* __restrict__ sym, int64_t* __restrict__ arcs, int64_t* __restrict__ dsts,
+                               int64_t* __restrict__ bad) {
+  const int lane = threadIdx.x & 31;
+  const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (b >= B) return;
+  const int64_t lo = off[b], hi = off[b + 1];
+  long long na = 0, nd = 0;
+  bool wrong = false;
+  for (int64_t i = lo + lane; i < hi; i += 32) {
+    const int32_t a = ids[i];
+    sym[i] = a;
+    if (a < 0 || a >= m) {
+      wrong = true;
+    } else {
+      na += sym_arc[a + 1] - sym_arc[a];
+      nd += sym_seg[a + 1] - sym_seg[a];
+    }
+  }
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) {
+    na += __shfl_xor_sync(0xffffffffu, na, d);
+    nd += __shfl_xor_sync(0xffffffffu, nd, d);
+  }
+  if (lane == 0) {
+    arcs[b] = na;
+    dsts[b] = nd;
+  }
+  if (wrong) *bad = 1;
+}
+
+// Step lists of one wave for the per-position kernels, built on the host.
 // Tokens of a string are consecutive (token p = position t of string b is
 // p = off_b + t - 1); the tokens of position t are listed string by string.
-int build_wave(fst_plan_s* P, Wave& W, const int64_t* h_off, const int32_t* hid, HostWave& H) {
+void build_steps(fst_plan_s* P, Wave& W, const std::vector<int32_t>& sym, const std::vector<int32_t>& bn,
+                 const std::vector<int64_t>& boff, HostWave& H) {
   fst_s* f = P->fst;
-  W.Bw = W.b1 - W.b0;
-  W.tok0 = h_off[W.b0];
-  W.ntok = h_off[W.b1] - W.tok0;
-  std::vector<int64_t> boff(W.Bw);
-  std::vector<int32_t> bn(W.Bw);
-  W.tmax = 0;
-  for (int32_t b = 0; b < W.Bw; ++b) {
-    boff[b] = h_off[W.b0 + b] - W.tok0;
-    bn[b] = (int32_t)(h_off[W.b0 + b + 1] - h_off[W.b0 + b]);
-    W.tmax = std::max(W.tmax, bn[b]);
-  }
-  std::vector<int32_t> sym(W.ntok), tb(W.ntok), step_tok;
+  std::vector<int32_t> tb(W.ntok), step_tok;
   std::vector<int64_t> stf(W.ntok);
   step_tok.reserve(W.ntok);
   for (int32_t b = 0; b < W.Bw; ++b)
-    for (int32_t i = 0; i < bn[b]; ++i) {
-      sym[boff[b] + i] = hid[W.tok0 + boff[b] + i];
-      tb[boff[b] + i] = b;
-    }
+    for (int32_t i = 0; i < bn[b]; ++i) tb[boff[b] + i] = b;
   // strings sorted by length (descending) so that the tokens of position t
   // are a prefix of that order: string b has a token at t iff n_b >= t
   std::vector<int32_t> order(W.Bw);
@@ -253,7 +293,6 @@ int build_wave(fst_plan_s* P, Wave& W, const int64_t* h_off, const int32_t* hid,
   std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return bn[x] > bn[y]; });
   W.step0.assign(W.tmax + 2, 0);
   W.stage = 0;
-  W.pool_bound = 0;
   int32_t live = W.Bw;
   for (int32_t t = 1; t <= W.tmax; ++t) {
     while (live > 0 && bn[order[live - 1]] < t) --live;
@@ -265,9 +304,7 @@ int build_wave(fst_plan_s* P, Wave& W, const int64_t* h_off, const int32_t* hid,
       step_tok.push_back((int32_t)p);
       stf[p] = accf;
       // distinct destinations of the symbol's arcs: the most a token can stage
-      const int64_t D = f->fwd.h_sym_seg[a + 1] - f->fwd.h_sym_seg[a];
-      accf += D;
-      W.pool_bound += D;
+      accf += f->fwd.h_sym_seg[a + 1] - f->fwd.h_sym_seg[a];
     }
     W.stage = std::max(W.stage, accf);
   }
@@ -275,13 +312,9 @@ int build_wave(fst_plan_s* P, Wave& W, const int64_t* h_off, const int32_t* hid,
   int64_t busiest = 1;
   for (int32_t t = 1; t <= W.tmax; ++t) busiest = std::max<int64_t>(busiest, W.step0[t + 1] - W.step0[t]);
   W.grid_est = (int32_t)std::min<int64_t>((int64_t)f->num_sms * 8, (busiest * 64 + 255) / 256);
-  H.sym = std::move(sym);
   H.tb = std::move(tb);
   H.step_tok = std::move(step_tok);
-  H.bn = std::move(bn);
   H.stf = std::move(stf);
-  H.boff = std::move(boff);
-  return FST_OK;
 }
 
 // The suggested threshold of the direction switch (fst_plan_set_pull(-1)):
@@ -290,46 +323,136 @@ int build_wave(fst_plan_s* P, Wave& W, const int64_t* h_off, const int32_t* hid,
 // win.
 int32_t pull_default(const fst_s* f) { return std::max<int32_t>(2048, f->Q / 2); }
 
-// The waves' token tables in the plan's token arena (grown when the one
-// taken over from a donor is too small), uploaded with one copy.
-int upload_tokens(fst_plan_s* P, std::vector<HostWave>& hw, cudaStream_t s) {
+// Words of the compact accumulator tables of `slots` slots each.
+int64_t htab_words(const fst_plan_s* P, int64_t slots) {
+  return slots * (2 * 2 * (int64_t)P->acc_stride + (P->want_fb ? 3 * 2 : 0));
+}
+
+// The waves' step lists in the plan's step arena, uploaded with one copy.
+int upload_steps(fst_plan_s* P, std::vector<HostWave>& hw, cudaStream_t s) {
   auto up16 = [](int64_t b) { return (b + 15) & ~(int64_t)15; };
   int64_t total = 0;
-  for (size_t i = 0; i < P->waves.size(); ++i) {
-    const Wave& W = P->waves[i];
-    total += up16(8 * (int64_t)W.Bw) + up16(4 * (int64_t)W.Bw) + up16(4 * W.ntok) * 3 + up16(8 * W.ntok) +
-             up16(4 * ((int64_t)W.tmax + 2));
-  }
+  for (const Wave& W : P->waves)
+    total += up16(4 * W.ntok) * 2 + up16(8 * W.ntok) + up16(4 * ((int64_t)W.tmax + 2));
   total = std::max<int64_t>(total, 16);
-  if (total > P->cap_tok) {
-    dfree(P->tok_arena);
-    P->cap_tok = 0;
-    int rc = dalloc(&P->tok_arena, total);
-    if (rc) return rc;
-    P->cap_tok = total;
-    P->store_bytes += total;
-    P->bytes += total;
-  }
+  int rc = dalloc(&P->step_arena, total);
+  if (rc) return rc;
+  P->bytes += total;
   std::vector<unsigned char> h((size_t)total);
   int64_t at = 0;
   auto put = [&](auto** dptr, const void* src, int64_t bytes) {
-    *dptr = (std::remove_pointer_t<decltype(dptr)>)(P->tok_arena + at);
+    *dptr = (std::remove_pointer_t<decltype(dptr)>)(P->step_arena + at);
     if (bytes > 0) memcpy(h.data() + at, src, (size_t)bytes);
     at += up16(bytes);
   };
   for (size_t i = 0; i < P->waves.size(); ++i) {
     Wave& W = P->waves[i];
     HostWave& H = hw[i];
-    put(&W.bw_off, H.boff.data(), 8 * (int64_t)W.Bw);
-    put(&W.bw_n, H.bn.data(), 4 * (int64_t)W.Bw);
-    put(&W.tok_sym, H.sym.data(), 4 * W.ntok);
     put(&W.tok_b, H.tb.data(), 4 * W.ntok);
     put(&W.step_tok, H.step_tok.data(), 4 * W.ntok);
     put(&W.stf, H.stf.data(), 8 * W.ntok);
     put(&W.d_step0, W.step0.data(), 4 * ((int64_t)W.tmax + 2));
   }
-  FST_CUDA(cudaMemcpyAsync(P->tok_arena, h.data(), (size_t)at, cudaMemcpyHostToDevice, s));
+  FST_CUDA(cudaMemcpyAsync(P->step_arena, h.data(), (size_t)at, cudaMemcpyHostToDevice, s));
   FST_CUDA(cudaStreamSynchronize(s));
+  return FST_OK;
+}
+
+// The step lists and accumulators of the per-position kernels, for the
+// settings that take them (the persistent driver, the direction switch, a
+// capped table).  Synchronises; nothing to do the second time.
+int plan_steps(fst_plan_s* P) {
+  if (P->steps) return FST_OK;
+  fst_s* f = P->fst;
+  const cudaStream_t s = 0;
+  int rc = FST_OK;
+  std::vector<HostWave> hw(P->waves.size());
+  P->max_stage = 0;
+  P->hslots = 0;
+  for (size_t i = 0; i < P->waves.size(); ++i) {
+    Wave& w = P->waves[i];
+    std::vector<int32_t> sym((size_t)std::max<int64_t>(w.ntok, 1)), bn((size_t)w.Bw);
+    std::vector<int64_t> boff((size_t)w.Bw);
+    FST_CUDA(cudaMemcpy(sym.data(), w.tok_sym, (size_t)w.ntok * 4, cudaMemcpyDeviceToHost));
+    FST_CUDA(cudaMemcpy(bn.data(), w.bw_n, (size_t)w.Bw * 4, cudaMemcpyDeviceToHost));
+    FST_CUDA(cudaMemcpy(boff.data(), w.bw_off, (size_t)w.Bw * 8, cudaMemcpyDeviceToHost));
+    build_steps(P, w, sym, bn, boff, hw[i]);
+    P->max_stage = std::max(P->max_stage, w.stage);
+    // compact accumulators at half load (a power of two; slots are named
+    // by int32 indices)
+    int64_t busiest = 0;
+    for (int32_t t = 1; t <= w.tmax; ++t) busiest = std::max<int64_t>(busiest, w.step0[t + 1] - w.step0[t]);
+    const int64_t live = std::min(w.stage, std::max(busiest * LIVE_PER_TOKEN, LIVE_FLOOR));
+    int64_t slots = 1024;
+    while (slots < 2 * live && slots < ((int64_t)1 << 30)) slots <<= 1;
+    P->hslots = std::max(P->hslots, slots);
+  }
+  P->cap_stage = P->max_stage;
+  P->cap_hslots = P->compact ? P->hslots : 0;
+  const int64_t na = P->compact ? 0 : P->max_bw * 2 * (int64_t)f->Q;
+  const int64_t nt = P->max_ntok;
+  const int64_t nh = P->compact ? htab_words(P, P->cap_hslots) : 0;
+  do {
+    if (P->compact) {
+      if ((rc = alloc_track(P, &P->htab, nh))) break;
+      if (P->want_fb && (rc = alloc_track(P, &P->bslot, P->pool_cap))) break;
+    } else {
+      if ((rc = alloc_track(P, &P->acc, na * P->acc_stride))) break;
+      if (P->want_fb && (rc = alloc_track(P, &P->beta, na))) break;
+      if (P->want_vit && (rc = alloc_track(P, &P->vmap, na))) break;
+      if (P->want_fb) {
+        // the direction switch's dense vectors, and the destination-ordered
+        // slice records it reads
+        if ((rc = alloc_track(P, &P->dvec, (int64_t)DENSE_SLOTS * 2 * f->Q)) ||
+            (rc = alloc_track(P, &P->dslot, nt)) ||
+            (rc = alloc_track(P, &P->dlist, ((int64_t)P->max_len + 2) * DENSE_SLOTS)) ||
+            (rc = alloc_track(P, &P->dcnt, (int64_t)P->max_len + 2)))
+          break;
+        if ((rc = launch_fill_neg_inf(P->dvec, (int64_t)DENSE_SLOTS * 2 * f->Q, s))) break;
+        if ((rc = slice_records_dst(f, s))) break;
+      }
+    }
+    if ((rc = alloc_track(P, &P->stage, P->max_stage)) || (rc = alloc_track(P, &P->stage_b, P->max_stage)) ||
+        (rc = alloc_track(P, &P->scnt, nt)) || (rc = alloc_track(P, &P->pool_top, 1)) ||
+        (rc = alloc_track(P, &P->slot_base, nt)) ||
+        (rc = alloc_track(P, &P->step_rng, 2 * ((int64_t)P->max_len + 2))) ||
+        (rc = alloc_track(P, &P->flags_d, 2)) || (rc = alloc_track(P, &P->esum, nt)) ||
+        (rc = alloc_track(P, &P->gbar, 2)))
+      break;
+    // the accumulators start at zero and every run leaves them so
+    cudaError_t ce = cudaSuccess;
+    if (P->acc) ce = cudaMemsetAsync(P->acc, 0, (size_t)std::max<int64_t>(na * P->acc_stride, 1) * 8, s);
+    if (ce == cudaSuccess && P->beta) ce = cudaMemsetAsync(P->beta, 0, (size_t)std::max<int64_t>(na, 1) * 8, s);
+    if (ce == cudaSuccess && P->htab) ce = cudaMemsetAsync(P->htab, 0, (size_t)std::max<int64_t>(nh, 1) * 8, s);
+    if (ce == cudaSuccess && P->dcnt)
+      ce = cudaMemsetAsync(P->dcnt, 0, (size_t)((int64_t)P->max_len + 2) * 4, s);
+    // position ranges start empty (a backward step reads those of a later
+    // position to empty its tables)
+    if (ce == cudaSuccess)
+      ce = cudaMemsetAsync(P->step_rng, 0, (size_t)(2 * ((int64_t)P->max_len + 2)) * 8, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(P->flags_d, 0, 8, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(P->pool_top, 0, 8, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(P->gbar, 0, 8, s);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+    if (ce != cudaSuccess) rc = cuda_fail(ce, "plan storage");
+  } while (0);
+  if (!rc) rc = upload_steps(P, hw, s);
+  if (rc) {
+#define PLAN_FREE(x) dfree(P->x);
+    PLAN_STEPS(PLAN_FREE)
+#undef PLAN_FREE
+    return rc;
+  }
+  P->steps = true;
+  return FST_OK;
+}
+// The same for a plan or each of its parts.
+int plan_steps_all(fst_plan_s* P) {
+  if (P->parts.empty()) return plan_steps(P);
+  for (fst_plan_s* q : P->parts) {
+    const int rc = plan_steps(q);
+    if (rc) return rc;
+  }
   return FST_OK;
 }
 
@@ -397,6 +520,38 @@ FrontierState wave_state(fst_plan_s* P, const Wave& W, const float* gweight) {
   S.gweight = gweight ? gweight + W.b0 : nullptr;
   S.bw_n = W.bw_n;
   S.bw_off = W.bw_off;
+  return S;
+}
+
+// Whether a run takes the string kernels: the launch driver without the
+// settings that only the per-position kernels have.
+bool string_path(const fst_plan_s* P) {
+  return P->driver == FST_DRIVER_LAUNCH && P->pull_min == 0 && P->table_limit == 0;
+}
+
+// Pool entries a group of the string kernels reserves at a time; a capped
+// pool is handed out range by range, so that the cap counts live entries.
+constexpr int32_t POOL_CHUNK = 64;
+
+StringWork string_work(fst_plan_s* P, const Wave& W, bool viterbi) {
+  StringWork K;
+  K.Bw = W.Bw;
+  K.ctl = P->str_ctl;
+  K.kept = P->str_kept;
+  K.fe_light = (int64_t)P->str_groups2 * P->fst->Q;
+  K.dirty = P->str_dirty;
+  K.dense = viterbi ? P->str_dense_v : P->str_dense_f;
+  K.dval = P->str_dval;
+  K.dstage = P->str_stage;
+  K.fe = P->str_fe;
+  K.groups2 = P->str_groups2;
+  K.chunk = P->pool_limit > 0 ? 0 : POOL_CHUNK;
+  return K;
+}
+FrontierState string_state(fst_plan_s* P, const Wave& W, const float* gweight) {
+  FrontierState S = wave_state(P, W, gweight);
+  S.flags = P->str_ctl + CTL_FLAGS;
+  S.pool_top = (int64_t*)(P->str_ctl + CTL_TOP);
   return S;
 }
 
@@ -472,10 +627,6 @@ void plan_ran(fst_plan_s* P, cudaStream_t s) {
 
 // State that starts every pass of a wave at zero.  A pass whose pool
 // overflowed left staged accumulators behind: they are cleared first.
-int64_t htab_words(const fst_plan_s* P, int64_t slots) {
-  return slots * (2 * 2 * (int64_t)P->acc_stride + (P->want_fb ? 3 * 2 : 0));
-}
-
 int wave_begin(fst_plan_s* P, const Wave& W, cudaStream_t s, bool fb) {
   int rc;
   if (P->compact) {
@@ -511,8 +662,18 @@ int run_viterbi_wave(fst_plan_s* P, const Wave& W, float* d_scores, int32_t* d_p
                      int32_t* d_status, cudaStream_t s) {
   fst_s* f = P->fst;
   int rc;
-  plan_learn(P, s);
   const LayoutView L = view_of(f->bwd);
+  P->str_last = string_path(P);
+  if (P->str_last) {
+    const FrontierState S = string_state(P, W, nullptr);
+    PROF(FST_PROF_VIT_STEP, launch_string_forward(true, L, W.tok_sym, S, string_work(P, W, true), f->num_sms, s));
+    PROF(FST_PROF_VIT_FINAL,
+         launch_vit_final(S, W.Bw, d_scores + W.b0, P->jfinal, d_status ? d_status + W.b0 : nullptr, s));
+    PROF(FST_PROF_BACKTRACE, launch_string_trace(S, f->olabel, W.Bw, P->jfinal, d_paths + W.tok0,
+                                                 d_olabels ? d_olabels + W.tok0 : nullptr, s));
+    return FST_OK;
+  }
+  plan_learn(P, s);
   const TokenView T = wave_tokens(W);
   const FrontierState S = wave_state(P, W, nullptr);
   if ((rc = wave_begin(P, W, s, false))) return rc;
@@ -540,8 +701,15 @@ PullView pull_view(const fst_plan_s* P) {
 int run_forward_wave(fst_plan_s* P, const Wave& W, cudaStream_t s, int32_t* d_status) {
   fst_s* f = P->fst;
   int rc;
-  plan_learn(P, s);
   const LayoutView L = view_of(f->bwd);
+  P->str_last = string_path(P);
+  if (P->str_last) {
+    const FrontierState S = string_state(P, W, nullptr);
+    PROF(FST_PROF_FWD_STEP, launch_string_forward(false, L, W.tok_sym, S, string_work(P, W, false), f->num_sms, s));
+    PROF(FST_PROF_FB_FINAL, launch_fb_final(S, W.Bw, P->logz + W.b0, d_status ? d_status + W.b0 : nullptr, s));
+    return FST_OK;
+  }
+  plan_learn(P, s);
   const TokenView T = wave_tokens(W);
   const FrontierState S = wave_state(P, W, nullptr);
   if ((rc = wave_begin(P, W, s, true))) return rc;
@@ -569,7 +737,9 @@ int run_backward_wave(fst_plan_s* P, const Wave& W, const float* d_weights, bool
   const TokenView T = wave_tokens(W);
   const FrontierState S = wave_state(P, W, d_weights);
   const CountView C{1, nullptr, nullptr, P->cnt64, states ? P->start64 : nullptr, states ? P->final64 : nullptr};
-  if (P->driver == FST_DRIVER_PERSISTENT) {
+  if (P->str_last) {
+    PROF(FST_PROF_BWD_STEP, launch_string_backward(L, W.tok_sym, S, C, string_work(P, W, false), f->num_sms, s));
+  } else if (P->driver == FST_DRIVER_PERSISTENT) {
     if (P->gbar) FST_CUDA(cudaMemsetAsync(P->gbar, 0, 4, s));  // arrivals; a timed-out forward pass leaves them
     if (W.tmax >= 1)
       PROF(FST_PROF_BWD_STEP,
@@ -618,10 +788,8 @@ inline cudaStream_t as_stream(void* p) { return (cudaStream_t)p; }
 
 }  // namespace
 
-static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_t B, int64_t mem_budget_bytes,
-                      int32_t flags, cudaStream_t s, fst_plan_s* donor, fst_plan_t** out);
-
-static bool part_threads_on();
+static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, const int64_t* h_off, int32_t B,
+                      int64_t mem_budget_bytes, int32_t flags, cudaStream_t s, fst_plan_s* donor, fst_plan_t** out);
 
 // The most parts a plan may have for its parts' step kernels to run chained
 // (FSTGPU_CHAIN_PARTS, default 1: parts run unchained, where one part's
@@ -639,8 +807,9 @@ static int32_t chain_parts_max() {
 // equal token counts, each an ordinary plan with its own stream; the count
 // accumulators (and the expected start and final states) are the parent's,
 // shared by the parts (their float64 atomics add up across parts).
-static int plan_create_parts(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_t B, int64_t budget,
-                             int32_t flags, cudaStream_t s, int32_t nparts, fst_plan_s* donor, fst_plan_t** out) {
+static int plan_create_parts(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, const int64_t* h_off, int32_t B,
+                             int64_t budget, int32_t flags, cudaStream_t s, int32_t nparts, fst_plan_s* donor,
+                             fst_plan_t** out) {
   // an earlier plan of as many parts lends each part's storage to the new
   // part of the same index, and its shared count accumulators
   std::unique_ptr<fst_plan_s> donor_owner(donor);
@@ -649,7 +818,7 @@ static int plan_create_parts(fst_t* f, const int32_t* hid, const int64_t* h_off,
   std::unique_ptr<fst_plan_s> P(new fst_plan_s());
   P->fst = f;
   P->B = B;
-  P->N = h_off[B];
+  P->N = h_off[B] - h_off[0];
   P->flags = flags;
   P->want_vit = !(flags & FST_PLAN_NO_VITERBI);
   P->want_fb = !(flags & FST_PLAN_NO_FB);
@@ -676,48 +845,16 @@ static int plan_create_parts(fst_t* f, const int32_t* hid, const int64_t* h_off,
       pd[i]->borrowed_counts = false;
     }
   }
-  // what the parts would otherwise each set up on the handle or read from
-  // the device: the destination-ordered slice records (dense accumulators
-  // with forward-backward) and the budget, taken once before they are built
-  if (P->want_fb && (flags & FST_PLAN_DENSE_ACC) && (rc = slice_records_dst(f, s))) {
-    for (fst_plan_s* q : pd) delete q;
-    return rc;
-  }
   const int64_t part_budget = budget > 0 ? std::max<int64_t>(budget / nparts, 1) : default_budget();
-  // the parts are built in parallel, one host thread each (the caller's
-  // building part 0; one after the other when FSTGPU_PART_THREADS=0):
-  // their host tables and uploads are independent
   std::vector<fst_plan_t*> sub((size_t)nparts, nullptr);
-  std::vector<int> prc((size_t)nparts, FST_OK);
-  std::vector<std::string> perr((size_t)nparts);
-  const int dev = f->device;
-  auto build_part = [&](int32_t i) {
-    if (i > 0 && cudaSetDevice(dev) != cudaSuccess) {
-      prc[i] = cuda_fail(cudaGetLastError(), "part thread");
-      perr[i] = fst_last_error();
-      delete pd[i];
-      return;
-    }
-    std::vector<int64_t> off((size_t)(bs[i + 1] - bs[i]) + 1);
-    for (int32_t b = bs[i]; b <= bs[i + 1]; ++b) off[b - bs[i]] = h_off[b] - h_off[bs[i]];
-    prc[i] = plan_build(f, hid + h_off[bs[i]], off.data(), bs[i + 1] - bs[i], part_budget,
-                        (flags & 0xff) | PLAN_PART, s, pd[i], &sub[i]);
-    if (prc[i]) perr[i] = fst_last_error();
-  };
-  {
-    std::vector<std::thread> th;
-    const bool threads = part_threads_on();
-    for (int32_t i = 1; i < nparts && threads; ++i) th.emplace_back(build_part, i);
-    build_part(0);
-    for (int32_t i = 1; i < nparts && !threads; ++i) build_part(i);
-    for (std::thread& t : th) t.join();
-  }
   rc = FST_OK;
   for (int32_t i = 0; i < nparts; ++i) {
-    if (prc[i] && !rc) {
-      rc = prc[i];
-      set_error("%s", perr[i].c_str());
+    if (rc) {
+      delete pd[i];
+      continue;
     }
+    rc = plan_build(f, d_ids, d_offsets + bs[i], h_off + bs[i], bs[i + 1] - bs[i], part_budget,
+                    (flags & 0xff) | PLAN_PART, s, pd[i], &sub[i]);
   }
   if (rc) {
     for (fst_plan_t* q : sub) delete q;
@@ -769,11 +906,11 @@ static int plan_create_parts(fst_t* f, const int32_t* hid, const int64_t* h_off,
   return FST_OK;
 }
 
-// fn(i) for every part i: from one host thread per part (the caller's
-// taking part 0), so that the parts' launches are issued in parallel, or
-// one after the other while the stream is being recorded into a graph, or
-// when FSTGPU_PART_THREADS=0 (a profiler that selects launches by a range
-// of the calling thread then sees them all).
+// fn(i) for every part i, one after the other; parts of per-position
+// launches (thousands of them) from one host thread per part (the caller's
+// taking part 0), unless the stream is being recorded into a graph or
+// FSTGPU_PART_THREADS=0 (a profiler that selects launches by a range of the
+// calling thread then sees them all).
 static bool part_threads_on() {
   static const bool on = [] {
     const char* e = std::getenv("FSTGPU_PART_THREADS");
@@ -785,7 +922,7 @@ template <class Fn>
 static int parts_each(fst_plan_s* P, cudaStream_t s, Fn fn) {
   const size_t n = P->parts.size();
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  bool threads = n > 1 && part_threads_on();
+  bool threads = n > 1 && !string_path(P->parts[0]) && part_threads_on();
   if (threads && (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) {
     (void)cudaGetLastError();
     threads = false;
@@ -845,30 +982,24 @@ static int plan_create(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets,
   const int64_t N = h_off[B];
   if (N >= ((int64_t)1 << 31)) { set_error("too many tokens"); return FST_ERR_UNSUPPORTED; }
   if (N > 0 && !d_ids) { set_error("ids is NULL"); return FST_ERR_INVALID_ARG; }
-  std::vector<int32_t> hid((size_t)std::max<int64_t>(N, 1));
-  if (N > 0) {
-    FST_CUDA(cudaMemcpyAsync(hid.data(), d_ids, (size_t)N * 4, cudaMemcpyDeviceToHost, s));
-    FST_CUDA(cudaStreamSynchronize(s));
-  }
-  for (int64_t i = 0; i < N; ++i)
-    if (hid[i] < 0 || hid[i] >= f->m) {
-      set_error("a symbol id is outside [0, %d)", f->m);
-      return FST_ERR_INVALID_ARG;
-    }
-  return plan_build(f, hid.data(), h_off.data(), B, mem_budget_bytes, flags, s, donor_owner.release(), out);
+  return plan_build(f, d_ids, d_offsets, h_off.data(), B, mem_budget_bytes, flags, s, donor_owner.release(), out);
 }
 
-// Plan building from host arrays (symbols checked; h_off[0] = 0).
-// `donor` (owned: always released here) is an earlier plan of the same
-// handle whose device storage is taken over when it is large enough, so
-// that repeated batch calls neither allocate nor clear it again.
-static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_t B, int64_t mem_budget_bytes,
-                      int32_t flags, cudaStream_t s, fst_plan_s* donor, fst_plan_t** out) {
+// Plan building: strings b of ids [h_off[b], h_off[b+1]), the offsets
+// checked (d_offsets the same on the device).  The symbols are copied into
+// the plan, checked and summed up on the device.  `donor` (owned: always
+// released here) is an earlier plan of the same handle whose device storage
+// is taken over when it is large enough, so that repeated batch calls
+// neither allocate nor clear it again.
+static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, const int64_t* h_off, int32_t B,
+                      int64_t mem_budget_bytes, int32_t flags, cudaStream_t s, fst_plan_s* donor, fst_plan_t** out) {
   std::unique_ptr<fst_plan_s> donor_owner(donor);
   *out = nullptr;
-  const int64_t N = h_off[B];
+  const int64_t N = h_off[B] - h_off[0];
   const int32_t nparts = std::min<int32_t>((flags >> 8) & 0xff, std::max(B, 1));
-  if (nparts > 1) return plan_create_parts(f, hid, h_off, B, mem_budget_bytes, flags, s, nparts, donor_owner.release(), out);
+  if (nparts > 1)
+    return plan_create_parts(f, d_ids, d_offsets, h_off, B, mem_budget_bytes, flags, s, nparts, donor_owner.release(),
+                             out);
   if (donor && !donor->parts.empty()) donor_owner.reset();  // a parts plan lends nothing to a single plan
   fst_plan_s* P = new fst_plan_s();
   P->fst = f;
@@ -878,11 +1009,7 @@ static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_
   P->want_vit = !(flags & FST_PLAN_NO_VITERBI);
   P->want_fb = !(flags & FST_PLAN_NO_FB);
   int rc = FST_OK;
-  std::vector<HostWave> hw;
   do {
-    // relaxations of one pass (the paper's definition: every arc of every slice)
-    P->relax = 0;
-    for (int64_t i = 0; i < N; ++i) P->relax += f->h_sym_arc[hid[i] + 1] - f->h_sym_arc[hid[i]];
     // waves: consecutive strings whose memory fits the budget.  Default: a
     // quarter of the device memory free now, at most 32 GiB and at least
     // 256 MiB (the GPU may be shared; fst_set_batch_budget raises it)
@@ -903,6 +1030,9 @@ static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_
           Wave w;
           w.b0 = b0;
           w.b1 = b;
+          w.Bw = b - b0;
+          w.tok0 = h_off[b0] - h_off[0];
+          w.ntok = h_off[b] - h_off[b0];
           P->waves.push_back(w);
         }
         b0 = b;
@@ -910,17 +1040,68 @@ static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_
       }
       acc += need;
     }
+    // the strings' lengths and offsets inside their wave, the sums over
+    // their symbols, and the symbols
+    const int64_t words = 2 * ((int64_t)B * 3 + 1) + B + 1;  // 4-byte words before the symbols
+    const int64_t arena = (words + N + 4) * 4;
+    if (donor_owner && donor_owner->cap_tok >= arena) {
+      std::swap(P->tok_arena, donor_owner->tok_arena);
+      P->cap_tok = donor_owner->cap_tok;
+    } else {
+      if ((rc = dalloc(&P->tok_arena, arena))) break;
+      P->cap_tok = arena;
+    }
+    P->store_bytes += P->cap_tok;
+    P->bytes += P->cap_tok;
+    int64_t* a_off = (int64_t*)P->tok_arena;
+    int64_t* a_arcs = a_off + B;
+    int64_t* a_dsts = a_arcs + B;
+    int64_t* a_bad = a_dsts + B;
+    int32_t* a_n = (int32_t*)(a_bad + 1);
+    int32_t* a_sym = a_n + B + 1;
+    std::vector<unsigned char> head((size_t)(words * 4), 0);
+    int64_t* h_boff = (int64_t*)head.data();
+    int32_t* h_n = (int32_t*)(head.data() + ((unsigned char*)a_n - P->tok_arena));
+    for (Wave& w : P->waves) {
+      for (int32_t b = w.b0; b < w.b1; ++b) {
+        h_boff[b] = h_off[b] - h_off[w.b0];
+        h_n[b] = (int32_t)(h_off[b + 1] - h_off[b]);
+        w.tmax = std::max(w.tmax, h_n[b]);
+      }
+      w.bw_off = a_off + w.b0;
+      w.bw_n = a_n + w.b0;
+      w.tok_sym = a_sym + w.tok0;
+    }
+    std::vector<int64_t> sums((size_t)2 * B + 1, 0);
+    cudaError_t e = cudaMemcpyAsync(P->tok_arena, head.data(), head.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && B > 0) {
+      k_string_stats<<<(unsigned)((B + 7) / 8), 256, 0, s>>>(d_ids, d_offsets, B, f->m, f->sym_arc, f->fwd.sym_seg,
+                                                            a_sym - h_off[0], a_arcs, a_dsts, a_bad);
+      e = cudaGetLastError();
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(sums.data(), a_arcs, sums.size() * 8, cudaMemcpyDeviceToHost, s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+      rc = cuda_fail(e, "plan tokens");
+      break;
+    }
+    if (sums[2 * (size_t)B]) {
+      set_error("a symbol id is outside [0, %d)", f->m);
+      rc = FST_ERR_INVALID_ARG;
+      break;
+    }
+    // relaxations of one pass (the paper's definition: every arc of every slice)
+    for (int32_t b = 0; b < B; ++b) P->relax += sums[b];
     if ((flags & FST_PLAN_SINGLE_WAVE) && P->waves.size() > 1) {
       set_error("the batch needs %d waves under a budget of %lld bytes", (int)P->waves.size(), (long long)budget);
       rc = FST_ERR_OOM;
       break;
     }
     for (Wave& w : P->waves) {
-      hw.emplace_back();
-      if ((rc = build_wave(P, w, h_off, hid, hw.back()))) break;
+      for (int32_t b = w.b0; b < w.b1; ++b) w.pool_bound += sums[(size_t)B + b];
       P->max_bw = std::max<int64_t>(P->max_bw, w.Bw);
       P->max_ntok = std::max<int64_t>(P->max_ntok, w.ntok);
-      P->max_stage = std::max(P->max_stage, w.stage);
       P->max_len = std::max(P->max_len, w.tmax);
       // live pool: its exact bound when that is small, else the larger of
       // POOL_PER_TOKEN entries per token and a quarter of the budget (at
@@ -930,100 +1111,69 @@ static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_
                                     std::min(std::max(budget / 4, (int64_t)256 << 20), (int64_t)4 << 30) / ebytes);
       // pool entries are named by int32 indices
       P->pool_cap = std::max(P->pool_cap, std::min(std::min(w.pool_bound, want), (int64_t)INT32_MAX));
-      // compact accumulators at half load (a power of two; slots are named
-      // by int32 indices)
-      int64_t busiest = 0;
-      for (int32_t t = 1; t <= w.tmax; ++t) busiest = std::max<int64_t>(busiest, w.step0[t + 1] - w.step0[t]);
-      const int64_t live = std::min(w.stage, std::max(busiest * LIVE_PER_TOKEN, LIVE_FLOOR));
-      int64_t slots = 1024;
-      while (slots < 2 * live && slots < ((int64_t)1 << 30)) slots <<= 1;
-      P->hslots = std::max(P->hslots, slots);
     }
-    if (rc) break;
+    // what the string kernels' chunks may leave unused
+    P->pool_cap = std::min<int64_t>(P->pool_cap + P->pool_cap / 3 + 3 * POOL_CHUNK * std::min<int64_t>(P->max_bw, 64 * f->num_sms),
+                                    (int64_t)INT32_MAX);
     P->acc_stride = P->want_fb ? 2 : 1;
+    // the last level's blocks of the string kernels: at most two per SM, one
+    // per string, within a quarter of the budget
+    const int64_t per_group = (int64_t)f->Q * ((P->want_vit ? 16 : 0) + (P->want_fb ? 32 : 0) + 4);
+    const int32_t groups2 = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>(std::min<int64_t>(P->max_bw, 2 * f->num_sms), budget / 4 / per_group));
+    const int64_t fe = P->want_vit ? (int64_t)groups2 * f->Q + string_light_entries(f->num_sms) : 0;
     fst_plan_s* d = donor_owner.get();
-    if (d && d->fst == f && d->want_fb == P->want_fb && d->want_vit == P->want_vit && d->compact == P->compact &&
-        (!P->compact || d->cap_hslots >= P->hslots) && (P->compact || d->cap_bw >= P->max_bw) &&
-        d->cap_nt >= P->max_ntok && d->cap_stage >= P->max_stage && d->pool_cap >= P->pool_cap &&
-        d->cap_len >= P->max_len && d->cap_B >= B) {
-      // take the donor's storage: its accumulators are zero (or, after an
-      // overflow, cleared by the next pass through the moved error flag)
+    if (d && d->fst == f && d->want_fb == P->want_fb && d->want_vit == P->want_vit && d->cap_bw >= P->max_bw &&
+        d->cap_nt >= P->max_ntok && d->pool_cap >= P->pool_cap && d->cap_B >= B && d->cap_fe >= fe &&
+        d->str_groups2 >= groups2) {
+      // take the donor's storage: its accumulators are zero
+      unsigned char* own = P->tok_arena;
 #define PLAN_MOVE(x) P->x = d->x; d->x = nullptr;
       PLAN_STORAGE(PLAN_MOVE)
 #undef PLAN_MOVE
+      dfree(P->tok_arena);  // the donor's, when it was too small
+      P->tok_arena = own;
       P->cap_bw = d->cap_bw;
       P->cap_nt = d->cap_nt;
-      P->cap_stage = d->cap_stage;
-      P->cap_len = d->cap_len;
       P->cap_B = d->cap_B;
-      P->cap_hslots = d->cap_hslots;
-      P->cap_tok = d->cap_tok;
+      P->str_groups2 = d->str_groups2;
+      P->cap_fe = d->cap_fe;
       P->pool_cap = d->pool_cap;
-      P->store_bytes = d->store_bytes;
-      P->bytes += d->store_bytes;
+      P->store_bytes += d->store_bytes - d->cap_tok;
+      P->bytes += d->store_bytes - d->cap_tok;
       break;
     }
     donor_owner.reset();  // too small (or none): release its memory first
     P->cap_bw = P->max_bw;
     P->cap_nt = P->max_ntok;
-    P->cap_stage = P->max_stage;
-    P->cap_len = P->max_len;
     P->cap_B = B;
-    P->cap_hslots = P->compact ? P->hslots : 0;
-    const int64_t na = P->compact ? 0 : P->max_bw * 2 * (int64_t)f->Q;
+    P->str_groups2 = groups2;
+    P->cap_fe = fe;
     const int64_t nt = P->max_ntok;
-    const int64_t nh = P->compact ? htab_words(P, P->cap_hslots) : 0;
-    if (P->compact) {
-      if ((rc = alloc_store(P, &P->htab, nh))) break;
-      if (P->want_fb && (rc = alloc_store(P, &P->bslot, P->pool_cap))) break;
-    } else {
-      if ((rc = alloc_store(P, &P->acc, na * P->acc_stride))) break;
-      if (P->want_fb && (rc = alloc_store(P, &P->beta, na))) break;
-      if (P->want_vit && (rc = alloc_store(P, &P->vmap, na))) break;
-      if (P->want_fb) {
-        // the direction switch's dense vectors, and the destination-ordered
-        // slice records it reads
-        if ((rc = alloc_store(P, &P->dvec, (int64_t)DENSE_SLOTS * 2 * f->Q)) ||
-            (rc = alloc_store(P, &P->dslot, nt)) ||
-            (rc = alloc_store(P, &P->dlist, ((int64_t)P->max_len + 2) * DENSE_SLOTS)) ||
-            (rc = alloc_store(P, &P->dcnt, (int64_t)P->max_len + 2)))
-          break;
-        if ((rc = launch_fill_neg_inf(P->dvec, (int64_t)DENSE_SLOTS * 2 * f->Q, s))) break;
-        // (a part's parent has set them up before building its parts)
-        if (!(flags & PLAN_PART) && (rc = slice_records_dst(f, s))) break;
-      }
-    }
-    // forward: arcs on the next symbol; Viterbi with dense accumulators:
-    // the predecessor entry
-    if ((P->want_fb || !P->compact) && (rc = alloc_store(P, &P->pool_n, P->pool_cap))) break;
-    if ((rc = alloc_store(P, &P->stage, P->max_stage)) || (rc = alloc_store(P, &P->stage_b, P->max_stage)) ||
-        (rc = alloc_store(P, &P->scnt, nt)) || (rc = alloc_store(P, &P->pool_q, P->pool_cap)) ||
-        (rc = alloc_store(P, &P->pool_x, P->pool_cap)) || (rc = alloc_store(P, &P->pool_v, P->pool_cap)) ||
+    const int64_t gq = (int64_t)groups2 * f->Q;
+    if ((rc = alloc_store(P, &P->str_ctl, string_ctl_words((int32_t)P->max_bw, groups2))) ||
+        (rc = alloc_store(P, &P->str_dirty, groups2)) ||
+        (rc = alloc_store(P, &P->str_kept, P->want_fb ? P->max_bw * string_kept_values() : 1)) ||
+        (rc = alloc_store(P, &P->str_stage, gq)))
+      break;
+    if (P->want_vit && ((rc = alloc_store(P, &P->str_dense_v, gq)) || (rc = alloc_store(P, &P->str_fe, fe)))) break;
+    if (P->want_fb && ((rc = alloc_store(P, &P->str_dense_f, 2 * gq)) || (rc = alloc_store(P, &P->str_dval, 2 * gq)))) break;
+    if ((rc = alloc_store(P, &P->pool_q, P->pool_cap)) || (rc = alloc_store(P, &P->pool_x, P->pool_cap)) ||
+        (rc = alloc_store(P, &P->pool_n, P->pool_cap)) || (rc = alloc_store(P, &P->pool_v, P->pool_cap)) ||
         (rc = alloc_store(P, &P->pool_base, nt)) || (rc = alloc_store(P, &P->pool_cnt, nt)) ||
-        (rc = alloc_store(P, &P->pool_top, 1)) || (rc = alloc_store(P, &P->slot_base, nt)) ||
-        (rc = alloc_store(P, &P->step_rng, 2 * ((int64_t)P->max_len + 2))) ||
-        (rc = alloc_store(P, &P->flags_d, 2)) || (rc = alloc_store(P, &P->mkey, nt)) ||
-        (rc = alloc_store(P, &P->ekey, nt)) || (rc = alloc_store(P, &P->csum, nt)) ||
-        (rc = alloc_store(P, &P->esum, nt)) || (rc = alloc_store(P, &P->jfinal, P->max_bw)) ||
-        (rc = alloc_store(P, &P->logz, B)) || (rc = alloc_store(P, &P->gbar, 2)))
+        (rc = alloc_store(P, &P->mkey, nt)) || (rc = alloc_store(P, &P->ekey, nt)) ||
+        (rc = alloc_store(P, &P->csum, nt)) || (rc = alloc_store(P, &P->jfinal, P->max_bw)) ||
+        (rc = alloc_store(P, &P->logz, B)))
       break;
     if (P->want_fb && !(flags & PLAN_PART) &&
         ((rc = alloc_store(P, &P->cnt64, f->A)) || (rc = alloc_store(P, &P->start64, f->Q)) ||
          (rc = alloc_store(P, &P->final64, f->Q))))
       break;
     // the accumulators start at zero and every run leaves them so
-    cudaError_t ce = cudaSuccess;
-    if (P->acc) ce = cudaMemsetAsync(P->acc, 0, (size_t)std::max<int64_t>(na * P->acc_stride, 1) * 8, s);
-    if (ce == cudaSuccess && P->beta) ce = cudaMemsetAsync(P->beta, 0, (size_t)std::max<int64_t>(na, 1) * 8, s);
-    if (ce == cudaSuccess && P->htab) ce = cudaMemsetAsync(P->htab, 0, (size_t)std::max<int64_t>(nh, 1) * 8, s);
-    if (ce == cudaSuccess && P->dcnt)
-      ce = cudaMemsetAsync(P->dcnt, 0, (size_t)((int64_t)P->max_len + 2) * 4, s);
-    // position ranges start empty (a backward step reads those of a later
-    // position to empty its tables)
-    if (ce == cudaSuccess)
-      ce = cudaMemsetAsync(P->step_rng, 0, (size_t)(2 * ((int64_t)P->max_len + 2)) * 8, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(P->flags_d, 0, 8, s);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(P->gbar, 0, 8, s);
+    cudaError_t ce = cudaMemsetAsync(P->str_dirty, 0, (size_t)groups2 * 4, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(P->str_ctl, 0, CTL_WORDS * 4, s);
+    if (ce == cudaSuccess && P->str_dense_v) ce = cudaMemsetAsync(P->str_dense_v, 0, (size_t)gq * 8, s);
+    if (ce == cudaSuccess && P->str_dense_f) ce = cudaMemsetAsync(P->str_dense_f, 0, (size_t)gq * 16, s);
     // per-token pool ranges start empty: a run that stops early leaves the
     // later positions' ranges as the previous run (or this clear) left them
     if (ce == cudaSuccess) ce = cudaMemsetAsync(P->pool_base, 0, (size_t)std::max<int64_t>(nt, 1) * 8, s);
@@ -1031,7 +1181,6 @@ static int plan_build(fst_t* f, const int32_t* hid, const int64_t* h_off, int32_
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess) rc = cuda_fail(ce, "plan storage");
   } while (0);
-  if (!rc) rc = upload_tokens(P, hw, s);
   if (rc) {
     delete P;
     return rc;
@@ -1081,6 +1230,11 @@ extern "C" int fst_plan_info(const fst_plan_t* P, int32_t* num_strings, int64_t*
       vl += 4;
       // overflow clear, forward pass, final, backward pass
       fl += w.tmax >= 1 ? 4 : 3;
+      continue;
+    }
+    if (string_path(P)) {
+      vl += 3;  // the string kernel, final, trace
+      fl += 3;  // forward, final, backward
       continue;
     }
     // overflow clear, first push, one step per position, final, backtrace
@@ -1256,42 +1410,15 @@ static void put_cached(fst_t* f, int kind, fst_plan_s* p) {
   delete old;
 }
 
-// Plan flags of a batch call (kind 0: Viterbi, 1: forward-backward): the
-// handle's setting (fst_set_batch_plan) or, by default, stream-parallel
-// parts by batch size (one Viterbi part per 32 strings, at most 2 and at
-// most 400 / the longest string; one forward-backward part per 8 strings,
-// at most 4 and at most 1,600 / the longest string) and dense accumulators
-// when they fit the budget in one wave.
-static int batch_flags(fst_t* f, int kind, const int64_t* d_offsets, int32_t B, cudaStream_t s, int32_t* flags) {
+// Plan flags of a batch call (kind 0: Viterbi, 1: forward-backward): by
+// default one part (the string kernels fill the GPU), and compact
+// accumulators, which lay down nothing until the per-position kernels are
+// asked for; the handle's setting (fst_set_batch_plan) overrides both.
+static int32_t batch_flags(const fst_t* f, int kind) {
   int32_t fl = kind == 0 ? FST_PLAN_NO_FB : FST_PLAN_NO_VITERBI;
-  std::vector<int64_t> h_off((size_t)B + 1, 0);
-  if (B > 0) {
-    FST_CUDA(cudaMemcpyAsync(h_off.data(), d_offsets, (size_t)(B + 1) * 8, cudaMemcpyDeviceToHost, s));
-    FST_CUDA(cudaStreamSynchronize(s));
-  }
-  int64_t tmax = 1;
-  for (int32_t b = 0; b < B; ++b) tmax = std::max(tmax, h_off[b + 1] - h_off[b]);
-  const int64_t N = h_off[B];
-  int32_t parts = f->batch_parts[kind];
-  if (parts <= 0) {
-    // by batch size, and few enough that a run stays near 400 (Viterbi) or
-    // 1,600 (forward-backward) position launches: the parts of a long
-    // string's batch multiply launches that the host issues one by one
-    const int64_t by_len = (kind == 0 ? 400 : 1600) / tmax;
-    parts = (int32_t)std::max<int64_t>(
-        1, std::min<int64_t>(kind == 0 ? std::min(2, B / 32) : std::min(4, B / 8), by_len));
-  }
-  if (parts > 1) fl |= FST_PLAN_PARTS(parts);
-  int32_t layout = f->batch_layout;
-  if (layout < 0) {
-    const int64_t budget = f->batch_budget > 0 ? f->batch_budget : default_budget();
-    const int64_t need = (dense_bytes_per_string(f, kind == 1, kind == 0) + 64) * (int64_t)B +
-                         (TOKEN_BYTES + POOL_PER_TOKEN * 20) * N;
-    layout = need <= budget ? 1 : 0;
-  }
-  if (layout == 1) fl |= FST_PLAN_DENSE_ACC;
-  *flags = fl;
-  return FST_OK;
+  if (f->batch_parts[kind] > 1) fl |= FST_PLAN_PARTS(f->batch_parts[kind]);
+  if (f->batch_layout == 1) fl |= FST_PLAN_DENSE_ACC;
+  return fl;
 }
 
 extern "C" int fst_set_batch_plan(fst_t* f, int32_t parts_viterbi, int32_t parts_fb, int32_t layout, int32_t graph) {
@@ -1349,10 +1476,7 @@ extern "C" int fst_viterbi_batch(fst_t* f, const int32_t* d_ids, const int64_t* 
   if (!f) { set_error("fst is NULL"); return FST_ERR_INVALID_ARG; }
   if (B < 0 || !d_offsets) { set_error("fst_viterbi_batch: bad arguments"); return FST_ERR_INVALID_ARG; }
   fst_plan_t* P = nullptr;
-  int32_t flags = 0;
-  int rc = batch_flags(f, 0, d_offsets, B, as_stream(stream), &flags);
-  if (rc) return rc;
-  rc = plan_create(f, d_ids, d_offsets, B, f->batch_budget, flags, stream, take_cached(f, 0), &P);
+  int rc = plan_create(f, d_ids, d_offsets, B, f->batch_budget, batch_flags(f, 0), stream, take_cached(f, 0), &P);
   if (rc) return rc;
   int64_t vl = 0;
   fst_plan_info(P, nullptr, nullptr, nullptr, nullptr, nullptr, &vl, nullptr, nullptr);
@@ -1371,10 +1495,7 @@ extern "C" int fst_forward_backward_batch(fst_t* f, const int32_t* d_ids, const 
   if (!f) { set_error("fst is NULL"); return FST_ERR_INVALID_ARG; }
   if (B < 0 || !d_offsets) { set_error("fst_forward_backward_batch: bad arguments"); return FST_ERR_INVALID_ARG; }
   fst_plan_t* P = nullptr;
-  int32_t flags = 0;
-  int rc = batch_flags(f, 1, d_offsets, B, as_stream(stream), &flags);
-  if (rc) return rc;
-  rc = plan_create(f, d_ids, d_offsets, B, f->batch_budget, flags, stream, take_cached(f, 1), &P);
+  int rc = plan_create(f, d_ids, d_offsets, B, f->batch_budget, batch_flags(f, 1), stream, take_cached(f, 1), &P);
   if (rc) return rc;
   int64_t fl = 0;
   fst_plan_info(P, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, &fl, nullptr);
@@ -1403,6 +1524,14 @@ extern "C" int fst_plan_live_work(fst_plan_t* P, int64_t* entries, int64_t* arcs
     return FST_OK;
   }
   cudaStream_t s = as_stream(stream);
+  if (P->str_last) {
+    unsigned long long live[2];
+    FST_CUDA(cudaMemcpyAsync(live, P->str_ctl + CTL_LIVE, sizeof(live), cudaMemcpyDeviceToHost, s));
+    FST_CUDA(cudaStreamSynchronize(s));
+    if (entries) *entries = (int64_t)live[0];
+    if (arcs) *arcs = P->want_fb ? (int64_t)live[1] : -1;
+    return FST_OK;
+  }
   int64_t top = 0;
   FST_CUDA(cudaMemcpyAsync(&top, P->pool_top, 8, cudaMemcpyDeviceToHost, s));
   FST_CUDA(cudaStreamSynchronize(s));
@@ -1440,13 +1569,28 @@ extern "C" int fst_plan_limit_pool(fst_plan_t* P, int64_t entries) {
 
 extern "C" int fst_plan_set_pull(fst_plan_t* P, int64_t min_live) {
   if (!P || min_live < -1) { set_error("fst_plan_set_pull: bad arguments"); return FST_ERR_INVALID_ARG; }
-  P->pull_min = min_live;
-  for (fst_plan_s* q : P->parts) q->pull_min = min_live;
+  // only dense accumulators have the direction switch
+  if (min_live != 0 && (P->flags & FST_PLAN_DENSE_ACC) && P->want_fb) {
+    const int rc = plan_steps_all(P);
+    if (rc) return rc;
+    P->pull_min = min_live;
+    for (fst_plan_s* q : P->parts) q->pull_min = min_live;
+  } else {
+    P->pull_min = 0;
+    for (fst_plan_s* q : P->parts) q->pull_min = 0;
+  }
   return FST_OK;
 }
 
 extern "C" int fst_plan_limit_table(fst_plan_t* P, int64_t slots) {
   if (!P || slots < 0) { set_error("fst_plan_limit_table: bad arguments"); return FST_ERR_INVALID_ARG; }
+  // only compact accumulators have tables to cap
+  if (slots > 0 && !(P->flags & FST_PLAN_DENSE_ACC)) {
+    const int rc = plan_steps_all(P);
+    if (rc) return rc;
+  } else {
+    slots = 0;
+  }
   P->table_limit = slots;
   for (fst_plan_s* q : P->parts) q->table_limit = slots;
   return FST_OK;
@@ -1454,6 +1598,10 @@ extern "C" int fst_plan_limit_table(fst_plan_t* P, int64_t slots) {
 
 extern "C" int fst_plan_table_slots(const fst_plan_t* P, int64_t* slots) {
   if (!P || !slots) { set_error("fst_plan_table_slots: bad arguments"); return FST_ERR_INVALID_ARG; }
+  if (!(P->flags & FST_PLAN_DENSE_ACC)) {
+    const int rc = plan_steps_all(const_cast<fst_plan_t*>(P));
+    if (rc) return rc;
+  }
   int64_t n = P->compact ? P->cap_hslots : 0;
   for (const fst_plan_s* q : P->parts) n = std::max(n, q->compact ? q->cap_hslots : 0);
   *slots = n;
@@ -1481,6 +1629,8 @@ extern "C" int fst_plan_set_driver(fst_plan_t* P, int32_t driver, int32_t grid_b
       set_error("a grid of %d blocks cannot be co-resident (at most %d)", grid_blocks, cap);
       return FST_ERR_UNSUPPORTED;
     }
+    const int rc = plan_steps_all(P);
+    if (rc) return rc;
   }
   P->driver = driver;
   P->persist_grid = grid_blocks;
@@ -1610,7 +1760,8 @@ extern "C" int fst_plan_autotune(fst_plan_t* P, void* stream, int32_t flags, int
           (rc = dalloc(&d_logz, P->B)) || (rc = dalloc(&d_counts, f->A)))
         break;
       std::vector<TuneConf> cands;
-      for (int32_t d : {16, 64, 256}) cands.push_back(TuneConf{FST_DRIVER_LAUNCH, 0, d, 0.0});
+      cands.push_back(TuneConf{FST_DRIVER_LAUNCH, 0, 64, 0.0});
+      if ((rc = plan_steps(P))) break;
       int dev = 0, coop = 0;
       if (cudaGetDevice(&dev) == cudaSuccess &&
           cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop) {
@@ -1649,6 +1800,7 @@ extern "C" int fst_plan_autotune(fst_plan_t* P, void* stream, int32_t flags, int
     g_tune[key] = best;
     tune_store_file(key, best);
   }
+  if (best.driver == FST_DRIVER_PERSISTENT && (rc = plan_steps(P))) return rc;
   P->driver = best.driver;
   P->persist_grid = best.grid;
   P->density = best.density;

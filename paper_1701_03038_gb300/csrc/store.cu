@@ -130,10 +130,12 @@ __global__ void k_seg_len(const int64_t* __restrict__ seg_first, int64_t nseg, i
 }
 
 // Insert every segment (symbol, state) -> (first position, length) into the
-// open-addressing table; one thread per segment.
+// bucketed table; one thread per segment.
 __global__ void k_hash_insert(const int64_t* __restrict__ sym_seg, int32_t m, const int32_t* __restrict__ seg_state,
                               const int32_t* __restrict__ seg_pos, const int32_t* __restrict__ seg_len,
-                              int64_t nseg, ulonglong2* __restrict__ tab, int64_t mask) {
+                              int64_t nseg, const int32_t* __restrict__ other, const float* __restrict__ theta,
+                              const int32_t* __restrict__ arc_id, SegSlot* __restrict__ tab, int64_t buckets,
+                              uint32_t* __restrict__ seg_slot) {
   const int64_t sg = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (sg >= nseg) return;
   int32_t lo = 0, hi = m;  // symbol of segment sg: last a with sym_seg[a] <= sg
@@ -142,15 +144,28 @@ __global__ void k_hash_insert(const int64_t* __restrict__ sym_seg, int32_t m, co
     if (sym_seg[mid] <= sg) lo = mid; else hi = mid;
   }
   const uint64_t k = seg_hash_key(lo, seg_state[sg]);
-  uint64_t h = seg_hash_slot(k, mask);
-  for (int64_t probe = 0; probe <= mask; ++probe) {
-    const unsigned long long old = atomicCAS(&tab[h].x, ~0ull, (unsigned long long)k);
-    if (old == ~0ull || old == k) {
-      tab[h].y = ((unsigned long long)(uint32_t)seg_len[sg] << 32) | (unsigned long long)(uint32_t)seg_pos[sg];
+  uint64_t b = seg_bucket(k, buckets);
+  for (int64_t probe = 0; probe < buckets; ++probe) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      SegSlot* t = tab + 2 * b + h;
+      if (atomicCAS(&t->key, ~0ull, (unsigned long long)k) != ~0ull) continue;
+      const int32_t i = seg_pos[sg];
+      // (another segment may mark the bucket spilled at the same time: the
+      // slot starts with a zero `at`)
+      atomicOr(&t->at, ((unsigned long long)(uint32_t)seg_len[sg] << 32) | (unsigned long long)(uint32_t)i);
+      t->arc = make_int4(other[i], __float_as_int(theta[i]), arc_id[i], 0);
+      seg_slot[sg] = (uint32_t)(2 * b + h);
       return;
     }
-    h = (h + 1) & (uint64_t)mask;
+    atomicOr(&tab[2 * b].at, SPILLED);
+    b = b + 1 < (uint64_t)buckets ? b + 1 : 0;
   }
+}
+
+__global__ void k_hash_clear(SegSlot* __restrict__ tab, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    *(ulonglong2*)&tab[i].key = make_ulonglong2(~0ull, 0ull);
 }
 
 __global__ void k_scatter_arcs(const uint32_t* __restrict__ perm, const int64_t* __restrict__ hd,
@@ -224,6 +239,13 @@ __global__ void k_set_weights(const int32_t* __restrict__ id, const float* __res
   if (i >= P) return;
   const int32_t k = id[i];
   theta[i] = k >= 0 ? th_by_id[k] : -INFINITY;
+}
+
+// The weight of every segment's first arc in its (symbol, state) slot.
+__global__ void k_set_first(const uint32_t* __restrict__ seg_slot, const int32_t* __restrict__ seg_pos,
+                            const float* __restrict__ theta, int64_t nseg, SegSlot* __restrict__ tab) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nseg) tab[seg_slot[i]].arc.y = __float_as_int(theta[seg_pos[i]]);
 }
 
 __global__ void k_set_weights64(const int32_t* __restrict__ id, const double* __restrict__ th_by_id, int64_t P,
@@ -353,7 +375,8 @@ int build_layout(fst_s* f, Layout& L, const int32_t* d_il, const int32_t* seg_st
 
 void free_layout(Layout& L) {
   dfree(L.other); dfree(L.theta); dfree(L.arc_id); dfree(L.theta64); dfree(L.win);
-  dfree(L.seg_state); dfree(L.seg_pos); dfree(L.seg_len); dfree(L.seg_hash); dfree(L.arcs); dfree(L.sym_win); dfree(L.sym_seg); dfree(L.sym_lseg);
+  dfree(L.seg_state); dfree(L.seg_pos); dfree(L.seg_len); dfree(L.seg_hash);
+  dfree(L.seg_slot); dfree(L.arcs); dfree(L.sym_win); dfree(L.sym_seg); dfree(L.sym_lseg);
   dfree(L.sym_lwin);
   free(L.h_sym_win); free(L.h_sym_seg); free(L.h_sym_lseg); free(L.h_sym_lwin);
   L.h_sym_win = L.h_sym_seg = L.h_sym_lseg = L.h_sym_lwin = nullptr;
@@ -381,14 +404,12 @@ int build_store(fst_s* f, const int32_t* d_src, const int32_t* d_dst, const int3
   // kernels find a live state's arcs on a symbol with about one probe
   {
     Layout& L = f->bwd;
-    int64_t size = 2;
-    while (size < 2 * std::max<int64_t>(L.nseg, 1)) size <<= 1;
-    if ((rc = dalloc(&L.seg_hash, size))) return rc;
-    L.hash_mask = size - 1;
-    FST_CUDA(cudaMemsetAsync(L.seg_hash, 0xff, (size_t)size * sizeof(ulonglong2), s));
+    L.buckets = std::min<int64_t>(1 + 3 * std::max<int64_t>(L.nseg, 1) / 2, ((int64_t)1 << 31) - 1);  // (32-bit slots)
+    if ((rc = dalloc(&L.seg_hash, 2 * L.buckets)) || (rc = dalloc(&L.seg_slot, L.nseg))) return rc;
+    k_hash_clear<<<(unsigned)std::min<int64_t>(blocks_for(2 * L.buckets), 152 * 16), TB, 0, s>>>(L.seg_hash, 2 * L.buckets);
     if (L.nseg > 0)
       k_hash_insert<<<blocks_for(L.nseg), TB, 0, s>>>(L.sym_seg, f->m, L.seg_state, L.seg_pos, L.seg_len, L.nseg,
-                                                      L.seg_hash, L.hash_mask);
+                                                      L.other, L.theta, L.arc_id, L.seg_hash, L.buckets, L.seg_slot);
     if ((rc = dalloc(&L.arcs, L.P))) return rc;
     if (L.P > 0) k_pack_arcs<<<blocks_for(L.P), TB, 0, s>>>(L.other, L.theta, L.arc_id, L.P, L.arcs);
     FST_CUDA(cudaStreamSynchronize(s));
@@ -401,6 +422,8 @@ int set_layout_weights(fst_s* f, const float* d_theta_by_id, cudaStream_t s) {
   for (Layout* L : Ls) {
     if (L->P > 0) k_set_weights<<<blocks_for(L->P), TB, 0, s>>>(L->arc_id, d_theta_by_id, L->P, L->theta);
     if (L->P > 0 && L->arcs) k_pack_arcs<<<blocks_for(L->P), TB, 0, s>>>(L->other, L->theta, L->arc_id, L->P, L->arcs);
+    if (L->nseg > 0 && L->seg_hash)
+      k_set_first<<<blocks_for(L->nseg), TB, 0, s>>>(L->seg_slot, L->seg_pos, L->theta, L->nseg, L->seg_hash);
   }
   FST_CUDA(cudaGetLastError());
   return FST_OK;
