@@ -41,6 +41,33 @@ int grid_for(int64_t work_warps, int block_threads, int num_sms, int max_blocks_
   if (need > cap) need = cap;
   return (int)(need < 1 ? 1 : need);
 }
+int Scratch::take(fst_s* h, size_t need) {
+  f = h;
+  {
+    std::lock_guard<std::mutex> lock(*f->batch_mu);
+    if (f->scratch_bytes >= need) {
+      p = (char*)f->scratch;
+      bytes = f->scratch_bytes;
+      f->scratch = nullptr;
+      f->scratch_bytes = 0;
+      return FST_OK;
+    }
+  }
+  const int rc = dalloc(&p, (int64_t)need);
+  if (!rc) bytes = need;
+  return rc;
+}
+Scratch::~Scratch() {
+  if (!p) return;
+  if (bytes <= SCRATCH_KEEP) {
+    std::lock_guard<std::mutex> lock(*f->batch_mu);
+    if (bytes > f->scratch_bytes) {
+      std::swap(*(void**)&p, f->scratch);
+      std::swap(bytes, f->scratch_bytes);
+    }
+  }
+  if (p) cudaFree(p);
+}
 int LaunchProfile::read(double* ms_by_kind, int64_t* launches_by_kind) {
   double ms[FST_PROF_KINDS] = {0};
   int64_t cnt[FST_PROF_KINDS] = {0};
@@ -453,6 +480,7 @@ extern "C" int fst_destroy(fst_t* f) {
   f->batch_mu = nullptr;
   delete f->pair_keys;
   f->pair_keys = nullptr;
+  dfree(f->scratch);
   dfree(f->slice_arcs);
   dfree(f->slice_arcs_src);
   dfree(f->slice_keys);

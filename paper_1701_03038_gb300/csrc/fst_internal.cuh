@@ -155,6 +155,10 @@ struct fst_s {
   // pair of each of its input symbols, ((uint64)ilabel << 32 | olabel), sorted
   std::vector<uint64_t>* pair_keys = nullptr;
   std::mutex* batch_mu = nullptr;
+  // working memory of the last lattice or product call, lent to the next
+  // (scratch_take, scratch_put)
+  void* scratch = nullptr;
+  size_t scratch_bytes = 0;
   // the paper's slice-wide relaxation (fst_viterbi_slice): per-arc records
   // {src, dst, id} in the destination-segmented layout's order, and the
   // packed keys of every position of the last string
@@ -291,6 +295,26 @@ int build_store(fst_s* f, const int32_t* d_src, const int32_t* d_dst, const int3
 void free_layout(Layout& L);
 int set_layout_weights(fst_s* f, const float* d_theta_by_id, cudaStream_t s);
 int set_layout_weights64(fst_s* f, const double* d_theta_by_id, cudaStream_t s);
+
+// Working memory of a call, from the handle (the last call's, when it is
+// large enough and no other call has it) or newly allocated; given back to
+// the handle, which keeps one block of at most SCRATCH_KEEP bytes.  get()
+// cuts 256-byte aligned pieces off it.
+constexpr size_t SCRATCH_KEEP = (size_t)512 << 20;
+struct Scratch {
+  fst_s* f = nullptr;
+  char* p = nullptr;
+  size_t bytes = 0, at = 0;
+  int take(fst_s* f, size_t need);
+  template <class T>
+  T* get(int64_t n) {
+    T* r = (T*)(p + at);
+    at += piece(n * (int64_t)sizeof(T));
+    return r;
+  }
+  static size_t piece(int64_t b) { return ((size_t)(b > 0 ? b : 1) + 255) & ~(size_t)255; }
+  ~Scratch();
+};
 
 int grid_for(int64_t work_warps, int block_threads, int num_sms, int max_blocks_per_sm);
 

@@ -10,16 +10,24 @@
 //
 // Matrices are dense Q x Q log-weights (-inf = no arc), one per symbol of
 // the string (parallel arcs combined: log-sum for the weight, max for the
-// best path).  A product entry is log sum_k exp(A[i][k] + B[k][j]) (an
-// online log-sum-exp over k, in float32) or max_k A[i][k] + B[k][j].  The
-// Viterbi score so obtained is the best path's weight with its float32
-// additions associated in tree order rather than left to right.
+// best path).  A product entry is log sum_k exp(A[i][k] + B[k][j]) or max_k
+// A[i][k] + B[k][j].  The sums are taken in the linear domain: with r_i the
+// largest entry of row i and c_j that of column j, exp(A - r) and exp(B - c)
+// are multiplied as matrices and r_i + c_j + log of the sum is the entry --
+// Q^2 exponentials a product where adding the logs one by one takes Q^3.  A
+// sum so small that terms may have underflowed (the largest A + B far below
+// r + c) is taken again in the log domain.  The Viterbi score is the best
+// path's weight with its float32 additions associated in tree order rather
+// than left to right.
+//
+// A level of the tree is one launch over its products, both semirings side by
+// side.  What bounds a call on 64 states and 1,000 symbols is the chain of
+// its ten levels; all products together are 0.5 GFLOP.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
-#include <map>
 #include <vector>
 
 #include "fst_internal.cuh"
@@ -29,15 +37,18 @@ using namespace fstgpu;
 namespace {
 
 constexpr int TB = 256;
-constexpr int TILE = 16;  // output tile TILE x TILE, one thread per entry
-constexpr int KC = 16;    // k chunk staged in shared memory
+constexpr int TILE = 64;   // output tile TILE x TILE, 4 x 4 entries a thread
+constexpr int KC = 64;     // k chunk staged in shared memory
 constexpr int PREFIX_MAX_STATES = 512;
+// sums below this may have lost terms to underflow (a lost term is below
+// 2^-126, and there are at most 512 of them)
+constexpr float TINY = 1e-30f;
 
 __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
 
 __global__ void k_fill(float* __restrict__ p, int64_t n, float v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = v;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    p[i] = v;
 }
 
 // log(e^a + e^b) with -inf handled.
@@ -48,77 +59,159 @@ __device__ __forceinline__ float log_add(float a, float b) {
   return hi + log1pf(expf(lo - hi));
 }
 
-// The dense matrices of one symbol: every arc of its slice adds into
-// M[src][dst] (log-sum: a compare-and-swap loop; max: order keys).
-__global__ void k_dense(const int4* __restrict__ arcs, const float* __restrict__ theta, int64_t i0, int64_t np,
-                        int32_t Q, float* __restrict__ msum, uint32_t* __restrict__ mmax) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= np) return;
-  const int4 a = __ldg(arcs + i0 + i);
-  if (a.z < 0) return;
-  const float th = __ldg(theta + i0 + i);
-  if (th == neg_inf()) return;
-  const int64_t e = (int64_t)a.x * Q + a.y;
-  atomicMax(mmax + e, fkey(th));
-  unsigned int* u = (unsigned int*)(msum + e);
-  unsigned int old = *u, seen;
-  do {
-    seen = old;
-    const float r = log_add(__uint_as_float(seen), th);
-    if (__float_as_uint(r) == seen) break;
-    old = atomicCAS(u, seen, __float_as_uint(r));
-  } while (old != seen);
+// The dense matrices of the symbols syms[blockIdx.y] (both filled with
+// -inf): every arc of the slice adds into M[src][dst] (log-sum: a
+// compare-and-swap loop; max: atomics on the float's bits, ordered as
+// integers for v >= 0 and reversed as unsigned ones below).
+__global__ void k_dense(const int4* __restrict__ arcs, const float* __restrict__ theta,
+                        const int64_t* __restrict__ sym_win, const int32_t* __restrict__ syms, int32_t Q,
+                        float* __restrict__ msum, float* __restrict__ mmax) {
+  const int32_t a = syms[blockIdx.y];
+  const int64_t i1 = sym_win[a + 1] * WIN;
+  for (int64_t i = sym_win[a] * WIN + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < i1;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int4 r = __ldg(arcs + i);
+    if (r.z < 0) continue;
+    const float th = __ldg(theta + i);
+    if (th == neg_inf()) continue;
+    const int64_t e = (int64_t)blockIdx.y * Q * Q + (int64_t)r.x * Q + r.y;
+    if (th >= 0.f) atomicMax((int*)(mmax + e), __float_as_int(th));
+    else atomicMin((unsigned int*)(mmax + e), __float_as_uint(th));
+    unsigned int* u = (unsigned int*)(msum + e);
+    unsigned int old = *u, seen;
+    do {
+      seen = old;
+      const float v = log_add(__uint_as_float(seen), th);
+      if (__float_as_uint(v) == seen) break;
+      old = atomicCAS(u, seen, __float_as_uint(v));
+    } while (old != seen);
+  }
 }
 
-// Order keys (0 = no arc) to float32 values.
-__global__ void k_keys_to_values(const uint32_t* __restrict__ k, int64_t n, float* __restrict__ v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = k[i] ? fkey_inv(k[i]) : neg_inf();
-}
-
-// out[p] = lhs[p] (x) rhs[p] for every pair p (blockIdx.y), one TILE x TILE
-// tile of the result per block (blockIdx.x); MAXPLUS picks the semiring.
-template <bool MAXPLUS>
-__global__ void __launch_bounds__(TILE * TILE) k_mul(const float* const* __restrict__ lhs,
-                                                     const float* const* __restrict__ rhs,
-                                                     float* __restrict__ out, int32_t Q) {
-  __shared__ float As[TILE][KC + 1];
+// One level of the tree: matrix 2p times matrix 2p + 1 of the level below,
+// for every p (blockIdx.y), one TILE x TILE tile of the result per block
+// (blockIdx.x), the log-sum and the max-plus products side by side
+// (blockIdx.z).  The matrices below are in[slot[k]] (slot null: in[k]); a
+// last matrix without a partner is carried up as it is.
+__global__ void __launch_bounds__(TB) k_mul(const float* __restrict__ in_sum, const float* __restrict__ in_max,
+                                            const int32_t* __restrict__ slot, int32_t count,
+                                            float* __restrict__ out_sum, float* __restrict__ out_max, int32_t Q) {
+  __shared__ float As[KC][TILE + 1];  // A transposed: [k][row]
   __shared__ float Bs[KC][TILE + 1];
+  __shared__ float rmax[TILE], cmax[TILE];
+  const bool maxplus = blockIdx.z != 0;
+  const int64_t QQ = (int64_t)Q * Q;
+  const float* in = maxplus ? in_max : in_sum;
+  float* out = (maxplus ? out_max : out_sum) + (int64_t)blockIdx.y * QQ;
+  const int32_t ka = 2 * blockIdx.y, kb = ka + 1;
+  const float* A = in + (slot ? slot[ka] : ka) * QQ;
   const int32_t tiles = (Q + TILE - 1) / TILE;
-  const int32_t ti = blockIdx.x / tiles, tj = blockIdx.x % tiles;
-  const int32_t r = threadIdx.x / TILE, c = threadIdx.x % TILE;
-  const int32_t i = ti * TILE + r, j = tj * TILE + c;
-  const float* A = lhs[blockIdx.y];
-  const float* B = rhs[blockIdx.y];
-  float m = neg_inf(), s = 0.f;  // log-sum: running max and sum of exp(v - m); max-plus: m
-  for (int32_t k0 = 0; k0 < Q; k0 += KC) {
-    // stage A[ti rows][k0..k0+KC) and B[k0..k0+KC)[tj cols]
-    {
-      const int32_t rr = threadIdx.x / KC, kk = threadIdx.x % KC;  // TILE * KC == blockDim
-      const int32_t ai = ti * TILE + rr, ak = k0 + kk;
-      As[rr][kk] = (ai < Q && ak < Q) ? A[(int64_t)ai * Q + ak] : neg_inf();
-      const int32_t bk = k0 + threadIdx.x / TILE, bj = tj * TILE + threadIdx.x % TILE;
-      Bs[threadIdx.x / TILE][threadIdx.x % TILE] = (bk < Q && bj < Q) ? B[(int64_t)bk * Q + bj] : neg_inf();
+  const int32_t i0 = ((int32_t)blockIdx.x / tiles) * TILE, j0 = ((int32_t)blockIdx.x % tiles) * TILE;
+  if (kb >= count) {
+    for (int32_t e = threadIdx.x; e < TILE * TILE; e += TB) {
+      const int32_t i = i0 + e / TILE, j = j0 + e % TILE;
+      if (i < Q && j < Q) out[(int64_t)i * Q + j] = A[(int64_t)i * Q + j];
     }
-    __syncthreads();
+    return;
+  }
+  const float* B = in + (slot ? slot[kb] : kb) * QQ;
+  // (the thread's 4 x 4 entries: rows ty + 16 u, columns tx + 16 v)
+  const int32_t tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto load = [&](int32_t k0) {
+    for (int32_t e = threadIdx.x; e < TILE * KC; e += TB) {
+      const int32_t i = i0 + e / KC, k = k0 + e % KC;
+      As[e % KC][e / KC] = (i < Q && k < Q) ? __ldg(A + (int64_t)i * Q + k) : neg_inf();
+      const int32_t kk = k0 + e / TILE, j = j0 + e % TILE;
+      Bs[e / TILE][e % TILE] = (kk < Q && j < Q) ? __ldg(B + (int64_t)kk * Q + j) : neg_inf();
+    }
+  };
+  if (!maxplus) {
+    // row and column maxima (0 stands for -inf: nothing to scale)
+    for (int32_t r = warp; r < TILE; r += TB / 32) {
+      float m = neg_inf(), c = neg_inf();
+      for (int32_t k = lane; k < Q; k += 32) {
+        if (i0 + r < Q) m = fmaxf(m, __ldg(A + (int64_t)(i0 + r) * Q + k));
+        if (j0 + r < Q) c = fmaxf(c, __ldg(B + (int64_t)k * Q + j0 + r));
+      }
 #pragma unroll
-    for (int kk = 0; kk < KC; ++kk) {
-      const float a = As[r][kk], b = Bs[kk][c];
-      if (a == neg_inf() || b == neg_inf()) continue;
-      const float v = a + b;
-      if (MAXPLUS) {
-        m = fmaxf(m, v);
-      } else if (v > m) {
-        s = s * expf(m - v) + 1.f;  // m == -inf gives s * 0 + 1
-        m = v;
-      } else {
-        s += expf(v - m);
+      for (int d = 16; d >= 1; d >>= 1) {
+        m = fmaxf(m, __shfl_xor_sync(FULL, m, d));
+        c = fmaxf(c, __shfl_xor_sync(FULL, c, d));
+      }
+      if (lane == 0) {
+        rmax[r] = m;
+        cmax[r] = c;
       }
     }
     __syncthreads();
   }
-  if (i < Q && j < Q)
-    out[((int64_t)blockIdx.y * Q + i) * Q + j] = MAXPLUS ? m : (m == neg_inf() ? m : m + logf(s));
+  float acc[4][4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[u][v] = maxplus ? neg_inf() : 0.f;
+  for (int32_t k0 = 0; k0 < Q; k0 += KC) {
+    if (k0 > 0) __syncthreads();
+    load(k0);
+    __syncthreads();
+    if (!maxplus) {
+      for (int32_t e = threadIdx.x; e < TILE * KC; e += TB) {
+        const int32_t k = e / TILE, x = e % TILE;
+        const float a = As[k][x], b = Bs[k][x];
+        As[k][x] = a == neg_inf() ? 0.f : expf(a - rmax[x]);
+        Bs[k][x] = b == neg_inf() ? 0.f : expf(b - cmax[x]);
+      }
+      __syncthreads();
+    }
+    const int32_t kn = min(KC, Q - k0);
+#pragma unroll 4
+    for (int32_t k = 0; k < kn; ++k) {
+      float a[4], b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[u] = As[k][ty + 16 * u];
+        b[u] = Bs[k][tx + 16 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = maxplus ? fmaxf(acc[u][v], a[u] + b[v]) : fmaf(a[u], b[v], acc[u][v]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int32_t i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
+      if (i >= Q || j >= Q) continue;
+      float r = acc[u][v];
+      if (!maxplus) {
+        const float rm = rmax[ty + 16 * u], cm = cmax[tx + 16 * v];
+        if (rm == neg_inf() || cm == neg_inf()) {
+          r = neg_inf();
+        } else if (r >= TINY) {
+          r = rm + cm + logf(r);
+        } else {
+          // terms may have underflowed: the log-sum one by one
+          float m = neg_inf(), s = 0.f;
+          for (int32_t k = 0; k < Q; ++k) {
+            const float x = __ldg(A + (int64_t)i * Q + k), y = __ldg(B + (int64_t)k * Q + j);
+            if (x == neg_inf() || y == neg_inf()) continue;
+            const float w = x + y;
+            if (w > m) {
+              s = s * expf(m - w) + 1.f;  // m == -inf gives s * 0 + 1
+              m = w;
+            } else {
+              s += expf(w - m);
+            }
+          }
+          r = m == neg_inf() ? m : m + logf(s);
+        }
+      }
+      out[(int64_t)i * Q + j] = r;
+    }
+  }
 }
 
 // log Z = LSE_{i,j}(theta_s[i] + P[i][j] + theta_f[j]) (float64) and the
@@ -182,19 +275,6 @@ __global__ void k_close(const float* __restrict__ P, const float* __restrict__ V
   }
 }
 
-struct DevMem {
-  std::vector<void*> p;
-  template <class T>
-  int get(T** out, int64_t n) {
-    int rc = dalloc(out, n);
-    if (!rc) p.push_back((void*)*out);
-    return rc;
-  }
-  ~DevMem() {
-    for (void* x : p) cudaFree(x);
-  }
-};
-
 struct DevGuard {
   int old = -1;
   explicit DevGuard(int dev) {
@@ -207,7 +287,11 @@ struct DevGuard {
   }
 };
 
-inline unsigned nb(int64_t n) { return (unsigned)std::max<int64_t>(1, (n + TB - 1) / TB); }
+// Window offsets of the symbols on the device, in the order slice_view
+// chose.
+inline const int64_t* slice_sym_win(const fst_s* f) {
+  return f->slice_order == FST_SLICE_BY_SOURCE ? f->bwd.sym_win : f->fwd.sym_win;
+}
 
 }  // namespace
 
@@ -228,96 +312,76 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
   DevGuard g(f->device);
   cudaStream_t s = 0;
   const int64_t Q = f->Q, QQ = Q * Q;
-  DevMem mem;
   int rc;
-  double* d_logz = nullptr;
-  float* d_best = nullptr;
-  if ((rc = mem.get(&d_logz, 1)) || (rc = mem.get(&d_best, 1))) return rc;
+  Scratch mem;
+  struct Out {
+    double logz;
+    float best, pad;
+  } h;
   if (n == 0) {
-    k_close<<<1, TB, 0, s>>>(nullptr, nullptr, f->Q, f->theta_s, f->theta_f, d_logz, d_best);
+    if ((rc = mem.take(f, Scratch::piece(sizeof(Out))))) return rc;
+    Out* d_out = mem.get<Out>(1);
+    k_close<<<1, TB, 0, s>>>(nullptr, nullptr, f->Q, f->theta_s, f->theta_f, &d_out->logz, &d_out->best);
+    FST_CUDA(cudaGetLastError());
+    FST_CUDA(cudaMemcpy(&h, d_out, sizeof(h), cudaMemcpyDeviceToHost));
   } else {
     SliceView sv;
     if ((rc = slice_view(f, s, &sv))) return rc;
-    // one dense pair (log-sum, max) per distinct symbol
-    std::map<int32_t, int32_t> slot;
-    for (int32_t i = 0; i < n; ++i) slot.emplace(ids[i], (int32_t)slot.size());
-    const int64_t U = (int64_t)slot.size(), half = (n + 1) / 2;
-    float *dsum = nullptr, *dmax = nullptr, *bufs[4] = {nullptr, nullptr, nullptr, nullptr};
-    uint32_t* keys = nullptr;
-    const float** d_ptr = nullptr;
-    if ((rc = mem.get(&dsum, U * QQ)) || (rc = mem.get(&dmax, U * QQ)) || (rc = mem.get(&keys, U * QQ)) ||
-        (rc = mem.get(&bufs[0], half * QQ)) || (rc = mem.get(&bufs[1], half * QQ)) ||
-        (rc = mem.get(&bufs[2], half * QQ)) || (rc = mem.get(&bufs[3], half * QQ)) ||
-        (rc = mem.get(&d_ptr, 2 * half)))
+    // one dense pair (log-sum, max) per distinct symbol: the matrix of each
+    // position, then the symbols, in one upload
+    std::vector<int32_t> syms(ids, ids + n), up((size_t)n);
+    std::sort(syms.begin(), syms.end());
+    syms.erase(std::unique(syms.begin(), syms.end()), syms.end());
+    int64_t longest = 1;
+    for (int32_t i = 0; i < n; ++i)
+      up[i] = (int32_t)(std::lower_bound(syms.begin(), syms.end(), ids[i]) - syms.begin());
+    for (const int32_t a : syms) longest = std::max(longest, (sv.h_sym_win[a + 1] - sv.h_sym_win[a]) * (int64_t)WIN);
+    const int64_t U = (int64_t)syms.size(), l1 = ((int64_t)n + 1) / 2, l2 = (l1 + 1) / 2;
+    up.insert(up.end(), syms.begin(), syms.end());
+    if ((rc = mem.take(f, Scratch::piece(sizeof(Out)) + Scratch::piece((int64_t)up.size() * 4) +
+                              Scratch::piece(2 * U * QQ * 4) + 2 * Scratch::piece(l1 * QQ * 4) +
+                              2 * Scratch::piece(l2 * QQ * 4))))
       return rc;
-    k_fill<<<nb(U * QQ), TB, 0, s>>>(dsum, U * QQ, -INFINITY);
-    FST_CUDA(cudaMemsetAsync(keys, 0, (size_t)(U * QQ) * 4, s));
-    for (const auto& kv : slot) {
-      const int32_t a = kv.first;
-      const int64_t i0 = sv.h_sym_win[a] * WIN, np = (sv.h_sym_win[a + 1] - sv.h_sym_win[a]) * WIN;
-      if (np)
-        k_dense<<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, f->Q, dsum + kv.second * QQ,
-                                      keys + kv.second * QQ);
-    }
-    k_keys_to_values<<<nb(U * QQ), TB, 0, s>>>(keys, U * QQ, dmax);
+    Out* d_out = mem.get<Out>(1);
+    int32_t* d_slot = mem.get<int32_t>((int64_t)up.size());
+    float* dsum = mem.get<float>(2 * U * QQ);
+    float* dmax = dsum + U * QQ;
+    // the levels' results take turns: the odd levels' in the larger buffers
+    float* buf_s[2] = {mem.get<float>(l1 * QQ), mem.get<float>(l2 * QQ)};
+    float* buf_m[2] = {mem.get<float>(l1 * QQ), mem.get<float>(l2 * QQ)};
+    FST_CUDA(cudaMemcpyAsync(d_slot, up.data(), up.size() * 4, cudaMemcpyHostToDevice, s));
+    k_fill<<<(unsigned)std::min<int64_t>((2 * U * QQ + TB - 1) / TB, 8 * (int64_t)f->num_sms), TB, 0, s>>>(
+        dsum, 2 * U * QQ, -INFINITY);
+    for (int64_t u0 = 0; u0 < U; u0 += 65535)
+      k_dense<<<dim3((unsigned)std::min<int64_t>((longest + TB - 1) / TB, 64), (unsigned)std::min<int64_t>(65535, U - u0)),
+                TB, 0, s>>>(sv.arcs, sv.theta, slice_sym_win(f), d_slot + n + u0, f->Q, dsum + u0 * QQ,
+                            dmax + u0 * QQ);
     FST_CUDA(cudaGetLastError());
-    // the product tree, both semirings side by side: level by level,
-    // adjacent pairs multiplied, an odd last matrix carried up
-    std::vector<const float*> cur_s(n), cur_m(n);
-    for (int32_t i = 0; i < n; ++i) {
-      cur_s[i] = dsum + slot[ids[i]] * QQ;
-      cur_m[i] = dmax + slot[ids[i]] * QQ;
-    }
-    int parity = 0;
+    // the product tree: level by level, adjacent pairs multiplied
+    const float *cur_s = dsum, *cur_m = dmax;
+    const int32_t* slot = d_slot;
+    int64_t count = n;
     const int32_t tiles = (int32_t)((Q + TILE - 1) / TILE);
-    while (cur_s.size() > 1) {
-      const int64_t pairs = (int64_t)cur_s.size() / 2;
-      float* out_s = bufs[parity];
-      float* out_m = bufs[2 + parity];
-      for (int sem = 0; sem < 2; ++sem) {
-        const std::vector<const float*>& cur = sem ? cur_m : cur_s;
-        std::vector<const float*> h(2 * pairs);
-        for (int64_t p = 0; p < pairs; ++p) {
-          h[p] = cur[2 * p];
-          h[pairs + p] = cur[2 * p + 1];
-        }
-        FST_CUDA(cudaMemcpyAsync(d_ptr, h.data(), (size_t)(2 * pairs) * sizeof(float*), cudaMemcpyHostToDevice, s));
-        for (int64_t p0 = 0; p0 < pairs; p0 += 65535) {
-          const int64_t cnt = std::min<int64_t>(65535, pairs - p0);
-          const dim3 grid((unsigned)(tiles * tiles), (unsigned)cnt);
-          float* out = (sem ? out_m : out_s) + p0 * QQ;
-          if (sem)
-            k_mul<true><<<grid, TILE * TILE, 0, s>>>(d_ptr + p0, d_ptr + pairs + p0, out, f->Q);
-          else
-            k_mul<false><<<grid, TILE * TILE, 0, s>>>(d_ptr + p0, d_ptr + pairs + p0, out, f->Q);
-        }
-        FST_CUDA(cudaGetLastError());
-        // the pointer table is rewritten for the other semiring only after
-        // these launches have read it
-        FST_CUDA(cudaStreamSynchronize(s));
+    for (int level = 0; count > 1 || slot; ++level) {
+      float *out_s = buf_s[level & 1], *out_m = buf_m[level & 1];
+      const int64_t pairs = (count + 1) / 2;
+      for (int64_t p0 = 0; p0 < pairs; p0 += 65535) {
+        const int64_t cnt = std::min<int64_t>(65535, pairs - p0);
+        k_mul<<<dim3((unsigned)(tiles * tiles), (unsigned)cnt, 2), TB, 0, s>>>(
+            slot ? cur_s : cur_s + 2 * p0 * QQ, slot ? cur_m : cur_m + 2 * p0 * QQ, slot ? slot + 2 * p0 : nullptr,
+            (int32_t)(count - 2 * p0), out_s + p0 * QQ, out_m + p0 * QQ, f->Q);
       }
-      std::vector<const float*> nxt_s(pairs), nxt_m(pairs);
-      for (int64_t p = 0; p < pairs; ++p) {
-        nxt_s[p] = out_s + p * QQ;
-        nxt_m[p] = out_m + p * QQ;
-      }
-      if (cur_s.size() % 2) {
-        // carry the odd one into this level's buffer (the buffer it sits in
-        // is overwritten by the next level's products)
-        FST_CUDA(cudaMemcpyAsync(out_s + pairs * QQ, cur_s.back(), (size_t)QQ * 4, cudaMemcpyDeviceToDevice, s));
-        FST_CUDA(cudaMemcpyAsync(out_m + pairs * QQ, cur_m.back(), (size_t)QQ * 4, cudaMemcpyDeviceToDevice, s));
-        nxt_s.push_back(out_s + pairs * QQ);
-        nxt_m.push_back(out_m + pairs * QQ);
-      }
-      cur_s.swap(nxt_s);
-      cur_m.swap(nxt_m);
-      parity ^= 1;
+      cur_s = out_s;
+      cur_m = out_m;
+      slot = nullptr;
+      count = pairs;
     }
-    k_close<<<1, TB, 0, s>>>(cur_s[0], cur_m[0], f->Q, f->theta_s, f->theta_f, d_logz, d_best);
+    k_close<<<1, TB, 0, s>>>(cur_s, cur_m, f->Q, f->theta_s, f->theta_f, &d_out->logz, &d_out->best);
+    FST_CUDA(cudaGetLastError());
+    FST_CUDA(cudaMemcpy(&h, d_out, sizeof(h), cudaMemcpyDeviceToHost));
   }
-  FST_CUDA(cudaGetLastError());
-  FST_CUDA(cudaMemcpy(log_z, d_logz, 8, cudaMemcpyDeviceToHost));
-  FST_CUDA(cudaMemcpy(best_score, d_best, 4, cudaMemcpyDeviceToHost));
+  *log_z = h.logz;
+  *best_score = h.best;
   if (*log_z == -INFINITY) {
     set_error("no accepting path");
     return FST_ERR_NO_PATH;
