@@ -6,7 +6,6 @@
 #include "kernels.cuh"
 
 namespace fstgpu {
-namespace {
 
 // Error bits of a run (FrontierState::flags[1]): the live pool overflowed,
 // or a grid barrier of a persistent pass gave up waiting.
@@ -24,8 +23,8 @@ __device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); 
 // compiles every check away.
 enum : int { CHK_STAGE = 1, CHK_POOL_WRITE = 2, CHK_POOL_READ = 3, CHK_ACC = 4, CHK_ARC = 5, CHK_TOKEN = 6 };
 #ifdef FST_DEBUG
-__device__ unsigned long long g_dbg[4];  // violations, code, index, bound (one record per source file)
-__device__ __noinline__ bool in_bounds_slow(int code, long long i, long long n) {
+static __device__ unsigned long long g_dbg[4];  // violations, code, index, bound (one record per source file)
+static __device__ __noinline__ bool in_bounds_slow(int code, long long i, long long n) {
   if (atomicAdd(&g_dbg[0], 1ull) == 0ull) {
     g_dbg[1] = (unsigned long long)code;
     g_dbg[2] = (unsigned long long)i;
@@ -102,6 +101,19 @@ __device__ __forceinline__ Arcs find_arcs(const LayoutView& L, int32_t a, int32_
   return seg_find(L, p, nullptr);
 }
 
+// Chained launches of the per-position kernels (programmatic dependent
+// launch).  A step kernel launched with programmatic stream serialization
+// may be scheduled while the previous kernel of its stream still runs.  Its
+// first instruction waits until that kernel has completed and its writes
+// are visible (griddepcontrol.wait), so no access of the step precedes it;
+// then it lets the next position's kernel be scheduled in turn.  What
+// overlaps is the launch and block scheduling of position t+1 with the work
+// of position t.  Launched without the attribute, both do nothing.
+__device__ __forceinline__ void chain_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ void add_count(const CountView& C, int32_t id, float g) {
   if (C.batched) {
     atomicAdd(C.cnt64 + id, (double)g);
@@ -117,5 +129,4 @@ __device__ __forceinline__ void add_count(const CountView& C, int32_t id, float 
   }
 }
 
-}  // namespace
 }  // namespace fstgpu

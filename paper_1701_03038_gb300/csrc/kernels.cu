@@ -555,19 +555,6 @@ __device__ __forceinline__ void first_position(const LayoutView& L, const TokenV
   ranges_last_block(T, V, S, S.scnt, S.pool_top, S.pool_cap, S.slot_base, S.pool_base, S.pool_cnt, S.step_rng + 2);
 }
 
-// Chained launches of the per-position kernels (programmatic dependent
-// launch).  A step kernel launched with programmatic stream serialization
-// may be scheduled while the previous kernel of its stream still runs.  Its
-// first instruction waits until that kernel has completed and its writes
-// are visible (griddepcontrol.wait), so no access of the step precedes it;
-// then it lets the next position's kernel be scheduled in turn.  What
-// overlaps is the launch and block scheduling of position t+1 with the work
-// of position t.  Launched without the attribute, both do nothing.
-__device__ __forceinline__ void chain_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 __global__ void __launch_bounds__(KT) k_vit_first(LayoutView L, TokenView T, StepView V, FrontierState S) {
   __shared__ BlockScratch<PushCtx> sh;
   chain_enter();

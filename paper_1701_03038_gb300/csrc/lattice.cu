@@ -22,11 +22,13 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
 
 #include "fst_internal.cuh"
+#include "frontier.cuh"
 
 using namespace fstgpu;
 
@@ -35,7 +37,28 @@ namespace {
 constexpr int TB = 256;
 inline unsigned nb(int64_t n) { return (unsigned)std::max<int64_t>(1, (n + TB - 1) / TB); }
 
-__device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
+// The lattice's edges on the device, grouped by the node they go into (or
+// come out of), each group in increasing edge id.  pre[j] counts the padded
+// arcs of the edges before position j, so that one launch covers all edges
+// of a node: flat arc pre[lo] + i belongs to the last edge with pre <= it.
+// The slices are whole 128-arc windows, so a warp's 32 arcs are one edge's.
+struct EdgeRec {
+  int64_t i0;     // first arc record of the edge's symbol
+  int32_t id;     // caller's edge id
+  int32_t from, to;
+  float w;
+};
+struct EdgeView {
+  const EdgeRec* e;
+  const int64_t* pre;
+};
+__device__ __forceinline__ int32_t edge_of(const EdgeView& G, int32_t lo, int32_t hi, int64_t x) {
+  while (hi - lo > 1) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (__ldg(G.pre + mid) <= x) lo = mid; else hi = mid;
+  }
+  return lo;
+}
 
 // Start node: the start weights as keys (no incoming arc: low word 0).
 __global__ void k_lat_vit_init(const float* __restrict__ theta_s, int32_t Q, unsigned long long* __restrict__ keys0) {
@@ -45,41 +68,48 @@ __global__ void k_lat_vit_init(const float* __restrict__ theta_s, int32_t Q, uns
   keys0[q] = v == neg_inf() ? 0ull : ((unsigned long long)fkey(v) << 32);
 }
 
-// One edge u -> v: every arc of its slice with a live source.
-__global__ void k_lat_vit_edge(const int4* __restrict__ arcs, const float* __restrict__ theta, int64_t i0, int64_t np,
-                               const unsigned long long* __restrict__ keys_u, float w,
-                               unsigned long long* __restrict__ keys_v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= np) return;
-  const int4 a = __ldg(arcs + i0 + i);
-  if (a.z < 0) return;
-  const unsigned long long kp = keys_u[a.x];
-  if (!kp) return;
-  const float c = __fadd_rn(__fadd_rn(fkey_inv((uint32_t)(kp >> 32)), __ldg(theta + i0 + i)), w);
-  if (c == neg_inf()) return;
-  atomicMax(keys_v + a.y, ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)a.z));
+// The edges [lo, hi) into a node: every arc of their slices with a live
+// source.
+__global__ void __launch_bounds__(TB) k_lat_vit_node(EdgeView G, int32_t lo, int32_t hi,
+                                                     const int4* __restrict__ arcs, const float* __restrict__ theta,
+                                                     int32_t Q, unsigned long long* __restrict__ keys) {
+  chain_enter();
+  const int64_t p0 = __ldg(G.pre + lo), p1 = __ldg(G.pre + hi);
+  for (int64_t x = p0 + (int64_t)blockIdx.x * TB + threadIdx.x; x < p1; x += (int64_t)gridDim.x * TB) {
+    const int32_t j = edge_of(G, lo, hi, x);
+    const EdgeRec e = G.e[j];
+    const int64_t i = e.i0 + (x - __ldg(G.pre + j));
+    const int4 a = __ldg(arcs + i);
+    if (a.z < 0) continue;
+    const unsigned long long kp = keys[(int64_t)e.from * Q + a.x];
+    if (!kp) continue;
+    const float c = __fadd_rn(__fadd_rn(fkey_inv((uint32_t)(kp >> 32)), __ldg(theta + i)), e.w);
+    if (c == neg_inf()) continue;
+    atomicMax(keys + (int64_t)e.to * Q + a.y, ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)a.z));
+  }
 }
 
 __device__ __forceinline__ float key_score(unsigned long long k) {
   return k ? fkey_inv((uint32_t)(k >> 32)) : neg_inf();
 }
 
-// Best end state (lowest id on ties), then the backtrace by thread 0: at
-// node v in state q the key names the best arc k; the edge is the lowest id
-// into v that reads k's symbol and reaches the same score through it.  At
-// most N-1 steps (each moves to a lower node).
-__global__ void k_lat_vit_final(const unsigned long long* __restrict__ keys, int32_t N, int32_t Q,
-                                const float* __restrict__ theta_f, const int32_t* __restrict__ in_off,
-                                const int32_t* __restrict__ in_edge, const int32_t* __restrict__ efrom,
-                                const int32_t* __restrict__ elabel, const float* __restrict__ eweight,
-                                const int32_t* __restrict__ il_by_id, const float* __restrict__ th_by_id,
-                                const int32_t* __restrict__ src_by_id, float* __restrict__ score,
-                                int32_t* __restrict__ edge_path, int32_t* __restrict__ arc_path,
-                                int32_t* __restrict__ path_len) {
-  __shared__ unsigned long long red[TB / 32];
+// Best end state (lowest id on ties), then the backtrace by warp 0: at node
+// v in state q the key names the best arc k; the edge is the lowest id into
+// v that reads k's symbol (k is among its source's arcs on the edge's symbol)
+// and reaches the same score through it -- a lane per edge.  At most N-1
+// steps (each moves to a lower node).  out: score, path length, the edges,
+// the arcs (both from the end back).
+__global__ void __launch_bounds__(1024) k_lat_vit_final(LayoutView L, EdgeView G, const int32_t* __restrict__ in_off,
+                                                        const int32_t* __restrict__ elabel,
+                                                        const unsigned long long* __restrict__ keys, int32_t N,
+                                                        int32_t Q, const float* __restrict__ theta_f,
+                                                        const int32_t* __restrict__ src_by_id,
+                                                        int32_t* __restrict__ out) {
+  __shared__ unsigned long long red[32];
+  const int lane = threadIdx.x & 31;
   const unsigned long long* last = keys + (int64_t)(N - 1) * Q;
   unsigned long long best = 0ull;
-  for (int32_t q = threadIdx.x; q < Q; q += TB) {
+  for (int32_t q = threadIdx.x; q < Q; q += blockDim.x) {
     const float c = __fadd_rn(key_score(last[q]), theta_f[q]);
     if (c == neg_inf()) continue;
     const unsigned long long k = ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)q);
@@ -90,11 +120,17 @@ __global__ void k_lat_vit_final(const unsigned long long* __restrict__ keys, int
     const unsigned long long o = __shfl_xor_sync(FULL, best, d);
     best = o > best ? o : best;
   }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
+  if (lane == 0) red[threadIdx.x >> 5] = best;
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int w = 0; w < TB / 32; ++w) best = red[w] > best ? red[w] : best;
-  *score = best ? fkey_inv((uint32_t)(best >> 32)) : neg_inf();
+  if (threadIdx.x >= 32) return;
+  best = lane < (int)(blockDim.x >> 5) ? red[lane] : 0ull;
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(FULL, best, d);
+    best = o > best ? o : best;
+  }
+  int32_t* edge_path = out + 2;
+  int32_t* arc_path = edge_path + (N > 1 ? N - 1 : 1);
   int32_t len = 0;
   if (best) {
     int32_t v = N - 1, q = (int32_t)(~(uint32_t)best);
@@ -103,83 +139,111 @@ __global__ void k_lat_vit_final(const unsigned long long* __restrict__ keys, int
       const int32_t k = (int32_t)(~(uint32_t)kv);
       if (!kv || k < 0) { len = -1; break; }
       const float s = key_score(kv);
-      const int32_t src = src_by_id[k];
-      int32_t e_best = -1;
-      for (int32_t j = in_off[v]; j < in_off[v + 1]; ++j) {  // edges into v, by increasing id
-        const int32_t e = in_edge[j];
-        if (elabel[e] != il_by_id[k]) continue;
-        const float vu = key_score(keys[(int64_t)efrom[e] * Q + src]);
-        if (vu == neg_inf()) continue;
-        if (__fadd_rn(__fadd_rn(vu, th_by_id[k]), eweight[e]) == s) { e_best = e; break; }
+      const int32_t src = __ldg(src_by_id + k);
+      int32_t e_best = -1, from = 0;
+      const int32_t lo = __ldg(in_off + v), hi = __ldg(in_off + v + 1);
+      for (int32_t j0 = lo; j0 < hi && e_best < 0; j0 += 32) {  // edges into v, by increasing id
+        const int32_t j = j0 + lane;
+        bool hit = false;
+        EdgeRec e{0, 0, 0, 0, 0.f};
+        if (j < hi) {
+          e = G.e[j];
+          const float vu = key_score(keys[(int64_t)e.from * Q + src]);
+          const Arcs r = find_arcs(L, __ldg(elabel + e.id), src);
+          if (vu != neg_inf())
+            for (int32_t i = 0; i < r.len; ++i) {
+              const int4 a = __ldg(L.arcs + r.pos + i);
+              if (a.z == k) hit = __fadd_rn(__fadd_rn(vu, __int_as_float(a.y)), e.w) == s;
+            }
+        }
+        const uint32_t hits = __ballot_sync(FULL, hit);
+        if (hits) {
+          e_best = __shfl_sync(FULL, e.id, __ffs(hits) - 1);
+          from = __shfl_sync(FULL, e.from, __ffs(hits) - 1);
+        }
       }
       if (e_best < 0) { len = -1; break; }
-      edge_path[len] = e_best;
-      arc_path[len] = k;
+      if (lane == 0) {
+        edge_path[len] = e_best;
+        arc_path[len] = k;
+      }
       ++len;
-      v = efrom[e_best];
+      v = from;
       q = src;
     }
   }
-  *path_len = len;
+  if (lane == 0) {
+    out[0] = __float_as_int(best ? fkey_inv((uint32_t)(best >> 32)) : neg_inf());
+    out[1] = len;
+  }
 }
 
-// Forward and backward relaxations of one edge (float64 values), in two
-// phases: the exact maximum of each target, then the fixed-point sum.
-// fwd: target = destination, value = tab_u[src] + w + theta;
-// bwd: target = source, value = w + theta + tab_v[dst].
-template <bool FWD, bool SUM>
-__global__ void k_lat_lse_edge(const int4* __restrict__ arcs, const float* __restrict__ theta, int64_t i0, int64_t np,
-                               const double* __restrict__ tab, double w, unsigned long long* __restrict__ maxk,
-                               unsigned long long* __restrict__ sum) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= np) return;
-  const int4 a = __ldg(arcs + i0 + i);
-  if (a.z < 0) return;
-  const double x = tab[FWD ? a.x : a.y];
-  const float th = __ldg(theta + i0 + i);
-  if (x == -INFINITY || th == neg_inf()) return;
-  const double v = x + w + (double)th;
-  const int32_t tgt = FWD ? a.y : a.x;
-  if (!SUM)
-    atomicMax(maxk + tgt, dkey(v));
-  else
-    atomicAdd(sum + tgt, fix_exp64(v, dkey_inv(maxk[tgt])));
+// A node's values in the forward and backward passes: {fixed-point sum,
+// order key of the maximum} per state, the value formed where it is read (a
+// sum that is one term takes no logarithm), so that no pass over the states
+// stands between the nodes.
+__device__ __forceinline__ double lse_value(const ulonglong2* __restrict__ tab, int64_t i) {
+  const ulonglong2 x = __ldcg(tab + i);
+  return x.y ? fix_log_sum64(dkey_inv(x.y), x.x) : -INFINITY;
 }
-
-// tab[q] = max + log(sum) (or -inf), and the accumulators back to zero.
-__global__ void k_lat_lse_finish(unsigned long long* __restrict__ maxk, unsigned long long* __restrict__ sum,
-                                 int32_t Q, double* __restrict__ tab) {
+__global__ void k_lat_lse_init(const float* __restrict__ in, int32_t Q, ulonglong2* __restrict__ tab) {
   const int32_t q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= Q) return;
-  const unsigned long long m = maxk[q];
-  tab[q] = m ? fix_log_sum64(dkey_inv(m), sum[q]) : -INFINITY;
-  maxk[q] = 0ull;
-  sum[q] = 0ull;
+  const float v = in[q];
+  tab[q] = v == neg_inf() ? make_ulonglong2(0ull, 0ull) : make_ulonglong2(1099511627776ull, dkey((double)v));  // 2^40
 }
 
-__global__ void k_lat_from_f32(const float* __restrict__ in, int32_t Q, double* __restrict__ out) {
-  const int32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < Q) out[q] = (double)in[q];
+// Forward (or backward) relaxation of all edges [lo, hi) into (out of) a
+// node, in two phases: the exact maximum of each target, then the
+// fixed-point sums.
+// FWD: target = destination, value = tab[from][src] + w + theta;
+// else: target = source, value = tab[to][dst] + w + theta.
+template <bool FWD, bool SUM>
+__global__ void __launch_bounds__(TB) k_lat_lse_node(EdgeView G, int32_t lo, int32_t hi,
+                                                     const int4* __restrict__ arcs, const float* __restrict__ theta,
+                                                     int32_t Q, ulonglong2* __restrict__ tab) {
+  chain_enter();
+  const int64_t p0 = __ldg(G.pre + lo), p1 = __ldg(G.pre + hi);
+  for (int64_t x = p0 + (int64_t)blockIdx.x * TB + threadIdx.x; x < p1; x += (int64_t)gridDim.x * TB) {
+    const int32_t j = edge_of(G, lo, hi, x);
+    const EdgeRec e = G.e[j];
+    const int64_t i = e.i0 + (x - __ldg(G.pre + j));
+    const int4 a = __ldg(arcs + i);
+    if (a.z < 0) continue;
+    const float th = __ldg(theta + i);
+    if (dead32(th)) continue;
+    const double u = lse_value(tab, (int64_t)(FWD ? e.from : e.to) * Q + (FWD ? a.x : a.y));
+    if (dead64(u)) continue;
+    const double v = u + (double)e.w + (double)th;
+    if (dead64(v)) continue;
+    unsigned long long* t = (unsigned long long*)(tab + (int64_t)(FWD ? e.to : e.from) * Q + (FWD ? a.y : a.x));
+    if (!SUM) atomicMax(t + 1, dkey(v));
+    else atomicAdd(t, fix_exp64(v, dkey_inv(__ldcg(t + 1))));
+  }
 }
 
 // log Z = LSE_q(alpha_end[q] + theta_f[q]) in float64 (one block).
-__global__ void k_lat_logz(const double* __restrict__ alpha_end, const float* __restrict__ theta_f, int32_t Q,
-                           double* __restrict__ logz) {
-  __shared__ double red[TB / 32];
+__global__ void __launch_bounds__(1024) k_lat_logz(const ulonglong2* __restrict__ end, const float* __restrict__ theta_f,
+                                                   int32_t Q, double* __restrict__ logz) {
+  chain_enter();
+  __shared__ double red[32];
+  const int nw = blockDim.x >> 5;
   double m = -INFINITY;
-  for (int32_t q = threadIdx.x; q < Q; q += TB) m = fmax(m, alpha_end[q] + (double)theta_f[q]);
+  for (int32_t q = threadIdx.x; q < Q; q += blockDim.x)
+    if (!dead32(theta_f[q])) m = fmax(m, lse_value(end, q) + (double)theta_f[q]);
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) m = fmax(m, __shfl_xor_sync(FULL, m, d));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   m = red[0];
-  for (int w = 1; w < TB / 32; ++w) m = fmax(m, red[w]);
+  for (int w = 1; w < nw; ++w) m = fmax(m, red[w]);
   __syncthreads();
   double s = 0.0;
   if (m != -INFINITY)
-    for (int32_t q = threadIdx.x; q < Q; q += TB) {
-      const double v = alpha_end[q] + (double)theta_f[q];
-      if (v != -INFINITY) s += exp(v - m);
+    for (int32_t q = threadIdx.x; q < Q; q += blockDim.x) {
+      if (dead32(theta_f[q])) continue;
+      const double v = lse_value(end, q) + (double)theta_f[q];
+      if (!dead64(v)) s += exp(v - m);
     }
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(FULL, s, d);
@@ -187,52 +251,52 @@ __global__ void k_lat_logz(const double* __restrict__ alpha_end, const float* __
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < TB / 32; ++w) t += red[w];
+    for (int w = 0; w < nw; ++w) t += red[w];
     *logz = m == -INFINITY ? -INFINITY : m + log(t);
   }
 }
 
-// Posteriors through edge e: exp(alpha[u][src] + w + theta + beta[v][dst] - log Z)
-// to each arc's count and to the edge's posterior.
-__global__ void k_lat_post(const int4* __restrict__ arcs, const float* __restrict__ theta, int64_t i0, int64_t np,
-                           const double* __restrict__ alpha_u, const double* __restrict__ beta_v, double w,
-                           const double* __restrict__ logz, double* __restrict__ cnt, double* __restrict__ epost) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double g = 0.0;
-  if (i < np) {
-    const int4 a = __ldg(arcs + i0 + i);
-    const float th = a.z >= 0 ? __ldg(theta + i0 + i) : neg_inf();
-    const double lz = *logz;
-    if (a.z >= 0 && th != neg_inf() && lz != -INFINITY) {
-      const double al = alpha_u[a.x], be = beta_v[a.y];
-      if (al != -INFINITY && be != -INFINITY) {
-        g = exp(al + w + (double)th + be - lz);
-        atomicAdd(cnt + a.z, g);
+// Posteriors through every edge: exp(alpha[u][src] + w + theta + beta[v][dst]
+// - log Z) to each arc's count and to the edge's posterior.
+__global__ void __launch_bounds__(TB) k_lat_post(EdgeView G, int32_t E, const int4* __restrict__ arcs,
+                                                 const float* __restrict__ theta, int32_t Q,
+                                                 const ulonglong2* __restrict__ alpha,
+                                                 const ulonglong2* __restrict__ beta, const double* __restrict__ logz,
+                                                 double* __restrict__ cnt, double* __restrict__ epost) {
+  chain_enter();
+  const double lz = *logz;
+  if (lz == -INFINITY) return;
+  const int64_t p1 = __ldg(G.pre + E);
+  // (whole warps: p1 is a multiple of 128)
+  for (int64_t x = (int64_t)blockIdx.x * TB + threadIdx.x; x < p1; x += (int64_t)gridDim.x * TB) {
+    const int32_t j = edge_of(G, 0, E, x);
+    const EdgeRec e = G.e[j];
+    const int64_t i = e.i0 + (x - __ldg(G.pre + j));
+    const int4 a = __ldg(arcs + i);
+    const float th = __ldg(theta + i);
+    double g = 0.0;
+    if (a.z >= 0 && !dead32(th)) {
+      const double al = lse_value(alpha, (int64_t)e.from * Q + a.x);
+      if (!dead64(al)) {
+        const double be = lse_value(beta, (int64_t)e.to * Q + a.y);
+        if (!dead64(be)) {
+          g = exp(al + (double)e.w + (double)th + be - lz);
+          atomicAdd(cnt + a.z, g);
+        }
       }
     }
-  }
+    if (!__any_sync(FULL, g != 0.0)) continue;
 #pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) g += __shfl_xor_sync(FULL, g, d);
-  if ((threadIdx.x & 31) == 0 && g != 0.0) atomicAdd(epost, g);
+    for (int d = 16; d >= 1; d >>= 1) g += __shfl_xor_sync(FULL, g, d);
+    if ((threadIdx.x & 31) == 0) atomicAdd(epost + e.id, g);
+  }
 }
 
+// Counts of the arcs, then posteriors of the edges, to float32.
 __global__ void k_lat_to_f32(const double* __restrict__ in, int64_t n, float* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (float)in[i];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = (float)in[i];
 }
-
-struct DevMem {
-  std::vector<void*> p;
-  template <class T>
-  int get(T** out, int64_t n) {
-    int rc = dalloc(out, n);
-    if (!rc) p.push_back((void*)*out);
-    return rc;
-  }
-  ~DevMem() {
-    for (void* x : p) cudaFree(x);
-  }
-};
 
 struct DevGuard {
   int old = -1;
@@ -296,11 +360,37 @@ int check_lattice(const fst_s* f, int32_t N, int32_t E, const int32_t* from, con
   return FST_OK;
 }
 
-template <class T>
-int upload(DevMem& mem, T** d, const T* h, int64_t n) {
-  int rc = mem.get(d, n);
-  if (rc) return rc;
-  if (n > 0) FST_CUDA(cudaMemcpy(*d, h, (size_t)n * sizeof(T), cudaMemcpyHostToDevice));
+// One host image of the device's edge tables: the edges grouped by
+// destination node, and (both) by source node too, their arcs counted.
+struct EdgeTables {
+  std::vector<EdgeRec> e;
+  std::vector<int64_t> pre;
+  void add(const SliceView& sv, const std::vector<int32_t>& order, int32_t E, const int32_t* from, const int32_t* to,
+           const int32_t* label, const float* weight) {
+    int64_t x = 0;
+    for (int32_t j = 0; j < E; ++j) {
+      const int32_t k = order[j], a = label[k];
+      e.push_back(EdgeRec{sv.h_sym_win[a] * (int64_t)WIN, k, from[k], to[k], weight[k]});
+      pre.push_back(x);
+      x += (sv.h_sym_win[a + 1] - sv.h_sym_win[a]) * (int64_t)WIN;
+    }
+    pre.push_back(x);
+  }
+};
+
+// A launch over n flat arcs, chained to the one before it.
+template <class... KArgs, class... Args>
+int launch_arcs(void (*kernel)(KArgs...), int64_t n, int num_sms, cudaStream_t s, Args... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + TB - 1) / TB, 8 * (int64_t)num_sms)));
+  cfg.blockDim = dim3(TB);
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  FST_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
   return FST_OK;
 }
 
@@ -320,51 +410,50 @@ extern "C" int fst_lattice_viterbi(fst_t* f, int32_t num_nodes, int32_t num_edge
   cudaStream_t s = 0;
   SliceView sv;
   if ((rc = slice_view(f, s, &sv))) return rc;
-  const int64_t Q = f->Q, N = num_nodes, E = num_edges;
-  DevMem mem;
-  unsigned long long* keys = nullptr;
-  int32_t *d_in_off = nullptr, *d_in_edge = nullptr, *d_from = nullptr, *d_label = nullptr, *il = nullptr;
-  int32_t *d_epath = nullptr, *d_apath = nullptr, *d_len = nullptr;
-  float *d_w = nullptr, *th = nullptr, *d_score = nullptr;
-  if ((rc = mem.get(&keys, N * Q)) || (rc = mem.get(&il, std::max<int64_t>(f->A, 1))) ||
-      (rc = mem.get(&th, std::max<int64_t>(f->A, 1))) || (rc = mem.get(&d_score, 1)) || (rc = mem.get(&d_len, 1)) ||
-      (rc = mem.get(&d_epath, std::max<int64_t>(N - 1, 1))) || (rc = mem.get(&d_apath, std::max<int64_t>(N - 1, 1))) ||
-      (rc = upload(mem, &d_in_off, H.in_off.data(), N + 1)) ||
-      (rc = upload(mem, &d_in_edge, H.in_edge.data(), std::max<int64_t>(E, 1))) ||
-      (rc = upload(mem, &d_from, from, E)) || (rc = upload(mem, &d_label, label, E)) ||
-      (rc = upload(mem, &d_w, weight, E)))
+  const int64_t Q = f->Q, N = num_nodes, E = num_edges, np = std::max<int64_t>(N - 1, 1);
+  EdgeTables T;
+  T.add(sv, H.in_edge, num_edges, from, to, label, weight);
+  Scratch mem;
+  if ((rc = mem.take(f, Scratch::piece(N * Q * 8) + Scratch::piece(E * (int64_t)sizeof(EdgeRec)) +
+                            Scratch::piece((E + 1) * 8) + Scratch::piece((N + 1) * 4) + Scratch::piece(E * 4) +
+                            Scratch::piece((2 + 2 * np) * 4))))
     return rc;
-  if ((rc = arcs_by_id(f, il, nullptr, th, s))) return rc;
+  unsigned long long* keys = mem.get<unsigned long long>(N * Q);
+  EdgeRec* d_e = mem.get<EdgeRec>(E);
+  int64_t* d_pre = mem.get<int64_t>(E + 1);
+  int32_t* d_in = mem.get<int32_t>(N + 1);
+  int32_t* d_label = mem.get<int32_t>(E);
+  int32_t* d_out = mem.get<int32_t>(2 + 2 * np);
+  if (E > 0) {
+    FST_CUDA(cudaMemcpyAsync(d_e, T.e.data(), (size_t)E * sizeof(EdgeRec), cudaMemcpyHostToDevice, s));
+    FST_CUDA(cudaMemcpyAsync(d_label, label, (size_t)E * 4, cudaMemcpyHostToDevice, s));
+  }
+  FST_CUDA(cudaMemcpyAsync(d_pre, T.pre.data(), (size_t)(E + 1) * 8, cudaMemcpyHostToDevice, s));
+  FST_CUDA(cudaMemcpyAsync(d_in, H.in_off.data(), (size_t)(N + 1) * 4, cudaMemcpyHostToDevice, s));
   FST_CUDA(cudaMemsetAsync(keys, 0, (size_t)(N * Q) * 8, s));
+  const EdgeView G{d_e, d_pre};
   k_lat_vit_init<<<nb(Q), TB, 0, s>>>(f->theta_s, f->Q, keys);
-  // node by node: every edge into v, in increasing id
-  for (int32_t v = 1; v < N; ++v)
-    for (int32_t j = H.in_off[v]; j < H.in_off[v + 1]; ++j) {
-      const int32_t e = H.in_edge[j], a = label[e];
-      const int64_t i0 = sv.h_sym_win[a] * WIN, np = (sv.h_sym_win[a + 1] - sv.h_sym_win[a]) * WIN;
-      if (np)
-        k_lat_vit_edge<<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, keys + (int64_t)from[e] * Q, weight[e],
-                                             keys + (int64_t)v * Q);
-    }
-  k_lat_vit_final<<<1, TB, 0, s>>>(keys, num_nodes, f->Q, f->theta_f, d_in_off, d_in_edge, d_from, d_label, d_w, il,
-                                   th, f->src_by_id, d_score, d_epath, d_apath, d_len);
+  // node by node: every edge into v
+  for (int32_t v = 1; v < N; ++v) {
+    const int32_t lo = H.in_off[v], hi = H.in_off[v + 1];
+    const int64_t n = T.pre[hi] - T.pre[lo];
+    if (n && (rc = launch_arcs(k_lat_vit_node, n, f->num_sms, s, G, lo, hi, sv.arcs, sv.theta, f->Q, keys))) return rc;
+  }
+  k_lat_vit_final<<<1, 1024, 0, s>>>(view_of(f->bwd), G, d_in, d_label, keys, num_nodes, f->Q, f->theta_f,
+                                     f->src_by_id, d_out);
   FST_CUDA(cudaGetLastError());
-  int32_t len = 0;
-  FST_CUDA(cudaMemcpy(best_score, d_score, 4, cudaMemcpyDeviceToHost));
-  FST_CUDA(cudaMemcpy(&len, d_len, 4, cudaMemcpyDeviceToHost));
+  std::vector<int32_t> h((size_t)(2 + 2 * np));
+  FST_CUDA(cudaMemcpy(h.data(), d_out, h.size() * 4, cudaMemcpyDeviceToHost));
+  memcpy(best_score, &h[0], 4);
+  const int32_t len = h[1];
   if (len < 0) {
     set_error("fst_lattice_viterbi: the backtrace found no edge reaching the recorded score");
     return FST_ERR_STATE;
   }
   // the path was recorded from the end node back: reverse it
-  std::vector<int32_t> he(std::max(len, 1)), ha(std::max(len, 1));
-  if (len > 0) {
-    FST_CUDA(cudaMemcpy(he.data(), d_epath, (size_t)len * 4, cudaMemcpyDeviceToHost));
-    FST_CUDA(cudaMemcpy(ha.data(), d_apath, (size_t)len * 4, cudaMemcpyDeviceToHost));
-  }
   for (int32_t i = 0; i < len; ++i) {
-    edge_path[i] = he[len - 1 - i];
-    arc_path[i] = ha[len - 1 - i];
+    edge_path[i] = h[(size_t)(2 + len - 1 - i)];
+    arc_path[i] = h[(size_t)(2 + np + len - 1 - i)];
   }
   *path_len = len;
   if (*best_score == -INFINITY) {
@@ -388,79 +477,65 @@ extern "C" int fst_lattice_forward_backward(fst_t* f, int32_t num_nodes, int32_t
   cudaStream_t s = 0;
   SliceView sv;
   if ((rc = slice_view(f, s, &sv))) return rc;
-  const int64_t Q = f->Q, N = num_nodes, E = num_edges, A = std::max<int64_t>(f->A, 1);
-  DevMem mem;
-  double *alpha = nullptr, *beta = nullptr, *d_logz = nullptr, *cnt = nullptr, *epost = nullptr;
-  unsigned long long *maxk = nullptr, *sum = nullptr;
-  if ((rc = mem.get(&alpha, N * Q)) || (rc = mem.get(&beta, N * Q)) || (rc = mem.get(&d_logz, 1)) ||
-      (rc = mem.get(&maxk, Q)) || (rc = mem.get(&sum, Q)) || (rc = mem.get(&cnt, A)) ||
-      (rc = mem.get(&epost, std::max<int64_t>(E, 1))))
+  const int64_t Q = f->Q, N = num_nodes, E = num_edges, A = f->A;
+  EdgeTables T;  // by destination node, then by source node
+  T.add(sv, H.in_edge, num_edges, from, to, label, weight);
+  T.add(sv, H.out_edge, num_edges, from, to, label, weight);
+  // the values of both passes, log Z, and the counts of the arcs and the
+  // posteriors of the edges side by side, as float64 and as float32
+  Scratch mem;
+  if ((rc = mem.take(f, Scratch::piece((2 * N * Q + (A + E + 2) / 2) * 16) + Scratch::piece((A + E) * 4 + 8) +
+                            Scratch::piece(2 * E * (int64_t)sizeof(EdgeRec)) + Scratch::piece(2 * (E + 1) * 8))))
     return rc;
-  FST_CUDA(cudaMemsetAsync(maxk, 0, (size_t)Q * 8, s));
-  FST_CUDA(cudaMemsetAsync(sum, 0, (size_t)Q * 8, s));
-  FST_CUDA(cudaMemsetAsync(cnt, 0, (size_t)A * 8, s));
-  FST_CUDA(cudaMemsetAsync(epost, 0, (size_t)std::max<int64_t>(E, 1) * 8, s));
-  auto slice = [&](int32_t a, int64_t* i0, int64_t* np) {
-    *i0 = sv.h_sym_win[a] * WIN;
-    *np = (sv.h_sym_win[a + 1] - sv.h_sym_win[a]) * WIN;
-  };
+  ulonglong2* alpha = mem.get<ulonglong2>(2 * N * Q + (A + E + 2) / 2);
+  ulonglong2* beta = alpha + N * Q;
+  double* d_logz = (double*)(beta + N * Q);
+  double* cnt = d_logz + 1;
+  double* epost = cnt + A;
+  float* out = mem.get<float>(A + E + 2);
+  EdgeRec* d_e = mem.get<EdgeRec>(2 * E);
+  int64_t* d_pre = mem.get<int64_t>(2 * (E + 1));
+  FST_CUDA(cudaMemsetAsync(alpha, 0, (size_t)(2 * N * Q) * 16 + 8 + (size_t)(A + E) * 8, s));
+  if (E > 0) FST_CUDA(cudaMemcpyAsync(d_e, T.e.data(), (size_t)(2 * E) * sizeof(EdgeRec), cudaMemcpyHostToDevice, s));
+  FST_CUDA(cudaMemcpyAsync(d_pre, T.pre.data(), (size_t)(2 * (E + 1)) * 8, cudaMemcpyHostToDevice, s));
+  const EdgeView Gi{d_e, d_pre}, Go{d_e + E, d_pre + E + 1};
+  const int64_t* pi = T.pre.data();
+  const int64_t* po = T.pre.data() + E + 1;
   // forward, node by node
-  k_lat_from_f32<<<nb(Q), TB, 0, s>>>(f->theta_s, f->Q, alpha);
+  k_lat_lse_init<<<nb(Q), TB, 0, s>>>(f->theta_s, f->Q, alpha);
   for (int32_t v = 1; v < N; ++v) {
-    for (int ph = 0; ph < 2; ++ph)
-      for (int32_t j = H.in_off[v]; j < H.in_off[v + 1]; ++j) {
-        const int32_t e = H.in_edge[j];
-        int64_t i0, np;
-        slice(label[e], &i0, &np);
-        if (!np) continue;
-        const double* tu = alpha + (int64_t)from[e] * Q;
-        if (ph == 0)
-          k_lat_lse_edge<true, false><<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, tu, weight[e], maxk, sum);
-        else
-          k_lat_lse_edge<true, true><<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, tu, weight[e], maxk, sum);
-      }
-    k_lat_lse_finish<<<nb(Q), TB, 0, s>>>(maxk, sum, f->Q, alpha + (int64_t)v * Q);
+    const int32_t lo = H.in_off[v], hi = H.in_off[v + 1];
+    const int64_t n = pi[hi] - pi[lo];
+    if (!n) continue;
+    if ((rc = launch_arcs(k_lat_lse_node<true, false>, n, f->num_sms, s, Gi, lo, hi, sv.arcs, sv.theta, f->Q, alpha)) ||
+        (rc = launch_arcs(k_lat_lse_node<true, true>, n, f->num_sms, s, Gi, lo, hi, sv.arcs, sv.theta, f->Q, alpha)))
+      return rc;
   }
-  k_lat_logz<<<1, TB, 0, s>>>(alpha + (N - 1) * Q, f->theta_f, f->Q, d_logz);
-  // backward, from the end node
-  k_lat_from_f32<<<nb(Q), TB, 0, s>>>(f->theta_f, f->Q, beta + (N - 1) * Q);
-  for (int32_t v = (int32_t)N - 2; v >= 0; --v) {
-    for (int ph = 0; ph < 2; ++ph)
-      for (int32_t j = H.out_off[v]; j < H.out_off[v + 1]; ++j) {
-        const int32_t e = H.out_edge[j];
-        int64_t i0, np;
-        slice(label[e], &i0, &np);
-        if (!np) continue;
-        const double* tv = beta + (int64_t)to[e] * Q;
-        if (ph == 0)
-          k_lat_lse_edge<false, false><<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, tv, weight[e], maxk, sum);
-        else
-          k_lat_lse_edge<false, true><<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, tv, weight[e], maxk, sum);
-      }
-    k_lat_lse_finish<<<nb(Q), TB, 0, s>>>(maxk, sum, f->Q, beta + (int64_t)v * Q);
-  }
-  // posteriors
-  for (int32_t e = 0; e < num_edges; ++e) {
-    int64_t i0, np;
-    slice(label[e], &i0, &np);
-    if (np)
-      k_lat_post<<<nb(np), TB, 0, s>>>(sv.arcs, sv.theta, i0, np, alpha + (int64_t)from[e] * Q,
-                                       beta + (int64_t)to[e] * Q, weight[e], d_logz, cnt, epost + e);
+  k_lat_logz<<<1, 1024, 0, s>>>(alpha + (N - 1) * Q, f->theta_f, f->Q, d_logz);
+  if (arc_posteriors || edge_posteriors) {
+    // backward, from the end node
+    k_lat_lse_init<<<nb(Q), TB, 0, s>>>(f->theta_f, f->Q, beta + (N - 1) * Q);
+    for (int32_t v = num_nodes - 2; v >= 0; --v) {
+      const int32_t lo = H.out_off[v], hi = H.out_off[v + 1];
+      const int64_t n = po[hi] - po[lo];
+      if (!n) continue;
+      if ((rc = launch_arcs(k_lat_lse_node<false, false>, n, f->num_sms, s, Go, lo, hi, sv.arcs, sv.theta, f->Q, beta)) ||
+          (rc = launch_arcs(k_lat_lse_node<false, true>, n, f->num_sms, s, Go, lo, hi, sv.arcs, sv.theta, f->Q, beta)))
+        return rc;
+    }
+    if (pi[E] && (rc = launch_arcs(k_lat_post, pi[E], f->num_sms, s, Gi, num_edges, sv.arcs, sv.theta, f->Q, alpha, beta,
+                                   d_logz, cnt, epost)))
+      return rc;
+    if (A + E > 0)
+      k_lat_to_f32<<<(unsigned)std::min<int64_t>(nb(A + E), 8 * (int64_t)f->num_sms), TB, 0, s>>>(cnt, A + E, out);
   }
   FST_CUDA(cudaGetLastError());
-  FST_CUDA(cudaMemcpy(log_z, d_logz, 8, cudaMemcpyDeviceToHost));
-  if (arc_posteriors && f->A > 0) {
-    float* tmp = nullptr;
-    if ((rc = mem.get(&tmp, f->A))) return rc;
-    k_lat_to_f32<<<nb(f->A), TB, 0, s>>>(cnt, f->A, tmp);
-    FST_CUDA(cudaMemcpy(arc_posteriors, tmp, (size_t)f->A * 4, cudaMemcpyDeviceToHost));
-  }
-  if (edge_posteriors && E > 0) {
-    float* tmp = nullptr;
-    if ((rc = mem.get(&tmp, E))) return rc;
-    k_lat_to_f32<<<nb(E), TB, 0, s>>>(epost, E, tmp);
-    FST_CUDA(cudaMemcpy(edge_posteriors, tmp, (size_t)E * 4, cudaMemcpyDeviceToHost));
-  }
+  FST_CUDA(cudaMemcpyAsync(log_z, d_logz, 8, cudaMemcpyDeviceToHost, s));
+  if (arc_posteriors && A > 0)
+    FST_CUDA(cudaMemcpyAsync(arc_posteriors, out, (size_t)A * 4, cudaMemcpyDeviceToHost, s));
+  if (edge_posteriors && E > 0)
+    FST_CUDA(cudaMemcpyAsync(edge_posteriors, out + A, (size_t)E * 4, cudaMemcpyDeviceToHost, s));
+  FST_CUDA(cudaStreamSynchronize(s));
   if (*log_z == -INFINITY) {
     set_error("no accepting path");
     return FST_ERR_NO_PATH;

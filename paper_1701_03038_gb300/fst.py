@@ -308,8 +308,9 @@ class Fst:
         of an acyclic input lattice (see fst_lattice_forward_backward)."""
         n, e, (a, b, c, d) = self._lattice_args(num_nodes, frm, to, label, weight)
         lz = np.zeros(1, np.float64)
-        cnt = np.zeros(max(self.num_arcs, 1), np.float32)
-        ep = np.zeros(max(e, 1), np.float32)
+        # (written whole by the call; fresh zeroed pages would be faulted in by the copy)
+        cnt = np.empty(max(self.num_arcs, 1), np.float32)
+        ep = np.empty(max(e, 1), np.float32)
         with torch.cuda.device(self.device):
             rc = self._lib.fst_lattice_forward_backward(self._h, n, e, _hptr(a), _hptr(b), _hptr(c), _hptr(d),
                                                         _hptr(lz), _hptr(cnt), _hptr(ep))
