@@ -42,7 +42,7 @@ __device__ __forceinline__ bool in_bounds(int, long long, long long) { return tr
 __device__ __forceinline__ float decode_max(uint32_t k) { return k ? fkey_inv(k) : neg_inf(); }
 
 // Order key of a float64 value rounded to float32 (0 = -inf, nothing).
-__device__ __forceinline__ uint32_t fkey64(double v) { return v == -INFINITY ? 0u : fkey((float)v); }
+__device__ __forceinline__ uint32_t fkey64(double v) { return dead64(v) ? 0u : fkey(fx_narrow(v)); }
 
 // The arcs out of state q on symbol a: their first position and count (0
 // when none), from the (symbol, state) table.  In two steps, so that the
@@ -116,7 +116,7 @@ __device__ __forceinline__ void chain_enter() {
 
 __device__ __forceinline__ void add_count(const CountView& C, int32_t id, float g) {
   if (C.batched) {
-    atomicAdd(C.cnt64 + id, (double)g);
+    atomicAdd(C.cnt64 + id, fx_widen(g));
   } else {
     // compensated float32 summation (one string: one writer per arc and
     // step; read through L2, as a persistent pass meets the same arc at

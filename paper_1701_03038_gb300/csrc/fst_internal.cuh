@@ -24,6 +24,7 @@
 #include <string>
 #include <vector>
 
+#include "fixmath.cuh"
 #include "fstgpu.h"
 
 namespace fstgpu {
@@ -221,6 +222,11 @@ __device__ __forceinline__ double dkey_inv(unsigned long long k) {
   return __longlong_as_double((long long)u);
 }
 
+// -inf tests on the bit patterns: integer compares (a float64 compare takes
+// the float64 pipe, narrow on this part).
+__device__ __forceinline__ bool dead64(double v) { return __double_as_longlong(v) == (long long)0xfff0000000000000ull; }
+__device__ __forceinline__ bool dead32(float v) { return __float_as_uint(v) == 0xff800000u; }
+
 // exp(v - m), v <= m, as a 2^-40 fixed-point integer: sums of these are exact
 // and so independent of the order in which they are added.  A sum of fewer
 // than 2^24 terms cannot overflow (the store refuses longer segments).  The
@@ -228,26 +234,22 @@ __device__ __forceinline__ double dkey_inv(unsigned long long k) {
 // carried from position to position are float64 (a float32 value rounds by
 // up to 2^-24 of its size at every position, and over a 200-position string
 // those roundings shift alpha + beta - log Z by ~1e-5, the whole posterior
-// tolerance), and so is the term, whose relative error would otherwise add
-// to the same drift.  The maximal term is exactly 2^40 and costs no
-// exponential (most destinations of a sparse frontier have one live arc;
-// float64 arithmetic is scarce on this GPU).
+// tolerance), and so is their difference.  The maximal term is exactly 2^40.
+// The exponential is fixmath.cuh's: the float64 one bounded the large
+// positions (a chunk of 1,024 destinations took 30,000 cycles in the float64
+// logarithm alone, 6,000 with integers).
 __device__ __forceinline__ unsigned long long fix_exp64(double v, double m) {
-  if (v == -INFINITY) return 0ull;
-  if (v == m) return 1099511627776ull;  // 2^40
-  return __double2ull_rn(exp(v - m) * 1099511627776.0);
+  if (dead64(v)) return 0ull;
+  if (__double_as_longlong(v) == __double_as_longlong(m)) return 1099511627776ull;  // 2^40
+  return fx_exp40(v - m);
 }
-// -inf tests on the bit patterns: integer compares (a float64 compare takes
-// the float64 pipe, narrow on this part).
-__device__ __forceinline__ bool dead64(double v) { return __double_as_longlong(v) == (long long)0xfff0000000000000ull; }
-__device__ __forceinline__ bool dead32(float v) { return __float_as_uint(v) == 0xff800000u; }
 
 // m + log(s / 2^40), in float64.  A sum that is the maximal term alone
 // (s = 2^40, the usual case on a sparse frontier: one live arc into the
 // state) is m itself and takes no logarithm.
 __device__ __forceinline__ double fix_log_sum64(double m, unsigned long long s) {
-  if (__double_as_longlong(m) == (long long)0xfff0000000000000ull || s == 0ull) return -INFINITY;
-  return s == 1099511627776ull ? m : m + log((double)s * 0x1p-40);
+  if (dead64(m) || s == 0ull) return -INFINITY;
+  return s == 1099511627776ull ? m : fx_add_log40(m, s);
 }
 
 
