@@ -261,7 +261,7 @@ struct alignas(128) StringJob {
   int32_t t, a, an;         // position, its symbol, the next symbol (-1: none)
   int32_t cnt, per;         // entries of t-1, entries a chunk
   int32_t nb;               // entries of t
-  long long base, nbase;    // their pool ranges
+  int32_t base, nbase;      // their pool ranges
   double K;                 // backward: C_{t-1} + E_t - log Z - m_{t-1}
   float shift, gw;          // m_{t-1} (forward) or e_t (backward); the string's weight
   int32_t single, last;     // every destination has one arc; t is the last position
@@ -284,7 +284,7 @@ struct StringWork {
 };
 // What a launch sees of it.
 struct StringQueue {
-  int32_t strings, heavy_blocks, owners;
+  int32_t strings, heavy_blocks, light_warps, owners;
   uint32_t* ctl;
   StringJob* jobs;
   uint32_t* ring;
