@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "frontier.cuh"
 #include "fst_internal.cuh"
 
 using namespace fstgpu;
@@ -37,16 +38,14 @@ using namespace fstgpu;
 namespace {
 
 constexpr int TB = 256;
-constexpr int TILE = 64;   // output tile TILE x TILE, 4 x 4 entries a thread
 constexpr int KC = 64;     // k chunk staged in shared memory
 constexpr int PREFIX_MAX_STATES = 512;
 // sums below this may have lost terms to underflow (a lost term is below
 // 2^-126, and there are at most 512 of them)
 constexpr float TINY = 1e-30f;
 
-__device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
-
-__global__ void k_fill(float* __restrict__ p, int64_t n, float v) {
+__global__ void k_fill(float* __restrict__ p, int64_t n, float v, uint32_t* __restrict__ zero) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *zero = 0u;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     p[i] = v;
 }
@@ -89,105 +88,132 @@ __global__ void k_dense(const int4* __restrict__ arcs, const float* __restrict__
 }
 
 // One level of the tree: matrix 2p times matrix 2p + 1 of the level below,
-// for every p (blockIdx.y), one TILE x TILE tile of the result per block
+// for every p (blockIdx.y), one T x T tile of the result per block
 // (blockIdx.x), the log-sum and the max-plus products side by side
 // (blockIdx.z).  The matrices below are in[slot[k]] (slot null: in[k]); a
 // last matrix without a partner is carried up as it is.
-__global__ void __launch_bounds__(TB) k_mul(const float* __restrict__ in_sum, const float* __restrict__ in_max,
-                                            const int32_t* __restrict__ slot, int32_t count,
-                                            float* __restrict__ out_sum, float* __restrict__ out_max, int32_t Q) {
-  __shared__ float As[KC][TILE + 1];  // A transposed: [k][row]
-  __shared__ float Bs[KC][TILE + 1];
-  __shared__ float rmax[TILE], cmax[TILE];
-  const bool maxplus = blockIdx.z != 0;
-  const int64_t QQ = (int64_t)Q * Q;
-  const float* in = maxplus ? in_max : in_sum;
-  float* out = (maxplus ? out_max : out_sum) + (int64_t)blockIdx.y * QQ;
-  const int32_t ka = 2 * blockIdx.y, kb = ka + 1;
-  const float* A = in + (slot ? slot[ka] : ka) * QQ;
-  const int32_t tiles = (Q + TILE - 1) / TILE;
-  const int32_t i0 = ((int32_t)blockIdx.x / tiles) * TILE, j0 = ((int32_t)blockIdx.x % tiles) * TILE;
-  if (kb >= count) {
-    for (int32_t e = threadIdx.x; e < TILE * TILE; e += TB) {
-      const int32_t i = i0 + e / TILE, j = j0 + e % TILE;
-      if (i < Q && j < Q) out[(int64_t)i * Q + j] = A[(int64_t)i * Q + j];
-    }
-    return;
-  }
-  const float* B = in + (slot ? slot[kb] : kb) * QQ;
-  // (the thread's 4 x 4 entries: rows ty + 16 u, columns tx + 16 v)
-  const int32_t tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+//
+// A thread holds T / 16 x T / 16 entries and reads both operands from shared
+// memory as vectors, four k at a time.  T = 64 needs the fewest reads and
+// exponentials a product; T = 32 spreads a product over four times the
+// blocks, for the levels that have too few to fill the GPU (the last eight
+// of ten on 64 states and 1,000 symbols).
+struct MulArgs {
+  const float *in_sum, *in_max;
+  const int32_t* slot;
+  float *out_sum, *out_max;
+  int32_t count, Q;
+};
+template <int T>
+struct MulShared {
+  static constexpr int PARTS = TB / T;
+  float A[T][KC + 4], B[KC][T + 4];
+  float rmax[T], cmax[T], part[PARTS][T];
+};
+template <int N>
+struct alignas(4 * N) Vec {
+  float v[N];
+};
+
+template <int T, bool MAX>
+__device__ __forceinline__ void mul_tile(MulShared<T>& sh, const float* A, const float* B, float* out, int32_t i0, int32_t j0, int32_t Q) {
+  constexpr int R = T / 16, PARTS = MulShared<T>::PARTS, LOADS = T * KC / TB;
+  const int32_t t = threadIdx.x, tx = t % 16, ty = t / 16;
   auto load = [&](int32_t k0) {
-    for (int32_t e = threadIdx.x; e < TILE * KC; e += TB) {
-      const int32_t i = i0 + e / KC, k = k0 + e % KC;
-      As[e % KC][e / KC] = (i < Q && k < Q) ? __ldg(A + (int64_t)i * Q + k) : neg_inf();
-      const int32_t kk = k0 + e / TILE, j = j0 + e % TILE;
-      Bs[e / TILE][e % TILE] = (kk < Q && j < Q) ? __ldg(B + (int64_t)kk * Q + j) : neg_inf();
+    float a[LOADS], b[LOADS];
+#pragma unroll
+    for (int u = 0; u < LOADS; ++u) {
+      const int32_t e = t + u * TB, i = i0 + e / KC, k = k0 + e % KC, kk = k0 + e / T, j = j0 + e % T;
+      a[u] = i < Q && k < Q ? __ldcg(A + (int64_t)i * Q + k) : neg_inf();
+      b[u] = kk < Q && j < Q ? __ldcg(B + (int64_t)kk * Q + j) : neg_inf();
+    }
+#pragma unroll
+    for (int u = 0; u < LOADS; ++u) {
+      const int32_t e = t + u * TB;
+      sh.A[e / KC][e % KC] = a[u];
+      sh.B[e / T][e % T] = b[u];
     }
   };
-  if (!maxplus) {
-    // row and column maxima (0 stands for -inf: nothing to scale)
-    for (int32_t r = warp; r < TILE; r += TB / 32) {
-      float m = neg_inf(), c = neg_inf();
-      for (int32_t k = lane; k < Q; k += 32) {
-        if (i0 + r < Q) m = fmaxf(m, __ldg(A + (int64_t)(i0 + r) * Q + k));
-        if (j0 + r < Q) c = fmaxf(c, __ldg(B + (int64_t)k * Q + j0 + r));
+  const bool once = Q <= KC;
+  load(0);
+  __syncthreads();
+  if (!MAX) {
+    // row and column maxima: PARTS threads a row (neighbours) and a column
+    const int32_t row = t / PARTS, rp = t % PARTS, col = t % T, cp = t / T;
+    float m = neg_inf(), c = neg_inf();
+    for (int32_t k0 = 0;;) {
+#pragma unroll 8
+      for (int k = 0; k < KC; k += PARTS) {
+        m = fmaxf(m, sh.A[row][k + rp]);
+        c = fmaxf(c, sh.B[k + cp][col]);
       }
+      if ((k0 += KC) >= Q) break;
+      __syncthreads();
+      load(k0);
+      __syncthreads();
+    }
 #pragma unroll
-      for (int d = 16; d >= 1; d >>= 1) {
-        m = fmaxf(m, __shfl_xor_sync(FULL, m, d));
-        c = fmaxf(c, __shfl_xor_sync(FULL, c, d));
-      }
-      if (lane == 0) {
-        rmax[r] = m;
-        cmax[r] = c;
-      }
+    for (int d = PARTS / 2; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, d));
+    if (rp == 0) sh.rmax[row] = m;
+    sh.part[cp][col] = c;
+    __syncthreads();
+    if (t < T) {
+      c = sh.part[0][t];
+#pragma unroll
+      for (int p = 1; p < PARTS; ++p) c = fmaxf(c, sh.part[p][t]);
+      sh.cmax[t] = c;
     }
     __syncthreads();
   }
-  float acc[4][4];
+  float acc[R][R];
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < R; ++u)
 #pragma unroll
-    for (int v = 0; v < 4; ++v) acc[u][v] = maxplus ? neg_inf() : 0.f;
+    for (int v = 0; v < R; ++v) acc[u][v] = MAX ? neg_inf() : 0.f;
   for (int32_t k0 = 0; k0 < Q; k0 += KC) {
-    if (k0 > 0) __syncthreads();
-    load(k0);
-    __syncthreads();
-    if (!maxplus) {
-      for (int32_t e = threadIdx.x; e < TILE * KC; e += TB) {
-        const int32_t k = e / TILE, x = e % TILE;
-        const float a = As[k][x], b = Bs[k][x];
-        As[k][x] = a == neg_inf() ? 0.f : expf(a - rmax[x]);
-        Bs[k][x] = b == neg_inf() ? 0.f : expf(b - cmax[x]);
+    if (!once && (k0 > 0 || !MAX)) {
+      __syncthreads();
+      load(k0);
+      __syncthreads();
+    }
+    if (!MAX) {
+#pragma unroll
+      for (int u = 0; u < LOADS; ++u) {
+        const int32_t e = t + u * TB;
+        float& a = sh.A[e / KC][e % KC];
+        float& b = sh.B[e / T][e % T];
+        a = a == neg_inf() ? 0.f : expf(a - sh.rmax[e / KC]);
+        b = b == neg_inf() ? 0.f : expf(b - sh.cmax[e % T]);
       }
       __syncthreads();
     }
-    const int32_t kn = min(KC, Q - k0);
-#pragma unroll 4
-    for (int32_t k = 0; k < kn; ++k) {
-      float a[4], b[4];
+    // (past Q the operands are 0, or -inf: they change nothing)
+    const int32_t kn = min(KC, (Q - k0 + 3) & ~3);
+    for (int32_t k = 0; k < kn; k += 4) {
+      Vec<4> a[R];
+      Vec<R> b[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = As[k][ty + 16 * u];
-        b[u] = Bs[k][tx + 16 * u];
-      }
+      for (int u = 0; u < R; ++u) a[u] = *(const Vec<4>*)&sh.A[R * ty + u][k];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int x = 0; x < 4; ++x) b[x] = *(const Vec<R>*)&sh.B[k + x][R * tx];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = maxplus ? fmaxf(acc[u][v], a[u] + b[v]) : fmaf(a[u], b[v], acc[u][v]);
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+#pragma unroll
+          for (int v = 0; v < R; ++v)
+            acc[u][v] = MAX ? fmaxf(acc[u][v], a[u].v[x] + b[x].v[v]) : fmaf(a[u].v[x], b[x].v[v], acc[u][v]);
     }
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < R; ++u) {
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int32_t i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
+    for (int v = 0; v < R; ++v) {
+      const int32_t i = i0 + R * ty + u, j = j0 + R * tx + v;
       if (i >= Q || j >= Q) continue;
       float r = acc[u][v];
-      if (!maxplus) {
-        const float rm = rmax[ty + 16 * u], cm = cmax[tx + 16 * v];
+      if (!MAX) {
+        const float rm = sh.rmax[R * ty + u], cm = sh.cmax[R * tx + v];
         if (rm == neg_inf() || cm == neg_inf()) {
           r = neg_inf();
         } else if (r >= TINY) {
@@ -196,7 +222,7 @@ __global__ void __launch_bounds__(TB) k_mul(const float* __restrict__ in_sum, co
           // terms may have underflowed: the log-sum one by one
           float m = neg_inf(), s = 0.f;
           for (int32_t k = 0; k < Q; ++k) {
-            const float x = __ldg(A + (int64_t)i * Q + k), y = __ldg(B + (int64_t)k * Q + j);
+            const float x = __ldcg(A + (int64_t)i * Q + k), y = __ldcg(B + (int64_t)k * Q + j);
             if (x == neg_inf() || y == neg_inf()) continue;
             const float w = x + y;
             if (w > m) {
@@ -214,65 +240,135 @@ __global__ void __launch_bounds__(TB) k_mul(const float* __restrict__ in_sum, co
   }
 }
 
-// log Z = LSE_{i,j}(theta_s[i] + P[i][j] + theta_f[j]) (float64) and the
-// best score max_{i,j} fl(fl(theta_s[i] + V[i][j]) + theta_f[j]); one block.
-// P == nullptr: the empty string (P and V the identity of their semiring).
-__global__ void k_close(const float* __restrict__ P, const float* __restrict__ V, int32_t Q,
-                        const float* __restrict__ ts, const float* __restrict__ tf, double* __restrict__ logz,
-                        float* __restrict__ best) {
-  __shared__ double red[TB / 32];
-  __shared__ float redf[TB / 32];
+template <int T>
+__global__ void __launch_bounds__(TB) k_mul(const MulArgs M) {
+  __shared__ MulShared<T> sh;
+  // (what the level below wrote is read with __ldcg: read-only loads may be
+  // moved up, over the wait)
+  chain_enter();
+  const bool maxplus = blockIdx.z != 0;
+  const int32_t Q = M.Q;
   const int64_t QQ = (int64_t)Q * Q;
-  auto val = [&](int64_t e, bool vit) -> float {
-    const int32_t i = (int32_t)(e / Q), j = (int32_t)(e % Q);
-    const float m = P ? (vit ? V[e] : P[e]) : (i == j ? 0.f : neg_inf());
-    if (ts[i] == neg_inf() || m == neg_inf() || tf[j] == neg_inf()) return neg_inf();
-    return __fadd_rn(__fadd_rn(ts[i], m), tf[j]);
-  };
-  double mx = -INFINITY;
-  float bf = neg_inf();
-  for (int64_t e = threadIdx.x; e < QQ; e += TB) {
-    const int32_t i = (int32_t)(e / Q), j = (int32_t)(e % Q);
-    const float m = P ? P[e] : (i == j ? 0.f : neg_inf());
-    if (ts[i] != neg_inf() && m != neg_inf() && tf[j] != neg_inf())
-      mx = fmax(mx, (double)ts[i] + (double)m + (double)tf[j]);
-    bf = fmaxf(bf, val(e, true));
+  const float* in = maxplus ? M.in_max : M.in_sum;
+  float* out = (maxplus ? M.out_max : M.out_sum) + (int64_t)blockIdx.y * QQ;
+  const int32_t ka = 2 * blockIdx.y, kb = ka + 1;
+  const float* A = in + (M.slot ? M.slot[ka] : ka) * QQ;
+  const int32_t tiles = (Q + T - 1) / T;
+  const int32_t i0 = ((int32_t)blockIdx.x / tiles) * T, j0 = ((int32_t)blockIdx.x % tiles) * T;
+  if (kb >= M.count) {
+    for (int32_t e = threadIdx.x; e < T * T; e += TB) {
+      const int32_t i = i0 + e / T, j = j0 + e % T;
+      if (i < Q && j < Q) out[(int64_t)i * Q + j] = __ldcg(A + (int64_t)i * Q + j);
+    }
+    return;
   }
-#pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) {
-    mx = fmax(mx, __shfl_xor_sync(FULL, mx, d));
-    bf = fmaxf(bf, __shfl_xor_sync(FULL, bf, d));
+  const float* B = in + (M.slot ? M.slot[kb] : kb) * QQ;
+  if (maxplus) mul_tile<T, true>(sh, A, B, out, i0, j0, Q);
+  else mul_tile<T, false>(sh, A, B, out, i0, j0, Q);
+}
+
+// What a call returns, and the blocks' parts of it.
+struct Part {
+  double m, sum;  // largest term, sum of exp(term - m)
+  float best, pad;
+};
+constexpr int CLOSE_BLOCKS = 64;
+struct Out {
+  double logz;
+  float best;
+  uint32_t done;
+  Part part[CLOSE_BLOCKS];
+};
+
+// log Z = LSE_{i,j}(theta_s[i] + P[i][j] + theta_f[j]) (float64) and the
+// best score max_{i,j} fl(fl(theta_s[i] + V[i][j]) + theta_f[j]).  A warp
+// takes a row at a time (rows of no start state cost one read), a block its
+// warps' rows, the last block to finish the blocks' parts in their order.
+// P == nullptr: the empty string (P and V the identity of their semiring).
+__device__ __forceinline__ void add_terms(double& m, double& s, double m2, double s2) {
+  if (m2 == -INFINITY) return;
+  if (m == -INFINITY) {
+    m = m2;
+    s = s2;
+    return;
   }
-  if ((threadIdx.x & 31) == 0) {
-    red[threadIdx.x >> 5] = mx;
-    redf[threadIdx.x >> 5] = bf;
-  }
-  __syncthreads();
-  mx = red[0];
-  bf = redf[0];
-  for (int w = 1; w < TB / 32; ++w) {
-    mx = fmax(mx, red[w]);
-    bf = fmaxf(bf, redf[w]);
-  }
-  __syncthreads();
-  double sum = 0.0;
-  if (mx != -INFINITY)
-    for (int64_t e = threadIdx.x; e < QQ; e += TB) {
-      const int32_t i = (int32_t)(e / Q), j = (int32_t)(e % Q);
-      const float m = P ? P[e] : (i == j ? 0.f : neg_inf());
-      if (ts[i] != neg_inf() && m != neg_inf() && tf[j] != neg_inf())
-        sum += exp((double)ts[i] + (double)m + (double)tf[j] - mx);
+  const double x = fmax(m, m2);
+  s = (m == x ? s : s * exp(m - x)) + (m2 == x ? s2 : s2 * exp(m2 - x));
+  m = x;
+}
+__global__ void __launch_bounds__(TB) k_close(const float* P, const float* V, int32_t Q,
+                                              const float* __restrict__ ts, const float* __restrict__ tf,
+                                              Out* __restrict__ o) {
+  constexpr int WARPS = TB / 32;
+  __shared__ Part part[WARPS];
+  chain_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double m = -INFINITY, s = 0.0;
+  float best = neg_inf();
+  for (int32_t i = (int32_t)blockIdx.x * WARPS + warp; i < Q; i += (int32_t)gridDim.x * WARPS) {
+    const float si = __ldg(ts + i);
+    if (si == neg_inf()) continue;
+    auto term = [&](int32_t j) -> double {
+      const float f = __ldg(tf + j), p = P ? __ldcg(P + (int64_t)i * Q + j) : (i == j ? 0.f : neg_inf());
+      return p == neg_inf() || f == neg_inf() ? -INFINITY : (double)si + (double)p + (double)f;
+    };
+    double rm = -INFINITY, rs = 0.0;
+    for (int32_t j = lane; j < Q; j += 32) {
+      rm = fmax(rm, term(j));
+      const float f = __ldg(tf + j), v = P ? __ldcg(V + (int64_t)i * Q + j) : (i == j ? 0.f : neg_inf());
+      if (v != neg_inf() && f != neg_inf()) best = fmaxf(best, __fadd_rn(__fadd_rn(si, v), f));
     }
 #pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(FULL, sum, d);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < TB / 32; ++w) t += red[w];
-    *logz = mx == -INFINITY ? -INFINITY : mx + log(t);
-    *best = bf;
+    for (int d = 16; d >= 1; d >>= 1) rm = fmax(rm, __shfl_xor_sync(FULL, rm, d));
+    if (rm == -INFINITY) continue;
+    for (int32_t j = lane; j < Q; j += 32) {
+      const double x = term(j);
+      if (x != -INFINITY) rs += exp(x - rm);
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) rs += __shfl_xor_sync(FULL, rs, d);
+    add_terms(m, s, rm, rs);
   }
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) best = fmaxf(best, __shfl_xor_sync(FULL, best, d));
+  if (lane == 0) part[warp] = Part{m, s, best, 0.f};
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < WARPS; ++w) {
+    add_terms(m, s, part[w].m, part[w].sum);
+    best = fmaxf(best, part[w].best);
+  }
+  if (gridDim.x > 1) {
+    o->part[blockIdx.x] = Part{m, s, best, 0.f};
+    __threadfence();
+    if (atomicAdd(&o->done, 1u) + 1u < gridDim.x) return;
+    __threadfence();
+    m = -INFINITY;
+    s = 0.0;
+    for (unsigned b = 0; b < gridDim.x; ++b) {
+      const volatile Part* q = o->part + b;
+      add_terms(m, s, q->m, q->sum);
+      best = fmaxf(best, q->best);
+    }
+  }
+  o->logz = m == -INFINITY ? -INFINITY : m + log(s);
+  o->best = best;
+}
+
+// A launch that begins while the one before it drains (chain_enter waits for it).
+template <class... KArgs, class... Args>
+int launch_after(void (*kernel)(KArgs...), dim3 grid, cudaStream_t s, Args... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(TB);
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  FST_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return FST_OK;
 }
 
 struct DevGuard {
@@ -314,15 +410,16 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
   const int64_t Q = f->Q, QQ = Q * Q;
   int rc;
   Scratch mem;
-  struct Out {
+  struct {
     double logz;
     float best, pad;
   } h;
   if (n == 0) {
     if ((rc = mem.take(f, Scratch::piece(sizeof(Out))))) return rc;
     Out* d_out = mem.get<Out>(1);
-    k_close<<<1, TB, 0, s>>>(nullptr, nullptr, f->Q, f->theta_s, f->theta_f, &d_out->logz, &d_out->best);
-    FST_CUDA(cudaGetLastError());
+    if ((rc = launch_after(k_close, dim3(1), s, (const float*)nullptr, (const float*)nullptr, f->Q,
+                           (const float*)f->theta_s, (const float*)f->theta_f, d_out)))
+      return rc;
     FST_CUDA(cudaMemcpy(&h, d_out, sizeof(h), cudaMemcpyDeviceToHost));
   } else {
     SliceView sv;
@@ -351,7 +448,7 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
     float* buf_m[2] = {mem.get<float>(l1 * QQ), mem.get<float>(l2 * QQ)};
     FST_CUDA(cudaMemcpyAsync(d_slot, up.data(), up.size() * 4, cudaMemcpyHostToDevice, s));
     k_fill<<<(unsigned)std::min<int64_t>((2 * U * QQ + TB - 1) / TB, 8 * (int64_t)f->num_sms), TB, 0, s>>>(
-        dsum, 2 * U * QQ, -INFINITY);
+        dsum, 2 * U * QQ, -INFINITY, &d_out->done);
     for (int64_t u0 = 0; u0 < U; u0 += 65535)
       k_dense<<<dim3((unsigned)std::min<int64_t>((longest + TB - 1) / TB, 64), (unsigned)std::min<int64_t>(65535, U - u0)),
                 TB, 0, s>>>(sv.arcs, sv.theta, slice_sym_win(f), d_slot + n + u0, f->Q, dsum + u0 * QQ,
@@ -361,23 +458,28 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
     const float *cur_s = dsum, *cur_m = dmax;
     const int32_t* slot = d_slot;
     int64_t count = n;
-    const int32_t tiles = (int32_t)((Q + TILE - 1) / TILE);
     for (int level = 0; count > 1 || slot; ++level) {
       float *out_s = buf_s[level & 1], *out_m = buf_m[level & 1];
       const int64_t pairs = (count + 1) / 2;
       for (int64_t p0 = 0; p0 < pairs; p0 += 65535) {
         const int64_t cnt = std::min<int64_t>(65535, pairs - p0);
-        k_mul<<<dim3((unsigned)(tiles * tiles), (unsigned)cnt, 2), TB, 0, s>>>(
-            slot ? cur_s : cur_s + 2 * p0 * QQ, slot ? cur_m : cur_m + 2 * p0 * QQ, slot ? slot + 2 * p0 : nullptr,
-            (int32_t)(count - 2 * p0), out_s + p0 * QQ, out_m + p0 * QQ, f->Q);
+        const MulArgs M{slot ? cur_s : cur_s + 2 * p0 * QQ, slot ? cur_m : cur_m + 2 * p0 * QQ,
+                        slot ? slot + 2 * p0 : nullptr, out_s + p0 * QQ, out_m + p0 * QQ, (int32_t)(count - 2 * p0), f->Q};
+        const int32_t t64 = (f->Q + 63) / 64, t32 = (f->Q + 31) / 32;
+        // (the large tiles once they fill every SM twice)
+        rc = 2 * cnt * t64 * t64 >= 2 * f->num_sms
+                 ? launch_after(k_mul<64>, dim3((unsigned)(t64 * t64), (unsigned)cnt, 2), s, M)
+                 : launch_after(k_mul<32>, dim3((unsigned)(t32 * t32), (unsigned)cnt, 2), s, M);
+        if (rc) return rc;
       }
       cur_s = out_s;
       cur_m = out_m;
       slot = nullptr;
       count = pairs;
     }
-    k_close<<<1, TB, 0, s>>>(cur_s, cur_m, f->Q, f->theta_s, f->theta_f, &d_out->logz, &d_out->best);
-    FST_CUDA(cudaGetLastError());
+    if ((rc = launch_after(k_close, dim3((unsigned)std::min<int64_t>((Q + 7) / 8, CLOSE_BLOCKS)), s, cur_s, cur_m, f->Q,
+                           (const float*)f->theta_s, (const float*)f->theta_f, d_out)))
+      return rc;
     FST_CUDA(cudaMemcpy(&h, d_out, sizeof(h), cudaMemcpyDeviceToHost));
   }
   *log_z = h.logz;
