@@ -60,6 +60,31 @@ __device__ __forceinline__ int32_t edge_of(const EdgeView& G, int32_t lo, int32_
   return lo;
 }
 
+// One flat arc of a node's edges: its edge, record and weight.  None of it
+// changes during a call, so a chained launch reads its first ones before it
+// waits for the launch before it.
+struct FlatArc {
+  EdgeRec e;
+  int4 a;
+  float th;
+};
+__device__ __forceinline__ FlatArc flat_arc(const EdgeView& G, int32_t lo, int32_t hi, const int4* __restrict__ arcs,
+                                            const float* __restrict__ theta, int64_t x) {
+  FlatArc f;
+  const int32_t j = edge_of(G, lo, hi, x);
+  f.e = G.e[j];
+  const int64_t i = f.e.i0 + (x - __ldg(G.pre + j));
+  f.a = __ldg(arcs + i);
+  f.th = __ldg(theta + i);
+  return f;
+}
+// The launch after this one may begin (it waits for this one's end, and so
+// for all before), and this one's inputs are there.
+__device__ __forceinline__ void chain_through() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Start node: the start weights as keys (no incoming arc: low word 0).
 __global__ void k_lat_vit_init(const float* __restrict__ theta_s, int32_t Q, unsigned long long* __restrict__ keys0) {
   const int32_t q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -73,19 +98,22 @@ __global__ void k_lat_vit_init(const float* __restrict__ theta_s, int32_t Q, uns
 __global__ void __launch_bounds__(TB) k_lat_vit_node(EdgeView G, int32_t lo, int32_t hi,
                                                      const int4* __restrict__ arcs, const float* __restrict__ theta,
                                                      int32_t Q, unsigned long long* __restrict__ keys) {
-  chain_enter();
-  const int64_t p0 = __ldg(G.pre + lo), p1 = __ldg(G.pre + hi);
-  for (int64_t x = p0 + (int64_t)blockIdx.x * TB + threadIdx.x; x < p1; x += (int64_t)gridDim.x * TB) {
-    const int32_t j = edge_of(G, lo, hi, x);
-    const EdgeRec e = G.e[j];
-    const int64_t i = e.i0 + (x - __ldg(G.pre + j));
-    const int4 a = __ldg(arcs + i);
-    if (a.z < 0) continue;
-    const unsigned long long kp = keys[(int64_t)e.from * Q + a.x];
-    if (!kp) continue;
-    const float c = __fadd_rn(__fadd_rn(fkey_inv((uint32_t)(kp >> 32)), __ldg(theta + i)), e.w);
-    if (c == neg_inf()) continue;
-    atomicMax(keys + (int64_t)e.to * Q + a.y, ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)a.z));
+  const int64_t p1 = __ldg(G.pre + hi), step = (int64_t)gridDim.x * TB;
+  int64_t x = __ldg(G.pre + lo) + (int64_t)blockIdx.x * TB + threadIdx.x;
+  FlatArc f{};
+  if (x < p1) f = flat_arc(G, lo, hi, arcs, theta, x);
+  chain_through();
+  while (x < p1) {
+    if (f.a.z >= 0) {
+      const unsigned long long kp = __ldcg(keys + (int64_t)f.e.from * Q + f.a.x);
+      if (kp) {
+        const float c = __fadd_rn(__fadd_rn(fkey_inv((uint32_t)(kp >> 32)), f.th), f.e.w);
+        if (c != neg_inf())
+          atomicMax(keys + (int64_t)f.e.to * Q + f.a.y,
+                    ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)f.a.z));
+      }
+    }
+    if ((x += step) < p1) f = flat_arc(G, lo, hi, arcs, theta, x);
   }
 }
 
@@ -93,23 +121,25 @@ __device__ __forceinline__ float key_score(unsigned long long k) {
   return k ? fkey_inv((uint32_t)(k >> 32)) : neg_inf();
 }
 
-// Best end state (lowest id on ties), then the backtrace by warp 0: at node
-// v in state q the key names the best arc k; the edge is the lowest id into
-// v that reads k's symbol (k is among its source's arcs on the edge's symbol)
-// and reaches the same score through it -- a lane per edge.  At most N-1
-// steps (each moves to a lower node).  out: score, path length, the edges,
-// the arcs (both from the end back).
-__global__ void __launch_bounds__(1024) k_lat_vit_final(LayoutView L, EdgeView G, const int32_t* __restrict__ in_off,
-                                                        const int32_t* __restrict__ elabel,
-                                                        const unsigned long long* __restrict__ keys, int32_t N,
-                                                        int32_t Q, const float* __restrict__ theta_f,
-                                                        const int32_t* __restrict__ src_by_id,
-                                                        int32_t* __restrict__ out) {
-  __shared__ unsigned long long red[32];
+// Best end state (lowest id on ties), over all blocks, then the backtrace by
+// a warp of the last of them: at node v in state q the key names the best arc
+// k; the edge is the lowest id into v that reads k's symbol (k is among its
+// source's arcs on the edge's symbol) and reaches the same score through it
+// -- a lane per edge.  At most N-1 steps (each moves to a lower node).
+// out: score, path length, the edges, the arcs (both from the end back).
+// end: {best key, blocks done}, both 0 before.  (One block over 50,000 states
+// and 30 nodes took 108 us, most of it the states.)
+__global__ void __launch_bounds__(TB) k_lat_vit_final(LayoutView L, EdgeView G, const int32_t* __restrict__ in_off,
+                                                      const int32_t* __restrict__ elabel,
+                                                      const unsigned long long* __restrict__ keys, int32_t N,
+                                                      int32_t Q, const float* __restrict__ theta_f,
+                                                      const int32_t* __restrict__ src_by_id,
+                                                      unsigned long long* __restrict__ end, int32_t* __restrict__ out) {
+  __shared__ unsigned long long red[TB / 32];
   const int lane = threadIdx.x & 31;
   const unsigned long long* last = keys + (int64_t)(N - 1) * Q;
   unsigned long long best = 0ull;
-  for (int32_t q = threadIdx.x; q < Q; q += blockDim.x) {
+  for (int32_t q = (int32_t)(blockIdx.x * TB + threadIdx.x); q < Q; q += (int32_t)(gridDim.x * TB)) {
     const float c = __fadd_rn(key_score(last[q]), theta_f[q]);
     if (c == neg_inf()) continue;
     const unsigned long long k = ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)q);
@@ -123,12 +153,18 @@ __global__ void __launch_bounds__(1024) k_lat_vit_final(LayoutView L, EdgeView G
   if (lane == 0) red[threadIdx.x >> 5] = best;
   __syncthreads();
   if (threadIdx.x >= 32) return;
-  best = lane < (int)(blockDim.x >> 5) ? red[lane] : 0ull;
-#pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) {
-    const unsigned long long o = __shfl_xor_sync(FULL, best, d);
-    best = o > best ? o : best;
+  if (lane == 0) {
+    for (int w = 1; w < TB / 32; ++w) best = red[w] > best ? red[w] : best;
+    if (best) atomicMax(end, best);
+    __threadfence();
+    const bool done = atomicAdd(end + 1, 1ull) + 1ull == gridDim.x;
+    __threadfence();
+    red[0] = done ? 1ull : 0ull;
+    red[1] = __ldcg(end);
   }
+  __syncwarp();
+  if (!red[0]) return;
+  best = red[1];
   int32_t* edge_path = out + 2;
   int32_t* arc_path = edge_path + (N > 1 ? N - 1 : 1);
   int32_t len = 0;
@@ -137,23 +173,29 @@ __global__ void __launch_bounds__(1024) k_lat_vit_final(LayoutView L, EdgeView G
     for (int32_t step = 0; step < N - 1 && v != 0; ++step) {
       const unsigned long long kv = keys[(int64_t)v * Q + q];
       const int32_t k = (int32_t)(~(uint32_t)kv);
+      const int32_t lo = __ldg(in_off + v), hi = __ldg(in_off + v + 1);
       if (!kv || k < 0) { len = -1; break; }
       const float s = key_score(kv);
       const int32_t src = __ldg(src_by_id + k);
       int32_t e_best = -1, from = 0;
-      const int32_t lo = __ldg(in_off + v), hi = __ldg(in_off + v + 1);
       for (int32_t j0 = lo; j0 < hi && e_best < 0; j0 += 32) {  // edges into v, by increasing id
         const int32_t j = j0 + lane;
         bool hit = false;
         EdgeRec e{0, 0, 0, 0, 0.f};
         if (j < hi) {
           e = G.e[j];
+          SegProbe<true> pr;
+          seg_load(L, __ldg(elabel + e.id), src, pr);
           const float vu = key_score(keys[(int64_t)e.from * Q + src]);
-          const Arcs r = find_arcs(L, __ldg(elabel + e.id), src);
+          int4 a = make_int4(0, 0, -1, 0);
+          const Arcs r = seg_find(L, pr, &a);
           if (vu != neg_inf())
             for (int32_t i = 0; i < r.len; ++i) {
-              const int4 a = __ldg(L.arcs + r.pos + i);
-              if (a.z == k) hit = __fadd_rn(__fadd_rn(vu, __int_as_float(a.y)), e.w) == s;
+              if (i > 0) a = __ldg(L.arcs + r.pos + i);
+              if (a.z == k) {
+                hit = __fadd_rn(__fadd_rn(vu, __int_as_float(a.y)), e.w) == s;
+                break;
+              }
             }
         }
         const uint32_t hits = __ballot_sync(FULL, hit);
@@ -193,67 +235,103 @@ __global__ void k_lat_lse_init(const float* __restrict__ in, int32_t Q, ulonglon
   tab[q] = v == neg_inf() ? make_ulonglong2(0ull, 0ull) : make_ulonglong2(1099511627776ull, dkey((double)v));  // 2^40
 }
 
-// Forward (or backward) relaxation of all edges [lo, hi) into (out of) a
-// node, in two phases: the exact maximum of each target, then the
-// fixed-point sums.
-// FWD: target = destination, value = tab[from][src] + w + theta;
-// else: target = source, value = tab[to][dst] + w + theta.
-template <bool FWD, bool SUM>
-__global__ void __launch_bounds__(TB) k_lat_lse_node(EdgeView G, int32_t lo, int32_t hi,
+// Step by step both passes at once: the forward relaxation of all edges into
+// a node (F.lo .. F.hi of its edges) and the backward one of all edges out of
+// another (B), which need nothing of each other.  Two phases a step: the
+// exact maximum of each target, then the fixed-point sums.
+// Forward: target = destination, value = tab[from][src] + w + theta;
+// backward: target = source, value = tab[to][dst] + w + theta.
+// A launch is bound by its own latency (a lookup, a value, an atomic); with
+// the passes one after the other a call on 30 nodes took 116 of them, now 58.
+struct StepSide {
+  EdgeView G;
+  int32_t lo, hi;
+  int64_t n;  // flat arcs
+  ulonglong2* tab;
+};
+template <bool SUM>
+__device__ __forceinline__ void lse_arc(const FlatArc& f, bool fwd, ulonglong2* tab, int32_t Q) {
+  if (f.a.z < 0 || dead32(f.th)) return;
+  const double u = lse_value(tab, (int64_t)(fwd ? f.e.from : f.e.to) * Q + (fwd ? f.a.x : f.a.y));
+  if (dead64(u)) return;
+  const double v = u + (double)f.e.w + (double)f.th;
+  if (dead64(v)) return;
+  unsigned long long* t = (unsigned long long*)(tab + (int64_t)(fwd ? f.e.to : f.e.from) * Q + (fwd ? f.a.y : f.a.x));
+  if (!SUM) atomicMax(t + 1, dkey(v));
+  else atomicAdd(t, fix_exp64(v, dkey_inv(__ldcg(t + 1))));
+}
+template <bool SUM>
+__global__ void __launch_bounds__(TB) k_lat_lse_step(const __grid_constant__ StepSide F,
+                                                     const __grid_constant__ StepSide B,
                                                      const int4* __restrict__ arcs, const float* __restrict__ theta,
-                                                     int32_t Q, ulonglong2* __restrict__ tab) {
-  chain_enter();
-  const int64_t p0 = __ldg(G.pre + lo), p1 = __ldg(G.pre + hi);
-  for (int64_t x = p0 + (int64_t)blockIdx.x * TB + threadIdx.x; x < p1; x += (int64_t)gridDim.x * TB) {
-    const int32_t j = edge_of(G, lo, hi, x);
-    const EdgeRec e = G.e[j];
-    const int64_t i = e.i0 + (x - __ldg(G.pre + j));
-    const int4 a = __ldg(arcs + i);
-    if (a.z < 0) continue;
-    const float th = __ldg(theta + i);
-    if (dead32(th)) continue;
-    const double u = lse_value(tab, (int64_t)(FWD ? e.from : e.to) * Q + (FWD ? a.x : a.y));
-    if (dead64(u)) continue;
-    const double v = u + (double)e.w + (double)th;
-    if (dead64(v)) continue;
-    unsigned long long* t = (unsigned long long*)(tab + (int64_t)(FWD ? e.to : e.from) * Q + (FWD ? a.y : a.x));
-    if (!SUM) atomicMax(t + 1, dkey(v));
-    else atomicAdd(t, fix_exp64(v, dkey_inv(__ldcg(t + 1))));
+                                                     int32_t Q) {
+  // (the sides have whole 128-arc windows: a warp's arcs are one side's)
+  const int64_t n = F.n + B.n, step = (int64_t)gridDim.x * TB;
+  int64_t x = (int64_t)blockIdx.x * TB + threadIdx.x;
+  auto get = [&]() {
+    return x < F.n ? flat_arc(F.G, F.lo, F.hi, arcs, theta, __ldg(F.G.pre + F.lo) + x)
+                   : flat_arc(B.G, B.lo, B.hi, arcs, theta, __ldg(B.G.pre + B.lo) + x - F.n);
+  };
+  FlatArc f{};
+  if (x < n) f = get();
+  chain_through();
+  while (x < n) {
+    const bool fwd = x < F.n;
+    lse_arc<SUM>(f, fwd, fwd ? F.tab : B.tab, Q);
+    if ((x += step) < n) f = get();
   }
 }
 
-// log Z = LSE_q(alpha_end[q] + theta_f[q]) in float64 (one block).
-__global__ void __launch_bounds__(1024) k_lat_logz(const ulonglong2* __restrict__ end, const float* __restrict__ theta_f,
-                                                   int32_t Q, double* __restrict__ logz) {
+// log Z = LSE_q(alpha_end[q] + theta_f[q]) in float64: every block a part
+// (its largest value and the sum of the exponentials below it), the last of
+// them the parts in their order.  (One block over 50,000 states took 113 us.)
+struct LogzPart {
+  double m, s;
+};
+constexpr int LOGZ_BLOCKS = 128;
+__global__ void __launch_bounds__(TB) k_lat_logz(const ulonglong2* __restrict__ end, const float* __restrict__ theta_f,
+                                                 int32_t Q, LogzPart* __restrict__ part, uint32_t* __restrict__ done,
+                                                 double* __restrict__ logz) {
   chain_enter();
-  __shared__ double red[32];
-  const int nw = blockDim.x >> 5;
-  double m = -INFINITY;
-  for (int32_t q = threadIdx.x; q < Q; q += blockDim.x)
-    if (!dead32(theta_f[q])) m = fmax(m, lse_value(end, q) + (double)theta_f[q]);
+  __shared__ double red[TB / 32];
+  auto over = [&](double x, bool sum) {  // the block's largest value, or its sum
 #pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) m = fmax(m, __shfl_xor_sync(FULL, m, d));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  m = red[0];
-  for (int w = 1; w < nw; ++w) m = fmax(m, red[w]);
-  __syncthreads();
-  double s = 0.0;
+    for (int d = 16; d >= 1; d >>= 1) {
+      const double y = __shfl_xor_sync(FULL, x, d);
+      x = sum ? x + y : fmax(x, y);
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+    __syncthreads();
+    x = red[0];
+    for (int w = 1; w < TB / 32; ++w) x = sum ? x + red[w] : fmax(x, red[w]);
+    return x;
+  };
+  auto value = [&](int32_t q) { return dead32(theta_f[q]) ? -INFINITY : lse_value(end, q) + (double)theta_f[q]; };
+  const int32_t q0 = (int32_t)(blockIdx.x * TB + threadIdx.x), step = (int32_t)(gridDim.x * TB);
+  double m = -INFINITY, s = 0.0;
+  for (int32_t q = q0; q < Q; q += step) m = fmax(m, value(q));
+  m = over(m, false);
   if (m != -INFINITY)
-    for (int32_t q = threadIdx.x; q < Q; q += blockDim.x) {
-      if (dead32(theta_f[q])) continue;
-      const double v = lse_value(end, q) + (double)theta_f[q];
+    for (int32_t q = q0; q < Q; q += step) {
+      const double v = value(q);
       if (!dead64(v)) s += exp(v - m);
     }
-#pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(FULL, s, d);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
+  s = over(s, true);
+  __shared__ bool last;
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += red[w];
-    *logz = m == -INFINITY ? -INFINITY : m + log(t);
+    part[blockIdx.x] = LogzPart{m, s};
+    __threadfence();
+    last = atomicAdd(done, 1u) + 1u == gridDim.x;
+    __threadfence();
   }
+  __syncthreads();
+  if (!last) return;
+  const bool mine = threadIdx.x < gridDim.x;  // (a thread a part)
+  const double pm = mine ? __ldcg(&part[threadIdx.x].m) : -INFINITY, ps = mine ? __ldcg(&part[threadIdx.x].s) : 0.0;
+  m = over(pm, false);
+  s = over(m == -INFINITY || pm == -INFINITY ? 0.0 : pm == m ? ps : ps * exp(pm - m), true);
+  if (threadIdx.x == 0) *logz = m == -INFINITY ? -INFINITY : m + log(s);
 }
 
 // Posteriors through every edge: exp(alpha[u][src] + w + theta + beta[v][dst]
@@ -261,19 +339,18 @@ __global__ void __launch_bounds__(1024) k_lat_logz(const ulonglong2* __restrict_
 __global__ void __launch_bounds__(TB) k_lat_post(EdgeView G, int32_t E, const int4* __restrict__ arcs,
                                                  const float* __restrict__ theta, int32_t Q,
                                                  const ulonglong2* __restrict__ alpha,
-                                                 const ulonglong2* __restrict__ beta, const double* __restrict__ logz,
+                                                 const ulonglong2* __restrict__ beta, const double* logz,
                                                  double* __restrict__ cnt, double* __restrict__ epost) {
   chain_enter();
-  const double lz = *logz;
+  const double lz = __ldcg(logz);
   if (lz == -INFINITY) return;
   const int64_t p1 = __ldg(G.pre + E);
   // (whole warps: p1 is a multiple of 128)
   for (int64_t x = (int64_t)blockIdx.x * TB + threadIdx.x; x < p1; x += (int64_t)gridDim.x * TB) {
-    const int32_t j = edge_of(G, 0, E, x);
-    const EdgeRec e = G.e[j];
-    const int64_t i = e.i0 + (x - __ldg(G.pre + j));
-    const int4 a = __ldg(arcs + i);
-    const float th = __ldg(theta + i);
+    const FlatArc f = flat_arc(G, 0, E, arcs, theta, x);
+    const EdgeRec& e = f.e;
+    const int4 a = f.a;
+    const float th = f.th;
     double g = 0.0;
     if (a.z >= 0 && !dead32(th)) {
       const double al = lse_value(alpha, (int64_t)e.from * Q + a.x);
@@ -378,14 +455,16 @@ struct EdgeTables {
   }
 };
 
-// A launch over n flat arcs, chained to the one before it.
+// A launch over n flat arcs, chained to the one before it; half the blocks
+// an SM holds, so that the next launch's fit beside them.
+constexpr int LAT_BLOCKS = 4;
 template <class... KArgs, class... Args>
 int launch_arcs(void (*kernel)(KArgs...), int64_t n, int num_sms, cudaStream_t s, Args... args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + TB - 1) / TB, 8 * (int64_t)num_sms)));
+  cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + TB - 1) / TB, LAT_BLOCKS * (int64_t)num_sms)));
   cfg.blockDim = dim3(TB);
   cfg.stream = s;
   cfg.attrs = at;
@@ -414,11 +493,11 @@ extern "C" int fst_lattice_viterbi(fst_t* f, int32_t num_nodes, int32_t num_edge
   EdgeTables T;
   T.add(sv, H.in_edge, num_edges, from, to, label, weight);
   Scratch mem;
-  if ((rc = mem.take(f, Scratch::piece(N * Q * 8) + Scratch::piece(E * (int64_t)sizeof(EdgeRec)) +
+  if ((rc = mem.take(f, Scratch::piece((N * Q + 2) * 8) + Scratch::piece(E * (int64_t)sizeof(EdgeRec)) +
                             Scratch::piece((E + 1) * 8) + Scratch::piece((N + 1) * 4) + Scratch::piece(E * 4) +
                             Scratch::piece((2 + 2 * np) * 4))))
     return rc;
-  unsigned long long* keys = mem.get<unsigned long long>(N * Q);
+  unsigned long long* keys = mem.get<unsigned long long>(N * Q + 2);
   EdgeRec* d_e = mem.get<EdgeRec>(E);
   int64_t* d_pre = mem.get<int64_t>(E + 1);
   int32_t* d_in = mem.get<int32_t>(N + 1);
@@ -430,7 +509,7 @@ extern "C" int fst_lattice_viterbi(fst_t* f, int32_t num_nodes, int32_t num_edge
   }
   FST_CUDA(cudaMemcpyAsync(d_pre, T.pre.data(), (size_t)(E + 1) * 8, cudaMemcpyHostToDevice, s));
   FST_CUDA(cudaMemcpyAsync(d_in, H.in_off.data(), (size_t)(N + 1) * 4, cudaMemcpyHostToDevice, s));
-  FST_CUDA(cudaMemsetAsync(keys, 0, (size_t)(N * Q) * 8, s));
+  FST_CUDA(cudaMemsetAsync(keys, 0, (size_t)(N * Q + 2) * 8, s));
   const EdgeView G{d_e, d_pre};
   k_lat_vit_init<<<nb(Q), TB, 0, s>>>(f->theta_s, f->Q, keys);
   // node by node: every edge into v
@@ -439,8 +518,8 @@ extern "C" int fst_lattice_viterbi(fst_t* f, int32_t num_nodes, int32_t num_edge
     const int64_t n = T.pre[hi] - T.pre[lo];
     if (n && (rc = launch_arcs(k_lat_vit_node, n, f->num_sms, s, G, lo, hi, sv.arcs, sv.theta, f->Q, keys))) return rc;
   }
-  k_lat_vit_final<<<1, 1024, 0, s>>>(view_of(f->bwd), G, d_in, d_label, keys, num_nodes, f->Q, f->theta_f,
-                                     f->src_by_id, d_out);
+  k_lat_vit_final<<<std::min(nb(Q), (unsigned)f->num_sms), TB, 0, s>>>(view_of(f->bwd), G, d_in, d_label, keys, num_nodes,
+                                                                       f->Q, f->theta_f, f->src_by_id, keys + N * Q, d_out);
   FST_CUDA(cudaGetLastError());
   std::vector<int32_t> h((size_t)(2 + 2 * np));
   FST_CUDA(cudaMemcpy(h.data(), d_out, h.size() * 4, cudaMemcpyDeviceToHost));
@@ -481,48 +560,46 @@ extern "C" int fst_lattice_forward_backward(fst_t* f, int32_t num_nodes, int32_t
   EdgeTables T;  // by destination node, then by source node
   T.add(sv, H.in_edge, num_edges, from, to, label, weight);
   T.add(sv, H.out_edge, num_edges, from, to, label, weight);
-  // the values of both passes, log Z, and the counts of the arcs and the
-  // posteriors of the edges side by side, as float64 and as float32
+  // the values of both passes, log Z (with its count of finished blocks and
+  // their parts), and the counts of the arcs and the posteriors of the edges
+  // side by side, as float64 and as float32
   Scratch mem;
-  if ((rc = mem.take(f, Scratch::piece((2 * N * Q + (A + E + 2) / 2) * 16) + Scratch::piece((A + E) * 4 + 8) +
+  if ((rc = mem.take(f, Scratch::piece((2 * N * Q + (A + E + 3) / 2) * 16) + Scratch::piece((A + E) * 4 + 8) +
+                            Scratch::piece(LOGZ_BLOCKS * (int64_t)sizeof(LogzPart)) +
                             Scratch::piece(2 * E * (int64_t)sizeof(EdgeRec)) + Scratch::piece(2 * (E + 1) * 8))))
     return rc;
-  ulonglong2* alpha = mem.get<ulonglong2>(2 * N * Q + (A + E + 2) / 2);
+  ulonglong2* alpha = mem.get<ulonglong2>(2 * N * Q + (A + E + 3) / 2);
   ulonglong2* beta = alpha + N * Q;
   double* d_logz = (double*)(beta + N * Q);
-  double* cnt = d_logz + 1;
+  uint32_t* d_done = (uint32_t*)(d_logz + 1);
+  double* cnt = d_logz + 2;
   double* epost = cnt + A;
   float* out = mem.get<float>(A + E + 2);
+  LogzPart* d_part = mem.get<LogzPart>(LOGZ_BLOCKS);
   EdgeRec* d_e = mem.get<EdgeRec>(2 * E);
   int64_t* d_pre = mem.get<int64_t>(2 * (E + 1));
-  FST_CUDA(cudaMemsetAsync(alpha, 0, (size_t)(2 * N * Q) * 16 + 8 + (size_t)(A + E) * 8, s));
+  FST_CUDA(cudaMemsetAsync(alpha, 0, (size_t)(2 * N * Q) * 16 + 16 + (size_t)(A + E) * 8, s));
   if (E > 0) FST_CUDA(cudaMemcpyAsync(d_e, T.e.data(), (size_t)(2 * E) * sizeof(EdgeRec), cudaMemcpyHostToDevice, s));
   FST_CUDA(cudaMemcpyAsync(d_pre, T.pre.data(), (size_t)(2 * (E + 1)) * 8, cudaMemcpyHostToDevice, s));
   const EdgeView Gi{d_e, d_pre}, Go{d_e + E, d_pre + E + 1};
   const int64_t* pi = T.pre.data();
   const int64_t* po = T.pre.data() + E + 1;
-  // forward, node by node
+  // node by node, forward and (for the posteriors) backward from the end
+  const bool post = arc_posteriors || edge_posteriors;
   k_lat_lse_init<<<nb(Q), TB, 0, s>>>(f->theta_s, f->Q, alpha);
+  if (post) k_lat_lse_init<<<nb(Q), TB, 0, s>>>(f->theta_f, f->Q, beta + (N - 1) * Q);
   for (int32_t v = 1; v < N; ++v) {
-    const int32_t lo = H.in_off[v], hi = H.in_off[v + 1];
-    const int64_t n = pi[hi] - pi[lo];
-    if (!n) continue;
-    if ((rc = launch_arcs(k_lat_lse_node<true, false>, n, f->num_sms, s, Gi, lo, hi, sv.arcs, sv.theta, f->Q, alpha)) ||
-        (rc = launch_arcs(k_lat_lse_node<true, true>, n, f->num_sms, s, Gi, lo, hi, sv.arcs, sv.theta, f->Q, alpha)))
+    const int32_t u = num_nodes - 1 - v;
+    const StepSide F{Gi, H.in_off[v], H.in_off[v + 1], pi[H.in_off[v + 1]] - pi[H.in_off[v]], alpha};
+    const StepSide B{Go, H.out_off[u], H.out_off[u + 1], post ? po[H.out_off[u + 1]] - po[H.out_off[u]] : 0, beta};
+    if (F.n + B.n == 0) continue;
+    if ((rc = launch_arcs(k_lat_lse_step<false>, F.n + B.n, f->num_sms, s, F, B, sv.arcs, sv.theta, f->Q)) ||
+        (rc = launch_arcs(k_lat_lse_step<true>, F.n + B.n, f->num_sms, s, F, B, sv.arcs, sv.theta, f->Q)))
       return rc;
   }
-  k_lat_logz<<<1, 1024, 0, s>>>(alpha + (N - 1) * Q, f->theta_f, f->Q, d_logz);
-  if (arc_posteriors || edge_posteriors) {
-    // backward, from the end node
-    k_lat_lse_init<<<nb(Q), TB, 0, s>>>(f->theta_f, f->Q, beta + (N - 1) * Q);
-    for (int32_t v = num_nodes - 2; v >= 0; --v) {
-      const int32_t lo = H.out_off[v], hi = H.out_off[v + 1];
-      const int64_t n = po[hi] - po[lo];
-      if (!n) continue;
-      if ((rc = launch_arcs(k_lat_lse_node<false, false>, n, f->num_sms, s, Go, lo, hi, sv.arcs, sv.theta, f->Q, beta)) ||
-          (rc = launch_arcs(k_lat_lse_node<false, true>, n, f->num_sms, s, Go, lo, hi, sv.arcs, sv.theta, f->Q, beta)))
-        return rc;
-    }
+  k_lat_logz<<<std::min(nb(Q), (unsigned)LOGZ_BLOCKS), TB, 0, s>>>(alpha + (N - 1) * Q, f->theta_f, f->Q, d_part, d_done,
+                                                                    d_logz);
+  if (post) {
     if (pi[E] && (rc = launch_arcs(k_lat_post, pi[E], f->num_sms, s, Gi, num_edges, sv.arcs, sv.theta, f->Q, alpha, beta,
                                    d_logz, cnt, epost)))
       return rc;
