@@ -171,7 +171,8 @@ struct PlainWs {
   unsigned long long* acc = nullptr;    // [2][Q] x 2 words (sum, maximum), zero between runs
   double* beta = nullptr;               // [2][Q] backward values
   int32_t* vmap = nullptr;              // [2][Q]
-  int32_t *tok_sym = nullptr, *tok_b = nullptr;
+  int32_t* tokens = nullptr;            // [1 + cap_n] the length and the symbols: one upload
+  int32_t *bw_n = nullptr, *tok_sym = nullptr, *tok_b = nullptr;
   int32_t* iota = nullptr;              // step list: token t-1 is the only slot of position t
   int32_t* step0 = nullptr;             // [cap_n + 2] step offsets of the persistent passes: step0[t] = t - 1
   uint32_t* gbar = nullptr;             // [2] grid barrier of the persistent passes
@@ -182,27 +183,40 @@ struct PlainWs {
   int32_t* pool_cnt = nullptr;
   uint32_t *mkey = nullptr, *ekey = nullptr;
   double *csum = nullptr, *esum = nullptr;
-  int32_t *paths = nullptr, *olabels = nullptr;
+  // [4 + 2 cap_n] log Z (two words), status, score, path, output labels: one
+  // download of the first 4 + 2 n (olabels stands at 4 + n for a call of n)
+  int32_t* result = nullptr;
+  double* logz = nullptr;
+  int32_t *status = nullptr, *paths = nullptr, *olabels = nullptr;
+  float* score = nullptr;
   int64_t cap_n = 0;
   int32_t *stage = nullptr, *stage_b = nullptr;
   int64_t cap_stage = 0;
   int32_t *pool_q = nullptr, *pool_x = nullptr, *pool_n = nullptr;
   double* pool_v = nullptr;             // Viterbi scores (float32) or forward values (float64)
   int64_t cap_pool = 0;
-  float *cnt = nullptr, *comp = nullptr, *counts_out = nullptr;
-  int32_t *jfinal = nullptr, *status = nullptr, *bw_n = nullptr;
-  float* score = nullptr;
-  double* logz = nullptr;
+  float* counts_out = nullptr;
+  int32_t* jfinal = nullptr;
   int64_t* bw_off = nullptr;
   int64_t* pool_top = nullptr;
   uint32_t* flags = nullptr;
   bool last_fb = false;                 // the last call was forward-backward (pool_n holds arc counts)
+  // the string kernels' (plain_string): a string is their whole batch
+  uint32_t *str_ctl = nullptr, *str_dirty = nullptr;
+  double *str_kept = nullptr, *str_dval = nullptr;
+  unsigned long long *str_dense_v = nullptr, *str_dense_f = nullptr;
+  int32_t* str_stage = nullptr;
+  int2* str_fe = nullptr;
+  double* cnt64 = nullptr;
+  bool str_last = false;                // the last call took them
   ~PlainWs() {
-    dfree(acc); dfree(beta); dfree(vmap); dfree(tok_sym); dfree(tok_b); dfree(iota); dfree(zero64);
+    dfree(str_ctl); dfree(str_dirty); dfree(str_kept); dfree(str_dval); dfree(str_dense_v); dfree(str_dense_f);
+    dfree(str_stage); dfree(str_fe); dfree(cnt64);
+    dfree(acc); dfree(beta); dfree(vmap); dfree(tokens); dfree(tok_b); dfree(iota); dfree(zero64);
     dfree(step0); dfree(gbar); dfree(slot_base); dfree(step_rng); dfree(scnt); dfree(pool_base); dfree(pool_cnt); dfree(mkey); dfree(ekey);
-    dfree(csum); dfree(esum); dfree(paths); dfree(olabels); dfree(stage); dfree(stage_b); dfree(pool_q);
-    dfree(pool_x); dfree(pool_n); dfree(pool_v); dfree(cnt); dfree(comp); dfree(counts_out); dfree(jfinal); dfree(status);
-    dfree(bw_n); dfree(score); dfree(logz); dfree(bw_off); dfree(pool_top); dfree(flags);
+    dfree(csum); dfree(esum); dfree(result); dfree(stage); dfree(stage_b); dfree(pool_q);
+    dfree(pool_x); dfree(pool_n); dfree(pool_v); dfree(counts_out); dfree(jfinal);
+    dfree(bw_off); dfree(pool_top); dfree(flags);
   }
 };
 
@@ -215,8 +229,7 @@ int plain_init(fst_s* f) {
   const int64_t Q = f->Q;
   int rc;
   if ((rc = dalloc(&w->acc, 4 * Q)) || (rc = dalloc(&w->beta, 2 * Q)) || (rc = dalloc(&w->vmap, 2 * Q)) ||
-      (rc = dalloc(&w->jfinal, 1)) || (rc = dalloc(&w->status, 1)) || (rc = dalloc(&w->score, 1)) ||
-      (rc = dalloc(&w->logz, 1)) || (rc = dalloc(&w->bw_n, 1)) || (rc = dalloc(&w->bw_off, 1)) ||
+      (rc = dalloc(&w->jfinal, 1)) || (rc = dalloc(&w->bw_off, 1)) ||
       (rc = dalloc(&w->pool_top, 1)) || (rc = dalloc(&w->flags, 2)) || (rc = dalloc(&w->gbar, 2)))
     return rc;
   FST_CUDA(cudaMemset(w->acc, 0, (size_t)4 * Q * sizeof(unsigned long long)));
@@ -233,9 +246,9 @@ int plain_reserve(PlainWs* w, int64_t n, int64_t stage, int64_t pool) {
   int rc;
   if (n > w->cap_n) {
     const int64_t c = std::max<int64_t>(n, 2 * w->cap_n);
-    dfree(w->tok_sym); dfree(w->tok_b); dfree(w->iota); dfree(w->step0); dfree(w->zero64); dfree(w->slot_base);
+    dfree(w->tokens); dfree(w->tok_b); dfree(w->iota); dfree(w->step0); dfree(w->zero64); dfree(w->slot_base);
     dfree(w->step_rng); dfree(w->scnt); dfree(w->pool_base); dfree(w->pool_cnt); dfree(w->mkey); dfree(w->ekey);
-    dfree(w->csum); dfree(w->esum); dfree(w->paths); dfree(w->olabels);
+    dfree(w->csum); dfree(w->esum); dfree(w->result);
     w->cap_n = 0;
     if ((rc = dalloc(&w->iota, c)) || (rc = dalloc(&w->slot_base, c)) || (rc = dalloc(&w->step_rng, 2 * (c + 2))) ||
         (rc = dalloc(&w->step0, c + 2)))
@@ -247,11 +260,20 @@ int plain_reserve(PlainWs* w, int64_t n, int64_t stage, int64_t pool) {
       FST_CUDA(cudaMemcpy(w->iota, io.data(), (size_t)c * 4, cudaMemcpyHostToDevice));
       FST_CUDA(cudaMemcpy(w->step0, s0.data(), (size_t)(c + 2) * 4, cudaMemcpyHostToDevice));
     }
-    if ((rc = dalloc(&w->tok_sym, c)) || (rc = dalloc(&w->tok_b, c)) || (rc = dalloc(&w->zero64, c)) ||
+    if ((rc = dalloc(&w->tokens, 1 + c)) || (rc = dalloc(&w->tok_b, c)) || (rc = dalloc(&w->zero64, c)) ||
         (rc = dalloc(&w->scnt, c)) || (rc = dalloc(&w->pool_base, c)) || (rc = dalloc(&w->pool_cnt, c)) ||
         (rc = dalloc(&w->mkey, c)) || (rc = dalloc(&w->ekey, c)) || (rc = dalloc(&w->csum, c)) ||
-        (rc = dalloc(&w->esum, c)) || (rc = dalloc(&w->paths, c)) || (rc = dalloc(&w->olabels, c)))
+        (rc = dalloc(&w->esum, c)) || (rc = dalloc(&w->result, 4 + 2 * c)))
       return rc;
+    w->bw_n = w->tokens;
+    w->tok_sym = w->tokens + 1;
+    w->logz = (double*)w->result;
+    w->status = w->result + 2;
+    w->score = (float*)(w->result + 3);
+    w->paths = w->result + 4;
+    // (a run that stops early leaves the later positions' ranges as they were)
+    FST_CUDA(cudaMemset(w->pool_base, 0, (size_t)c * sizeof(int64_t)));
+    FST_CUDA(cudaMemset(w->pool_cnt, 0, (size_t)c * sizeof(int32_t)));
     FST_CUDA(cudaMemset(w->tok_b, 0, (size_t)c * sizeof(int32_t)));
     FST_CUDA(cudaMemset(w->zero64, 0, (size_t)c * sizeof(int64_t)));
     w->cap_n = c;
@@ -276,8 +298,10 @@ int plain_reserve(PlainWs* w, int64_t n, int64_t stage, int64_t pool) {
   return FST_OK;
 }
 
-// Upload the tokens of one string and start a run.
-int plain_tokens(fst_s* f, const int32_t* ids, int32_t n, cudaStream_t s) {
+// Upload the tokens of one string and start a run; *strings: it takes the
+// string kernels (the launch driver, unless the pool is past their 31-bit
+// entry numbers).
+int plain_tokens(fst_s* f, const int32_t* ids, int32_t n, cudaStream_t s, bool* strings) {
   PlainWs* w = f->plain;
   int64_t stage = 1, pool = 1;
   for (int32_t i = 0; i < n; ++i) {
@@ -289,16 +313,63 @@ int plain_tokens(fst_s* f, const int32_t* ids, int32_t n, cudaStream_t s) {
     stage = std::max(stage, D);
     pool += D;
   }
-  int rc = plain_reserve(w, std::max(n, 1), stage, pool);
+  // (what the chunks of a light warp and a heavy block may leave unused)
+  const int64_t spare = pool / 3 + 4 * POOL_CHUNK;
+  *strings = f->plain_fb_driver == FST_DRIVER_LAUNCH && pool + spare < INT32_MAX;
+  int rc = plain_reserve(w, std::max(n, 1), stage, *strings ? pool + spare : pool);
   if (rc) return rc;
+  w->olabels = w->paths + n;
+  w->str_last = *strings;
+  std::vector<int32_t> up((size_t)n + 1);
+  up[0] = n;
+  std::copy(ids, ids + n, up.begin() + 1);
+  FST_CUDA(cudaMemcpyAsync(w->tokens, up.data(), up.size() * 4, cudaMemcpyHostToDevice, s));
+  if (*strings) return FST_OK;
   const size_t n4 = (size_t)std::max(n, 1) * 4;
-  if (n > 0) FST_CUDA(cudaMemcpyAsync(w->tok_sym, ids, (size_t)n * 4, cudaMemcpyHostToDevice, s));
-  FST_CUDA(cudaMemcpyAsync(w->bw_n, &n, 4, cudaMemcpyHostToDevice, s));
   FST_CUDA(cudaMemsetAsync(w->scnt, 0, n4, s));
   FST_CUDA(cudaMemsetAsync(w->mkey, 0, n4, s));
   FST_CUDA(cudaMemsetAsync(w->ekey, 0, n4, s));
   FST_CUDA(cudaMemsetAsync(w->pool_top, 0, 8, s));
   FST_CUDA(cudaMemsetAsync(w->flags, 0, 8, s));
+  return FST_OK;
+}
+
+// Storage of the string kernels for one string: one heavy block owns dense
+// accumulators (the others help with its large positions).
+int plain_string(fst_s* f, bool viterbi, StringWork* K) {
+  PlainWs* w = f->plain;
+  const int64_t Q = f->Q;
+  int rc;
+  if (!w->str_ctl) {
+    const int64_t ctl = string_ctl_words(1, 1);
+    if ((rc = dalloc(&w->str_dirty, 2)) || (rc = dalloc(&w->str_kept, string_kept_values())) ||
+        (rc = dalloc(&w->str_stage, Q)))
+      return rc;
+    FST_CUDA(cudaMemset(w->str_dirty, 0, 8));
+    if ((rc = dalloc(&w->str_ctl, ctl))) return rc;
+    FST_CUDA(cudaMemset(w->str_ctl, 0, (size_t)ctl * 4));
+  }
+  if (viterbi && !w->str_dense_v) {
+    dfree(w->str_fe);
+    if ((rc = dalloc(&w->str_fe, Q + string_light_entries(f->num_sms))) || (rc = dalloc(&w->str_dense_v, Q))) return rc;
+    FST_CUDA(cudaMemset(w->str_dense_v, 0, (size_t)Q * 8));
+  }
+  if (!viterbi && !w->str_dense_f) {
+    dfree(w->str_dval);
+    if ((rc = dalloc(&w->str_dval, 2 * Q)) || (rc = dalloc(&w->str_dense_f, 2 * Q))) return rc;
+    FST_CUDA(cudaMemset(w->str_dense_f, 0, (size_t)Q * 16));
+  }
+  K->Bw = 1;
+  K->ctl = w->str_ctl;
+  K->dirty = w->str_dirty + (viterbi ? 0 : 1);
+  K->kept = w->str_kept;
+  K->dense = viterbi ? w->str_dense_v : w->str_dense_f;
+  K->dval = w->str_dval;
+  K->dstage = w->str_stage;
+  K->fe = w->str_fe;
+  K->fe_light = Q;
+  K->groups2 = 1;
+  K->chunk = POOL_CHUNK;
   return FST_OK;
 }
 
@@ -344,7 +415,27 @@ FrontierState plain_state(fst_s* f) {
   S.gweight = nullptr;
   S.bw_n = w->bw_n;
   S.bw_off = w->bw_off;
+  if (w->str_last) {
+    S.flags = w->str_ctl + CTL_FLAGS;
+    S.pool_top = (int64_t*)(w->str_ctl + CTL_TOP);
+  }
   return S;
+}
+// Log Z, status and score of a call, and `words` words of path after them.
+int plain_result(fst_s* f, int64_t words, std::vector<int32_t>* h) {
+  h->resize((size_t)(4 + words));
+  FST_CUDA(cudaMemcpy(h->data(), f->plain->result, h->size() * 4, cudaMemcpyDeviceToHost));
+  const int32_t st = (*h)[2];
+  if (st == FST_ERR_TIMEOUT) {
+    set_error(f->plain->str_last ? "a block of the string kernels waited too long for the others"
+                                 : "a grid barrier of the persistent pass timed out");
+    return FST_ERR_TIMEOUT;
+  }
+  if (st != FST_OK) {
+    set_error("no accepting path");
+    return FST_ERR_NO_PATH;
+  }
+  return FST_OK;
 }
 
 // The single token of position t (slot t-1); x_t names the other position
@@ -668,12 +759,17 @@ static int fst_viterbi_frontier(fst_t* f, const int32_t* ids, int32_t n, float* 
   int rc;
   if ((rc = plain_init(f))) return rc;
   cudaStream_t s = 0;
-  if ((rc = plain_tokens(f, ids, n, s))) return rc;
+  bool strings;
+  if ((rc = plain_tokens(f, ids, n, s, &strings))) return rc;
   PlainWs* w = f->plain;
+  StringWork K;
+  if (strings && (rc = plain_string(f, true, &K))) return rc;
   const LayoutView L = view_of(f->bwd);
   const TokenView T = plain_tokview(w);
   const FrontierState S = plain_state(f);
-  if (f->plain_fb_driver == FST_DRIVER_PERSISTENT && n >= 1) {
+  if (strings) {
+    PLAIN_PROF(FST_PROF_VIT_STEP, launch_string_forward(true, L, w->tok_sym, S, K, f->num_sms, s));
+  } else if (f->plain_fb_driver == FST_DRIVER_PERSISTENT && n >= 1) {
     // one cooperative launch for all positions
     const int32_t pgrid = std::max(1, std::min(f->plain_fb_grid > 0 ? f->plain_fb_grid : f->num_sms,
                                                persist_grid_limit(0)));
@@ -687,24 +783,16 @@ static int fst_viterbi_frontier(fst_t* f, const int32_t* ids, int32_t n, float* 
       PLAIN_PROF(FST_PROF_VIT_STEP, launch_vit_step(L, T, plain_step(f, n, t, t + 1), S, s));
   }
   PLAIN_PROF(FST_PROF_VIT_FINAL, launch_vit_final(S, 1, w->score, w->jfinal, w->status, s));
-  PLAIN_PROF(FST_PROF_BACKTRACE, launch_backtrace(S, f->olabel, 1, w->jfinal, w->paths, w->olabels, s));
+  PLAIN_PROF(FST_PROF_BACKTRACE, strings ? launch_string_trace(S, f->olabel, 1, w->jfinal, w->paths, w->olabels, s)
+                                         : launch_backtrace(S, f->olabel, 1, w->jfinal, w->paths, w->olabels, s));
   w->last_fb = false;
-  int32_t st = 0;
-  FST_CUDA(cudaMemcpy(best_score, w->score, 4, cudaMemcpyDeviceToHost));
-  FST_CUDA(cudaMemcpy(&st, w->status, 4, cudaMemcpyDeviceToHost));
-  if (n > 0) {
-    FST_CUDA(cudaMemcpy(arc_path, w->paths, (size_t)n * 4, cudaMemcpyDeviceToHost));
-    if (olabels) FST_CUDA(cudaMemcpy(olabels, w->olabels, (size_t)n * 4, cudaMemcpyDeviceToHost));
-  }
-  if (st == FST_ERR_TIMEOUT) {
-    set_error("a grid barrier of the persistent pass timed out");
-    return FST_ERR_TIMEOUT;
-  }
-  if (st != FST_OK) {
-    set_error("no accepting path");
-    return FST_ERR_NO_PATH;
-  }
-  return FST_OK;
+  std::vector<int32_t> h;
+  rc = plain_result(f, 2 * (int64_t)n, &h);
+  if (rc != FST_OK && rc != FST_ERR_NO_PATH && rc != FST_ERR_TIMEOUT) return rc;
+  memcpy(best_score, &h[3], 4);
+  std::copy(h.begin() + 4, h.begin() + 4 + n, arc_path);
+  if (olabels) std::copy(h.begin() + 4 + n, h.end(), olabels);
+  return rc;
 }
 
 extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, double* log_z, float* arc_posteriors) {
@@ -727,12 +815,18 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
   }
   if ((rc = plain_init(f))) return rc;
   cudaStream_t s = 0;
-  if ((rc = plain_tokens(f, ids, n, s))) return rc;
+  bool strings;
+  if ((rc = plain_tokens(f, ids, n, s, &strings))) return rc;
   PlainWs* w = f->plain;
-  if (arc_posteriors && !w->cnt) {
-    if ((rc = dalloc(&w->cnt, f->A)) || (rc = dalloc(&w->comp, f->A)) || (rc = dalloc(&w->counts_out, f->A)))
-      return rc;
+  StringWork K;
+  if (strings && (rc = plain_string(f, false, &K))) return rc;
+  // counts: float64 sums (string kernels), or float32 ones with their
+  // compensation (one writer per arc and position), in the same storage
+  if (arc_posteriors && !w->cnt64) {
+    dfree(w->counts_out);
+    if ((rc = dalloc(&w->counts_out, f->A)) || (rc = dalloc(&w->cnt64, f->A))) return rc;
   }
+  float* const cnt = (float*)w->cnt64;
   const LayoutView L = view_of(f->bwd);
   const TokenView T = plain_tokview(w);
   const FrontierState S = plain_state(f);
@@ -743,7 +837,9 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
                                              std::min(persist_grid_limit(1), persist_grid_limit(2))));
   const WaveSteps D{w->step0, n};
   const GridSync G{w->gbar, 0u, 2000000000ull};
-  if (persist) {
+  if (strings) {
+    PLAIN_PROF(FST_PROF_FWD_STEP, launch_string_forward(false, L, w->tok_sym, S, K, f->num_sms, s));
+  } else if (persist) {
     FST_CUDA(cudaMemsetAsync(w->gbar, 0, 8, s));
     PLAIN_PROF(FST_PROF_FWD_STEP, launch_fwd_persist(L, T, D, S, pgrid, G, s));
   } else {
@@ -756,10 +852,11 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
   PLAIN_PROF(FST_PROF_FB_FINAL, launch_fb_final(S, 1, w->logz, w->status, s));
   w->last_fb = true;
   if (arc_posteriors) {
-    const CountView C{0, w->cnt, w->comp, nullptr};
-    FST_CUDA(cudaMemsetAsync(w->cnt, 0, (size_t)std::max<int64_t>(f->A, 1) * 4, s));
-    FST_CUDA(cudaMemsetAsync(w->comp, 0, (size_t)std::max<int64_t>(f->A, 1) * 4, s));
-    if (persist) {
+    const CountView C = strings ? CountView{1, nullptr, nullptr, w->cnt64} : CountView{0, cnt, cnt + f->A, nullptr};
+    FST_CUDA(cudaMemsetAsync(w->cnt64, 0, (size_t)std::max<int64_t>(f->A, 1) * 8, s));
+    if (strings) {
+      PLAIN_PROF(FST_PROF_BWD_STEP, launch_string_backward(L, w->tok_sym, S, C, K, f->num_sms, s));
+    } else if (persist) {
       FST_CUDA(cudaMemsetAsync(w->gbar, 0, 8, s));
       PLAIN_PROF(FST_PROF_BWD_STEP, launch_bwd_persist(L, T, D, S, C, pgrid, G, s));
     } else {
@@ -768,20 +865,12 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
     }
     PLAIN_PROF(FST_PROF_COUNTS, launch_counts_out(f->A, C, w->counts_out, s));
     if (f->A > 0)
-      FST_CUDA(cudaMemcpy(arc_posteriors, w->counts_out, (size_t)f->A * 4, cudaMemcpyDeviceToHost));
+      FST_CUDA(cudaMemcpyAsync(arc_posteriors, w->counts_out, (size_t)f->A * 4, cudaMemcpyDeviceToHost, s));
   }
-  int32_t st = 0;
-  FST_CUDA(cudaMemcpy(log_z, w->logz, 8, cudaMemcpyDeviceToHost));
-  FST_CUDA(cudaMemcpy(&st, w->status, 4, cudaMemcpyDeviceToHost));
-  if (st == FST_ERR_TIMEOUT) {
-    set_error("a grid barrier of the persistent pass timed out");
-    return FST_ERR_TIMEOUT;
-  }
-  if (st != FST_OK) {
-    set_error("no accepting path");
-    return FST_ERR_NO_PATH;
-  }
-  return FST_OK;
+  std::vector<int32_t> h;
+  rc = plain_result(f, 0, &h);
+  if (rc == FST_OK || rc == FST_ERR_NO_PATH || rc == FST_ERR_TIMEOUT) memcpy(log_z, h.data(), 8);
+  return rc;
 }
 
 // ============================================================ measurement
@@ -821,6 +910,13 @@ extern "C" int fst_live_work(fst_t* f, int64_t* entries, int64_t* arcs) {
   if (entries) *entries = 0;
   if (arcs) *arcs = w && w->last_fb ? 0 : -1;
   if (!w) return FST_OK;
+  if (w->str_last) {
+    unsigned long long live[2];
+    FST_CUDA(cudaMemcpy(live, w->str_ctl + CTL_LIVE, sizeof(live), cudaMemcpyDeviceToHost));
+    if (entries) *entries = (int64_t)live[0];
+    if (arcs && w->last_fb) *arcs = (int64_t)live[1];
+    return FST_OK;
+  }
   int64_t top = 0;
   FST_CUDA(cudaMemcpy(&top, w->pool_top, 8, cudaMemcpyDeviceToHost));
   top = std::min(top, w->cap_pool);

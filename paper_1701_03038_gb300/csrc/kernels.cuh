@@ -299,6 +299,9 @@ struct StringQueue {
   int64_t fe_light;
   int32_t chunk;
 };
+// Pool entries a group of the string kernels reserves at a time; a capped
+// pool is handed out range by range, so that the cap counts live entries.
+constexpr int32_t POOL_CHUNK = 64;
 int64_t string_ctl_words(int32_t Bw, int32_t groups2);
 int64_t string_light_entries(int num_sms);
 int32_t string_kept_values();

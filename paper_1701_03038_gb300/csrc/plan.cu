@@ -529,17 +529,13 @@ bool string_path(const fst_plan_s* P) {
   return P->driver == FST_DRIVER_LAUNCH && P->pull_min == 0 && P->table_limit == 0;
 }
 
-// Pool entries a group of the string kernels reserves at a time; a capped
-// pool is handed out range by range, so that the cap counts live entries.
-constexpr int32_t POOL_CHUNK = 64;
-
 StringWork string_work(fst_plan_s* P, const Wave& W, bool viterbi) {
   StringWork K;
   K.Bw = W.Bw;
   K.ctl = P->str_ctl;
   K.kept = P->str_kept;
   K.fe_light = (int64_t)P->str_groups2 * P->fst->Q;
-  K.dirty = P->str_dirty;
+  K.dirty = P->str_dirty + (viterbi ? 0 : P->str_groups2);  // (a mark per kind of accumulator)
   K.dense = viterbi ? P->str_dense_v : P->str_dense_f;
   K.dval = P->str_dval;
   K.dstage = P->str_stage;
@@ -1152,7 +1148,7 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
     const int64_t nt = P->max_ntok;
     const int64_t gq = (int64_t)groups2 * f->Q;
     if ((rc = alloc_store(P, &P->str_ctl, string_ctl_words((int32_t)P->max_bw, groups2))) ||
-        (rc = alloc_store(P, &P->str_dirty, groups2)) ||
+        (rc = alloc_store(P, &P->str_dirty, 2 * groups2)) ||
         (rc = alloc_store(P, &P->str_kept, P->want_fb ? P->max_bw * string_kept_values() : 1)) ||
         (rc = alloc_store(P, &P->str_stage, gq)))
       break;
@@ -1170,7 +1166,7 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
          (rc = alloc_store(P, &P->final64, f->Q))))
       break;
     // the accumulators start at zero and every run leaves them so
-    cudaError_t ce = cudaMemsetAsync(P->str_dirty, 0, (size_t)groups2 * 4, s);
+    cudaError_t ce = cudaMemsetAsync(P->str_dirty, 0, (size_t)groups2 * 8, s);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(P->str_ctl, 0, CTL_WORDS * 4, s);
     if (ce == cudaSuccess && P->str_dense_v) ce = cudaMemsetAsync(P->str_dense_v, 0, (size_t)gq * 8, s);
     if (ce == cudaSuccess && P->str_dense_f) ce = cudaMemsetAsync(P->str_dense_f, 0, (size_t)gq * 16, s);

@@ -260,7 +260,7 @@ class Fst:
                     or out.ndim != 1 or out.shape[0] < max(self.num_arcs, 1)):
                 raise ValueError(f"out must be a contiguous float32 array of at least {max(self.num_arcs, 1)} elements")
             posteriors = True
-        cnt = (out if out is not None else np.zeros(max(self.num_arcs, 1), np.float32)) if posteriors else None
+        cnt = (out if out is not None else np.empty(max(self.num_arcs, 1), np.float32)) if posteriors else None
         with torch.cuda.device(self.device):
             rc = self._lib.fst_forward_backward(self._h, _hptr(x), n, _hptr(lz),
                                                 _hptr(cnt) if posteriors else None)
