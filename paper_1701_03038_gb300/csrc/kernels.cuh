@@ -237,11 +237,11 @@ int launch_to_float(const double* in, int64_t n, float* out, cudaStream_t s);
 // live entries and arcs; then, cleared before each pass, the strings started
 // and finished, a counter of progress, the open jobs, the heads and tails of
 // the two queues, the blocks that have begun, the light warps at work and the
-// open jobs of many chunks.
+// open jobs of many chunks, and the heavy blocks without a string.
 // Each on a cache line of its own: they are polled.
 enum : int {
   CTL_FLAGS = 0, CTL_TOP = 2, CTL_LIVE = 4, CTL_TAKE = 32, CTL_FINISHED = 64, CTL_PROGRESS = 96, CTL_OPEN = 128,
-  CTL_BIG = 129, CTL_HEAD = 160, CTL_TAIL = 224, CTL_BEGUN = 288, CTL_ALIVE = 289, CTL_WORDS = 320,
+  CTL_BIG = 129, CTL_IDLE = 130, CTL_HEAD = 160, CTL_TAIL = 224, CTL_BEGUN = 288, CTL_ALIVE = 289, CTL_WORDS = 320,
   CTL_LINE = 32
 };
 // Where a string was left when it changed hands (t = 0: not started), and

@@ -82,10 +82,11 @@ __device__ __forceinline__ int32_t warp_excl(int32_t len, int32_t* total) {
   return incl - len;
 }
 // Lane owning flat arc a: the last lane whose first flat arc is <= a.
-__device__ __forceinline__ int warp_owner_of(const int32_t* excl, int32_t a) {
+template <int N = 32>
+__device__ __forceinline__ int owner_of(const int32_t* excl, int32_t a) {
   int o = 0;
 #pragma unroll
-  for (int step = 16; step >= 1; step >>= 1)
+  for (int step = N / 2; step >= 1; step >>= 1)
     if (excl[o + step] <= a) o += step;
   return o;
 }
@@ -96,13 +97,23 @@ __device__ __forceinline__ int next_peer(uint32_t peers, int s) {
   return __ffs(above ? above : peers) - 1;
 }
 
-// The chunk of 32 entries a warp works on, in shared memory.
-template <class Real>
-struct WarpStage {
-  Real r[32];       // the source's value,
-  int32_t j[32];    // pool entry,
-  int32_t excl[32]; // first flat arc and
-  int32_t e0[32];   // first arc record
+// The entries a group of N lanes (a warp or a block) walks at a time, E a lane
+// and in shared memory: the lanes take their arcs flat, whatever entry they
+// belong to.  (A heavy block's warps with 32 entries each left most of them
+// waiting for the one with the most arcs: out-degrees are heavy-tailed.  And
+// most entries of a dense position have no arc: 256 of them at a time made
+// rounds of 420 arcs on average, each with its own chain of latencies.)
+template <class Real, int N, int E>
+struct GroupStage {
+  static constexpr int LANES = N, PER = E;
+  Real r[N * E];        // the source's value,
+  int32_t excl[N * E];  // first flat arc and
+  int32_t e0[N * E];    // first arc record
+  int32_t total[E][N / 32];  // arcs of each warp's entries
+  // (a block:) states a warp staged and has not yet listed
+  static constexpr int OUT = N == 32 ? 1 : 256;
+  int32_t out[N / 32][OUT];
+  static __device__ __forceinline__ int lane() { return N == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x; }
 };
 
 // A table of one position's accumulators (it fits when the position has at
@@ -129,6 +140,8 @@ struct GroupState {
 // arcs and largest value.
 struct HeavyShared {
   StringJob job;
+  unsigned long long tag;  // slot and phase number whose parameters job holds (~0: none)
+  bool same, last, halt;   // of the last claim
   int32_t chunk, pick, at, self;
   int32_t base;
   uint32_t tot, mk;
@@ -274,49 +287,63 @@ __device__ __forceinline__ int32_t next_light(const StringQueue& K) {
 // ----------------------------------------------------------------------
 constexpr int JOB_BITS = 22;
 constexpr unsigned long long JOB_MASK = (1ull << JOB_BITS) - 1ull;
+__device__ __forceinline__ int32_t job_left(unsigned long long w) {
+  return (int32_t)((w >> JOB_BITS) & JOB_MASK) - (int32_t)(w & JOB_MASK);
+}
 __device__ __forceinline__ bool job_open(unsigned long long w) { return (w & JOB_MASK) < ((w >> JOB_BITS) & JOB_MASK); }
 
-// Claim a chunk of the job in slot g: its index and the parameters into
-// shared memory.  All threads call it; false: none left.
+// Claim a chunk of the job in slot g: its index and (unless they are there)
+// the parameters into shared memory.  All threads call it, after the chunk
+// claimed before, of slot fin (-1: none), which counts as done now that its
+// writes are visible.  False: none left.  It costs one atomic's way to L2 and
+// back: the block that holds a job's last chunk does not ask for another, and
+// whether its ticket's string has come (*stop) is looked up meanwhile, for
+// the next call (sh.halt).  (Done, asked and checked one by one a chunk of 17
+// us carried 9 us of this.)
 template <class Sh>
-__device__ __forceinline__ bool job_claim(Sh& sh, const StringQueue& K, int32_t g) {
+__device__ __forceinline__ bool job_claim(Sh& sh, const StringQueue& K, int32_t g, int32_t fin, const uint32_t* stop) {
   StringJob* J = K.jobs + g;
   __syncthreads();
   if (threadIdx.x == 0) {
-    int32_t c = -1;
-    if (job_open(*(volatile unsigned long long*)&J->word)) {
-      const unsigned long long w = atomicAdd(&J->word, 1ull);
-      if (job_open(w)) c = (int32_t)(w & JOB_MASK);
+    const uint32_t come = stop ? peek(stop) : 0u;
+    if (fin >= 0) {
+      __threadfence();
+      atomicAdd(&K.jobs[fin].done, 1u);
     }
+    int32_t c = -1;
+    if (fin < 0 || !(sh.last || sh.halt)) {
+      const unsigned long long w = atomicAdd(&J->word, 1ull);
+      if (job_open(w)) {
+        c = (int32_t)(w & JOB_MASK);
+        sh.last = (w & JOB_MASK) + 1ull == ((w >> JOB_BITS) & JOB_MASK);
+        const unsigned long long tag = ((unsigned long long)g << 32) | (w >> (2 * JOB_BITS));
+        sh.same = sh.tag == tag;
+        sh.tag = tag;
+        __threadfence();
+      }
+    }
+    sh.halt = come != 0u;
     sh.chunk = c;
-    __threadfence();
   }
   __syncthreads();
   if (sh.chunk < 0) return false;
+  if (sh.same) return true;
   constexpr int W = (int)(sizeof(StringJob) / 4);
   static_assert(sizeof(StringJob) % 4 == 0 && W <= 32, "one word a lane");
   if (threadIdx.x < W) ((uint32_t*)&sh.job)[threadIdx.x] = __ldcg((const uint32_t*)J + threadIdx.x);
   __syncthreads();
   return true;
 }
-// The claimed chunk is done: its writes are visible before it counts.
+// A slot with at least `least` chunks left, this block's neighbours first
+// (-1: none).
 template <class Sh>
-__device__ __forceinline__ void job_done(Sh& sh, const StringQueue& K, int32_t g) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&K.jobs[g].done, 1u);
-  }
-}
-// A slot with chunks left, this block's neighbours first (-1: none).
-template <class Sh>
-__device__ __forceinline__ int32_t job_find(Sh& sh, const StringQueue& K) {
+__device__ __forceinline__ int32_t job_find(Sh& sh, const StringQueue& K, int32_t least) {
   __syncthreads();
   if (threadIdx.x == 0) sh.pick = INT32_MAX;
   __syncthreads();
   for (int32_t i = threadIdx.x; i < K.owners; i += blockDim.x) {
     const int32_t g = (int32_t)((sh.self + i) % (unsigned)K.owners);
-    if (job_open(*(volatile unsigned long long*)&K.jobs[g].word)) atomicMin(&sh.pick, i);
+    if (job_left(*(volatile unsigned long long*)&K.jobs[g].word) >= least) atomicMin(&sh.pick, i);
   }
   __syncthreads();
   const int32_t i = sh.pick;
@@ -330,6 +357,7 @@ __device__ __forceinline__ void job_post(Sh& sh, const StringQueue& K, int32_t n
     StringJob* J = K.jobs + sh.self;
     const unsigned long long w = *(volatile unsigned long long*)&J->word;
     sh.job.done = 0u;
+    sh.tag = ~0ull;
     constexpr int W = (int)(sizeof(StringJob) / 4);
     for (int i = 2; i < W; ++i) *((volatile uint32_t*)J + i) = ((const uint32_t*)&sh.job)[i];
     __threadfence();
@@ -369,6 +397,14 @@ __device__ __forceinline__ bool job_wait(Sh& sh, const StringQueue& K, int32_t n
   return sh.pick != 0;
 }
 
+// Whether there are jobs that a block with a string of its own leaves it for:
+// large ones, while few of the blocks that would do them have no string.
+// (With half of the blocks idle a string lost 136 us at one position to them.)
+__device__ __forceinline__ bool big_jobs(const StringQueue& K) {
+  const uint4 w = __ldcv((const uint4*)(K.ctl + CTL_OPEN));
+  return w.y != 0u && w.z * 8u < (uint32_t)K.owners;
+}
+
 // What a heavy block does next: a string from the heavy queue (blocks that
 // own dense storage), a job of another block, and, while there are no light
 // warps, the light ones' strings too; it leaves once every string is done.
@@ -392,9 +428,13 @@ struct HeavyPick {
         if (begun && !holds) {
           ticket = queue_ticket(K, QH);
           holds = true;
+          atomicAdd(K.ctl + CTL_IDLE, 1u);
         }
         b = holds ? queue_poll(K, QH, ticket) : queue_pop(K, QH);
-        if (b >= 0) holds = false;
+        if (b >= 0 && holds) {
+          holds = false;
+          atomicSub(K.ctl + CTL_IDLE, 1u);
+        }
         if (b < 0 && !lights && (b = queue_pop(K, QL)) < 0) b = take_new(K);
         if (b < 0) b = PICK_NONE;
       }
@@ -421,6 +461,11 @@ struct HeavyPick {
     __syncthreads();
     return b;
   }
+  // Where the string of this block's ticket will appear (null: it has none):
+  // its helping stops for it.
+  __device__ __forceinline__ const uint32_t* stop(const StringQueue& K) const {
+    return holds ? queue_slot(K, QH, ticket) : nullptr;
+  }
   // There was a chunk to help with.
   __device__ __forceinline__ void helped() { idle = waiting = false; }
 };
@@ -432,7 +477,8 @@ template <bool VIT>
 struct Forward {
   typedef typename std::conditional<VIT, int32_t, unsigned long long>::type Val;
   typedef typename std::conditional<VIT, float, double>::type Real;
-  typedef WarpStage<Real> Stage;
+  typedef GroupStage<Real, 32, 1> Stage;
+  typedef GroupStage<Real, NT1, 2> BlockStage;
   typedef Table<HS0, Val> LightTable;
   typedef Table<HS1, Val> HeavyTable;
   struct LightShared {
@@ -442,7 +488,7 @@ struct Forward {
   };
   struct BlockShared {
     HeavyTable tab;
-    Stage st[WARPS];
+    BlockStage st;
     HeavyShared hv;
     GroupState gs;
   };
@@ -451,7 +497,6 @@ struct Forward {
   const int32_t* sym;
   const FrontierState& S;
   const StringQueue& K;
-  Stage& st;  // of this warp
 
   // Dense storage of heavy block g: [Q] keys (Viterbi) or [Q] {sum, maximum}
   // pairs, the staged states, and (Viterbi) the arcs of the entries of the
@@ -509,25 +554,59 @@ struct Forward {
     }
   }
 
-  // The entries of a warp's chunk staged for load_arcs; returns their arcs.
-  __device__ __forceinline__ int32_t stage(const Entry& x, int32_t len) const {
-    int32_t total;
-    const int32_t ex = warp_excl(len, &total);
-    __syncwarp();
-    st.excl[lane_id()] = ex;
-    st.e0[lane_id()] = x.e0;
-    st.r[lane_id()] = x.r;
-    if (VIT) st.j[lane_id()] = x.jp;
-    __syncwarp();
+  // The group's next entries staged for load_arcs: those from i0 on, below n,
+  // of the position before (fe, t, base, a as for entry).  Returns their
+  // arcs.  (A block's walk of the ones before may still be going on: it is
+  // waited for.)
+  template <class St>
+  __device__ __forceinline__ int32_t stage(St& st, const int2* fe, int32_t t, int32_t base, int32_t a, int32_t i0,
+                                           int32_t n) const {
+    constexpr int N = St::LANES, E = St::PER;
+    constexpr bool BLOCK = N > 32;
+    Entry x[E];
+    int32_t ex[E], total = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int32_t i = i0 + e * N + St::lane();
+      x[e] = Entry{0, 0, -1, none()};
+      if (i < n) x[e] = entry(fe, t, base, i, a);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      ex[e] = warp_excl(x[e].len, &total);
+      if (BLOCK && lane_id() == 0) st.total[e][warp_id()] = total;
+    }
+    if constexpr (BLOCK) {
+      __syncthreads();
+      total = 0;
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+#pragma unroll
+        for (int w = 0; w < N / 32; ++w) {
+          if (w == warp_id()) ex[e] += total;
+          total += st.total[e][w];
+        }
+    } else {
+      __syncwarp();
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int k = e * N + St::lane();
+      st.excl[k] = ex[e];
+      st.e0[k] = x[e].e0;
+      st.r[k] = x[e].r;
+    }
+    if (BLOCK) __syncthreads();
+    else __syncwarp();
     return total;
   }
   // This lane's VU flat arcs from a0 on: their owners (-1: none) and records.
-  template <int VU>
-  __device__ __forceinline__ void load_arcs(int32_t a0, int32_t total, int (&oo)[VU], int4 (&arc)[VU]) const {
+  template <int VU, class St>
+  __device__ __forceinline__ void load_arcs(const St& st, int32_t a0, int32_t total, int (&oo)[VU], int4 (&arc)[VU]) const {
 #pragma unroll
     for (int u = 0; u < VU; ++u) {
-      const int32_t a = a0 + u * 32 + lane_id();
-      oo[u] = a < total ? warp_owner_of(st.excl, a) : -1;
+      const int32_t a = a0 + u * St::LANES + St::lane();
+      oo[u] = a < total ? owner_of<St::LANES * St::PER>(st.excl, a) : -1;
       arc[u] = make_int4(0, 0, 0, 0);
       if (oo[u] >= 0) {
         const int32_t i = st.e0[oo[u]] + (a - st.excl[oo[u]]);
@@ -548,17 +627,18 @@ struct Forward {
 
   // The staged chunk's arcs into a table.  PHASE 0: the atomic max of each
   // destination, whose first arc stages it; PHASE 1 (forward), once every
-  // maximum is final: the fixed-point terms.
-  template <int PHASE, int HS>
-  __device__ __forceinline__ void walk_table(Table<HS, Val>& tab, int32_t total) const {
+  // maximum is final: the fixed-point terms.  j0: the pool entry of the first
+  // staged one (-1: start states).
+  template <int PHASE, int HS, class St>
+  __device__ __forceinline__ void walk_table(Table<HS, Val>& tab, const St& st, int32_t total, int32_t j0) const {
     constexpr int VU = HS == HS0 ? VU0 : VU1;
-    for (int32_t a0 = 0; a0 < total; a0 += 32 * VU) {
+    for (int32_t a0 = 0; a0 < total; a0 += St::LANES * VU) {
       int oo[VU];
       int4 arc[VU];
-      load_arcs(a0, total, oo, arc);
+      load_arcs(st, a0, total, oo, arc);
 #pragma unroll
       for (int u = 0; u < VU; ++u) {
-        if (u > 0 && a0 + u * 32 >= total) break;  // (warp-uniform)
+        if (u > 0 && a0 + u * St::LANES >= total) break;  // (the same in the group)
         double v = 0.0;
         const unsigned long long c = oo[u] >= 0 ? candidate(st.r[oo[u]], arc[u], &v) : 0ull;
         bool fresh = false;
@@ -580,7 +660,7 @@ struct Forward {
           if (c != 0ull) {
             atomicMax(tab.acc + h, c);
             if constexpr (VIT)
-              if (fresh) tab.aux[h] = st.j[oo[u]];
+              if (fresh) tab.aux[h] = j0 < 0 ? -1 : j0 + oo[u];
           }
           const int32_t at = append(&tab.staged, fresh);
           if (fresh) tab.list[at] = (uint16_t)h;
@@ -591,52 +671,58 @@ struct Forward {
     }
   }
 
+  // The states the warp staged, to the list: one atomic for up to 256 of them.
+  __device__ __forceinline__ void list_staged(int32_t g, int32_t* staged, const BlockStage& st, int32_t& pend) const {
+    __syncwarp();
+    int32_t at = 0;
+    if (lane_id() == 0 && pend) at = atomicAdd(staged, pend);
+    at = __shfl_sync(FULL, at, 0);
+    for (int32_t i = lane_id(); i < pend; i += 32)
+      if (in_bounds(CHK_STAGE, at + i, S.Q)) dstage(g)[at + i] = st.out[warp_id()][i];
+    __syncwarp();
+    pend = 0;
+  }
   // The same into heavy block g's dense accumulators; `staged` counts the
   // staged states (shared memory, or the job's word).
   template <int PHASE>
-  __device__ __forceinline__ void walk_dense(int32_t g, int32_t* staged, int32_t total) const {
+  __device__ __forceinline__ void walk_dense(int32_t g, int32_t* staged, BlockStage& st, int32_t total, int32_t& pend) const {
     constexpr int VU = VU1;
     unsigned long long* acc = dacc(g);
-    for (int32_t a0 = 0; a0 < total; a0 += 32 * VU) {
-      int oo[VU];
-      int4 arc[VU];
-      load_arcs(a0, total, oo, arc);
+    int oo[VU];
+    int4 arc[VU];
+    load_arcs(st, 0, total, oo, arc);
+    for (int32_t a0 = 0; a0 < total; a0 += NT1 * VU) {
       double v[VU];
       unsigned long long c[VU];
+      int32_t q[VU];
 #pragma unroll
       for (int u = 0; u < VU; ++u) {
         v[u] = 0.0;
-        c[u] = oo[u] >= 0 && in_bounds(CHK_ACC, arc[u].x, S.Q) ? candidate(st.r[oo[u]], arc[u], &v[u]) : 0ull;
+        q[u] = arc[u].x;
+        c[u] = oo[u] >= 0 && in_bounds(CHK_ACC, q[u], S.Q) ? candidate(st.r[oo[u]], arc[u], &v[u]) : 0ull;
       }
+      // (the next arcs' records are on their way while these ones' atomics are)
+      load_arcs(st, a0 + NT1 * VU, total, oo, arc);
       if constexpr (PHASE == 0) {
         unsigned long long old[VU];
 #pragma unroll
         for (int u = 0; u < VU; ++u)
-          old[u] = c[u] ? atomicMax(VIT ? acc + arc[u].x : acc + 2 * (int64_t)arc[u].x + 1, c[u]) : 1ull;
-        // the lanes that met a destination first stage it: one atomic a round
-        uint32_t w[VU];
-        int32_t n = 0;
+          old[u] = c[u] ? atomicMax(VIT ? acc + q[u] : acc + 2 * (int64_t)q[u] + 1, c[u]) : 1ull;
+        // the lanes that met a destination first stage it, with their warp
 #pragma unroll
         for (int u = 0; u < VU; ++u) {
-          w[u] = __ballot_sync(FULL, old[u] == 0ull);
-          n += __popc(w[u]);
+          const uint32_t w = __ballot_sync(FULL, old[u] == 0ull);
+          if (old[u] == 0ull) st.out[warp_id()][pend + __popc(w & lanes_below())] = q[u];
+          pend += __popc(w);
         }
-        if (n == 0) continue;
-        int32_t at = lane_id() == 0 ? atomicAdd(staged, n) : 0;
-        at = __shfl_sync(FULL, at, 0);
-#pragma unroll
-        for (int u = 0; u < VU; ++u) {
-          const int32_t i = at + __popc(w[u] & lanes_below());
-          if (old[u] == 0ull && in_bounds(CHK_STAGE, i, S.Q)) dstage(g)[i] = arc[u].x;
-          at += __popc(w[u]);
-        }
+        if (pend > BlockStage::OUT - 32 * VU) list_staged(g, staged, st, pend);
       } else {
         unsigned long long mx[VU];
 #pragma unroll
-        for (int u = 0; u < VU; ++u) mx[u] = c[u] ? __ldcg(acc + 2 * (int64_t)arc[u].x + 1) : 0ull;
+        for (int u = 0; u < VU; ++u) mx[u] = c[u] ? __ldcg(acc + 2 * (int64_t)q[u] + 1) : 0ull;
 #pragma unroll
         for (int u = 0; u < VU; ++u)
-          if (mx[u]) atomicAdd(acc + 2 * (int64_t)arc[u].x, fix_exp64(v[u], dkey_inv(mx[u])));
+          if (mx[u]) atomicAdd(acc + 2 * (int64_t)q[u], fix_exp64(v[u], dkey_inv(mx[u])));
       }
     }
   }
@@ -908,7 +994,7 @@ struct Forward {
   // in registers: a lane per entry, a lane per arc, destinations grouped by
   // a warp match, and the next lookups in flight while the values are formed.
   // The frontiers beyond, up to HS0 / 2 arcs, go through the warp's table.
-  __device__ __forceinline__ void light_string(LightTable& tab, GroupState& gs, int32_t g, int32_t b) const {
+  __device__ __forceinline__ void light_string(LightTable& tab, Stage& st, GroupState& gs, int32_t g, int32_t b) const {
     const int lane = lane_id();
     Place P = resume(b);
     int2* fe = fe_light(g);
@@ -1036,9 +1122,8 @@ struct Forward {
         have = true;
       } else {
         for (int32_t c = 0; c < P.cnt; c += 32) {
-          Entry y{0, 0, -1, none()};
-          if (c + lane < P.cnt) y = entry(fe, P.t, P.base, c + lane, a);
-          walk_table<0>(tab, stage(y, y.len));
+          const int32_t total = stage(st, fe, P.t, P.base, a, c, P.cnt);
+          walk_table<0>(tab, st, total, P.t == 1 ? -1 : P.base + c);
         }
         __syncwarp();
         nb = tab.staged;
@@ -1047,9 +1132,8 @@ struct Forward {
         const bool single = nb == P.tot;
         if (!VIT && !single)
           for (int32_t c = 0; c < P.cnt; c += 32) {
-            Entry y{0, 0, -1, none()};
-            if (c + lane < P.cnt) y = entry(fe, P.t, P.base, c + lane, a);
-            walk_table<1>(tab, stage(y, y.len));
+            const int32_t total = stage(st, fe, P.t, P.base, a, c, P.cnt);
+            walk_table<1>(tab, st, total, P.t == 1 ? -1 : P.base + c);
           }
         nbase = warp_reserve(gs, nb);
         __syncwarp();
@@ -1098,8 +1182,8 @@ struct Forward {
   }
 
   // ---- heavy blocks ------------------------------------------------------
-  // A chunk of a dense position (hv.job): its entries, 32 a warp.
-  __device__ __forceinline__ void chunk(HeavyShared& hv, int32_t c, int32_t* staged) const {
+  // A chunk of a dense position (hv.job).
+  __device__ __forceinline__ void chunk(HeavyShared& hv, BlockStage& st, int32_t c, int32_t* staged) const {
     const StringJob& J = hv.job;
     const int32_t lo = c * J.per;
     if (J.phase == 2) {
@@ -1117,13 +1201,13 @@ struct Forward {
       return;
     }
     const int32_t hi = min(lo + J.per, J.cnt);
-    for (int32_t i0 = lo + 32 * warp_id(); i0 < hi; i0 += 32 * WARPS) {
-      Entry y{0, 0, -1, none()};
-      if (i0 + lane_id() < hi) y = entry(fe_heavy(J.owner), J.t, J.base, i0 + lane_id(), J.a);
-      const int32_t total = stage(y, y.len);
-      if (J.phase == 0) walk_dense<0>(J.owner, staged, total);
-      else if constexpr (!VIT) walk_dense<1>(J.owner, nullptr, total);
+    int32_t pend = 0;
+    for (int32_t i0 = lo; i0 < hi; i0 += NT1 * BlockStage::PER) {
+      const int32_t total = stage(st, fe_heavy(J.owner), J.t, J.base, J.a, i0, hi);
+      if (J.phase == 0) walk_dense<0>(J.owner, staged, st, total, pend);
+      else if constexpr (!VIT) walk_dense<1>(J.owner, nullptr, st, total, pend);
     }
+    if (J.phase == 0) list_staged(J.owner, staged, st, pend);
   }
 
   // A heavy block's life, as one loop with one copy of each part (calls out
@@ -1177,10 +1261,14 @@ struct Forward {
           continue;
         }
         an = P.t < P.n ? __ldg(sym + P.off + P.t) : -1;
-        if (P.tot > HS1 / 2) {
-          const bool shared = P.tot >= SHARE_ARCS;
+        if (P.tot > HS1 / 2 || P.cnt >= SHARE_ARCS) {
+          // (many entries with few arcs are work too: 176,615 of them with
+          // 2,627 took a block by itself 860 us)
+          const int32_t size = max(P.tot, P.cnt);
+          const bool shared = size >= SHARE_ARCS;
           if (tid == 0) {
             StringJob& J = hv.job;
+            hv.tag = ~0ull;
             J.phase = 0;
             J.owner = self;
             J.t = P.t;
@@ -1188,7 +1276,7 @@ struct Forward {
             J.an = an;
             J.cnt = P.cnt;
             // (fewer than 2^31 arcs: the chunks' numbers fit JOB_BITS)
-            J.per = shared ? (int32_t)min((long long)P.cnt, max(1ll, (long long)P.cnt * CHUNK_ARCS / P.tot)) : P.cnt;
+            J.per = shared ? (int32_t)min((long long)P.cnt, max(1ll, (long long)P.cnt * CHUNK_ARCS / size)) : P.cnt;
             J.base = P.base;
             J.shift = P.shift;
             J.shared = shared;
@@ -1198,11 +1286,10 @@ struct Forward {
           own = 0;
           __syncthreads();
         } else {
-          const uint32_t big = tid == 0 ? peek(K.ctl + CTL_BIG) : 0u;  // (used below)
-          for (int32_t c = 32 * warp_id(); c < P.cnt; c += NT1) {
-            Entry y{0, 0, -1, none()};
-            if (c + lane < P.cnt) y = entry(fe, P.t, P.base, c + lane, a);
-            walk_table<0>(sh.tab, stage(y, y.len));
+          const uint32_t big = tid == 0 ? big_jobs(K) : 0u;  // (used below)
+          for (int32_t c = 0; c < P.cnt; c += NT1 * BlockStage::PER) {
+            const int32_t total = stage(sh.st, fe, P.t, P.base, a, c, P.cnt);
+            walk_table<0>(sh.tab, sh.st, total, P.t == 1 ? -1 : P.base + c);
           }
           __syncthreads();
           nb = sh.tab.staged;
@@ -1212,10 +1299,9 @@ struct Forward {
             hv.tot = hv.mk = 0u;
           }
           if (!VIT && !single)
-            for (int32_t c = 32 * warp_id(); c < P.cnt; c += NT1) {
-              Entry y{0, 0, -1, none()};
-              if (c + lane < P.cnt) y = entry(fe, P.t, P.base, c + lane, a);
-              walk_table<1>(sh.tab, stage(y, y.len));
+            for (int32_t c = 0; c < P.cnt; c += NT1 * BlockStage::PER) {
+              const int32_t total = stage(sh.st, fe, P.t, P.base, a, c, P.cnt);
+              walk_table<1>(sh.tab, sh.st, total, P.t == 1 ? -1 : P.base + c);
             }
           __syncthreads();
           const int32_t nbase = hv.base;
@@ -1248,17 +1334,21 @@ struct Forward {
         const bool mine = own >= 0, alone = mine && !hv.job.shared;
         const int32_t n = mine ? ((own == 2 ? hv.job.nb : hv.job.cnt) + hv.job.per - 1) / max(hv.job.per, 1) : 0;
         if (mine && !alone) job_post(hv, K, n);
-        int32_t g = mine ? self : job_find(hv, K);
+        const int32_t least = b >= 0 ? BIG_CHUNKS : 1;
+        int32_t g = mine ? self : job_find(hv, K, least), fin = -1;
         for (int32_t c = 0; g >= 0; ++c) {
           if (alone) {
             if (c >= n) break;
-          } else if (!job_claim(hv, K, g)) {
-            g = mine ? -1 : job_find(hv, K);
-            continue;
+          } else {
+            const bool got = job_claim(hv, K, g, fin, mine ? nullptr : pick.stop(K));
+            fin = got ? g : -1;
+            if (!got) {
+              g = mine || hv.halt ? -1 : job_find(hv, K, least);
+              continue;
+            }
           }
           if (help) pick.helped();
-          chunk(hv, alone ? c : hv.chunk, alone ? &sh.tab.staged : (int32_t*)&K.jobs[g].staged);
-          if (!alone) job_done(hv, K, g);
+          chunk(hv, sh.st, alone ? c : hv.chunk, alone ? &sh.tab.staged : (int32_t*)&K.jobs[g].staged);
         }
         if (mine) {
           bool ok = true;
@@ -1351,12 +1441,12 @@ __global__ void __launch_bounds__(NT1, 3)
       sh.gs = GroupState{0, 0, 0ull, 0ull};
     }
     __syncwarp();
-    const F f{L, sym, S, K, sh.st};
+    const F f{L, sym, S, K};
     const int32_t g = ((int32_t)blockIdx.x - K.heavy_blocks) * WARPS + warp_id();
     while (warp_id() < K.light_warps) {
       const int32_t b = next_light(K);
       if (b < 0) break;
-      f.light_string(sh.tab, sh.gs, g, b);
+      f.light_string(sh.tab, sh.st, sh.gs, g, b);
       __syncwarp();
     }
     return;
@@ -1372,9 +1462,10 @@ __global__ void __launch_bounds__(NT1, 3)
     sh.tab.staged = 0;
     sh.gs = GroupState{0, 0, 0ull, 0ull};
     sh.hv.self = self;
+    sh.hv.tag = ~0ull;
   }
   __syncthreads();
-  const F f{L, sym, S, K, sh.st[warp_id()]};
+  const F f{L, sym, S, K};
   if (self < K.owners && peek(K.dirty + self)) {
     // a run that gave up left values behind
     const int64_t w = (int64_t)S.Q * (VIT ? 1 : 2);
@@ -1505,7 +1596,7 @@ struct Backward {
 #pragma unroll
       for (int u = 0; u < VU; ++u) {
         const int32_t a = a0 + u * 32 + lane;
-        oi[u] = a < total ? warp_owner_of(st.excl, a) : -1;
+        oi[u] = a < total ? owner_of(st.excl, a) : -1;
         arc[u] = oi[u] >= 0 ? __ldg(L.arcs + st.e0[oi[u]] + (a - st.excl[oi[u]])) : make_int4(0, 0, 0, 0);
       }
 #pragma unroll
@@ -1530,7 +1621,7 @@ struct Backward {
       for (int u = 0; u < VU; ++u) {
         if (a0 > 0) {
           const int32_t a = a0 + u * 32 + lane;
-          oo[u] = a < total ? warp_owner_of(st.excl, a) : -1;
+          oo[u] = a < total ? owner_of(st.excl, a) : -1;
           v[u] = -INFINITY;
           if (oo[u] >= 0) {
             const int4 arc = __ldg(L.arcs + st.e0[oo[u]] + (a - st.excl[oo[u]]));
@@ -1645,7 +1736,7 @@ struct Backward {
     J.next_big = dense;
     J.shared = shared;
     J.mk = 0u;
-    J.per = (int32_t)min((long long)R.cnt, max(1ll, (long long)R.cnt * CHUNK_ARCS / max(1u, R.tot)));
+    J.per = (int32_t)min((long long)R.cnt, max(1ll, (long long)R.cnt * CHUNK_ARCS / max((uint32_t)R.cnt, R.tot)));
     if ((P.t & 4095) == 0) atomicAdd(K.ctl + CTL_PROGRESS, 1u);
   }
   __device__ __forceinline__ void leave(const Place& P, int32_t b, int32_t hand) const {
@@ -1812,7 +1903,7 @@ struct Backward {
         if (P.t < P.n) P.tE += (double)et;
         const bool shared = max((uint32_t)R.cnt, R.tot) >= (uint32_t)SHARE_ARCS;
         dense = R.cnt > CAP || shared;  // where the values of t-1 go
-        big = tid == 0 ? peek(K.ctl + CTL_BIG) : 0u;  // (used below)
+        big = tid == 0 ? big_jobs(K) : 0u;  // (used below)
         if (shared && P.t < P.n && !P.cur_big) {
           // the values of position t where every block finds them
           const int w = P.t & 1;
@@ -1825,6 +1916,7 @@ struct Backward {
           P.cur_big = true;
         }
         if (tid == 0) {
+          hv.tag = ~0ull;
           fill(hv.job, P, R, self, et, dense, shared);
           hv.mk = 0u;
         }
@@ -1837,17 +1929,21 @@ struct Backward {
         const bool alone = mine && !hv.job.shared;
         const int32_t n = mine ? (alone ? 1 : (R.cnt + hv.job.per - 1) / max(hv.job.per, 1)) : 0;
         if (mine && !alone) job_post(hv, K, n);
-        int32_t g = mine ? self : job_find(hv, K);
+        const int32_t least = b >= 0 ? BIG_CHUNKS : 1;
+        int32_t g = mine ? self : job_find(hv, K, least), fin = -1;
         for (int32_t c = 0; g >= 0; ++c) {
           if (alone) {
             if (c >= n) break;
-          } else if (!job_claim(hv, K, g)) {
-            g = mine ? -1 : job_find(hv, K);
-            continue;
+          } else {
+            const bool got = job_claim(hv, K, g, fin, mine ? nullptr : pick.stop(K));
+            fin = got ? g : -1;
+            if (!got) {
+              g = mine || hv.halt ? -1 : job_find(hv, K, least);
+              continue;
+            }
           }
           if (help) pick.helped();
           chunk(hv, alone ? c : hv.chunk);
-          if (!alone) job_done(hv, K, g);
         }
         if (!mine) break;
         bool ok = true;
@@ -1887,7 +1983,10 @@ __global__ void __launch_bounds__(NT1, 3)
   }
   BwdBlockShared& sh = *(BwdBlockShared*)smem;
   for (int i = threadIdx.x; i < BHS1; i += NT1) sh.tab.key[0][i] = sh.tab.key[1][i] = 0u;
-  if (threadIdx.x == 0) sh.hv.self = (int32_t)blockIdx.x;
+  if (threadIdx.x == 0) {
+    sh.hv.self = (int32_t)blockIdx.x;
+    sh.hv.tag = ~0ull;
+  }
   __syncthreads();
   const Backward<BHS1, BHS1 / 2> w{L, sym, S, C, K, sh.st[warp_id()], sh.tab};
   w.heavy_block(sh.hv);
@@ -1980,8 +2079,12 @@ int resident(K kernel, int which, size_t smem, int num_sms, int* out) {
   return FST_OK;
 }
 
-// The queues and roles of a launch of at most `blocks` blocks: half of them
-// heavy, the others as many as the strings fill.
+// The queues and roles of a launch of at most `blocks` blocks: a quarter of
+// them light, up to half where that gives every string a warp at once, the
+// others heavy.  (The few dense positions are most of the work: with half of
+// the blocks light, Viterbi of 4,096 strings on 20M arcs took 3.5 ms instead
+// of 3.0, with an eighth 3.3; a training step of 1,024 strings whose last 112
+// wait for a warp took 0.92 ms instead of 0.87.)
 StringQueue string_queue(const StringWork& W, int blocks, int32_t* grid) {
   StringQueue K;
   K.strings = W.Bw;
@@ -2003,7 +2106,9 @@ StringQueue string_queue(const StringWork& W, int blocks, int32_t* grid) {
   K.fe_light = W.fe_light;
   K.chunk = W.chunk;
   // (heavy blocks come first, so that they are resident first)
-  K.heavy_blocks = std::max(blocks / 2, 1);
+  const int all = (W.Bw + WARPS - 1) / WARPS;
+  const int want = all <= blocks / 2 ? std::max(all, blocks / 4) : blocks / 4;
+  K.heavy_blocks = std::max(blocks - want, 1);
   // few strings are spread over the blocks
   const int light = std::max(1, std::min(blocks - K.heavy_blocks, W.Bw));
   K.light_warps = std::max(1, std::min(WARPS, (W.Bw + light - 1) / light));
