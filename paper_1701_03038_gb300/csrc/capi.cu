@@ -626,26 +626,24 @@ extern "C" int fst_set_weights(fst_t* f, const float* weight, int32_t weight_kin
   const int64_t A = f->A;
   if (A == 0) return FST_OK;
   const bool dev = (flags & FST_FLAG_DEVICE_PTRS) != 0;
-  float *d_w = nullptr, *d_theta = nullptr;
-  unsigned int* d_err = nullptr;
-  int rc = FST_OK;
-  do {
-    if (!dev) {
-      if ((rc = to_device(weight, &d_w, A))) break;
-    }
-    if ((rc = dalloc(&d_theta, A)) || (rc = dalloc(&d_err, 1))) break;
-    if (cudaMemset(d_err, 0, 4) != cudaSuccess) { rc = cuda_fail(cudaGetLastError(), "memset"); break; }
-    k_convert_arcs<<<nblk(A), TB>>>(nullptr, nullptr, nullptr, dev ? weight : d_w, A, f->Q, f->m, weight_kind,
-                                    d_theta, d_err);
-    if ((rc = read_err_flag(d_err, "fst_set_weights"))) break;
-    if ((rc = set_layout_weights(f, d_theta, 0))) break;
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) rc = cuda_fail(e, "fst_set_weights");
-  } while (0);
-  dfree(d_w);
-  dfree(d_theta);
-  dfree(d_err);
-  return rc;
+  // (kept from call to call: allocating it took as long as the kernels)
+  Scratch mem;
+  int rc = mem.take(f, Scratch::piece(A * 4) * (dev ? 1 : 2) + Scratch::piece(4));
+  if (rc) return rc;
+  float* d_theta = mem.get<float>(A);
+  unsigned int* d_err = mem.get<unsigned int>(1);
+  const float* d_w = weight;
+  if (!dev) {
+    float* up = mem.get<float>(A);
+    FST_CUDA(cudaMemcpy(up, weight, (size_t)A * 4, cudaMemcpyHostToDevice));
+    d_w = up;
+  }
+  FST_CUDA(cudaMemset(d_err, 0, 4));
+  k_convert_arcs<<<nblk(A), TB>>>(nullptr, nullptr, nullptr, d_w, A, f->Q, f->m, weight_kind, d_theta, d_err);
+  if ((rc = read_err_flag(d_err, "fst_set_weights"))) return rc;
+  if ((rc = set_layout_weights(f, d_theta, 0))) return rc;
+  FST_CUDA(cudaDeviceSynchronize());
+  return FST_OK;
 }
 
 extern "C" int fst_set_state_weights(fst_t* f, const float* start_weight, const float* final_weight,

@@ -46,6 +46,7 @@ namespace {
 
 constexpr int KT = 256;  // threads per block of the step kernels
 constexpr int FT = 256;  // threads per block of the final reductions
+constexpr int FU = 8;    // candidates a thread reads at a time
 
 // Owner of flat entry j among the n slots whose first entries base[0..n)
 // are nondecreasing with base[0] <= j: the last slot with base <= j.  The
@@ -1289,19 +1290,37 @@ __global__ void __launch_bounds__(FT) k_vit_final(FrontierState S, float* __rest
   const int64_t base = (n == 0 || err) ? 0 : S.pool_base[p];
   const int32_t* cand = n == 0 ? S.start_q : S.pool_q + base;
   const int32_t ncand = err ? 0 : (n == 0 ? S.nstart : S.pool_cnt[p]);
-  // best (score, lowest state) key; the low word holds ~state, and for the
-  // pool entry the search below finds the index
+  // best (score, lowest state) key; the low word holds ~state.  FU candidates
+  // a thread at a time: a string that ends with 200,000 of them is a chain of
+  // dependent reads otherwise (240 us of a batch, 60 so).
   unsigned long long best = 0ull;
-  for (int32_t i = threadIdx.x; i < ncand; i += FT) {
-    const int32_t q = cand[i];
-    if (q < 0) continue;
-    const float a = n == 0 ? __ldg(S.theta_s + q) : S.pool_v[base + i];
-    const float c = __fadd_rn(a, __ldg(S.theta_f + q));
-    if (c != neg_inf()) {
-      const unsigned long long key = ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)q);
-      best = key > best ? key : best;
+  int32_t at = -1;
+  for (int32_t i0 = threadIdx.x; i0 < ncand; i0 += FT * FU) {
+    int32_t q[FU];
+    float a[FU], f[FU];
+#pragma unroll
+    for (int u = 0; u < FU; ++u) {
+      const int32_t i = i0 + u * FT;
+      q[u] = i < ncand ? cand[i] : -1;
+      a[u] = i < ncand && n > 0 ? S.pool_v[base + i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < FU; ++u) {
+      f[u] = q[u] >= 0 ? __ldg(S.theta_f + q[u]) : neg_inf();
+      if (n == 0 && q[u] >= 0) a[u] = __ldg(S.theta_s + q[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < FU; ++u) {
+      const float c = __fadd_rn(a[u], f[u]);
+      if (q[u] < 0 || c == neg_inf()) continue;
+      const unsigned long long key = ((unsigned long long)fkey(c) << 32) | (unsigned long long)(~(uint32_t)q[u]);
+      if (key > best) {
+        best = key;
+        at = i0 + u * FT;
+      }
     }
   }
+  const unsigned long long own = best;
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) {
     const unsigned long long o = __shfl_xor_sync(FULL, best, d);
@@ -1312,16 +1331,13 @@ __global__ void __launch_bounds__(FT) k_vit_final(FrontierState S, float* __rest
   best = red[0];
   for (int w = 1; w < FT / 32; ++w) best = red[w] > best ? red[w] : best;
   const bool oom = err != 0u;
-  const int32_t qbest = best ? (int32_t)(~(uint32_t)best) : -1;
   if (threadIdx.x == 0) {
     scores[b] = (best && !oom) ? fkey_inv((uint32_t)(best >> 32)) : neg_inf();
     if (status) status[b] = err ? run_error(err) : (best ? FST_OK : FST_ERR_NO_PATH);
     if (!best || oom || n == 0) jfinal[b] = -1;
   }
   // the entry holding the best state (each state appears once per token)
-  if (best && !oom && n > 0)
-    for (int32_t i = threadIdx.x; i < ncand; i += FT)
-      if (cand[i] == qbest) jfinal[b] = (int32_t)(base + i);
+  if (best && own == best && !oom && n > 0) jfinal[b] = (int32_t)(base + at);
 }
 
 // One thread per string, from the last position back: each pool entry
@@ -1397,7 +1413,8 @@ __global__ void __launch_bounds__(FT) k_fb_final(FrontierState S, double* __rest
                                                  int32_t* __restrict__ status) {
   __shared__ double red_m[FT / 32];
   __shared__ unsigned long long red_lo[FT], red_hi[FT];
-  __shared__ double c_prev;
+  __shared__ double c_prev, pack[FT * FU];
+  __shared__ int32_t npack;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t b = blockIdx.x;
   const int32_t n = S.bw_n[b];
@@ -1432,17 +1449,34 @@ __global__ void __launch_bounds__(FT) k_fb_final(FrontierState S, double* __rest
   const int64_t base = (n == 0 || err) ? 0 : S.pool_base[p];
   const int32_t* cand = n == 0 ? S.start_q : S.pool_q + base;
   const int32_t ncand = err ? 0 : (n == 0 ? S.nstart : S.pool_cnt[p]);
-  auto value = [&](int32_t i) -> double {
-    const int32_t q = cand[i];
-    if (q < 0) return -INFINITY;
-    const double a = n == 0 ? (double)__ldg(S.theta_s + q) : S.pool_d[base + i];
-    return a + (double)__ldg(S.theta_f + q);
+  // The values of FU candidates a thread, -inf where there is none.
+  auto values = [&](int32_t i0, double (&v)[FU]) {
+    int32_t q[FU];
+#pragma unroll
+    for (int u = 0; u < FU; ++u) {
+      const int32_t i = i0 + u * FT;
+      q[u] = i < ncand ? cand[i] : -1;
+    }
+    float f[FU];
+#pragma unroll
+    for (int u = 0; u < FU; ++u) f[u] = q[u] >= 0 ? __ldg(S.theta_f + q[u]) : neg_inf();
+#pragma unroll
+    for (int u = 0; u < FU; ++u) {
+      v[u] = -INFINITY;
+      if (f[u] != neg_inf()) v[u] = (n == 0 ? (double)__ldg(S.theta_s + q[u]) : S.pool_d[base + i0 + u * FT]) + (double)f[u];
+    }
   };
   // the candidates sit in the pool in scheduling order: the sum is made
   // order-independent (bitwise repeatable) by adding exp(v - max) as
   // integers, in units of 2^-62
   double mx = -INFINITY;
-  for (int32_t i = threadIdx.x; i < ncand; i += FT) mx = fmax(mx, value(i));
+  for (int32_t i0 = threadIdx.x; i0 < ncand; i0 += FT * FU) {
+    double v[FU];
+    values(i0, v);
+#pragma unroll
+    for (int u = 0; u < FU; ++u)
+      if (!dead64(v[u])) mx = fmax(mx, v[u]);
+  }
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) mx = fmax(mx, __shfl_xor_sync(FULL, mx, d));
   if (lane == 0) red_m[warp] = mx;
@@ -1450,12 +1484,29 @@ __global__ void __launch_bounds__(FT) k_fb_final(FrontierState S, double* __rest
   for (int w = 0; w < FT / 32; ++w) mx = fmax(mx, red_m[w]);
   unsigned long long lo = 0ull, hi = 0ull;  // 128-bit accumulator
   if (mx != -INFINITY) {
-    for (int32_t i = threadIdx.x; i < ncand; i += FT) {
-      const double v = value(i);
-      if (v == -INFINITY) continue;
-      const unsigned long long u = __double2ull_rn(exp(v - mx) * 4611686018427387904.0);  // 2^62
-      lo += u;
-      hi += (lo < u) ? 1ull : 0ull;
+    // The live candidates (a tenth, where a tenth of the states are final) of
+    // a round, packed: an exponential occupies the float64 unit for a whole
+    // warp whatever the number of its lanes.
+    for (int32_t c0 = 0; c0 < ncand; c0 += FT * FU) {
+      if (threadIdx.x == 0) npack = 0;
+      __syncthreads();
+      double v[FU];
+      values(c0 + (int32_t)threadIdx.x, v);
+#pragma unroll
+      for (int u = 0; u < FU; ++u) {
+        const uint32_t on = __ballot_sync(FULL, !dead64(v[u]));
+        int32_t at = 0;
+        if (lane == 0 && on) at = atomicAdd(&npack, __popc(on));
+        at = __shfl_sync(FULL, at, 0) + __popc(on & ((1u << lane) - 1u));
+        if (!dead64(v[u])) pack[at] = v[u];
+      }
+      __syncthreads();
+      for (int32_t i = threadIdx.x; i < npack; i += FT) {
+        const unsigned long long u = __double2ull_rn(exp(pack[i] - mx) * 4611686018427387904.0);  // 2^62
+        lo += u;
+        hi += (lo < u) ? 1ull : 0ull;
+      }
+      __syncthreads();
     }
   }
   red_lo[threadIdx.x] = lo;

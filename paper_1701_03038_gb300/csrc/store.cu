@@ -233,12 +233,16 @@ __global__ void k_pack_arcs(const int32_t* __restrict__ other, const float* __re
   if (i < P) arcs[i] = make_int4(other[i], __float_as_int(theta[i]), arc_id[i], 0);
 }
 
+// The weights by caller id into a layout's order, and (arcs set) into its
+// packed records: one gather for both.
 __global__ void k_set_weights(const int32_t* __restrict__ id, const float* __restrict__ th_by_id, int64_t P,
-                              float* __restrict__ theta) {
+                              float* __restrict__ theta, const int32_t* __restrict__ other, int4* __restrict__ arcs) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= P) return;
   const int32_t k = id[i];
-  theta[i] = k >= 0 ? th_by_id[k] : -INFINITY;
+  const float th = k >= 0 ? th_by_id[k] : -INFINITY;
+  theta[i] = th;
+  if (arcs) arcs[i] = make_int4(other[i], __float_as_int(th), k, 0);
 }
 
 // The weight of every segment's first arc in its (symbol, state) slot.
@@ -420,8 +424,8 @@ int build_store(fst_s* f, const int32_t* d_src, const int32_t* d_dst, const int3
 int set_layout_weights(fst_s* f, const float* d_theta_by_id, cudaStream_t s) {
   Layout* Ls[2] = {&f->fwd, &f->bwd};
   for (Layout* L : Ls) {
-    if (L->P > 0) k_set_weights<<<blocks_for(L->P), TB, 0, s>>>(L->arc_id, d_theta_by_id, L->P, L->theta);
-    if (L->P > 0 && L->arcs) k_pack_arcs<<<blocks_for(L->P), TB, 0, s>>>(L->other, L->theta, L->arc_id, L->P, L->arcs);
+    if (L->P > 0)
+      k_set_weights<<<blocks_for(L->P), TB, 0, s>>>(L->arc_id, d_theta_by_id, L->P, L->theta, L->other, L->arcs);
     if (L->nseg > 0 && L->seg_hash)
       k_set_first<<<blocks_for(L->nseg), TB, 0, s>>>(L->seg_slot, L->seg_pos, L->theta, L->nseg, L->seg_hash);
   }

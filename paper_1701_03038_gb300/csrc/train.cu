@@ -36,7 +36,7 @@ __global__ void k_by_id(const int32_t* __restrict__ arc_id, const int32_t* __res
   const int32_t id = arc_id[i];
   if (id < 0) return;
   const int64_t w = i / WIN;
-  int32_t lo = 0, hi = m;  // last a with sym_win[a] <= w
+  int32_t lo = 0, hi = il_out ? m : 0;  // last a with sym_win[a] <= w
   while (hi - lo > 1) {
     const int32_t mid = (lo + hi) >> 1;
     if (sym_win[mid] <= w) lo = mid; else hi = mid;
@@ -59,15 +59,42 @@ __global__ void k_em_totals(const float* __restrict__ counts, const int32_t* __r
   atomicAdd(total + src[k], (double)c + alpha);
 }
 
+// ... the logarithm of every total beside it ...
+__global__ void k_em_logs(const double* __restrict__ total, int64_t Q, double2* __restrict__ tl) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < Q) tl[q] = make_double2(total[q], total[q] > 0.0 ? log(total[q]) : 0.0);
+}
 // ... and theta'_k = log((count_k + alpha) / total[src_k]); a state with a
-// zero total keeps its arcs' old log-weights.
+// zero total keeps its arcs' old log-weights.  A float64 division and
+// logarithm of every arc took 380 us on 5M arcs (the float64 unit); the
+// difference of the logarithms, one of them taken in integers, is within a
+// few units of 2^-52 of the quotient's, and a result below log 1/2 rounds to
+// float32 as that does.  Nearer to 0 the quotient is taken (at most four arcs
+// of a state reach a quarter of its total); a count that is all of it gives 0.
 __global__ void k_em_theta(const float* __restrict__ counts, const int32_t* __restrict__ src,
-                           const float* __restrict__ theta_old, const double* __restrict__ total, int64_t A,
+                           const float* __restrict__ theta_old, const double2* __restrict__ tl, int64_t A,
                            double alpha, float* __restrict__ out) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= A) return;
-  const double t = total[src[k]];
-  out[k] = t > 0.0 ? (float)log(((double)counts[k] + alpha) / t) : theta_old[k];
+  const double2 t = __ldg(tl + src[k]);
+  const uint64_t ut = fx_bits(t.x);
+  if ((int64_t)ut <= 0) {  // (totals are at least 0)
+    out[k] = theta_old[k];
+    return;
+  }
+  const double c = fx_widen(counts[k]) + alpha;
+  const uint64_t uc = fx_bits(c);
+  const int ec = (int)(uc >> 52);
+  if (uc == ut) {
+    out[k] = 0.f;
+  } else if (uc == 0ull) {
+    out[k] = -INFINITY;
+  } else if (ec == 0 || ec >= (int)(ut >> 52) - 1) {
+    out[k] = (float)log(c / t.x);
+  } else {
+    const double l = (double)fx_log58((uc << 11) | (1ull << 63)) * 3.469446951953614e-18;  // 2^-58
+    out[k] = fx_narrow(fma((double)(ec - 1023), 0.6931471805599453, l) - t.y);
+  }
 }
 
 // (input label, output label) key of every arc, with its id, for the sort.
@@ -143,17 +170,21 @@ extern "C" int fst_em_update(fst_t* f, const float* counts, float pseudo_count, 
   if (A == 0) return FST_OK;
   const bool dev = (flags & FST_FLAG_DEVICE_PTRS) != 0;
   cudaStream_t s = 0;
-  DevMem mem;
-  float *d_counts = nullptr, *d_out = nullptr, *d_old = nullptr;
-  double* total = nullptr;
-  unsigned int* err = nullptr;
+  // (kept from call to call: allocating it took as long as the kernels)
+  Scratch mem;
+  const int64_t Q = f->Q;
   int rc;
-  if ((rc = mem.get(&d_old, A)) || (rc = mem.get(&total, f->Q)) || (rc = mem.get(&err, 1))) return rc;
-  if (dev) {
-    d_counts = (float*)counts;
-    d_out = theta_out;
-  } else {
-    if ((rc = mem.get(&d_counts, A)) || (rc = mem.get(&d_out, A))) return rc;
+  if ((rc = mem.take(f, Scratch::piece(A * 4) + Scratch::piece(Q * 8) + Scratch::piece(Q * 16) + Scratch::piece(4) +
+                            (dev ? 0 : 2 * Scratch::piece(A * 4)))))
+    return rc;
+  float* d_old = mem.get<float>(A);
+  double* total = mem.get<double>(Q);
+  double2* tl = mem.get<double2>(Q);
+  unsigned int* err = mem.get<unsigned int>(1);
+  float *d_counts = (float*)counts, *d_out = theta_out;
+  if (!dev) {
+    d_counts = mem.get<float>(A);
+    d_out = mem.get<float>(A);
     FST_CUDA(cudaMemcpy(d_counts, counts, (size_t)A * 4, cudaMemcpyHostToDevice));
   }
   FST_CUDA(cudaMemsetAsync(total, 0, (size_t)f->Q * 8, s));
@@ -167,7 +198,8 @@ extern "C" int fst_em_update(fst_t* f, const float* counts, float pseudo_count, 
     set_error("fst_em_update: a count is negative, NaN or infinite");
     return FST_ERR_INVALID_ARG;
   }
-  k_em_theta<<<nblk(A), TB, 0, s>>>(d_counts, f->src_by_id, d_old, total, A, (double)pseudo_count, d_out);
+  k_em_logs<<<nblk(Q), TB, 0, s>>>(total, Q, tl);
+  k_em_theta<<<nblk(A), TB, 0, s>>>(d_counts, f->src_by_id, d_old, tl, A, (double)pseudo_count, d_out);
   FST_CUDA(cudaGetLastError());
   if (flags & FST_EM_APPLY) {
     if ((rc = set_layout_weights(f, d_out, s))) return rc;
