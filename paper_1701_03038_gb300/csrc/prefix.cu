@@ -241,7 +241,7 @@ __device__ __forceinline__ void mul_tile(MulShared<T>& sh, const float* A, const
 }
 
 template <int T>
-__global__ void __launch_bounds__(TB) k_mul(const MulArgs M) {
+__global__ void __launch_bounds__(TB, 3) k_mul(const MulArgs M) {
   __shared__ MulShared<T> sh;
   // (what the level below wrote is read with __ldcg: read-only loads may be
   // moved up, over the wait)
@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(TB) k_close(const float* P, const float* V, in
                                               Out* __restrict__ o) {
   constexpr int WARPS = TB / 32;
   __shared__ Part part[WARPS];
+  __shared__ bool last;
   chain_enter();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double m = -INFINITY, s = 0.0;
@@ -333,26 +334,43 @@ __global__ void __launch_bounds__(TB) k_close(const float* P, const float* V, in
   for (int d = 16; d >= 1; d >>= 1) best = fmaxf(best, __shfl_xor_sync(FULL, best, d));
   if (lane == 0) part[warp] = Part{m, s, best, 0.f};
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int w = 1; w < WARPS; ++w) {
-    add_terms(m, s, part[w].m, part[w].sum);
-    best = fmaxf(best, part[w].best);
-  }
-  if (gridDim.x > 1) {
-    o->part[blockIdx.x] = Part{m, s, best, 0.f};
-    __threadfence();
-    if (atomicAdd(&o->done, 1u) + 1u < gridDim.x) return;
-    __threadfence();
-    m = -INFINITY;
-    s = 0.0;
-    for (unsigned b = 0; b < gridDim.x; ++b) {
-      const volatile Part* q = o->part + b;
-      add_terms(m, s, q->m, q->sum);
-      best = fmaxf(best, q->best);
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < WARPS; ++w) {
+      add_terms(m, s, part[w].m, part[w].sum);
+      best = fmaxf(best, part[w].best);
+    }
+    if (gridDim.x > 1) {
+      o->part[blockIdx.x] = Part{m, s, best, 0.f};
+      __threadfence();
+      last = atomicAdd(&o->done, 1u) + 1u == gridDim.x;
     }
   }
-  o->logz = m == -INFINITY ? -INFINITY : m + log(s);
-  o->best = best;
+  // (the last block, or the only one)
+  if (threadIdx.x >= 32) return;
+  if (gridDim.x > 1) {
+    __syncwarp();
+    if (!last) return;
+    __threadfence();
+    // its first warp adds the parts up, two a lane at most, in a fixed order
+    m = -INFINITY;
+    s = 0.0;
+    best = neg_inf();
+    for (unsigned b = lane; b < gridDim.x; b += 32) {
+      const Part* q = o->part + b;
+      add_terms(m, s, __ldcg(&q->m), __ldcg(&q->sum));
+      best = fmaxf(best, __ldcg(&q->best));
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+      const double m2 = __shfl_xor_sync(FULL, m, d), s2 = __shfl_xor_sync(FULL, s, d);
+      add_terms(m, s, m2, s2);
+      best = fmaxf(best, __shfl_xor_sync(FULL, best, d));
+    }
+  }
+  if (lane == 0) {
+    o->logz = m == -INFINITY ? -INFINITY : m + log(s);
+    o->best = best;
+  }
 }
 
 // A launch that begins while the one before it drains (chain_enter waits for it).
@@ -434,6 +452,33 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
       up[i] = (int32_t)(std::lower_bound(syms.begin(), syms.end(), ids[i]) - syms.begin());
     for (const int32_t a : syms) longest = std::max(longest, (sv.h_sym_win[a + 1] - sv.h_sym_win[a]) * (int64_t)WIN);
     const int64_t U = (int64_t)syms.size(), l1 = ((int64_t)n + 1) / 2, l2 = (l1 + 1) / 2;
+    // The first level's products are those of pairs of symbols: with few
+    // symbols (U^2 at most half of the pairs) each pair that occurs is
+    // multiplied once, and the second level names its operands.  (500
+    // products of 64 states: 42 us, the 36 of 6 symbols: 8.)
+    const int64_t pairs = n / 2;
+    int64_t uniq = 0;  // distinct pairs (0: every pair by itself)
+    std::vector<int32_t> slot2;
+    if (pairs >= 2 && U * U <= pairs / 2) {
+      std::vector<int32_t> id((size_t)(U * U), -1), first;
+      for (int64_t p = 0; p < pairs; ++p) {
+        int32_t& k = id[(size_t)(up[2 * p] * U + up[2 * p + 1])];
+        if (k < 0) {
+          k = (int32_t)uniq++;
+          first.push_back(up[2 * p]);
+          first.push_back(up[2 * p + 1]);
+        }
+        slot2.push_back(k);
+      }
+      if (n & 1) {
+        first.push_back(up[n - 1]);
+        slot2.push_back((int32_t)uniq);
+      }
+      up = first;
+    }
+    const int64_t count0 = (int64_t)up.size();
+    up.insert(up.end(), slot2.begin(), slot2.end());
+    const int64_t at_syms = (int64_t)up.size();
     up.insert(up.end(), syms.begin(), syms.end());
     if ((rc = mem.take(f, Scratch::piece(sizeof(Out)) + Scratch::piece((int64_t)up.size() * 4) +
                               Scratch::piece(2 * U * QQ * 4) + 2 * Scratch::piece(l1 * QQ * 4) +
@@ -451,13 +496,13 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
         dsum, 2 * U * QQ, -INFINITY, &d_out->done);
     for (int64_t u0 = 0; u0 < U; u0 += 65535)
       k_dense<<<dim3((unsigned)std::min<int64_t>((longest + TB - 1) / TB, 64), (unsigned)std::min<int64_t>(65535, U - u0)),
-                TB, 0, s>>>(sv.arcs, sv.theta, slice_sym_win(f), d_slot + n + u0, f->Q, dsum + u0 * QQ,
+                TB, 0, s>>>(sv.arcs, sv.theta, slice_sym_win(f), d_slot + at_syms + u0, f->Q, dsum + u0 * QQ,
                             dmax + u0 * QQ);
     FST_CUDA(cudaGetLastError());
     // the product tree: level by level, adjacent pairs multiplied
     const float *cur_s = dsum, *cur_m = dmax;
     const int32_t* slot = d_slot;
-    int64_t count = n;
+    int64_t count = count0;
     for (int level = 0; count > 1 || slot; ++level) {
       float *out_s = buf_s[level & 1], *out_m = buf_m[level & 1];
       const int64_t pairs = (count + 1) / 2;
@@ -474,8 +519,8 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
       }
       cur_s = out_s;
       cur_m = out_m;
-      slot = nullptr;
-      count = pairs;
+      slot = uniq && level == 0 ? d_slot + count0 : nullptr;
+      count = slot ? (int64_t)slot2.size() : pairs;
     }
     if ((rc = launch_after(k_close, dim3((unsigned)std::min<int64_t>((Q + 7) / 8, CLOSE_BLOCKS)), s, cur_s, cur_m, f->Q,
                            (const float*)f->theta_s, (const float*)f->theta_f, d_out)))
