@@ -59,41 +59,45 @@ __global__ void k_em_totals(const float* __restrict__ counts, const int32_t* __r
   atomicAdd(total + src[k], (double)c + alpha);
 }
 
-// ... the logarithm of every total beside it ...
-__global__ void k_em_logs(const double* __restrict__ total, int64_t Q, double2* __restrict__ tl) {
+// ... the logarithm of every total beside it, in units of 2^-52 ...
+struct Total {
+  double t;
+  int64_t log;
+};
+__global__ void k_em_logs(const double* __restrict__ total, int64_t Q, Total* __restrict__ tl) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < Q) tl[q] = make_double2(total[q], total[q] > 0.0 ? log(total[q]) : 0.0);
+  if (q < Q) tl[q] = Total{total[q], total[q] > 0.0 ? __double2ll_rn(log(total[q]) * 4503599627370496.0) : 0};
 }
 // ... and theta'_k = log((count_k + alpha) / total[src_k]); a state with a
 // zero total keeps its arcs' old log-weights.  A float64 division and
 // logarithm of every arc took 380 us on 5M arcs (the float64 unit); the
-// difference of the logarithms, one of them taken in integers, is within a
-// few units of 2^-52 of the quotient's, and a result below log 1/2 rounds to
-// float32 as that does.  Nearer to 0 the quotient is taken (at most four arcs
-// of a state reach a quarter of its total); a count that is all of it gives 0.
+// difference of the logarithms, in integers, is within 2e-15, far below half
+// a unit of a float32 result that is not within 2^-16 of 0.  There the
+// quotient is taken; a count that is all of its total gives 0.
 __global__ void k_em_theta(const float* __restrict__ counts, const int32_t* __restrict__ src,
-                           const float* __restrict__ theta_old, const double2* __restrict__ tl, int64_t A,
+                           const float* __restrict__ theta_old, const Total* __restrict__ tl, int64_t A,
                            double alpha, float* __restrict__ out) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= A) return;
-  const double2 t = __ldg(tl + src[k]);
-  const uint64_t ut = fx_bits(t.x);
+  const Total t = tl[src[k]];
+  const uint64_t ut = fx_bits(t.t);
   if ((int64_t)ut <= 0) {  // (totals are at least 0)
     out[k] = theta_old[k];
     return;
   }
-  const double c = fx_widen(counts[k]) + alpha;
+  const double c = alpha != 0.0 ? fx_widen(counts[k]) + alpha : fx_widen(counts[k]);
   const uint64_t uc = fx_bits(c);
   const int ec = (int)(uc >> 52);
   if (uc == ut) {
     out[k] = 0.f;
   } else if (uc == 0ull) {
     out[k] = -INFINITY;
-  } else if (ec == 0 || ec >= (int)(ut >> 52) - 1) {
-    out[k] = (float)log(c / t.x);
   } else {
-    const double l = (double)fx_log58((uc << 11) | (1ull << 63)) * 3.469446951953614e-18;  // 2^-58
-    out[k] = fx_narrow(fma((double)(ec - 1023), 0.6931471805599453, l) - t.y);
+    // (e ln 2 in two parts: 2^-52 and the 2^-58 below it)
+    const int64_t e = ec - 1023, low = e * (FX_LN2_58 & 63) + fx_log58((uc << 11) | (1ull << 63));
+    const int64_t d = e * (FX_LN2_58 >> 6) + (low >> 6) - t.log;
+    const bool near = ec == 0 || (d < (1ll << 36) && d > -(1ll << 36));  // within 2^-16 of 0, or subnormal
+    out[k] = near ? (float)log(c / t.t) : fx_narrow((double)d * 2.220446049250313e-16);  // 2^-52
   }
 }
 
@@ -179,7 +183,7 @@ extern "C" int fst_em_update(fst_t* f, const float* counts, float pseudo_count, 
     return rc;
   float* d_old = mem.get<float>(A);
   double* total = mem.get<double>(Q);
-  double2* tl = mem.get<double2>(Q);
+  Total* tl = mem.get<Total>(Q);
   unsigned int* err = mem.get<unsigned int>(1);
   float *d_counts = (float*)counts, *d_out = theta_out;
   if (!dev) {
