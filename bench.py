@@ -63,9 +63,11 @@ WORKLOADS = {
 PERSIST_NAMES = {"vit": "k_vit_persist", "fwd": "k_fwd_persist", "bwd": "k_bwd_persist"}
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 # the files that decide what the step kernels read and write
-KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "store.cu", "fst_internal.cuh")  # the device code of the batched passes
+KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "store.cu", "fst_internal.cuh", "strings.cu", "frontier.cuh",
+                  "fixmath.cuh")  # the device code of the batched passes
 PASS_KERNELS = {"vit": ("vit_first", "vit_step"), "fwd": ("fwd_first", "fwd_sum", "fwd_step"),
                 "bwd": ("bwd_step",)}
+STRING_NAMES = {"vit": "k_str_forward", "fwd": "k_str_forward", "bwd": "k_str_backward"}  # one launch a pass
 KERNEL_NAMES = {"vit_first": "k_vit_first", "vit_step": "k_vit_step", "fwd_first": "k_fwd_first",
                 "fwd_sum": "k_fwd_sum", "fwd_step": "k_fwd_step", "bwd_step": "k_bwd_step",
                 "vit_final": "k_vit_final", "backtrace": "k_backtrace", "fb_final": "k_fb_final",
@@ -87,11 +89,11 @@ def parse_args(argv=None):
     ap.add_argument("--e2e-steps", type=int, default=2)
     ap.add_argument("--strings", type=int, default=0, help="use only the first N strings (profiling captures)")
     ap.add_argument("--parts-vit", type=int, default=0,
-                    help="stream-parallel parts of the Viterbi plan (0 = the batch calls' rule: one per 32 "
-                         "strings, at most 2 and 400 / the longest string)")
+                    help="stream-parallel parts of the Viterbi plan (0 = one; with --pull or the other drivers one "
+                         "per 32 strings, at most 2 and 400 / the longest string)")
     ap.add_argument("--parts-fb", type=int, default=0,
-                    help="stream-parallel parts of the forward-backward plan (0 = one per 8 strings, at most 8 "
-                         "and 1,600 / the longest string)")
+                    help="stream-parallel parts of the forward-backward plan (0 = one; with --pull or the other "
+                         "drivers one per 256 strings, at most 16)")
     ap.add_argument("--pull", type=int, default=0,
                     help="direction switch of the forward pass: live states from which a token pulls "
                          "(0 = off, the library default; -1 = half the states)")
@@ -103,7 +105,8 @@ def parse_args(argv=None):
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-graph", action="store_true", help="launch the timed steps from the host, not a CUDA graph")
     ap.add_argument("--driver", default="graph", choices=["graph", "persistent", "persistent-all", "autotune"],
-                    help="graph: one launch per position, the step replayed as a CUDA graph; persistent: the "
+                    help="graph: the string kernels, one launch a pass (per position with --pull), the step "
+                         "replayed as a CUDA graph; persistent: the "
                          "forward-backward plan as persistent passes (one cooperative launch each), the Viterbi "
                          "plan beside it on its own stream; persistent-all: both plans persistent, one after the "
                          "other; autotune: each plan's driver and grid chosen by fst_plan_autotune")
@@ -115,7 +118,7 @@ def parse_args(argv=None):
 
 
 def auto_parts(args, B, tmax):
-    """The plan parts of the graph-replayed device step: the arguments, or
+    """The plan parts of a step of the per-position kernels: the arguments, or
     by batch size: one Viterbi part per 32 strings, at most 2 and at most
     400 / tmax position launches' worth (tmax the longest string), and one
     forward-backward part per 256 strings, at most 16.  A graph replays the
@@ -280,6 +283,7 @@ def roofline(prof, live, peak, peak_src, traffic, stats=None, ids=None, persiste
          "frac": round(achieved / peak, 5), "traffic": None if tr is None else int(tr),
          "per": f"{dom} pass (all its launches)",
          "kernel": (PERSIST_NAMES[dom] if dom in persistent
+                    else STRING_NAMES[dom] if "fwd_sum" in prof and not prof["fwd_sum"][1]
                     else " + ".join(KERNEL_NAMES[x] for x in PASS_KERNELS[dom])),
          "launches": sum(prof[x][1] for x in PASS_KERNELS[dom]), "pass_ms": round(pass_ms[dom], 3),
          "algorithmic_bytes": int(alg[dom]),
@@ -539,7 +543,11 @@ def bench_batch(args, rank, world, dev, fa, strs, f, stats):
     ids = torch.from_numpy(strs.ids).to(dev)
     off = torch.from_numpy(strs.offsets).to(dev)
     acc = _lib.PLAN_DENSE_ACC if args.dense_acc else 0
-    args.parts_vit, args.parts_fb = auto_parts(args, strs.count, int(np.diff(strs.offsets).max(initial=1)))
+    if args.driver == "graph" and args.pull == 0:
+        # the string kernels fill the GPU with one part of any size
+        args.parts_vit, args.parts_fb = max(args.parts_vit, 1), max(args.parts_fb, 1)
+    else:
+        args.parts_vit, args.parts_fb = auto_parts(args, strs.count, int(np.diff(strs.offsets).max(initial=1)))
     plans_v = [f.plan(ids, off, mem_budget=budget, flags=PLAN_NO_FB | acc, parts=args.parts_vit)]
     plans_f = [f.plan(ids, off, mem_budget=budget, flags=PLAN_NO_VITERBI | acc, parts=args.parts_fb)]
     for p in plans_f:
@@ -635,8 +643,9 @@ def bench_batch(args, rank, world, dev, fa, strs, f, stats):
         "streams": f"a Viterbi plan of {args.parts_vit} and a forward-backward plan of {args.parts_fb} "
                    "stream-parallel parts; per-kernel times from one more step run serially",
         "launch": "CUDA graph replay" if graph is not None else "host launches",
-        "driver": {"viterbi": "persistent" if plans_v[0].driver()[0] else "one launch per position",
-                   "forward_backward": "persistent" if plans_f[0].driver()[0] else "one launch per position",
+        "driver": {"viterbi": "persistent" if plans_v[0].driver()[0] else "one launch per pass",
+                   "forward_backward": "persistent" if plans_f[0].driver()[0] else
+                   ("one launch per pass" if args.pull == 0 else "one launch per position"),
                    "grid": {"viterbi": plans_v[0].driver()[1], "forward_backward": plans_f[0].driver()[1]},
                    "concurrent": not serial, "autotune": tuned or None},
         "l2": "no flush: inputs larger than L2 (arc store and hash "
@@ -767,7 +776,8 @@ def plain_launches(f, strs, stats, coef) -> int:
     non-empty slice + final + output labels; the frontier Viterbi first +
     n steps + final + backtrace (one persistent pass + 2 with that
     driver); the frontier forward-backward first + n (sum + step) + final
-    + n backward steps + counts (persistent: 2 passes + 2)."""
+    + n backward steps + counts (persistent: 2 passes + 2).  The frontier
+    figures are those of one launch per position (string_launches)."""
     from paper_1701_03038_gb300 import _lib
     pm = f.plain_method()
     if pm["method"] == _lib.PLAIN_BLOCK:
@@ -786,6 +796,25 @@ def plain_launches(f, strs, stats, coef) -> int:
         else:
             total += (3 if n >= 1 else 2) if persist else n + 3 - (n == 0)
         total += (4 if n >= 1 else 2) if persist else 3 * n + 3 - (n == 0)
+    return total
+
+
+def string_launches(f, strs, stats, coef) -> int:
+    """The same where the handle's driver is the launch driver and its method
+    not the one-block kernels: the string kernels, Viterbi as forward +
+    final + trace, forward-backward as forward + final + backward + counts."""
+    from paper_1701_03038_gb300 import _lib
+    pm = f.plain_method()
+    if pm["method"] == _lib.PLAIN_BLOCK or pm["driver"] == _lib.DRIVER_PERSISTENT:
+        return plain_launches(f, strs, stats, coef)
+    total = 0
+    for b in range(strs.count):
+        x = strs.get(b)
+        n = len(x)
+        arcs = int(stats[0][x].sum())
+        slice_vit = pm["method"] == _lib.PLAIN_SLICE or (
+            pm["method"] == _lib.PLAIN_AUTO and coef[2] + coef[3] * n + coef[4] * arcs < coef[0] + coef[1] * n)
+        total += 4 + (int((stats[0][x] > 0).sum()) + 1 + (n > 0) if slice_vit else 3)
     return total
 
 
@@ -813,7 +842,7 @@ def bench_plain(args, rank, world, dev, fa, strs, f, stats):
             f.forward_backward(x, out=h_post)
 
     ms, clk = timed(step, args, world, dev, ClockSampler(int(str(dev).split(":")[-1])))
-    launches = plain_launches(f, strs, stats, coef)
+    launches = string_launches(f, strs, stats, coef)
     out = base_line(args, world, fa, strs, ms, relax_step, clk, args.steps * launches)
     out["config"].update({"parallelism": "replicas" if world > 1 else "1 GPU",
                           "launch": "host launches, one string at a time (fst_viterbi, fst_forward_backward; posteriors into a pinned host buffer)",
@@ -917,7 +946,7 @@ def bench_train(args, rank, world, dev, fa, strs, f, stats):
     out["config"].update({"relaxations_per_pass": relax_pass, "plan_gb": round(info["device_bytes"] / 2**30, 2),
                           "parallelism": "replicas" if world > 1 else "1 GPU",
                           "launch": "host launches (fst_set_weights between steps is synchronous)",
-                          "driver": {"forward_backward": "persistent" if plan.driver()[0] else "one launch per position",
+                          "driver": {"forward_backward": "persistent" if plan.driver()[0] else "one launch per pass",
                                      "grid": plan.driver()[1], "autotune": tuned},
                           "l2": "no flush: arc store, plan storage and the 2M-arc count vector exceed L2"})
     plan.profile(True)

@@ -179,8 +179,10 @@ FST_API int fst_set_plain_method(fst_t* fst, int32_t method);
 FST_API int fst_autotune_plain(fst_t* fst, const int32_t* ids, const int64_t* offsets, int32_t B, double* coef);
 
 /* Driver of the single-string frontier kernels (fst_forward_backward, and
- * fst_viterbi when it uses them): FST_DRIVER_LAUNCH (one launch per
- * position and kernel kind, the default) or FST_DRIVER_PERSISTENT (one
+ * fst_viterbi when it uses them): FST_DRIVER_LAUNCH (the default: the
+ * string kernels, one launch per pass, in which warps and blocks run the
+ * whole string; a string whose live pool may pass 2^31 entries takes one
+ * launch per position and kernel kind) or FST_DRIVER_PERSISTENT (one
  * cooperative launch per pass, grid_blocks blocks, 0 = one per SM,
  * positions separated by bounded grid barriers; a barrier that times out
  * makes the call return FST_ERR_TIMEOUT).  fst_autotune_plain also picks
@@ -283,27 +285,30 @@ FST_API int fst_forward_backward_batch(fst_t* fst, const int32_t* d_ids, const i
 FST_API int fst_set_batch_budget(fst_t* fst, int64_t mem_budget_bytes);
 
 /* Plans of fst_viterbi_batch and fst_forward_backward_batch: parts_viterbi
- * and parts_fb stream-parallel parts (FST_PLAN_PARTS; 0 = by batch size:
- * one Viterbi part per 32 strings, at most 2 and at most 400 / n, one
- * forward-backward part per 8 strings, at most 4 and at most 1,600 / n,
- * n the longest string) and the accumulator layout (-1 = dense when
- * the dense accumulators and the live pool fit the batch budget in one
- * wave, else compact; 0 = compact; 1 = FST_PLAN_DENSE_ACC), and whether
+ * and parts_fb stream-parallel parts (FST_PLAN_PARTS; 0 = one part: the
+ * string kernels fill the device with one) and the layout that the plan's
+ * per-position kernels would take (-1 = dense when the dense accumulators
+ * and the live pool fit the batch budget in one wave, else compact; 0 =
+ * compact; 1 = FST_PLAN_DENSE_ACC), and whether
  * the run's launches are recorded into a CUDA graph that is then launched
  * (graph: 0 = no, 1 = yes, never on the legacy default stream or inside a
- * capture the caller began; -1 = the default, no: recording and
- * instantiating a run of thousands of launches measured slower than
- * issuing them).  The default is 0, 0, -1, -1.  A batch call keeps its
- * plan's device storage for the next call of the same kind (part by part).
- * Outside a graph capture, the parts of a plan issue their launches from
- * one host thread each. (Execution policy: no counterpart in the paper.) */
+ * capture the caller began; -1 = the default, no).  The default is 0, 0,
+ * -1, -1.  A batch call keeps its plan's device storage for the next call
+ * of the same kind (part by part).  Outside a graph capture, the parts of a
+ * plan whose kernels run per position issue their launches from one host
+ * thread each. (Execution policy: no counterpart in the paper.) */
 FST_API int fst_set_batch_plan(fst_t* fst, int32_t parts_viterbi, int32_t parts_fb, int32_t layout, int32_t graph);
 
 /* A plan holds everything a batch needs on the device for the per-position
- * loops of Alg. 1 and Alg. 2 (Sec. 5): the token lists of
- * every position (strings sorted by length), the accumulators, the live
- * pool of every position (states, values, backpointers or arcs) and the
- * per-token scalars.  The accumulators are hash tables keyed by (string,
+ * loops of Alg. 1 and Alg. 2 (Sec. 5): the strings, the live pool of
+ * every position (states, values, backpointers or arcs), the per-token
+ * scalars, and the string kernels' queues and accumulators (dense arrays
+ * of all states for at most two blocks per SM, within a quarter of the
+ * budget).  What only the per-position kernels need (the token lists of
+ * every position, their accumulators) is allocated by the call that first
+ * asks for them: fst_plan_set_driver (persistent), fst_plan_set_pull,
+ * fst_plan_limit_table, fst_plan_table_slots, fst_plan_autotune; those
+ * calls then synchronise.  These accumulators are hash tables keyed by (string,
  * state), sized for 128 live states per token of the busiest position (at
  * most the symbols' destination counts) at half load; a position that
  * holds more live states than a table fits ends the run with FST_ERR_OOM,
@@ -527,9 +532,14 @@ FST_API int fst_live_work(fst_t* fst, int64_t* entries, int64_t* arcs);
 FST_API int fst_plan_live_work(fst_plan_t* plan, int64_t* entries, int64_t* arcs, void* stream);
 
 /* How a plan advances its positions (the batched driver).
- *   FST_DRIVER_LAUNCH      one kernel launch per position and kernel kind
- *                          (the default; a run can be captured into a CUDA
- *                          graph and replayed).
+ *   FST_DRIVER_LAUNCH      the string kernels (the default): one launch
+ *                          per pass, in which a warp or block runs a string
+ *                          over all of its positions; a wait that sees no
+ *                          progress for 2 s ends the run with
+ *                          FST_ERR_TIMEOUT.  With the direction switch or a
+ *                          table limit one launch per position and kernel
+ *                          kind instead.  Either run can be captured into a
+ *                          CUDA graph and replayed.
  *   FST_DRIVER_PERSISTENT  one cooperative launch per pass (Viterbi, forward,
  *                          backward) of grid_blocks blocks (0 = the plan's
  *                          estimate), all co-resident, that runs every
