@@ -341,6 +341,7 @@ int plain_string(fst_s* f, bool viterbi, StringWork* K) {
   const int64_t Q = f->Q;
   int rc;
   if (!w->str_ctl) {
+    dfree(w->str_dirty); dfree(w->str_kept); dfree(w->str_stage);
     const int64_t ctl = string_ctl_words(1, 1);
     if ((rc = dalloc(&w->str_dirty, 2)) || (rc = dalloc(&w->str_kept, string_kept_values())) ||
         (rc = dalloc(&w->str_stage, Q)))

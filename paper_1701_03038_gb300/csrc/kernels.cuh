@@ -281,6 +281,7 @@ struct StringWork {
   int64_t fe_light;           // where the light warps' begin
   int32_t groups2;            // heavy blocks that run strings
   int32_t chunk;              // pool entries a group reserves at a time (0: each range by itself)
+  int32_t share = 1;          // launches like this one that run side by side
 };
 // What a launch sees of it.
 struct StringQueue {

@@ -194,6 +194,7 @@ struct fst_plan_s {
   // ranges, each run on its own stream; the plan itself then holds only the
   // count accumulators that the parts share
   std::vector<fst_plan_s*> parts;
+  int32_t share = 1;  // parts that run side by side with this one
   std::vector<int32_t> part_b0;
   std::vector<int64_t> part_tok0;
   std::vector<cudaStream_t> part_stream;
@@ -542,6 +543,7 @@ StringWork string_work(fst_plan_s* P, const Wave& W, bool viterbi) {
   K.fe = P->str_fe;
   K.groups2 = P->str_groups2;
   K.chunk = P->pool_limit > 0 ? 0 : POOL_CHUNK;
+  K.share = P->share;
   return K;
 }
 FrontierState string_state(fst_plan_s* P, const Wave& W, const float* gweight) {
@@ -858,6 +860,7 @@ static int plan_create_parts(fst_t* f, const int32_t* d_ids, const int64_t* d_of
   }
   for (int32_t i = 0; i < nparts; ++i) {
     sub[i]->chain = nparts <= chain_parts_max();
+    sub[i]->share = nparts;
     P->parts.push_back(sub[i]);
     P->part_b0.push_back(bs[i]);
     P->part_tok0.push_back(h_off[bs[i]]);

@@ -41,15 +41,15 @@ namespace fstgpu {
 namespace {
 
 // Arcs per lane in flight: a light warp's (its table serves at most 128
-// arcs) and a heavy block's.  More of them spill: with 4 and 4 a backward
-// pass over 4,096 strings of 5 to 200 symbols on 20M arcs takes 4.35 ms
-// instead of 3.80, and the forward passes are the same.
+// arcs) and a heavy block's.  More of them spill: with 4 a heavy block's
+// backward pass over 4,096 strings of 5 to 200 symbols on 20M arcs takes 18%
+// longer (2.7 ms with 2), and the forward passes (2.9 and 4.6 ms) are the same.
 constexpr int VU0 = 1, VU1 = 2;
 
 // Threads of a block (a light block runs NT1 / 32 strings), and the slots of
 // a light warp's and a heavy block's table.  The kernels are compiled for
-// three blocks an SM (80 registers a thread): two (128) cost the same
-// backward pass 5.5 ms, four (64) the 1,000-symbol strings 7%.
+// three blocks an SM (80 registers a thread): with two (128) the same
+// backward pass takes 40% longer, with four (64) the Viterbi pass 30%.
 constexpr int NT1 = 256, WARPS = NT1 / 32;
 constexpr int HS0 = 256, HS1 = 2048;
 // the same of the backward pass, whose light warps hold at most LIGHT_CAP
@@ -1297,6 +1297,7 @@ struct Forward {
           if (tid == 0) {
             hv.base = reserve(sh.gs, nb);
             hv.tot = hv.mk = 0u;
+            if (!light) hv.at = peek(K.ctl + CTL_ALIVE) != 0u;
           }
           if (!VIT && !single)
             for (int32_t c = 0; c < P.cnt; c += NT1 * BlockStage::PER) {
@@ -1326,6 +1327,7 @@ struct Forward {
           P.cnt = nbase < 0 ? 0 : nb;
           P.tot = (int32_t)hv.tot;
           mk = hv.mk;
+          light = hv.at != 0;  // (light blocks that began meanwhile)
           done = true;
         }
       }
@@ -1919,9 +1921,11 @@ struct Backward {
           hv.tag = ~0ull;
           fill(hv.job, P, R, self, et, dense, shared);
           hv.mk = 0u;
+          if (!light) hv.at = peek(K.ctl + CTL_ALIVE) != 0u;
         }
         mine = true;
         __syncthreads();
+        light = hv.at != 0;  // (light blocks that began meanwhile)
       }
       // the chunks: the own position's, all by itself or shared, or, between
       // two positions, others'
@@ -2085,7 +2089,11 @@ int resident(K kernel, int which, size_t smem, int num_sms, int* out) {
 // the blocks light, Viterbi of 4,096 strings on 20M arcs took 3.5 ms instead
 // of 3.0, with an eighth 3.3; a training step of 1,024 strings whose last 112
 // wait for a warp took 0.92 ms instead of 0.87.)
+// Launches of W.share parts on streams of their own divide the blocks among
+// them: blocks that wait for a place serve their strings late and by the
+// wrong role (sixteen forward-backward parts of 256 strings: 32 ms a step).
 StringQueue string_queue(const StringWork& W, int blocks, int32_t* grid) {
+  blocks = std::max(blocks / std::max(W.share, 1), 8);
   StringQueue K;
   K.strings = W.Bw;
   K.ctl = W.ctl;
