@@ -1,5 +1,5 @@
 """The parallel product over time against float64 matrix products: sizes round
-the edges of its tiles, odd numbers of matrices, and weights so far apart that
+the edges of its tiles, odd numbers of matrices, repeated pairs, and weights so far apart that
 the scaled sums underflow and are taken again."""
 import numpy as np
 import pytest
@@ -24,7 +24,8 @@ def _lse(x, axis):
 
 
 @pytest.mark.parametrize("spread", [1.0, 150.0])
-@pytest.mark.parametrize("Q,n", [(1, 3), (3, 1), (31, 2), (32, 5), (33, 6), (63, 9), (64, 17), (65, 13), (97, 7), (130, 33)])
+@pytest.mark.parametrize("Q,n", [(1, 3), (3, 1), (31, 2), (32, 5), (33, 6), (63, 9), (64, 17), (65, 13), (97, 7), (130, 33),
+                                 (5, 37), (9, 40), (33, 75), (64, 41)])  # (repeated pairs of symbols, even and odd)
 def test_product_over_time(Q, n, spread):
     from paper_1701_03038_gb300.fst import Fst
     rng = np.random.default_rng(1000 * Q + n)
