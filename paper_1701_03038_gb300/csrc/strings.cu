@@ -1262,6 +1262,7 @@ struct Forward {
         }
         an = P.t < P.n ? __ldg(sym + P.off + P.t) : -1;
         if (P.tot > HS1 / 2 || P.cnt >= SHARE_ARCS) {
+          __syncthreads();  // (every thread has read hv.tot, hv.mk and hv.at of the position before)
           // (many entries with few arcs are work too: 176,615 of them with
           // 2,627 took a block by itself 860 us)
           const int32_t size = max(P.tot, P.cnt);

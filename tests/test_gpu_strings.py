@@ -102,3 +102,37 @@ def test_string_kernels_match_per_position_kernels(fans, widths, count):
     for i in list(range(5)) + [strs.count - 1]:
         lo, hi = strs.offsets[i], strs.offsets[i + 1]
         assert_viterbi_equal(sc[i], pa[lo:hi], None, st[i], o.viterbi(strs.get(i)))
+
+
+def _same_as_per_position(f, strs, runs):
+    """The string kernels' outputs, run after run, against the persistent driver's."""
+    import torch
+    from paper_1701_03038_gb300 import _lib
+    ids, off = torch.from_numpy(strs.ids).cuda(), torch.from_numpy(strs.offsets).cuda()
+    B, N = strs.count, len(strs.ids)
+    p = f.plan(ids, off, flags=_lib.PLAN_DENSE_ACC)
+    p.set_driver(_lib.DRIVER_PERSISTENT)
+    p.viterbi()
+    p.forward_backward()
+    torch.cuda.synchronize()
+    q = f.plan(ids, off)
+    for _ in range(runs):
+        q.viterbi()
+        q.forward_backward()
+        torch.cuda.synchronize()
+        for k, n in (("status", B), ("scores", B), ("paths", N), ("olabels", N), ("logz", B)):
+            assert torch.equal(getattr(q, k)[:n], getattr(p, k)[:n]), k
+        # the same float32 posteriors added up in float64 in another order: at
+        # most one float32 rounding apart
+        np.testing.assert_allclose(q.counts.cpu().numpy(), p.counts.cpu().numpy(), rtol=2.0**-23, atol=1e-12)
+
+
+@pytest.mark.parametrize("count", [1, 40])
+def test_table_and_dense_positions_in_turn(fans, count):
+    # a heavy block's every change between its table and dense positions that
+    # it works through alone, with no other barrier between them
+    f, _ = fans
+    turn = [FAN + 9, STEP, GATHER, FAN + 13, GATHER, FAN + 12, STEP, STEP, GATHER]
+    out = [turn * (60 + b % 3) for b in range(count)]
+    off = np.concatenate([[0], np.cumsum([len(s) for s in out])]).astype(np.int64)
+    _same_as_per_position(f, synth.Strings(np.concatenate(out).astype(np.int32), off), 6)
