@@ -419,6 +419,7 @@ struct HeavyPick {
   uint64_t first = 0u;
   // All threads call it; *light: the light warps take light strings.
   __device__ __forceinline__ int32_t next(HeavyShared& hv, const StringQueue& K, bool* light) {
+    __syncthreads();  // (every thread has read hv.pick of a search that found no job)
     if (threadIdx.x == 0) {
       int32_t b = PICK_NONE;
       const bool begun = holds || all_begun(K);

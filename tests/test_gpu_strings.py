@@ -136,3 +136,14 @@ def test_table_and_dense_positions_in_turn(fans, count):
     out = [turn * (60 + b % 3) for b in range(count)]
     off = np.concatenate([[0], np.cumsum([len(s) for s in out])]).astype(np.int64)
     _same_as_per_position(f, synth.Strings(np.concatenate(out).astype(np.int32), off), 6)
+
+
+@pytest.mark.parametrize("count", [1, 3])
+def test_idle_blocks_look_for_jobs(fans, count):
+    # few strings of many shared positions: hundreds of blocks without a
+    # string find a job, or look for one that others have taken, at each
+    f, _ = fans
+    turn = [FAN + 15, SCATTER, STEP, GATHER, STEP, STEP]
+    out = [turn * (50 + b) for b in range(count)]
+    off = np.concatenate([[0], np.cumsum([len(s) for s in out])]).astype(np.int64)
+    _same_as_per_position(f, synth.Strings(np.concatenate(out).astype(np.int32), off), 6)
