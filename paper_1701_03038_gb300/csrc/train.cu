@@ -86,7 +86,7 @@ __global__ void k_em_theta(const float* __restrict__ counts, const int32_t* __re
     return;
   }
   const double c = alpha != 0.0 ? fx_widen(counts[k]) + alpha : fx_widen(counts[k]);
-  const uint64_t uc = fx_bits(c);
+  const uint64_t uc = fx_bits(c) & 0x7fffffffffffffffull;  // (a count may be -0)
   const int ec = (int)(uc >> 52);
   if (uc == ut) {
     out[k] = 0.f;

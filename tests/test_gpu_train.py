@@ -44,6 +44,32 @@ def test_em_update_matches_oracle():
         assert np.allclose(tot[used], 1.0, atol=1e-5)
 
 
+@pytest.mark.parametrize("alpha", [0.0, 0.5])
+def test_em_update_negative_zero_counts(alpha):
+    # the counts of arcs not used are -0 where a gradient was negated: the
+    # same log-weights as from +0, bit for bit, and what float64 gives
+    import torch
+    from paper_1701_03038_gb300.fst import Fst
+    fa, _ = _case()
+    f = Fst.from_arrays(fa)
+    rng = np.random.default_rng(11)
+    c = rng.uniform(0.0, 3.0, fa.num_arcs).astype(np.float32)
+    c[rng.random(fa.num_arcs) < 0.6] = 0.0
+    c[fa.src < fa.num_states // 8] = 0.0  # states of no count at all
+    neg = np.where(c == 0, np.float32(-0.0), c)
+    assert np.signbit(neg).any()
+    want = f.em_update(c, alpha)
+    got = [f.em_update(neg, alpha), f.em_update(torch.from_numpy(neg).cuda(), alpha).cpu().numpy(),
+           f.em_update(-torch.from_numpy(-c).cuda(), alpha).cpu().numpy()]
+    total = np.bincount(fa.src, weights=c.astype(np.float64) + alpha, minlength=fa.num_states)[fa.src]
+    with np.errstate(divide="ignore", invalid="ignore"):
+        ref = np.log((c.astype(np.float64) + alpha) / total)
+    ref = np.where(total > 0, ref, -fa.weight.astype(np.float64))
+    for g in got:
+        assert np.array_equal(g.view(np.uint32), want.view(np.uint32))
+    assert np.allclose(want, ref, rtol=2 ** -22, atol=1e-12)
+
+
 def test_em_apply_and_training_raises_likelihood():
     # EM iterations on the device (counts from the batched backward pass,
     # then the M-step installed with FST_EM_APPLY) beside the same
