@@ -25,6 +25,7 @@
 // its ten levels; all products together are 0.5 GFLOP.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -104,16 +105,23 @@ struct MulArgs {
   float *out_sum, *out_max;
   int32_t count, Q;
 };
-template <int T>
-struct MulShared {
-  static constexpr int PARTS = TB / T;
-  float A[T][KC + 4], B[KC][T + 4];
-  float rmax[T], cmax[T], part[PARTS][T];
-};
 template <int N>
 struct alignas(4 * N) Vec {
   float v[N];
 };
+template <int T>
+struct alignas(16) MulShared {
+  static constexpr int PARTS = TB / T;
+  float A[T][KC + 4], B[KC][T + 4];
+  float rmax[T], cmax[T], part[PARTS][T];
+};
+// The rows that a thread reads as vectors: four of A at once, T / 16 of B.
+template <class S>
+constexpr bool vector_rows(int r) {
+  return alignof(S) % alignof(Vec<4>) == 0 && offsetof(S, A) % alignof(Vec<4>) == 0 &&
+         sizeof(S::A[0]) % alignof(Vec<4>) == 0 && offsetof(S, B) % (4 * r) == 0 && sizeof(S::B[0]) % (4 * r) == 0;
+}
+static_assert(vector_rows<MulShared<32>>(2) && vector_rows<MulShared<64>>(4), "vector reads need aligned rows");
 
 template <int T, bool MAX>
 __device__ __forceinline__ void mul_tile(MulShared<T>& sh, const float* A, const float* B, float* out, int32_t i0, int32_t j0, int32_t Q) {
