@@ -14,9 +14,11 @@
 // A[i][k] + B[k][j].  The sums are taken in the linear domain: with r_i the
 // largest entry of row i and c_j that of column j, exp(A - r) and exp(B - c)
 // are multiplied as matrices and r_i + c_j + log of the sum is the entry --
-// Q^2 exponentials a product where adding the logs one by one takes Q^3.  A
-// sum so small that terms may have underflowed (the largest A + B far below
-// r + c) is taken again in the log domain.  The Viterbi score is the best
+// Q^2 exponentials a product where adding the logs one by one takes Q^3.  The
+// differences and that last sum carry their rounding errors along (Knuth's
+// error-free addition, TAOCP 2, 4.2.2): r + c may be far larger than the
+// entry.  A sum so small that terms may have underflowed (the largest A + B
+// far below r + c) is taken again in the log domain.  The Viterbi score is the best
 // path's weight with its float32 additions associated in tree order rather
 // than left to right.
 //
@@ -42,8 +44,8 @@ constexpr int TB = 256;
 constexpr int KC = 64;     // k chunk staged in shared memory
 constexpr int PREFIX_MAX_STATES = 512;
 // sums below this may have lost terms to underflow (a lost term is below
-// 2^-126, and there are at most 512 of them)
-constexpr float TINY = 1e-30f;
+// 2^-126, and the at most 512 of them below half a rounding of this)
+constexpr float TINY = 1e-28f;
 
 __global__ void k_fill(float* __restrict__ p, int64_t n, float v, uint32_t* __restrict__ zero) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *zero = 0u;
@@ -57,6 +59,40 @@ __device__ __forceinline__ float log_add(float a, float b) {
   if (b == neg_inf()) return a;
   const float hi = fmaxf(a, b), lo = fminf(a, b);
   return hi + log1pf(expf(lo - hi));
+}
+
+// The rounded sum and its error: a + b = s + e exactly.
+struct Sum2 {
+  float s, e;
+};
+__device__ __forceinline__ Sum2 add2(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return Sum2{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+
+// exp(x - m), x <= m: within the roundings of the exponential and of the
+// product, whatever the sizes of x and m.
+__device__ __forceinline__ float exp_below(float x, float m) {
+  if (x == neg_inf()) return 0.f;
+  const Sum2 d = add2(x, -m);
+  const float y = expf(d.s);
+  return y == 0.f ? 0.f : fmaf(y, d.e, y);  // (a difference that overflows has no error term)
+}
+
+// r + c + log x, x normal and positive, rounded about once: log x = k log 2 +
+// log f with f in [0.7, 1.42), k log 2 in a part that is exact for any k (log
+// 2 to 12 bits) and a small one.
+__device__ __forceinline__ float add_log(float r, float c, float x) {
+  constexpr float HI = 2839.f / 4096.f, LO = (float)(0.693147180559945309417 - 2839.0 / 4096.0);
+  const uint32_t u = __float_as_uint(x);
+  float f = __uint_as_float((u & 0x7fffffu) | 0x3f800000u), k = (float)((int32_t)(u >> 23) - 127);
+  if (f > 1.41f) {
+    f *= 0.5f;
+    k += 1.f;
+  }
+  const Sum2 a = add2(r, c), b = add2(a.s, k * HI);
+  if (isinf(b.s)) return b.s;
+  return b.s + ((a.e + b.e) + (k * LO + logf(f)));
 }
 
 // The dense matrices of the symbols syms[blockIdx.y] (both filled with
@@ -190,8 +226,8 @@ __device__ __forceinline__ void mul_tile(MulShared<T>& sh, const float* A, const
         const int32_t e = t + u * TB;
         float& a = sh.A[e / KC][e % KC];
         float& b = sh.B[e / T][e % T];
-        a = a == neg_inf() ? 0.f : expf(a - sh.rmax[e / KC]);
-        b = b == neg_inf() ? 0.f : expf(b - sh.cmax[e % T]);
+        a = exp_below(a, sh.rmax[e / KC]);
+        b = exp_below(b, sh.cmax[e % T]);
       }
       __syncthreads();
     }
@@ -225,7 +261,7 @@ __device__ __forceinline__ void mul_tile(MulShared<T>& sh, const float* A, const
         if (rm == neg_inf() || cm == neg_inf()) {
           r = neg_inf();
         } else if (r >= TINY) {
-          r = rm + cm + logf(r);
+          r = add_log(rm, cm, r);
         } else {
           // terms may have underflowed: the log-sum one by one
           float m = neg_inf(), s = 0.f;

@@ -64,3 +64,29 @@ def test_product_over_time(Q, n, spread):
     tol = 4 * levels * 2.0**-24 * (spread * n + 8.0)
     assert st == 0 and abs(lz - want) <= tol, (lz, want, tol)
     assert abs(best - vbest) <= tol, (best, vbest, tol)
+
+
+@pytest.mark.parametrize("Q", [4, 16, 33, 70])
+def test_scales_that_cancel(Q):
+    # rows and columns whose largest entries do not meet: the scales add up to
+    # 58, the entries of the product stay near 0 and are as accurate as there
+    from paper_1701_03038_gb300.fst import Fst
+    rng = np.random.default_rng(Q)
+    i, j = (x.ravel().astype(np.int32) for x in np.meshgrid(np.arange(Q), np.arange(Q), indexing="ij"))
+    start, final = np.full(Q, np.inf, np.float32), np.full(Q, np.inf, np.float32)
+    start[0] = final[Q - 1] = 0.0
+    for _ in range(12):
+        M = rng.uniform(-1.0, 1.0, (2, Q, Q)).astype(np.float32)
+        M[0, :, 0] += 29.0
+        M[1, 0] = -200.0
+        M[1, 1] += 29.0
+        M[0, :, 1] = -200.0
+        lab = np.repeat(np.arange(2), Q * Q).astype(np.int32)
+        fa = synth.FstArrays(Q, 2, 2, np.tile(i, 2), np.tile(j, 2), lab, lab, -M.ravel(), start, final)
+        lz, _, st = Fst.from_arrays(fa).prefix_log_z(np.array([0, 1], np.int32))
+        x = M[0, 0].astype(np.float64) + M[1, :, Q - 1].astype(np.float64)
+        want = np.log(np.exp(x - x.max()).sum()) + x.max()
+        # roundings, of 2^-24: two exponentials (within 2 ulp), Q additions, a
+        # logarithm and the sums of its parts, the result
+        tol = 2.0**-24 * (8 + Q + 4 + 2 * abs(want))
+        assert st == 0 and abs(lz - want) <= tol, (lz, want, lz - want, tol)
