@@ -535,8 +535,11 @@ FST_API int fst_plan_live_work(fst_plan_t* plan, int64_t* entries, int64_t* arcs
  *   FST_DRIVER_LAUNCH      the string kernels (the default): one launch
  *                          per pass, in which a warp or block runs a string
  *                          over all of its positions; a wait that sees no
- *                          progress for 2 s ends the run with
- *                          FST_ERR_TIMEOUT.  With the direction switch or a
+ *                          progress for barrier_timeout_us (0 = keep the
+ *                          current limit, 2 s by default) ends the run with
+ *                          FST_ERR_TIMEOUT in the status of every string of
+ *                          its wave, and the next run starts clean.  With
+ *                          the direction switch or a
  *                          table limit one launch per position and kernel
  *                          kind instead.  Either run can be captured into a
  *                          CUDA graph and replayed.

@@ -268,6 +268,10 @@ struct alignas(128) StringJob {
   int32_t cur_big, next_big;  // backward: the values of t and t-1 are in the dense arrays
   int32_t shared;           // its chunks are open to other blocks
 };
+// Waits of the string kernels give up after this long without progress
+// anywhere in the launch, unless a plan sets another limit: the run then
+// reports FST_ERR_TIMEOUT.
+constexpr uint64_t STRING_WAIT_NS = 2000000000ull;
 // Device storage of the string kernels.
 struct StringWork {
   int32_t Bw;
@@ -282,6 +286,7 @@ struct StringWork {
   int32_t groups2;            // heavy blocks that run strings
   int32_t chunk;              // pool entries a group reserves at a time (0: each range by itself)
   int32_t share = 1;          // launches like this one that run side by side
+  uint64_t limit_ns = STRING_WAIT_NS;  // waits give up after this long without progress
 };
 // What a launch sees of it.
 struct StringQueue {
@@ -299,6 +304,7 @@ struct StringQueue {
   int2* fe;
   int64_t fe_light;
   int32_t chunk;
+  uint64_t limit_ns;
 };
 // Pool entries a group of the string kernels reserves at a time; a capped
 // pool is handed out range by range, so that the cap counts live entries.

@@ -188,6 +188,7 @@ struct fst_plan_s {
   bool learned = false, ran = false;
   cudaEvent_t run_event = nullptr;   // recorded at the end of each run outside a graph capture
   uint64_t barrier_limit_ns = 2000000000ull;
+  uint64_t wait_limit_ns = STRING_WAIT_NS;  // of the string kernels
   uint32_t barrier_extra = 0;        // fault injection: blocks a barrier waits for beyond the grid
   uint32_t* gbar = nullptr;          // [2] grid barrier (arrivals, generation)
   // stream-parallel parts (FST_PLAN_PARTS): sub-plans over contiguous string
@@ -544,6 +545,7 @@ StringWork string_work(fst_plan_s* P, const Wave& W, bool viterbi) {
   K.groups2 = P->str_groups2;
   K.chunk = P->pool_limit > 0 ? 0 : POOL_CHUNK;
   K.share = P->share;
+  K.limit_ns = P->wait_limit_ns;
   return K;
 }
 FrontierState string_state(fst_plan_s* P, const Wave& W, const float* gweight) {
@@ -1633,7 +1635,13 @@ extern "C" int fst_plan_set_driver(fst_plan_t* P, int32_t driver, int32_t grid_b
   }
   P->driver = driver;
   P->persist_grid = grid_blocks;
-  if (barrier_timeout_us > 0) P->barrier_limit_ns = (uint64_t)barrier_timeout_us * 1000ull;
+  if (barrier_timeout_us > 0) {
+    P->barrier_limit_ns = (uint64_t)barrier_timeout_us * 1000ull;
+    if (driver == FST_DRIVER_LAUNCH) {
+      P->wait_limit_ns = P->barrier_limit_ns;
+      for (fst_plan_s* q : P->parts) q->wait_limit_ns = P->wait_limit_ns;
+    }
+  }
   return FST_OK;
 }
 

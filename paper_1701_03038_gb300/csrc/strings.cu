@@ -152,9 +152,6 @@ __device__ __forceinline__ uint64_t now_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Waits give up after this long without progress anywhere in the launch:
-// the run then reports FST_ERR_TIMEOUT.
-constexpr uint64_t WAIT_NS = 2000000000ull;
 constexpr uint64_t BEGIN_NS = 20000ull;
 
 __device__ __forceinline__ uint32_t peek(const uint32_t* p) { return *(const volatile uint32_t*)p; }
@@ -175,7 +172,7 @@ __device__ __forceinline__ void queue_push(const StringQueue& K, int q, int32_t 
   // (a slot a whole ring back has its reader, who empties it)
   const uint64_t t0 = now_ns();
   while (atomicCAS(slot, 0u, (uint32_t)b + 1u) != 0u) {
-    if (now_ns() - t0 > WAIT_NS) {
+    if (now_ns() - t0 > K.limit_ns) {
       atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
       return;
     }
@@ -204,7 +201,7 @@ __device__ __forceinline__ int32_t queue_pop(const StringQueue& K, int q) {
     for (;;) {  // (its writer has the number and is about to write)
       const int32_t b = queue_poll(K, q, h);
       if (b >= 0) return b;
-      if (now_ns() - t0 > WAIT_NS) {
+      if (now_ns() - t0 > K.limit_ns) {
         atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
         return -1;
       }
@@ -213,7 +210,7 @@ __device__ __forceinline__ int32_t queue_pop(const StringQueue& K, int q) {
   return -1;
 }
 
-// A worker's patience: true once nothing has moved for WAIT_NS.
+// A worker's patience: true once nothing has moved for the limit.
 struct Patience {
   uint64_t t0;
   uint32_t seen;
@@ -227,7 +224,7 @@ struct Patience {
       seen = p;
       t0 = now_ns();
     }
-    if (now_ns() - t0 <= WAIT_NS) return false;
+    if (now_ns() - t0 <= K.limit_ns) return false;
     atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
     return true;
   }
@@ -376,7 +373,7 @@ __device__ __forceinline__ bool job_wait(Sh& sh, const StringQueue& K, int32_t n
     const uint64_t t0 = now_ns();
     int32_t ok = 1;
     while (*(volatile uint32_t*)&J->done != (uint32_t)n) {
-      if (now_ns() - t0 > WAIT_NS) {
+      if (now_ns() - t0 > K.limit_ns) {
         atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
         *(volatile uint32_t*)(K.dirty + sh.self) = 1u;
         ok = 0;
@@ -2115,6 +2112,7 @@ StringQueue string_queue(const StringWork& W, int blocks, int32_t* grid) {
   K.fe = W.fe;
   K.fe_light = W.fe_light;
   K.chunk = W.chunk;
+  K.limit_ns = W.limit_ns;
   // (heavy blocks come first, so that they are resident first)
   const int all = (W.Bw + WARPS - 1) / WARPS;
   const int want = all <= blocks / 2 ? std::max(all, blocks / 4) : blocks / 4;

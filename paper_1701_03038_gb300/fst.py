@@ -510,7 +510,8 @@ class Plan:
 
     def set_driver(self, driver: int, grid_blocks: int = 0, barrier_timeout_us: int = 0):
         """Driver of the following runs: _lib.DRIVER_LAUNCH (one launch per
-        pass) or _lib.DRIVER_PERSISTENT (one cooperative launch per pass)."""
+        pass) or _lib.DRIVER_PERSISTENT (one cooperative launch per pass),
+        and how long its waits may see no progress (0: as before)."""
         with torch.cuda.device(self.fst.device):
             check(self._lib.fst_plan_set_driver(self._h, int(driver), int(grid_blocks), int(barrier_timeout_us)),
                   "fst_plan_set_driver")

@@ -178,6 +178,66 @@ def test_persistent_barrier_timeout_reports_and_recovers():
     assert_counts_close(pf.counts.cpu().numpy(), ofb["counts"], batch=True)
 
 
+def _chain_fst(states=64, symbols=3, wide=0):
+    """A ring whose symbols 0 .. symbols-1 each lead every state on by 1 + the
+    symbol, and (wide) one more symbol of `wide` arcs out of every state."""
+    q = np.arange(states)
+    parts = [(q, (q + 1 + a) % states, a) for a in range(symbols)]
+    if wide:
+        rng = np.random.default_rng(wide)
+        parts.append((np.repeat(q[:8], wide), rng.integers(0, states, 8 * wide), symbols))
+    src, dst = (np.concatenate([p[k] for p in parts]).astype(np.int32) for k in (0, 1))
+    lab = np.concatenate([np.full(len(p[0]), p[2]) for p in parts]).astype(np.int32)
+    w = np.random.default_rng(1).uniform(0.1, 2.0, len(src)).astype(np.float32)
+    start = np.full(states, np.inf, np.float32)
+    start[0] = 0.0
+    m = symbols + (1 if wide else 0)
+    return synth.FstArrays(states, m, m, src, dst, lab, lab, w, start, np.zeros(states, np.float32))
+
+
+def _plans(f, strs, **kw):
+    import torch
+    from paper_1701_03038_gb300._lib import PLAN_NO_FB, PLAN_NO_VITERBI
+    ids, off = torch.from_numpy(strs.ids).cuda(), torch.from_numpy(strs.offsets).cuda()
+    return f.plan(ids, off, flags=PLAN_NO_FB, **kw), f.plan(ids, off, flags=PLAN_NO_VITERBI, **kw)
+
+
+@pytest.mark.parametrize("parts", [1, 2])
+def test_string_waits_run_out_and_recover(parts):
+    # two strings of 20,000 one-arc positions (some 10 ms) under a limit of a
+    # microsecond: the workers without a string give up, the run reports
+    # FST_ERR_TIMEOUT everywhere, and with the limit back the same plans are
+    # exact
+    import torch
+    from paper_1701_03038_gb300 import _lib
+    from paper_1701_03038_gb300.fst import Fst
+    fa = _chain_fst()
+    f, o = Fst.from_arrays(fa), oracle.Fst(fa)
+    rng = np.random.default_rng(2)
+    n = 20_000
+    strs = synth.Strings(rng.integers(0, 3, 2 * n).astype(np.int32), np.array([0, n, 2 * n], np.int64))
+    pv, pf = _plans(f, strs, parts=parts)
+    for limit_us in (1, 2_000_000):
+        for p in (pv, pf):
+            p.set_driver(_lib.DRIVER_LAUNCH, 0, limit_us)
+        pv.viterbi()
+        pf.forward_backward()
+        torch.cuda.synchronize()
+        if limit_us == 1:
+            assert (pv.status[:2].cpu().numpy() == _lib.TIMEOUT).all()
+            assert (pf.status[:2].cpu().numpy() == _lib.TIMEOUT).all()
+            assert np.isneginf(pv.scores[:2].cpu().numpy()).all()
+            assert (pv.paths[:2 * n].cpu().numpy() == -1).all()
+            assert np.isneginf(pf.logz[:2].cpu().numpy()).all()
+    ofb = o.fb_batch(strs.ids, strs.offsets, nthreads=2)
+    for b in range(2):
+        lo, hi = strs.offsets[b], strs.offsets[b + 1]
+        assert_viterbi_equal(pv.scores[b].item(), pv.paths[lo:hi].cpu().numpy(), pv.olabels[lo:hi].cpu().numpy(),
+                             pv.status[b].item(), o.viterbi(strs.get(b)))
+        assert_logz_close(pf.logz[b].item(), ofb["logz"][b])
+    assert_counts_close(pf.counts.cpu().numpy(), ofb["counts"], batch=True)
+
+
 def test_fault_inject_rejects_bad_arguments():
     import torch
     from paper_1701_03038_gb300 import _lib
