@@ -156,6 +156,10 @@ constexpr uint64_t BEGIN_NS = 20000ull;
 
 __device__ __forceinline__ uint32_t peek(const uint32_t* p) { return *(const volatile uint32_t*)p; }
 
+// Whether a wait has run out: the run is over, and what others would have
+// brought may not come any more.
+__device__ __forceinline__ bool gave_up(const StringQueue& K) { return (peek(K.ctl + CTL_FLAGS + 1) & ERR_TIMEOUT) != 0u; }
+
 // The two string queues (QL light, QH heavy): rings whose slots hold string
 // + 1 (0 = empty).  A worker that may wait takes a ticket, the number of an
 // item that may still have to come, and polls that item's slot, which no
@@ -172,6 +176,7 @@ __device__ __forceinline__ void queue_push(const StringQueue& K, int q, int32_t 
   // (a slot a whole ring back has its reader, who empties it)
   const uint64_t t0 = now_ns();
   while (atomicCAS(slot, 0u, (uint32_t)b + 1u) != 0u) {
+    if (gave_up(K)) return;
     if (now_ns() - t0 > K.limit_ns) {
       atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
       return;
@@ -201,6 +206,7 @@ __device__ __forceinline__ int32_t queue_pop(const StringQueue& K, int q) {
     for (;;) {  // (its writer has the number and is about to write)
       const int32_t b = queue_poll(K, q, h);
       if (b >= 0) return b;
+      if (gave_up(K)) return -1;
       if (now_ns() - t0 > K.limit_ns) {
         atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
         return -1;
@@ -230,7 +236,7 @@ struct Patience {
   }
 };
 __device__ __forceinline__ bool all_done(const StringQueue& K) {
-  return peek(K.ctl + CTL_FINISHED) >= (uint32_t)K.strings || (peek(K.ctl + CTL_FLAGS + 1) & ERR_TIMEOUT) != 0u;
+  return peek(K.ctl + CTL_FINISHED) >= (uint32_t)K.strings || gave_up(K);
 }
 // A string is done (one thread, after the group's barrier).
 __device__ __forceinline__ void string_done(const StringQueue& K) {
@@ -278,9 +284,11 @@ __device__ __forceinline__ int32_t next_light(const StringQueue& K) {
 // claims chunks, between the positions of its own string or when it has
 // none; the owner claims them too, then waits for the chunks that
 // others hold.  A claimed chunk is being worked on by a running block, so
-// the wait needs no co-residency; it is bounded all the same (past the
-// limit the run reports FST_ERR_TIMEOUT, and the owner's accumulators are
-// cleared when its block next starts).
+// the wait needs no co-residency; it is bounded all the same: past the
+// limit the run reports FST_ERR_TIMEOUT, and the owner leaves the kernel.  It
+// takes nothing more, because the others go on with the chunks of its slot,
+// which a next position's staged states, counts and phases would meet; its
+// accumulators are cleared when its block next starts.
 // ----------------------------------------------------------------------
 constexpr int JOB_BITS = 22;
 constexpr unsigned long long JOB_MASK = (1ull << JOB_BITS) - 1ull;
@@ -1352,20 +1360,19 @@ struct Forward {
           chunk(hv, sh.st, alone ? c : hv.chunk, alone ? &sh.tab.staged : (int32_t*)&K.jobs[g].staged);
         }
         if (mine) {
-          bool ok = true;
           if (alone) __syncthreads();
-          else ok = job_wait(hv, K, n);
+          else if (!job_wait(hv, K, n)) return;
           if (own == 0) {
             nb = alone ? sh.tab.staged : (int32_t)hv.job.staged;
             single = nb == P.tot;
           }
           __syncthreads();
-          if (ok && own == 0 && !VIT && !single) {
+          if (own == 0 && !VIT && !single) {
             if (tid == 0) hv.job.phase = 1;
             own = 1;
           } else if (own < 2) {
             if (tid == 0) {
-              hv.base = ok ? reserve(sh.gs, nb) : -1;
+              hv.base = reserve(sh.gs, nb);
               hv.job.phase = 2;
               hv.job.nb = nb;
               hv.job.nbase = hv.base;
@@ -1378,18 +1385,17 @@ struct Forward {
             own = 2;
             if (P.base < 0) {
               // empty what was staged
-              if (ok)
-                for (int32_t i = tid; i < nb; i += NT1) {
-                  const int32_t d = __ldcg(dstage(self) + i);
-                  if (VIT) dacc(self)[d] = 0ull;
-                  else ((ulonglong2*)dacc(self))[d] = make_ulonglong2(0ull, 0ull);
-                }
+              for (int32_t i = tid; i < nb; i += NT1) {
+                const int32_t d = __ldcg(dstage(self) + i);
+                if (VIT) dacc(self)[d] = 0ull;
+                else ((ulonglong2*)dacc(self))[d] = make_ulonglong2(0ull, 0ull);
+              }
               P.cnt = P.tot = 0;
               done = true;
             }
           } else {
-            P.cnt = ok ? nb : 0;
-            P.tot = ok ? (int32_t)(alone ? hv.tot : hv.job.tot) : 0;
+            P.cnt = nb;
+            P.tot = (int32_t)(alone ? hv.tot : hv.job.tot);
             mk = alone ? hv.mk : hv.job.mk;
             done = true;
           }
@@ -1949,16 +1955,15 @@ struct Backward {
           chunk(hv, alone ? c : hv.chunk);
         }
         if (!mine) break;
-        bool ok = true;
         if (alone) __syncthreads();
-        else ok = job_wait(hv, K, n);
+        else if (!job_wait(hv, K, n)) return;
         P.ek = alone ? hv.mk : hv.job.mk;
         // the values of position t have been read: empty their table
         empty(P, tid, NT1);
         help = __syncthreads_or(big != 0u) != 0;
         P.cur_big = dense;
         P.cur_n = P.t > 1 ? R.cnt : 0;
-        P.t = ok ? P.t - 1 : 0;  // (0: given up)
+        --P.t;
         mine = false;
         if (!help) break;
       }

@@ -238,6 +238,45 @@ def test_string_waits_run_out_and_recover(parts):
     assert_counts_close(pf.counts.cpu().numpy(), ofb["counts"], batch=True)
 
 
+def test_shared_position_waits_run_out_and_recover():
+    # strings whose every position is shared out among the blocks, under a
+    # limit of a microsecond: owners stop waiting for chunks that others hold
+    # and leave their accumulators unclean; the runs after that are exact
+    import torch
+    from paper_1701_03038_gb300 import _lib
+    from paper_1701_03038_gb300.fst import Fst
+    fa = _chain_fst(states=20_000, wide=6_000)
+    f, o = Fst.from_arrays(fa), oracle.Fst(fa)
+    rng = np.random.default_rng(3)
+    B, n = 12, 120
+    x = rng.integers(0, 3, (B, n)).astype(np.int32)
+    x[:, 0] = 3
+    strs = synth.Strings(x.reshape(-1), np.arange(B + 1, dtype=np.int64) * n)
+    pv, pf = _plans(f, strs)
+    ov = [o.viterbi(strs.get(b)) for b in range(B)]
+    ofb = o.fb_batch(strs.ids, strs.offsets, nthreads=8)
+    for _ in range(3):
+        for p in (pv, pf):
+            p.set_driver(_lib.DRIVER_LAUNCH, 0, 1)
+        pv.viterbi()
+        pf.forward_backward()
+        torch.cuda.synchronize()
+        assert (pv.status[:B].cpu().numpy() == _lib.TIMEOUT).all()
+        assert (pf.status[:B].cpu().numpy() == _lib.TIMEOUT).all()
+        assert (pv.paths[:B * n].cpu().numpy() == -1).all()
+        for p in (pv, pf):
+            p.set_driver(_lib.DRIVER_LAUNCH, 0, 2_000_000)
+        pv.viterbi()
+        pf.forward_backward()
+        torch.cuda.synchronize()
+        for b in range(B):
+            lo, hi = strs.offsets[b], strs.offsets[b + 1]
+            assert_viterbi_equal(pv.scores[b].item(), pv.paths[lo:hi].cpu().numpy(), pv.olabels[lo:hi].cpu().numpy(),
+                                 pv.status[b].item(), ov[b])
+            assert_logz_close(pf.logz[b].item(), ofb["logz"][b])
+        assert_counts_close(pf.counts.cpu().numpy(), ofb["counts"], batch=True)
+
+
 def test_fault_inject_rejects_bad_arguments():
     import torch
     from paper_1701_03038_gb300 import _lib
