@@ -367,7 +367,10 @@ FST_API int fst_plan_forward(fst_plan_t* plan, double* d_logz, int32_t* d_status
 
 /* Backward pass and expected counts after fst_plan_forward on the same plan:
  * d_counts[k] = sum_b d_weights[b] * count_b(k) (d_weights NULL = all 1).
- * Returns FST_ERR_STATE if no forward pass preceded it. Alg. 2's backward and count loops. */
+ * Returns FST_ERR_STATE if no forward pass preceded it.  A backward pass
+ * that gives up waiting (FST_ERR_TIMEOUT, see fst_plan_set_driver) would
+ * leave partial counts: every count is NaN then, and the combined calls below
+ * report FST_ERR_TIMEOUT for every string. Alg. 2's backward and count loops. */
 FST_API int fst_plan_backward(fst_plan_t* plan, const float* d_weights, float* d_counts, void* stream);
 
 /* Forward and backward for every wave of the plan (any number of waves). Alg. 2. */

@@ -823,7 +823,7 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
   // compensation (one writer per arc and position), in the same storage
   if (arc_posteriors && !w->cnt64) {
     dfree(w->counts_out);
-    if ((rc = dalloc(&w->counts_out, f->A)) || (rc = dalloc(&w->cnt64, f->A))) return rc;
+    if ((rc = dalloc(&w->counts_out, f->A)) || (rc = dalloc(&w->cnt64, f->A + 1))) return rc;  // (and CountView::spoiled)
   }
   float* const cnt = (float*)w->cnt64;
   const LayoutView L = view_of(f->bwd);
@@ -851,8 +851,9 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
   PLAIN_PROF(FST_PROF_FB_FINAL, launch_fb_final(S, 1, w->logz, w->status, s));
   w->last_fb = true;
   if (arc_posteriors) {
-    const CountView C = strings ? CountView{1, nullptr, nullptr, w->cnt64} : CountView{0, cnt, cnt + f->A, nullptr};
-    FST_CUDA(cudaMemsetAsync(w->cnt64, 0, (size_t)std::max<int64_t>(f->A, 1) * 8, s));
+    CountView C = strings ? CountView{1, nullptr, nullptr, w->cnt64} : CountView{0, cnt, cnt + f->A, nullptr};
+    C.spoiled = w->cnt64 + f->A;
+    FST_CUDA(cudaMemsetAsync(w->cnt64, 0, (size_t)(f->A + 1) * 8, s));
     if (strings) {
       PLAIN_PROF(FST_PROF_BWD_STEP, launch_string_backward(L, w->tok_sym, S, C, K, f->num_sms, s));
     } else if (persist) {
@@ -862,7 +863,7 @@ extern "C" int fst_forward_backward(fst_t* f, const int32_t* ids, int32_t n, dou
       for (int32_t t = n; t >= 1; --t)
         PLAIN_PROF(FST_PROF_BWD_STEP, launch_bwd_step(L, T, plain_step(f, n, t, t - 1), S, C, s));
     }
-    PLAIN_PROF(FST_PROF_COUNTS, launch_counts_out(f->A, C, w->counts_out, s));
+    PLAIN_PROF(FST_PROF_COUNTS, launch_counts_out(f->A, C, w->counts_out, 1, w->status, s));
     if (f->A > 0)
       FST_CUDA(cudaMemcpyAsync(arc_posteriors, w->counts_out, (size_t)f->A * 4, cudaMemcpyDeviceToHost, s));
   }

@@ -1264,7 +1264,10 @@ __global__ void __launch_bounds__(KT) k_bwd_persist(LayoutView L, TokenView T, W
     StepView V = step_at(D, t, t - 1);
     V.y_t = t + 1 < D.tmax ? t + 1 : 0;
     bwd_position(L, T, V, S, C, sh);
-    if (!grid_sync(G, S.flags + 1)) return;
+    if (!grid_sync(G, S.flags + 1)) {
+      if (threadIdx.x == 0 && C.spoiled) *C.spoiled = __longlong_as_double(0x7fffffffffffffffll);
+      return;
+    }
   }
   if (compact(S) && D.tmax >= 2) bwd_clear_position(S, 1);
 }
@@ -1564,15 +1567,23 @@ __global__ void k_fill_neg_inf(double* __restrict__ p, int64_t n) {
     p[i] = -INFINITY;
 }
 
-__global__ void k_to_float(const double* __restrict__ in, int64_t n, float* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (float)in[i];
+// (a bit test: a float64 compare takes the narrow float64 unit)
+__device__ __forceinline__ bool is_spoiled(const double* spoiled) {
+  return spoiled && __double_as_longlong(__ldg(spoiled)) != 0ll;
 }
 
-__global__ void k_counts_out(int64_t A, CountView C, float* __restrict__ out) {
+__global__ void k_to_float(const double* __restrict__ in, int64_t n, float* __restrict__ out, const double* spoiled) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = is_spoiled(spoiled) ? __int_as_float(0x7fffffff) : (float)in[i];
+}
+
+__global__ void k_counts_out(int64_t A, CountView C, float* __restrict__ out, int32_t B, int32_t* __restrict__ status) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool bad = is_spoiled(C.spoiled);
+  if (bad && status)
+    for (int64_t b = i; b < B; b += (int64_t)gridDim.x * blockDim.x) status[b] = FST_ERR_TIMEOUT;
   if (i >= A) return;
-  out[i] = C.batched ? (float)C.cnt64[i] : __fsub_rn(C.cnt[i], C.comp[i]);
+  out[i] = bad ? __int_as_float(0x7fffffff) : C.batched ? (float)C.cnt64[i] : __fsub_rn(C.cnt[i], C.comp[i]);
 }
 
 __global__ void k_clear_if_overflow(const uint32_t* __restrict__ flag, unsigned long long* __restrict__ acc,
@@ -1790,9 +1801,9 @@ int launch_fb_final(const FrontierState& S, int32_t Bw, double* logz, int32_t* s
   return check_launch("k_fb_final");
 }
 
-int launch_counts_out(int64_t A, const CountView& C, float* out, cudaStream_t s) {
-  if (A <= 0) return FST_OK;
-  k_counts_out<<<(unsigned)((A + 255) / 256), 256, 0, s>>>(A, C, out);
+int launch_counts_out(int64_t A, const CountView& C, float* out, int32_t B, int32_t* status, cudaStream_t s) {
+  if (A <= 0 && !status) return FST_OK;
+  k_counts_out<<<(unsigned)std::max<int64_t>((A + 255) / 256, 1), 256, 0, s>>>(A, C, out, B, status);
   return check_launch("k_counts_out");
 }
 
@@ -1808,9 +1819,9 @@ int launch_fill_neg_inf(double* p, int64_t n, cudaStream_t s) {
   return check_launch("k_fill_neg_inf");
 }
 
-int launch_to_float(const double* in, int64_t n, float* out, cudaStream_t s) {
+int launch_to_float(const double* in, int64_t n, float* out, const double* spoiled, cudaStream_t s) {
   if (n <= 0) return FST_OK;
-  k_to_float<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, n, out);
+  k_to_float<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, n, out, spoiled);
   return check_launch("k_to_float");
 }
 

@@ -175,6 +175,7 @@ struct CountView {
   double* cnt64;
   double* start64;    // [Q] expected start states, or null
   double* final64;    // [Q] expected final states, or null
+  double* spoiled = nullptr;  // [1] NaN once a backward pass gave up waiting, else 0: the counts are partial
 };
 
 // First position (Viterbi and forward): the start states push their arcs
@@ -223,15 +224,17 @@ int launch_vit_final(const FrontierState& S, int32_t Bw, float* scores, int32_t*
 int launch_backtrace(const FrontierState& S, const int32_t* olabel_by_id, int32_t Bw, const int32_t* jfinal,
                      int32_t* paths, int32_t* olabels, cudaStream_t s);
 int launch_fb_final(const FrontierState& S, int32_t Bw, double* logz, int32_t* status, cudaStream_t s);
-int launch_counts_out(int64_t A, const CountView& C, float* out, cudaStream_t s);
+// Counts as float32, out[0..A); where a backward pass gave up, NaN, and
+// FST_ERR_TIMEOUT in status[0..B) (null: none).
+int launch_counts_out(int64_t A, const CountView& C, float* out, int32_t B, int32_t* status, cudaStream_t s);
 // Expected final states of every string (and expected start states of the
 // empty strings, whose paths start where they end), added to C.final64 and
 // C.start64 with the strings' weights.  Needs the forward pass and log Z.
 int launch_final_posteriors(const FrontierState& S, int32_t Bw, const CountView& C, cudaStream_t s);
 // p[i] = -inf, i < n.
 int launch_fill_neg_inf(double* p, int64_t n, cudaStream_t s);
-// out[i] = (float)in[i], i < n.
-int launch_to_float(const double* in, int64_t n, float* out, cudaStream_t s);
+// out[i] = (float)in[i], i < n; NaN where a backward pass gave up.
+int launch_to_float(const double* in, int64_t n, float* out, const double* spoiled, cudaStream_t s);
 // The string kernels (strings.cu): a warp or block runs one string over all
 // of its positions.  Control words of a wave's run: error flags, pool top,
 // live entries and arcs; then, cleared before each pass, the strings started
@@ -305,6 +308,7 @@ struct StringQueue {
   int64_t fe_light;
   int32_t chunk;
   uint64_t limit_ns;
+  double* spoiled;  // backward: CountView::spoiled
 };
 // Pool entries a group of the string kernels reserves at a time; a capped
 // pool is handed out range by range, so that the cap counts live entries.

@@ -736,7 +736,8 @@ int run_backward_wave(fst_plan_s* P, const Wave& W, const float* d_weights, bool
   const LayoutView L = view_of(f->bwd);
   const TokenView T = wave_tokens(W);
   const FrontierState S = wave_state(P, W, d_weights);
-  const CountView C{1, nullptr, nullptr, P->cnt64, states ? P->start64 : nullptr, states ? P->final64 : nullptr};
+  const CountView C{1, nullptr, nullptr, P->cnt64, states ? P->start64 : nullptr, states ? P->final64 : nullptr,
+                    P->cnt64 + f->A};
   if (P->str_last) {
     PROF(FST_PROF_BWD_STEP, launch_string_backward(L, W.tok_sym, S, C, string_work(P, W, false), f->num_sms, s));
   } else if (P->driver == FST_DRIVER_PERSISTENT) {
@@ -762,7 +763,7 @@ int run_backward_wave(fst_plan_s* P, const Wave& W, const float* d_weights, bool
 // Zero the count accumulators of a backward run.
 int counts_begin(fst_plan_s* P, bool states, cudaStream_t s) {
   fst_s* f = P->fst;
-  FST_CUDA(cudaMemsetAsync(P->cnt64, 0, (size_t)std::max<int64_t>(1, f->A) * 8, s));
+  FST_CUDA(cudaMemsetAsync(P->cnt64, 0, (size_t)(f->A + 1) * 8, s));  // (and CountView::spoiled)
   if (states) {
     FST_CUDA(cudaMemsetAsync(P->start64, 0, (size_t)f->Q * 8, s));
     FST_CUDA(cudaMemsetAsync(P->final64, 0, (size_t)f->Q * 8, s));
@@ -771,16 +772,15 @@ int counts_begin(fst_plan_s* P, bool states, cudaStream_t s) {
 }
 
 // Counts (and state posteriors) from their float64 accumulators to the
-// caller's float arrays.
-int counts_end(fst_plan_s* P, float* d_counts, float* d_start, float* d_final, cudaStream_t s) {
+// caller's float arrays, and the status of a backward pass that gave up.
+int counts_end(fst_plan_s* P, float* d_counts, float* d_start, float* d_final, int32_t* d_status, cudaStream_t s) {
   fst_s* f = P->fst;
   int rc;
-  if (d_counts) {
-    const CountView C{1, nullptr, nullptr, P->cnt64};
-    PROF(FST_PROF_COUNTS, launch_counts_out(f->A, C, d_counts, s));
-  }
-  if (d_start && (rc = launch_to_float(P->start64, f->Q, d_start, s))) return rc;
-  if (d_final && (rc = launch_to_float(P->final64, f->Q, d_final, s))) return rc;
+  CountView C{1, nullptr, nullptr, P->cnt64};
+  C.spoiled = P->cnt64 + f->A;
+  if (d_counts || d_status) PROF(FST_PROF_COUNTS, launch_counts_out(d_counts ? f->A : 0, C, d_counts, P->B, d_status, s));
+  if (d_start && (rc = launch_to_float(P->start64, f->Q, d_start, C.spoiled, s))) return rc;
+  if (d_final && (rc = launch_to_float(P->final64, f->Q, d_final, C.spoiled, s))) return rc;
   return FST_OK;
 }
 
@@ -875,7 +875,7 @@ static int plan_create_parts(fst_t* f, const int32_t* d_ids, const int64_t* d_of
     P->start64 = donor->start64;
     P->final64 = donor->final64;
     donor->cnt64 = donor->start64 = donor->final64 = nullptr;
-    P->bytes += (int64_t)(f->A + 2 * (int64_t)f->Q) * 8;
+    P->bytes += (int64_t)(f->A + 1 + 2 * (int64_t)f->Q) * 8;
     for (fst_plan_s* q : P->parts) {
       dfree(q->cnt64);
       dfree(q->start64);
@@ -886,7 +886,7 @@ static int plan_create_parts(fst_t* f, const int32_t* d_ids, const int64_t* d_of
       q->borrowed_counts = true;
     }
   } else if (P->want_fb) {
-    if ((rc = alloc_track(P.get(), &P->cnt64, f->A)) || (rc = alloc_track(P.get(), &P->start64, f->Q)) ||
+    if ((rc = alloc_track(P.get(), &P->cnt64, f->A + 1)) || (rc = alloc_track(P.get(), &P->start64, f->Q)) ||
         (rc = alloc_track(P.get(), &P->final64, f->Q)))
       return rc;
     for (fst_plan_s* q : P->parts) {
@@ -1167,7 +1167,7 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
         (rc = alloc_store(P, &P->logz, B)))
       break;
     if (P->want_fb && !(flags & PLAN_PART) &&
-        ((rc = alloc_store(P, &P->cnt64, f->A)) || (rc = alloc_store(P, &P->start64, f->Q)) ||
+        ((rc = alloc_store(P, &P->cnt64, f->A + 1)) || (rc = alloc_store(P, &P->start64, f->Q)) ||
          (rc = alloc_store(P, &P->final64, f->Q))))
       break;
     // the accumulators start at zero and every run leaves them so
@@ -1332,11 +1332,11 @@ extern "C" int fst_plan_backward_ex(fst_plan_t* P, const float* d_weights, float
     });
     if (rc) return rc;
     if ((rc = parts_join(P, s))) return rc;
-    return counts_end(P, d_counts, d_start, d_final, s);
+    return counts_end(P, d_counts, d_start, d_final, nullptr, s);
   }
   for (const Wave& W : P->waves)
     if ((rc = run_backward_wave(P, W, d_weights, states, s))) return rc;
-  return counts_end(P, d_counts, d_start, d_final, s);
+  return counts_end(P, d_counts, d_start, d_final, nullptr, s);
 }
 
 extern "C" int fst_plan_backward(fst_plan_t* P, const float* d_weights, float* d_counts, void* stream) {
@@ -1372,7 +1372,7 @@ extern "C" int fst_plan_forward_backward_ex(fst_plan_t* P, const float* d_weight
     });
     if (rc) return rc;
     if ((rc = parts_join(P, s))) return rc;
-    if (bwd && (rc = counts_end(P, d_counts, d_start, d_final, s))) return rc;
+    if (bwd && (rc = counts_end(P, d_counts, d_start, d_final, d_status, s))) return rc;
     P->forward_done = true;
     for (fst_plan_s* q : P->parts) P->forward_done = P->forward_done && q->forward_done;
     return FST_OK;
@@ -1382,7 +1382,7 @@ extern "C" int fst_plan_forward_backward_ex(fst_plan_t* P, const float* d_weight
     if (bwd && (rc = run_backward_wave(P, W, d_weights, states, s))) return rc;
   }
   if (P->B > 0) FST_CUDA(cudaMemcpyAsync(d_logz, P->logz, (size_t)P->B * 8, cudaMemcpyDeviceToDevice, s));
-  if (bwd && (rc = counts_end(P, d_counts, d_start, d_final, s))) return rc;
+  if (bwd && (rc = counts_end(P, d_counts, d_start, d_final, d_status, s))) return rc;
   P->forward_done = P->waves.size() <= 1;
   return FST_OK;
 }

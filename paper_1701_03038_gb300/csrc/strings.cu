@@ -159,6 +159,12 @@ __device__ __forceinline__ uint32_t peek(const uint32_t* p) { return *(const vol
 // Whether a wait has run out: the run is over, and what others would have
 // brought may not come any more.
 __device__ __forceinline__ bool gave_up(const StringQueue& K) { return (peek(K.ctl + CTL_FLAGS + 1) & ERR_TIMEOUT) != 0u; }
+// This wait has.  (The forward passes' final kernels read the flag; after a
+// backward pass the counts' kernel reads `spoiled`.)
+__device__ __forceinline__ void give_up(const StringQueue& K) {
+  atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
+  if (K.spoiled) *(volatile double*)K.spoiled = __longlong_as_double(0x7fffffffffffffffll);
+}
 
 // The two string queues (QL light, QH heavy): rings whose slots hold string
 // + 1 (0 = empty).  A worker that may wait takes a ticket, the number of an
@@ -178,7 +184,7 @@ __device__ __forceinline__ void queue_push(const StringQueue& K, int q, int32_t 
   while (atomicCAS(slot, 0u, (uint32_t)b + 1u) != 0u) {
     if (gave_up(K)) return;
     if (now_ns() - t0 > K.limit_ns) {
-      atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
+      give_up(K);
       return;
     }
   }
@@ -208,7 +214,7 @@ __device__ __forceinline__ int32_t queue_pop(const StringQueue& K, int q) {
       if (b >= 0) return b;
       if (gave_up(K)) return -1;
       if (now_ns() - t0 > K.limit_ns) {
-        atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
+        give_up(K);
         return -1;
       }
     }
@@ -231,7 +237,7 @@ struct Patience {
       t0 = now_ns();
     }
     if (now_ns() - t0 <= K.limit_ns) return false;
-    atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
+    give_up(K);
     return true;
   }
 };
@@ -382,7 +388,7 @@ __device__ __forceinline__ bool job_wait(Sh& sh, const StringQueue& K, int32_t n
     int32_t ok = 1;
     while (*(volatile uint32_t*)&J->done != (uint32_t)n) {
       if (now_ns() - t0 > K.limit_ns) {
-        atomicOr(K.ctl + CTL_FLAGS + 1, ERR_TIMEOUT);
+        give_up(K);
         *(volatile uint32_t*)(K.dirty + sh.self) = 1u;
         ok = 0;
         break;
@@ -2118,6 +2124,7 @@ StringQueue string_queue(const StringWork& W, int blocks, int32_t* grid) {
   K.fe_light = W.fe_light;
   K.chunk = W.chunk;
   K.limit_ns = W.limit_ns;
+  K.spoiled = nullptr;
   // (heavy blocks come first, so that they are resident first)
   const int all = (W.Bw + WARPS - 1) / WARPS;
   const int want = all <= blocks / 2 ? std::max(all, blocks / 4) : blocks / 4;
@@ -2171,7 +2178,8 @@ int launch_string_backward(const LayoutView& L, const int32_t* sym, const Fronti
   int32_t grid = 0;
   const int rc = resident(k_str_backward, 2, smem, num_sms, &blocks);
   if (rc) return rc;
-  const StringQueue K = string_queue(W, blocks, &grid);
+  StringQueue K = string_queue(W, blocks, &grid);
+  K.spoiled = C.spoiled;
   k_str_backward<<<(unsigned)grid, NT1, smem, s>>>(L, sym, S, C, K);
   return check_launch("k_str_backward");
 }

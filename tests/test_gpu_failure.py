@@ -277,6 +277,40 @@ def test_shared_position_waits_run_out_and_recover():
         assert_counts_close(pf.counts.cpu().numpy(), ofb["counts"], batch=True)
 
 
+@pytest.mark.parametrize("wide", [0, 6_000])
+def test_backward_pass_that_gives_up_spoils_the_counts(wide):
+    # a forward pass that ends, then a backward pass under a limit of a
+    # microsecond: its counts would be partial, and are NaN; the next pair of
+    # passes is exact
+    import torch
+    from paper_1701_03038_gb300 import _lib
+    from paper_1701_03038_gb300.fst import Fst
+    fa = _chain_fst(states=20_000 if wide else 64, wide=wide)
+    f, o = Fst.from_arrays(fa), oracle.Fst(fa)
+    rng = np.random.default_rng(4)
+    B, n = (6, 100) if wide else (2, 20_000)
+    x = rng.integers(0, 3, (B, n)).astype(np.int32)
+    if wide:
+        x[:, 0] = 3
+    strs = synth.Strings(x.reshape(-1), np.arange(B + 1, dtype=np.int64) * n)
+    _, pf = _plans(f, strs)
+    ofb = o.fb_batch(strs.ids, strs.offsets, nthreads=8)
+    for limit_us in (1, 2_000_000):
+        pf.set_driver(_lib.DRIVER_LAUNCH, 0, 2_000_000)
+        pf.forward()
+        pf.set_driver(_lib.DRIVER_LAUNCH, 0, limit_us)
+        pf.backward(torch.ones(B, device="cuda"), states=True)
+        torch.cuda.synchronize()
+        assert (pf.status[:B].cpu().numpy() == 0).all()
+        if limit_us == 1:
+            for c in (pf.counts, pf.start_counts, pf.final_counts):
+                assert np.isnan(c.cpu().numpy()).all()
+    for b in range(B):
+        assert_logz_close(pf.logz[b].item(), ofb["logz"][b])
+    assert_counts_close(pf.counts.cpu().numpy(), ofb["counts"], batch=True)
+    assert abs(pf.start_counts.sum().item() - B) < 1e-4 and abs(pf.final_counts.sum().item() - B) < 1e-4
+
+
 def test_fault_inject_rejects_bad_arguments():
     import torch
     from paper_1701_03038_gb300 import _lib
