@@ -244,6 +244,13 @@ struct Patience {
 __device__ __forceinline__ bool all_done(const StringQueue& K) {
   return peek(K.ctl + CTL_FINISHED) >= (uint32_t)K.strings || gave_up(K);
 }
+// A string went from position t0 to t1 (one thread): every 4,096 positions
+// count as progress, whichever way they were done.  (A run of one-arc
+// positions steps over most multiples of 4,096: without its report a string
+// of 3.5 million of them ran into the limit of those who wait.)
+__device__ __forceinline__ void report(const StringQueue& K, int32_t t0, int32_t t1) {
+  if ((t0 ^ t1) >> 12) atomicAdd(K.ctl + CTL_PROGRESS, 1u);
+}
 // A string is done (one thread, after the group's barrier).
 __device__ __forceinline__ void string_done(const StringQueue& K) {
   __threadfence();
@@ -991,9 +998,12 @@ struct Forward {
     P.tot = full ? 0 : nxt.len;
     P.base = base + k - 1;
     P.shift = shift;
-    if (!full && lane == 0) {
-      gs.live_e += (unsigned long long)k;
-      gs.live_a += (unsigned long long)(k - 1 + nxt.len);
+    if (lane == 0) {
+      report(K, P.t - k, P.t);
+      if (!full) {
+        gs.live_e += (unsigned long long)k;
+        gs.live_a += (unsigned long long)(k - 1 + nxt.len);
+      }
     }
     if (VIT && lane == 0) fe[0] = make_int2(nxt.pos, nxt.len);
     x = Entry{nxt.pos, lane == 0 ? P.tot : 0, P.base, r};
@@ -1179,7 +1189,7 @@ struct Forward {
         gs.live_e += (unsigned long long)nb;
         gs.live_a += (unsigned long long)P.tot;
         position_done(P, p, mk);
-        if ((P.t & 4095) == 0) atomicAdd(K.ctl + CTL_PROGRESS, 1u);
+        report(K, P.t - 1, P.t);
       }
       P.shift = decode_max(mk);
       a = an;
@@ -1414,7 +1424,7 @@ struct Forward {
           sh.gs.live_e += (unsigned long long)P.cnt;
           sh.gs.live_a += (unsigned long long)P.tot;
           position_done(P, P.off + P.t - 1, mk);
-          if ((P.t & 4095) == 0) atomicAdd(K.ctl + CTL_PROGRESS, 1u);
+          report(K, P.t - 1, P.t);
         }
         P.shift = decode_max(mk);
         a = an;
@@ -1750,7 +1760,7 @@ struct Backward {
     J.shared = shared;
     J.mk = 0u;
     J.per = (int32_t)min((long long)R.cnt, max(1ll, (long long)R.cnt * CHUNK_ARCS / max((uint32_t)R.cnt, R.tot)));
-    if ((P.t & 4095) == 0) atomicAdd(K.ctl + CTL_PROGRESS, 1u);
+    report(K, P.t - 1, P.t);
   }
   __device__ __forceinline__ void leave(const Place& P, int32_t b, int32_t hand) const {
     if (hand >= 0) {
@@ -1819,6 +1829,7 @@ struct Backward {
     __syncwarp();
     const int32_t last_q = __shfl_sync(FULL, q, m - 1);
     P.t -= m;
+    if (lane == 0) report(K, P.t, P.t + m);
     P.tE = tE;
     P.ek = fkey64(u);
     P.cur_n = 1;

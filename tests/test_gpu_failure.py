@@ -311,6 +311,34 @@ def test_backward_pass_that_gives_up_spoils_the_counts(wide):
     assert abs(pf.start_counts.sum().item() - B) < 1e-4 and abs(pf.final_counts.sum().item() - B) < 1e-4
 
 
+def test_long_runs_of_one_arc_positions_count_as_progress():
+    # a string whose passes take several times the limit: its positions are
+    # progress to the workers that wait, in both passes
+    import torch
+    from paper_1701_03038_gb300 import _lib
+    from paper_1701_03038_gb300.fst import Fst
+    fa = _chain_fst()
+    f, o = Fst.from_arrays(fa), oracle.Fst(fa)
+    n = 600_000  # (at least 0.2 us a position: 120 ms)
+    ids = np.random.default_rng(5).integers(0, 3, n + 5).astype(np.int32)
+    strs = synth.Strings(ids, np.array([0, n, n + 5], np.int64))
+    pv, pf = _plans(f, strs)
+    for p in (pv, pf):
+        p.set_driver(_lib.DRIVER_LAUNCH, 0, 25_000)
+    pv.viterbi()
+    pf.forward_backward()
+    torch.cuda.synchronize()
+    assert (pv.status[:2].cpu().numpy() == 0).all() and (pf.status[:2].cpu().numpy() == 0).all()
+    for b in range(2):
+        lo, hi = strs.offsets[b], strs.offsets[b + 1]
+        assert_viterbi_equal(pv.scores[b].item(), pv.paths[lo:hi].cpu().numpy(), pv.olabels[lo:hi].cpu().numpy(),
+                             pv.status[b].item(), o.viterbi(strs.get(b)))
+        # one path: its weight, and a posterior of 1 at every position
+        assert_logz_close(pf.logz[b].item(), -fa.weight[pv.paths[lo:hi].cpu().numpy()].astype(np.float64).sum())
+    used = np.bincount(pv.paths[:n + 5].cpu().numpy(), minlength=fa.num_arcs)
+    assert_counts_close(pf.counts.cpu().numpy(), used, batch=True)
+
+
 def test_fault_inject_rejects_bad_arguments():
     import torch
     from paper_1701_03038_gb300 import _lib
