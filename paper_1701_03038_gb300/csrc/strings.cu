@@ -57,6 +57,9 @@ constexpr int HS0 = 256, HS1 = 2048;
 constexpr int BHS0 = 128, BHS1 = 1024, LIGHT_CAP = 96;
 // a heavy block hands a string back at this many arcs and entries
 constexpr int LIGHT_ARCS = 64;
+// a light warp leaves a string with more start states to a heavy block, and a
+// block shares more than SHARE_ARCS of them out uncounted, in chunks of START_CHUNK
+constexpr int LIGHT_STARTS = HS0 / 2, START_CHUNK = NT1 * 2;
 // a position is shared among the heavy blocks from SHARE_ARCS arcs on, in
 // chunks of about CHUNK_ARCS; a block with a string of its own leaves it for
 // jobs of BIG_CHUNKS chunks
@@ -1022,8 +1025,12 @@ struct Forward {
     int2* fe = fe_light(g);
     uint32_t mk = 0u;
     int32_t a = P.n > 0 ? __ldg(sym + P.off + P.t - 1) : 0;
-    for (int32_t i = lane; i < P.cnt; i += 32) P.tot += resume_entry(P, fe, i, a);
-    P.tot = (int32_t)__reduce_add_sync(FULL, (unsigned)P.tot);
+    if (P.t == 1 && P.cnt > LIGHT_STARTS) {
+      P.tot = HS0;  // (more than it takes)
+    } else {
+      for (int32_t i = lane; i < P.cnt; i += 32) P.tot += resume_entry(P, fe, i, a);
+      P.tot = (int32_t)__reduce_add_sync(FULL, (unsigned)P.tot);
+    }
     __syncwarp();
     // this lane's entry (len 0: none), with its first arc when first.w is set
     Entry x{0, 0, -1, none()};
@@ -1226,6 +1233,7 @@ struct Forward {
     int32_t pend = 0;
     for (int32_t i0 = lo; i0 < hi; i0 += NT1 * BlockStage::PER) {
       const int32_t total = stage(st, fe_heavy(J.owner), J.t, J.base, J.a, i0, hi);
+      if (J.phase == 0 && J.t == 1 && J.shared && threadIdx.x == 0) atomicAdd(&K.jobs[J.owner].tot, (uint32_t)total);
       if (J.phase == 0) walk_dense<0>(J.owner, staged, st, total, pend);
       else if constexpr (!VIT) walk_dense<1>(J.owner, nullptr, st, total, pend);
     }
@@ -1262,13 +1270,20 @@ struct Forward {
           b = got;
           P = resume(b);
           a = P.n > 0 ? __ldg(sym + P.off + P.t - 1) : 0;
-          if (tid == 0) hv.tot = 0u;
-          __syncthreads();
-          for (int32_t i = tid; i < P.cnt; i += NT1) P.tot += resume_entry(P, fe, i, a);
-          P.tot = (int32_t)__reduce_add_sync(FULL, (unsigned)P.tot);
-          if (lane == 0 && P.tot) atomicAdd(&hv.tot, (uint32_t)P.tot);
-          __syncthreads();
-          P.tot = (int32_t)hv.tot;
+          if (P.t == 1 && P.cnt >= SHARE_ARCS) {
+            // many start states: their arcs are counted as they are walked
+            // (200,000 of them, looked up by one warp: a call of 6 symbols
+            // took 10.6 ms; shared out it takes 0.1)
+            P.tot = P.cnt;
+          } else {
+            if (tid == 0) hv.tot = 0u;
+            __syncthreads();
+            for (int32_t i = tid; i < P.cnt; i += NT1) P.tot += resume_entry(P, fe, i, a);
+            P.tot = (int32_t)__reduce_add_sync(FULL, (unsigned)P.tot);
+            if (lane == 0 && P.tot) atomicAdd(&hv.tot, (uint32_t)P.tot);
+            __syncthreads();
+            P.tot = (int32_t)hv.tot;
+          }
         }
       }
       bool done = false;  // position P.t is done
@@ -1300,6 +1315,7 @@ struct Forward {
             J.cnt = P.cnt;
             // (fewer than 2^31 arcs: the chunks' numbers fit JOB_BITS)
             J.per = shared ? (int32_t)min((long long)P.cnt, max(1ll, (long long)P.cnt * CHUNK_ARCS / size)) : P.cnt;
+            if (P.t == 1 && P.cnt >= SHARE_ARCS) J.per = max(START_CHUNK, P.cnt >> (JOB_BITS - 1));
             J.base = P.base;
             J.shift = P.shift;
             J.shared = shared;
@@ -1380,14 +1396,19 @@ struct Forward {
           else if (!job_wait(hv, K, n)) return;
           if (own == 0) {
             nb = alone ? sh.tab.staged : (int32_t)hv.job.staged;
+            if (!alone && P.t == 1) P.tot = (int32_t)hv.job.tot;  // (start states: counted now)
             single = nb == P.tot;
           }
           __syncthreads();
           if (own == 0 && !VIT && !single) {
-            if (tid == 0) hv.job.phase = 1;
+            if (tid == 0) {
+              hv.job.phase = 1;
+              hv.job.tot = 0u;
+            }
             own = 1;
           } else if (own < 2) {
             if (tid == 0) {
+              hv.job.tot = 0u;
               hv.base = reserve(sh.gs, nb);
               hv.job.phase = 2;
               hv.job.nb = nb;

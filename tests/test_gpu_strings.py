@@ -8,7 +8,7 @@ import pytest
 import oracle
 from paper_1701_03038_gb300 import synth
 
-from gpu_util import assert_viterbi_equal, ensure_built
+from gpu_util import assert_counts_close, assert_logz_close, assert_viterbi_equal, ensure_built
 
 pytestmark = pytest.mark.gpu
 
@@ -147,3 +147,37 @@ def test_idle_blocks_look_for_jobs(fans, count):
     out = [turn * (50 + b) for b in range(count)]
     off = np.concatenate([[0], np.cumsum([len(s) for s in out])]).astype(np.int64)
     _same_as_per_position(f, synth.Strings(np.concatenate(out).astype(np.int32), off), 6)
+
+
+@pytest.mark.parametrize("starts", [96, 97, 128, 129, 1000, 4095, 4096, 4097, 6000])
+def test_many_start_states(starts):
+    # the first position (and the last of the backward pass) over start states
+    # on both sides of every line: a table's entries, a light warp's, a block's
+    # by itself, shared out; few arcs, many, and none out of them
+    from paper_1701_03038_gb300.fst import Fst
+    rng = np.random.default_rng(starts)
+    q = np.arange(Q)
+    parts = [(q, (q + 1) % Q, 0), (q[::40], (q[::40] * 7) % Q, 1), (np.repeat(q, 3), rng.integers(0, Q, 3 * Q), 2),
+             (q[::40], q[::40] % 3, 3)]
+    src, dst = (np.concatenate([p[k] for p in parts]).astype(np.int32) for k in (0, 1))
+    lab = np.concatenate([np.full(len(p[0]), p[2]) for p in parts]).astype(np.int32)
+    w = rng.uniform(0.1, 4.0, len(src)).astype(np.float32)
+    start = np.full(Q, np.inf, np.float32)
+    start[rng.choice(Q, starts, replace=False)] = rng.uniform(0.0, 2.0, starts)
+    fa = synth.FstArrays(Q, 5, 5, src, dst, lab, lab, w, start, rng.uniform(0.0, 2.0, Q).astype(np.float32))
+    f, o = Fst.from_arrays(fa), oracle.Fst(fa)
+    out = [[], [0], [1], [2], [3], [4], [1, 0, 0], [2, 1, 0], [3, 0, 2, 2], [0, 2, 1], [4, 0], [2, 4, 1]]
+    out += [list(rng.integers(0, 4, int(rng.integers(1, 9)))) for _ in range(40)]
+    off = np.concatenate([[0], np.cumsum([len(s) for s in out])]).astype(np.int64)
+    strs = synth.Strings(np.concatenate([np.asarray(s, np.int32) for s in out]).astype(np.int32), off)
+    _same_as_per_position(f, strs, 2)
+    from paper_1701_03038_gb300 import _lib
+    f.set_plain_method(_lib.PLAIN_FRONTIER)
+    for s in out[:8]:
+        x = np.asarray(s, np.int32)
+        score, path, olab, st = f.viterbi(x)
+        assert_viterbi_equal(score, path, olab, st, o.viterbi(x))
+        ofb = o.forward_backward(x)
+        lz, cnt, _ = f.forward_backward(x)
+        assert_logz_close(lz, ofb["logz"])
+        assert_counts_close(cnt, ofb["counts"])
