@@ -181,8 +181,9 @@ FST_API int fst_autotune_plain(fst_t* fst, const int32_t* ids, const int64_t* of
 /* Driver of the single-string frontier kernels (fst_forward_backward, and
  * fst_viterbi when it uses them): FST_DRIVER_LAUNCH (the default: the
  * string kernels, one launch per pass, in which warps and blocks run the
- * whole string; a string whose live pool may pass 2^31 entries takes one
- * launch per position and kernel kind) or FST_DRIVER_PERSISTENT (one
+ * whole string; a string whose live pool may pass 2^31 entries, or whose
+ * symbols' slices are expected to keep its frontier wide, takes one launch
+ * per position and kernel kind) or FST_DRIVER_PERSISTENT (one
  * cooperative launch per pass, grid_blocks blocks, 0 = one per SM,
  * positions separated by bounded grid barriers; a barrier that times out
  * makes the call return FST_ERR_TIMEOUT).  fst_autotune_plain also picks

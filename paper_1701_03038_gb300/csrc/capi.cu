@@ -298,9 +298,41 @@ int plain_reserve(PlainWs* w, int64_t n, int64_t stage, int64_t pool) {
   return FST_OK;
 }
 
+// Whether launches per position run one string faster than the string
+// kernels.  A position of more than a heavy block's table takes those two or
+// three phases, each shared out to blocks that must first find it (32 us a
+// position in Viterbi, 55 forward), and the launches 15 and 30 us; every
+// narrower position is theirs at 2 to 10 us.  So the launches take a string
+// when a third of its positions are expected to be that large, unless so
+// many arcs meet in each destination (more than 12 a live state) that the
+// launches' atomics collide -- which the string kernels' do too past half a
+// million arcs.  30 symbols, Viterbi and forward, by launches and by string
+// kernels: 20,000 states of 2 arcs a state and symbol 524 and 1,067 us, 922
+// and 1,904; 8 arcs 781 and 1,100, 1,556 and 2,042; 20 arcs 1,252 and 1,169,
+// 2,621 and 2,225; 100,000 states of 20 arcs 1,506 and 2,589, 3,927 and 5,207.
+// The frontier's expected width: live states have their slice's average arcs,
+// which hit its destinations at random.
+bool plain_by_launches(const fst_s* f, const int32_t* ids, int32_t n) {
+  double live = f->nstart, large = 0.0, from = 0.0, arcs = 0.0;
+  for (int32_t i = 0; i < n; ++i) {
+    const double A = (double)(f->h_sym_arc[ids[i] + 1] - f->h_sym_arc[ids[i]]);
+    const double D = (double)(f->fwd.h_sym_seg[ids[i] + 1] - f->fwd.h_sym_seg[ids[i]]);
+    if (A <= 0.0) break;
+    const double x = std::min(live / f->Q, 1.0) * A;
+    if (x > STRING_TABLE_ARCS) {
+      large += 1.0;
+      from += live;
+      arcs += x;
+    }
+    live = std::max(1.0, x < D / 20.0 ? x : D * (1.0 - std::pow(std::max(0.0, 1.0 - x / A), A / D)));
+  }
+  if (large * 3.0 <= n) return false;
+  return arcs <= 12.0 * from || arcs >= 5e5 * large;
+}
+
 // Upload the tokens of one string and start a run; *strings: it takes the
 // string kernels (the launch driver, unless the pool is past their 31-bit
-// entry numbers).
+// entry numbers or launches per position are faster).
 int plain_tokens(fst_s* f, const int32_t* ids, int32_t n, cudaStream_t s, bool* strings) {
   PlainWs* w = f->plain;
   int64_t stage = 1, pool = 1;
@@ -315,7 +347,7 @@ int plain_tokens(fst_s* f, const int32_t* ids, int32_t n, cudaStream_t s, bool* 
   }
   // (what the chunks of a light warp and a heavy block may leave unused)
   const int64_t spare = pool / 3 + 4 * POOL_CHUNK;
-  *strings = f->plain_fb_driver == FST_DRIVER_LAUNCH && pool + spare < INT32_MAX;
+  *strings = f->plain_fb_driver == FST_DRIVER_LAUNCH && pool + spare < INT32_MAX && !plain_by_launches(f, ids, n);
   int rc = plain_reserve(w, std::max(n, 1), stage, *strings ? pool + spare : pool);
   if (rc) return rc;
   w->olabels = w->paths + n;

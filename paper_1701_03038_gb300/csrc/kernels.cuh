@@ -310,6 +310,9 @@ struct StringQueue {
   uint64_t limit_ns;
   double* spoiled;  // backward: CountView::spoiled
 };
+// Arcs out of a position's live states up to which a heavy block takes its
+// table in shared memory, half of the table's slots.
+constexpr int32_t STRING_TABLE_ARCS = 1024;
 // Pool entries a group of the string kernels reserves at a time; a capped
 // pool is handed out range by range, so that the cap counts live entries.
 constexpr int32_t POOL_CHUNK = 64;

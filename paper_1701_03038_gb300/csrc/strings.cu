@@ -51,7 +51,7 @@ constexpr int VU0 = 1, VU1 = 2;
 // three blocks an SM (80 registers a thread): with two (128) the same
 // backward pass takes 40% longer, with four (64) the Viterbi pass 30%.
 constexpr int NT1 = 256, WARPS = NT1 / 32;
-constexpr int HS0 = 256, HS1 = 2048;
+constexpr int HS0 = 256, HS1 = 2 * STRING_TABLE_ARCS;
 // the same of the backward pass, whose light warps hold at most LIGHT_CAP
 // states
 constexpr int BHS0 = 128, BHS1 = 1024, LIGHT_CAP = 96;

@@ -388,3 +388,35 @@ def test_block_method_small_fsts():
     with pytest.raises(_lib.FstError) as ei:
         _fst(big).set_plain_method(_lib.PLAIN_BLOCK)
     assert ei.value.code == _lib.UNSUPPORTED
+
+
+@pytest.mark.parametrize("growth,launches", [(0.5, False), (2.0, True), (8.0, True), (20.0, False)])
+def test_wide_frontiers_by_launches_or_string_kernels(growth, launches):
+    # single strings on one handle, taking the string kernels and the launches
+    # per position in turn: which of the two by the arcs per state of the
+    # symbols 0..2 (3 has few arcs), the results as the oracle's either way
+    rng = np.random.default_rng(int(growth * 10))
+    Q, A = 3000, int(3000 * growth)
+    src, dst = (rng.integers(0, Q, 3 * A).astype(np.int32) for _ in range(2))
+    lab = np.repeat(np.arange(3), A).astype(np.int32)
+    q = np.arange(0, Q, 3, dtype=np.int32)
+    src, dst = np.concatenate([src, q]), np.concatenate([dst, (q * 3) % Q]).astype(np.int32)
+    lab = np.concatenate([lab, np.full(len(q), 3, np.int32)])
+    w = rng.uniform(0.1, 3.0, len(src)).astype(np.float32)
+    start = np.full(Q, np.inf, np.float32)
+    start[:60] = rng.uniform(0.0, 1.0, 60)
+    fa = synth.FstArrays(Q, 4, 4, src, dst, lab, lab, w, start, rng.uniform(0.0, 1.0, Q).astype(np.float32))
+    f, o = _fst(fa), oracle.Fst(fa)
+    wide = rng.integers(0, 3, 24).astype(np.int32)
+    third = np.concatenate([np.full(16, 3), rng.integers(0, 3, 9)]).astype(np.int32)
+    f.profile(True)
+    for x, large in ((wide, True), (np.full(9, 3, np.int32), False), (wide[:1], False), (wide, True),
+                     (third, None), (np.zeros(0, np.int32), False), (wide[::-1].copy(), True)):
+        f.profile_read()
+        check_string(f, o, x)
+        by = f.profile_read()
+        if large is not None and len(x):
+            assert by["vit_step"][1] == (len(x) if launches and large else 1), by
+            assert by["fwd_step"][1] == (len(x) if launches and large else 1), by
+            assert by["bwd_step"][1] == (len(x) if launches and large else 1), by
+    f.profile(False)
