@@ -118,39 +118,44 @@ __device__ __forceinline__ void load_arcs(ArcRegs& R, const int4* __restrict__ a
     R.th[k] = i < sl.i1 ? __ldg(theta + i) : 0.f;
   }
 }
-// The slices of a pass's positions, t, t + d, t + 2 d and on: a symbol, its
+__device__ __forceinline__ Slice slice_at(const int64_t* __restrict__ sym_win, const int32_t* __restrict__ ids,
+                                          int32_t n, int32_t t) {
+  return (t >= 1 && t <= n) ? slice_of(sym_win, __ldg(ids + t - 1)) : Slice{0, 0};
+}
+// The slices of Viterbi's positions, t, t + 1, t + 2 and on: a symbol, its
 // slice's bounds and its arcs are reads that depend on each other, so each
-// position's are taken a position after the one before (Viterbi of 50 symbols
-// on 1,000 states, 400 arcs a slice: 66.8 us with the three in one position,
-// 63.3 so; the barriers and the shared-memory atomics are most of the rest).
+// position's are taken a position after the one before (a call on 50 symbols,
+// 1,000 states and 400 arcs a slice: 81.6 us with the three in one position,
+// 79.3 so, in turn; the barriers and the shared-memory atomics are most of the
+// rest.  The forward-backward kernels lose by it: 141.8 us a call, 140.5 without).
 struct SliceRun {
   const int64_t* __restrict__ sym_win;
   const int32_t* __restrict__ ids;
-  int32_t n, t, d;
+  int32_t n, t;
   int32_t a;        // the symbol three positions on
   Slice now, next, after;
   __device__ __forceinline__ int32_t symbol(int32_t u) const { return u >= 1 && u <= n ? __ldg(ids + u - 1) : -1; }
   __device__ __forceinline__ Slice slice(int32_t x) const { return x >= 0 ? slice_of(sym_win, x) : Slice{0, 0}; }
-  __device__ __forceinline__ SliceRun(const int64_t* w, const int32_t* i, int32_t n_, int32_t t_, int32_t d_)
-      : sym_win(w), ids(i), n(n_), t(t_), d(d_) {
+  __device__ __forceinline__ SliceRun(const int64_t* w, const int32_t* i, int32_t n_, int32_t t_)
+      : sym_win(w), ids(i), n(n_), t(t_) {
     now = slice(symbol(t));
-    next = slice(symbol(t + d));
-    after = slice(symbol(t + 2 * d));
-    a = symbol(t + 3 * d);
+    next = slice(symbol(t + 1));
+    after = slice(symbol(t + 2));
+    a = symbol(t + 3);
   }
   // What the next position but two needs, asked for at the start of one ...
   struct Ahead {
     Slice s;
     int32_t a;
   };
-  __device__ __forceinline__ Ahead ahead() const { return Ahead{slice(a), symbol(t + 4 * d)}; }
+  __device__ __forceinline__ Ahead ahead() const { return Ahead{slice(a), symbol(t + 4)}; }
   // ... and taken up at its end.
   __device__ __forceinline__ void step(const Ahead& h) {
     now = next;
     next = after;
     after = h.s;
     a = h.a;
-    t += d;
+    ++t;
   }
 };
 
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(BT, 1) k_block_viterbi(const int4* __restrict_
     v[q] = __ldg(theta_s + q);
   }
   ArcRegs cur, nxt;
-  SliceRun run(sym_win, ids, n, 1, 1);
+  SliceRun run(sym_win, ids, n, 1);
   load_arcs(cur, arcs, theta, run.now);
   __syncthreads();
   for (int32_t t = 1; t <= n; ++t) {
@@ -304,13 +309,11 @@ __device__ void block_forward(const int4* __restrict__ arcs, const float* __rest
     alpha[q] = a[q];
   }
   ArcRegs cur, nxt;
-  SliceRun run(sym_win, ids, n, 1, 1);
-  load_arcs(cur, arcs, theta, run.now);
+  load_arcs(cur, arcs, theta, slice_at(sym_win, ids, n, 1));
   __syncthreads();
   for (int32_t t = 1; t <= n; ++t) {
-    const Slice sl = run.now;
-    load_arcs(nxt, arcs, theta, run.next);
-    const SliceRun::Ahead ahead = run.ahead();
+    const Slice sl = slice_at(sym_win, ids, n, t);
+    load_arcs(nxt, arcs, theta, slice_at(sym_win, ids, n, t + 1));
     // an arc counts when its source is live and its weight finite (then
     // the sum is finite too)
 #pragma unroll
@@ -353,7 +356,6 @@ __device__ void block_forward(const int4* __restrict__ arcs, const float* __rest
     }
     __syncthreads();
     cur = nxt;
-    run.step(ahead);
   }
   // log Z = log sum_q exp(alpha_n[q] + theta_f[q]): exact maximum, then a
   // float64 sum in a fixed order
@@ -392,13 +394,11 @@ __device__ void block_backward(const int4* __restrict__ arcs, const float* __res
     beta[(int64_t)n * Q + q] = a[q];
   }
   ArcRegs cur, nxt;
-  SliceRun run(sym_win, ids, n, n, -1);
-  load_arcs(cur, arcs, theta, run.now);
+  load_arcs(cur, arcs, theta, slice_at(sym_win, ids, n, n));
   __syncthreads();
   for (int32_t t = n; t >= 1; --t) {
-    const Slice sl = run.now;
-    load_arcs(nxt, arcs, theta, run.next);
-    const SliceRun::Ahead ahead = run.ahead();
+    const Slice sl = slice_at(sym_win, ids, n, t);
+    load_arcs(nxt, arcs, theta, slice_at(sym_win, ids, n, t - 1));
 #pragma unroll
     for (int k = 0; k < KR; ++k) {
       if (cur.r[k].z < 0 || dead32(cur.th[k])) continue;
@@ -439,7 +439,6 @@ __device__ void block_backward(const int4* __restrict__ arcs, const float* __res
     }
     __syncthreads();
     cur = nxt;
-    run.step(ahead);
   }
 }
 
