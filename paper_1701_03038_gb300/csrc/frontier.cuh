@@ -3,6 +3,7 @@
 // per string over all positions).
 #pragma once
 
+#include "debug_record.cuh"
 #include "kernels.cuh"
 
 namespace fstgpu {
@@ -35,6 +36,16 @@ static __device__ __noinline__ bool in_bounds_slow(int code, long long i, long l
 __device__ __forceinline__ bool in_bounds(int code, long long i, long long n) {
   return (i >= 0 && i < n) ? true : in_bounds_slow(code, i, n);
 }
+// (this file's record, read with the others')
+static int debug_read_own(DebugCounts* out) {
+  unsigned long long h[4] = {0, 0, 0, 0};
+  FST_CUDA(cudaMemcpyFromSymbol(h, g_dbg, sizeof(h)));
+  *out = DebugCounts{h[0], h[1], h[2], h[3]};
+  for (unsigned long long& x : h) x = 0;
+  FST_CUDA(cudaMemcpyToSymbol(g_dbg, h, sizeof(h)));
+  return FST_OK;
+}
+static DebugRecord g_dbg_record(debug_read_own);
 #else
 __device__ __forceinline__ bool in_bounds(int, long long, long long) { return true; }
 #endif

@@ -1725,21 +1725,13 @@ int launch_persist(K kernel, int* cap_cache, int32_t grid, GridSync G, cudaStrea
 
 int debug_read(int64_t* violations, int32_t* code, int64_t* index, int64_t* bound) {
 #ifdef FST_DEBUG
-  unsigned long long h[4] = {0, 0, 0, 0};
-  FST_CUDA(cudaMemcpyFromSymbol(h, g_dbg, sizeof(h)));
-  const unsigned long long z[4] = {0, 0, 0, 0};
-  FST_CUDA(cudaMemcpyToSymbol(g_dbg, z, sizeof(z)));
-  unsigned long long g[4] = {0, 0, 0, 0};
-  const int rc = string_debug_read(g);
+  DebugCounts d;
+  const int rc = debug_read_all(&d);
   if (rc) return rc;
-  g[0] += h[0];
-  if (h[0])
-    for (int i = 1; i < 4; ++i) g[i] = h[i];
-  for (int i = 0; i < 4; ++i) h[i] = g[i];
-  if (violations) *violations = (int64_t)h[0];
-  if (code) *code = (int32_t)h[1];
-  if (index) *index = (int64_t)h[2];
-  if (bound) *bound = (int64_t)h[3];
+  if (violations) *violations = (int64_t)d.violations;
+  if (code) *code = (int32_t)d.code;
+  if (index) *index = (int64_t)d.index;
+  if (bound) *bound = (int64_t)d.bound;
   return FST_OK;
 #else
   (void)violations; (void)code; (void)index; (void)bound;

@@ -333,10 +333,6 @@ int launch_string_backward(const LayoutView& L, const int32_t* sym, const Fronti
 // launch_vit_final.
 int launch_string_trace(const FrontierState& S, const int32_t* olabel_by_id, int32_t Bw, const int32_t* jfinal,
                         int32_t* paths, int32_t* olabels, cudaStream_t s);
-#ifdef FST_DEBUG
-int string_debug_read(unsigned long long* h);  // as debug_read, of strings.cu
-#endif
-
 // Bounds-checked build (compiled with FST_DEBUG): the kernels check every
 // computed index into the staging buffers, the live pool, the dense
 // accumulators and the arc records against its buffer's size, count the

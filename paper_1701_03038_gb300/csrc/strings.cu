@@ -2223,13 +2223,4 @@ int launch_string_trace(const FrontierState& S, const int32_t* olabel_by_id, int
   return check_launch("k_str_trace");
 }
 
-#ifdef FST_DEBUG
-int string_debug_read(unsigned long long* h) {
-  FST_CUDA(cudaMemcpyFromSymbol(h, g_dbg, 4 * sizeof(unsigned long long)));
-  const unsigned long long z[4] = {0, 0, 0, 0};
-  FST_CUDA(cudaMemcpyToSymbol(g_dbg, z, sizeof(z)));
-  return FST_OK;
-}
-#endif
-
 }  // namespace fstgpu
