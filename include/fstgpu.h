@@ -625,8 +625,9 @@ FST_API int fst_plan_set_pull(fst_plan_t* plan, int64_t min_live);
  * build_debug) checks, in the frontier kernels, every computed index into
  * the staging buffers, the live pool, the dense accumulators and the arc
  * records against its buffer's size; a violation is counted, the first is
- * recorded (code: 1 staging, 2 pool write, 3 pool read, 4 dense
- * accumulator, 5 arc record; its index and the bound) and the access is
+ * recorded (code: 1 staging and what a string's worker keeps from position
+ * to position, 2 pool write, 3 pool read, 4 dense accumulator or backward
+ * value, 5 arc record; its index and the bound) and the access is
  * skipped.  This call reads the record (host outputs, any may be NULL) and
  * clears it.  FST_ERR_UNSUPPORTED in a normal build. (No counterpart in the paper.) */
 FST_API int fst_debug_checks(int64_t* violations, int32_t* code, int64_t* index, int64_t* bound);

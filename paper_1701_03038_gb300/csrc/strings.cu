@@ -528,6 +528,11 @@ struct Forward {
   __device__ __forceinline__ int2* fe_heavy(int32_t g) const { return K.fe + (int64_t)g * S.Q; }
   __device__ __forceinline__ int2* fe_light(int32_t g) const { return K.fe + K.fe_light + (int64_t)g * (HS0 / 2); }
 
+  // The arcs of entry i (cap: the entries that fe holds).
+  __device__ __forceinline__ void put_arcs(int2* fe, int32_t cap, int32_t i, const Arcs& x) const {
+    if (in_bounds(CHK_STAGE, i, cap)) fe[i] = make_int2(x.pos, x.len);
+  }
+
   struct Entry {
     int32_t e0, len, jp;
     Real r;
@@ -547,6 +552,7 @@ struct Forward {
       x = Entry{s.pos, s.len, -1, real(__ldg(S.theta_s + q))};
     } else {
       x.jp = base + i;
+      if (!in_bounds(CHK_POOL_READ, x.jp, S.pool_cap)) return Entry{0, 0, -1, none()};
       if constexpr (VIT) {
         const int2 s = __ldcg(fe + i);
         x.e0 = s.x;
@@ -813,7 +819,7 @@ struct Forward {
     x.jp = base + i;
     if (VIT) {
       put(base + i, d, x.r, (int32_t)(~(uint32_t)acc), single ? (int32_t)aux : -2);
-      fe[i] = make_int2(nxt.pos, nxt.len);
+      put_arcs(fe, HS == HS0 ? HS0 / 2 : S.Q, i, nxt);
     } else {
       put(base + i, d, x.r, nxt.pos, nxt.len);
     }
@@ -847,6 +853,8 @@ struct Forward {
     for (int u = 0; u < RU; ++u) {
       x[u] = make_ulonglong2(0ull, 0ull);
       if (d[u] < 0) continue;
+      if (!in_bounds(CHK_ACC, d[u], S.Q)) d[u] = -1;
+      if (d[u] < 0) continue;
       if (VIT) x[u].y = __ldcg(acc + d[u]);
       else x[u] = __ldcg((const ulonglong2*)acc + d[u]);
       if (an >= 0) seg_load(L, an, d[u], p[u]);
@@ -859,7 +867,7 @@ struct Forward {
       if constexpr (VIT) {
         acc[d[u]] = 0ull;
         put(base + i, d[u], fkey_inv((uint32_t)(x[u].y >> 32)), (int32_t)(~(uint32_t)x[u].y), -2);
-        fe_heavy(g)[i] = make_int2(nxt.pos, nxt.len);
+        put_arcs(fe_heavy(g), S.Q, i, nxt);
       } else {
         ((ulonglong2*)acc)[d[u]] = make_ulonglong2(0ull, 0ull);
         const double r = fix_log_sum64(dkey_inv(x[u].y) - fx_widen(shift), single ? 1099511627776ull : x[u].x);
@@ -894,10 +902,10 @@ struct Forward {
   }
   // The arcs of entry i that a string goes on with: the Viterbi entries'
   // are looked up again.
-  __device__ __forceinline__ int32_t resume_entry(const Place& P, int2* fe, int32_t i, int32_t a) const {
+  __device__ __forceinline__ int32_t resume_entry(const Place& P, int2* fe, int32_t cap, int32_t i, int32_t a) const {
     if (VIT && P.t > 1) {
       const Arcs x = find_arcs(L, a, __ldcg(S.pool_q + P.base + i));
-      fe[i] = make_int2(x.pos, x.len);
+      put_arcs(fe, cap, i, x);
       return x.len;
     }
     return entry(fe, P.t, P.base, i, a).len;
@@ -1028,7 +1036,7 @@ struct Forward {
     if (P.t == 1 && P.cnt > LIGHT_STARTS) {
       P.tot = HS0;  // (more than it takes)
     } else {
-      for (int32_t i = lane; i < P.cnt; i += 32) P.tot += resume_entry(P, fe, i, a);
+      for (int32_t i = lane; i < P.cnt; i += 32) P.tot += resume_entry(P, fe, HS0 / 2, i, a);
       P.tot = (int32_t)__reduce_add_sync(FULL, (unsigned)P.tot);
     }
     __syncwarp();
@@ -1085,7 +1093,10 @@ struct Forward {
           arc.w = __shfl_sync(FULL, first.w, o);
           if (k != 0) arc.w = 0;
         }
-        if (on && !arc.w) arc = __ldg(L.arcs + e);
+        if (on && !arc.w) {
+          if (in_bounds(CHK_ARC, e, L.P)) arc = __ldg(L.arcs + e);
+          else on = false;
+        }
         double v = 0.0;
         const unsigned long long c = on ? candidate(r, arc, &v) : 0ull;
         on = c != 0ull;
@@ -1139,7 +1150,7 @@ struct Forward {
           x.jp = nbase + i;
           if (VIT) {
             put(nbase + i, arc.x, x.r, (int32_t)(~(uint32_t)c), jp);
-            fe[i] = make_int2(nxt.pos, nxt.len);
+            put_arcs(fe, HS0 / 2, i, nxt);
           } else {
             put(nbase + i, arc.x, x.r, nxt.pos, nxt.len);
           }
@@ -1278,7 +1289,7 @@ struct Forward {
           } else {
             if (tid == 0) hv.tot = 0u;
             __syncthreads();
-            for (int32_t i = tid; i < P.cnt; i += NT1) P.tot += resume_entry(P, fe, i, a);
+            for (int32_t i = tid; i < P.cnt; i += NT1) P.tot += resume_entry(P, fe, S.Q, i, a);
             P.tot = (int32_t)__reduce_add_sync(FULL, (unsigned)P.tot);
             if (lane == 0 && P.tot) atomicAdd(&hv.tot, (uint32_t)P.tot);
             __syncthreads();
@@ -1596,6 +1607,7 @@ struct Backward {
       if (atomicCAS(tab.key[w] + h, 0u, k) == 0u) break;
       h = (h + 1) & (HS - 1);
     }
+    if (!in_bounds(CHK_STAGE, i, CAP)) return;
     tab.val[w][h] = v;
     tab.list[w][i] = (uint16_t)h;
   }
@@ -1641,6 +1653,7 @@ struct Backward {
       for (int u = 0; u < VU; ++u) {
         const int32_t a = a0 + u * 32 + lane;
         oi[u] = a < total ? owner_of(st.excl, a) : -1;
+        if (oi[u] >= 0 && !in_bounds(CHK_ARC, (long long)st.e0[oi[u]] + (a - st.excl[oi[u]]), L.P)) oi[u] = -1;
         arc[u] = oi[u] >= 0 ? __ldg(L.arcs + st.e0[oi[u]] + (a - st.excl[oi[u]])) : make_int4(0, 0, 0, 0);
       }
 #pragma unroll
@@ -1667,7 +1680,7 @@ struct Backward {
           const int32_t a = a0 + u * 32 + lane;
           oo[u] = a < total ? owner_of(st.excl, a) : -1;
           v[u] = -INFINITY;
-          if (oo[u] >= 0) {
+          if (oo[u] >= 0 && in_bounds(CHK_ARC, (long long)st.e0[oo[u]] + (a - st.excl[oo[u]]), L.P)) {
             const int4 arc = __ldg(L.arcs + st.e0[oo[u]] + (a - st.excl[oo[u]]));
             v[u] = term(J, arc);
             id[u] = arc.z;
@@ -1687,8 +1700,11 @@ struct Backward {
       const double uv = fix_log_sum64(m, st.acc[lane]);
       if (J.t > 1) {
         const int w = (J.t & 1) ^ 1;
-        if (HEAVY && J.next_big) dval(J.owner, w)[q] = uv;
-        else insert(w, i, q, uv);
+        if (HEAVY && J.next_big) {
+          if (in_bounds(CHK_ACC, q, S.Q)) dval(J.owner, w)[q] = uv;
+        } else {
+          insert(w, i, q, uv);
+        }
         ek = fkey64(uv);
       } else if (C.start64 && uv != -INFINITY) {
         // the item is a start state q, log beta_0[q] = u + E_1
@@ -1738,6 +1754,7 @@ struct Backward {
     double* kept = K.kept + (int64_t)b * LIGHT_CAP;
     const int64_t base = P.t < P.n ? __ldg(S.pool_base + P.off + P.t - 1) : 0;
     for (int32_t i = first; i < P.cur_n; i += step) {
+      if (!in_bounds(CHK_STAGE, i, LIGHT_CAP)) continue;
       if (HEAVY && P.cur_big) {
         kept[i] = __ldcg(dval(g, w) + __ldg(S.pool_q + base + i));
       } else {
@@ -1817,7 +1834,8 @@ struct Backward {
     if (lane < m && in_bounds(CHK_POOL_READ, base, S.pool_cap)) {
       q = __ldg(S.pool_q + base);
       ra = __ldg(S.pool_d + base);
-      arc = __ldg(L.arcs + __ldg(S.pool_x + base));
+      const int32_t e = __ldg(S.pool_x + base);
+      if (in_bounds(CHK_ARC, e, L.P)) arc = __ldg(L.arcs + e);
       mprev = decode_max(__ldg(S.mkey + p - 1));
       pre = __ldg(S.csum + p - 1);
     }

@@ -83,3 +83,41 @@ def test_debug_build_has_no_violations(tmp_path):
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
     line = [x for x in r.stdout.splitlines() if x.startswith("VIOLATIONS")][-1]
     assert line.split()[1] == "0", line
+
+
+WIDE = textwrap.dedent("""
+    import sys
+    sys.path.insert(0, {root!r}); sys.path.insert(0, {tests!r})
+    import numpy as np, torch
+    import test_gpu_strings as T
+    from paper_1701_03038_gb300 import synth, _lib
+    from paper_1701_03038_gb300.fst import Fst, debug_checks
+
+    # frontiers across every line between the string kernels' parts, handed
+    # from worker to worker in both passes
+    f, o = T.fans.__wrapped__()
+    strs = T._strings(list(range(16)), 60)
+    T._same_as_per_position(f, strs, 2)
+    f.set_plain_method(_lib.PLAIN_FRONTIER)
+    for b in range(0, 60, 7):
+        f.viterbi(strs.get(b)); f.forward_backward(strs.get(b))
+    # a lattice (its lookups have checks of their own)
+    n = 12
+    frm, to = np.repeat(np.arange(n), 2).astype(np.int32), np.repeat(np.arange(1, n + 1), 2).astype(np.int32)
+    lab = np.tile(np.array([T.STEP, T.SCATTER], np.int32), n)
+    wt = np.zeros(2 * n, np.float32)
+    f.lattice_viterbi(n + 1, frm, to, lab, wt); f.lattice_forward_backward(n + 1, frm, to, lab, wt)
+    r = debug_checks()
+    print("VIOLATIONS", r["violations"], r["code"], r["index"], r["bound"])
+""")
+
+
+def test_debug_build_wide_frontiers_and_lattices(tmp_path):
+    from paper_1701_03038_gb300 import build
+    lib = build.build_debug(str(tmp_path / "libfstgpu_debug.so"))
+    env = dict(os.environ, FSTGPU_LIB=lib)
+    script = WIDE.format(root=ROOT, tests=os.path.join(ROOT, "tests"))
+    r = subprocess.run([sys.executable, "-c", script], env=env, cwd=ROOT, capture_output=True, text=True, timeout=1200)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    line = [x for x in r.stdout.splitlines() if x.startswith("VIOLATIONS")][-1]
+    assert line.split()[1] == "0", line
