@@ -1859,9 +1859,21 @@ struct Backward {
       u = x;
       et = fx_narrow(x);
     }
-    if (lane < m && !dead64(my_x)) {
+    const bool on = lane < m && !dead64(my_x);
+    float g = 0.f;
+    if (on) {
       const double K0 = (pre + my_tE - P.lz) - (double)mprev;
-      add_count(C, arc.z, __expf(fx_narrow(ra + my_x + K0)) * P.gw);
+      g = __expf(fx_narrow(ra + my_x + K0)) * P.gw;
+    }
+    // A string by itself: positions that use the same arc add to it one after
+    // the other, so that its counts are the same bits every time (everywhere
+    // else an arc has one writer a position, and barriers between positions).
+    const uint32_t same = K.strings == 1 ? __match_any_sync(FULL, on ? arc.z : -1 - lane) : 1u << lane;
+    const int rank = __popc(same & lanes_below());
+    const int ranks = (int)__reduce_max_sync(FULL, (unsigned)rank);
+    for (int r = 0; r <= ranks; ++r) {
+      if (on && rank == r) add_count(C, arc.z, g);
+      __syncwarp();
     }
     // the table: the values of position P.t out, the last one in
     empty(P, lane, 32);

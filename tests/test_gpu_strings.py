@@ -181,3 +181,28 @@ def test_many_start_states(starts):
         lz, cnt, _ = f.forward_backward(x)
         assert_logz_close(lz, ofb["logz"])
         assert_counts_close(cnt, ofb["counts"])
+
+
+def test_counts_of_one_string_are_repeatable(fans):
+    # a string by itself adds its float64 counts in the order of its positions,
+    # also where a run of one-arc positions uses an arc again and again
+    from paper_1701_03038_gb300 import _lib
+    from paper_1701_03038_gb300.fst import Fst
+    rng = np.random.default_rng(6)
+    q = np.arange(8)
+    fan = rng.integers(0, 8, 64)
+    src = np.concatenate([q, np.repeat(q, 8), q]).astype(np.int32)
+    dst = np.concatenate([(q + 1) % 8, fan, np.zeros(8, int)]).astype(np.int32)
+    lab = np.concatenate([np.zeros(8), np.ones(64), np.full(8, 2)]).astype(np.int32)
+    start = np.full(8, np.inf, np.float32)
+    start[0] = 0.0
+    small = Fst.from_arrays(synth.FstArrays(8, 3, 3, src, dst, lab, lab, rng.uniform(0.1, 2.0, 80).astype(np.float32), start,
+                                            np.zeros(8, np.float32)))
+    runs = np.concatenate([[1] * 5 + [2] + [0] * int(rng.integers(40, 90)) for _ in range(12)]).astype(np.int32)
+    f, _ = fans
+    wide = _strings(list(range(16)), 12)
+    for h, x in [(small, runs)] + [(f, wide.get(b)) for b in (8, 11)]:
+        h.set_plain_method(_lib.PLAIN_FRONTIER)
+        want = h.forward_backward(x)[1].view(np.uint32)
+        for _ in range(8):
+            assert np.array_equal(h.forward_backward(x)[1].view(np.uint32), want)
