@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <array>
 #include <chrono>
+#include <memory>
 #include <vector>
 
 #include "fst_internal.cuh"
@@ -224,19 +225,29 @@ namespace {
 
 int plain_init(fst_s* f) {
   if (f->plain) return FST_OK;
-  PlainWs* w = new PlainWs();
-  f->plain = w;
-  const int64_t Q = f->Q;
+  std::unique_ptr<PlainWs> w(new PlainWs());
   int rc;
-  if ((rc = dalloc(&w->acc, 4 * Q)) || (rc = dalloc(&w->beta, 2 * Q)) || (rc = dalloc(&w->vmap, 2 * Q)) ||
-      (rc = dalloc(&w->jfinal, 1)) || (rc = dalloc(&w->bw_off, 1)) ||
-      (rc = dalloc(&w->pool_top, 1)) || (rc = dalloc(&w->flags, 2)) || (rc = dalloc(&w->gbar, 2)))
+  if ((rc = dalloc(&w->jfinal, 1)) || (rc = dalloc(&w->bw_off, 1)) || (rc = dalloc(&w->pool_top, 1)) ||
+      (rc = dalloc(&w->flags, 2)) || (rc = dalloc(&w->gbar, 2)))
     return rc;
-  FST_CUDA(cudaMemset(w->acc, 0, (size_t)4 * Q * sizeof(unsigned long long)));
-  FST_CUDA(cudaMemset(w->beta, 0, (size_t)2 * Q * sizeof(double)));
   FST_CUDA(cudaMemset(w->bw_off, 0, sizeof(int64_t)));
   FST_CUDA(cudaMemset(w->flags, 0, 2 * sizeof(uint32_t)));
+  f->plain = w.release();
   return FST_OK;
+}
+
+// The accumulators of the per-position kernels, on their first use (56 bytes
+// a state, beside the string kernels' 52).
+int plain_steps(fst_s* f) {
+  PlainWs* w = f->plain;
+  if (w->vmap) return FST_OK;
+  dfree(w->acc); dfree(w->beta);
+  const int64_t Q = f->Q;
+  int rc;
+  if ((rc = dalloc(&w->acc, 4 * Q)) || (rc = dalloc(&w->beta, 2 * Q))) return rc;
+  FST_CUDA(cudaMemset(w->acc, 0, (size_t)4 * Q * sizeof(unsigned long long)));
+  FST_CUDA(cudaMemset(w->beta, 0, (size_t)2 * Q * sizeof(double)));
+  return dalloc(&w->vmap, 2 * Q);
 }
 
 // Grow the per-string buffers: n tokens, a staging buffer for the largest
@@ -350,6 +361,7 @@ int plain_tokens(fst_s* f, const int32_t* ids, int32_t n, cudaStream_t s, bool* 
   *strings = f->plain_fb_driver == FST_DRIVER_LAUNCH && pool + spare < INT32_MAX && !plain_by_launches(f, ids, n);
   int rc = plain_reserve(w, std::max(n, 1), stage, *strings ? pool + spare : pool);
   if (rc) return rc;
+  if (!*strings && (rc = plain_steps(f))) return rc;
   w->olabels = w->paths + n;
   w->str_last = *strings;
   std::vector<int32_t> up((size_t)n + 1);

@@ -420,3 +420,30 @@ def test_wide_frontiers_by_launches_or_string_kernels(growth, launches):
             assert by["fwd_step"][1] == (len(x) if launches and large else 1), by
             assert by["bwd_step"][1] == (len(x) if launches and large else 1), by
     f.profile(False)
+
+
+def test_accumulators_of_the_launches_come_on_first_use():
+    # a handle whose single strings all take the string kernels holds no
+    # accumulators of the per-position kernels (56 bytes a state); the first
+    # string that takes those lays them down
+    import torch
+    Q = 2_000_000
+    q = np.arange(Q, dtype=np.int32)
+    src, dst = np.concatenate([q, q, q[:3000]]), np.concatenate([(q + 1) % Q, (q * 3) % Q, np.arange(3000)]).astype(np.int32)
+    lab = np.concatenate([np.zeros(Q), np.ones(Q), np.full(3000, 2)]).astype(np.int32)
+    start = np.full(Q, np.inf, np.float32)
+    start[:2000] = 0.5
+    fa = synth.FstArrays(Q, 3, 3, src.astype(np.int32), dst, lab, lab, np.ones(len(src), np.float32), start,
+                         np.zeros(Q, np.float32))
+    f, o = _fst(fa), oracle.Fst(fa)
+    narrow = np.array([2, 2], np.int32)  # (three arcs expected out of 2,000 of 2M states)
+    wide = np.array([0, 1, 0, 1, 1], np.int32)
+    free = lambda: torch.cuda.mem_get_info()[0]  # noqa: E731
+    before = free()
+    f.viterbi(narrow)
+    f.forward_backward(narrow, posteriors=False)
+    held = before - free()
+    assert held < 80 * Q, held  # (the string kernels' 52, and 10 MB)
+    for x in (wide, narrow, wide):
+        check_string(f, o, x)
+    assert before - free() >= held + 56 * Q
