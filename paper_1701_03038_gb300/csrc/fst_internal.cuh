@@ -26,6 +26,7 @@
 
 #include "fixmath.cuh"
 #include "fstgpu.h"
+#include "seg_table.cuh"
 
 namespace fstgpu {
 
@@ -50,14 +51,15 @@ struct __align__(16) WinMeta {
 // brings the arc too.  A key that finds its bucket full goes to the next
 // ones, and marks its own as spilled (SPILLED in the first slot's `at`), so
 // that a lookup that misses reads on only past a spilled bucket; with three
-// slots a segment about 3% of the buckets are.  (One slot after another at
-// up to half load, a warp's 32 lookups waited for the longest of their probe
-// sequences: 7,000 cycles in the readout of a large position.)
+// slots a segment (seg_table.cuh) about 3% of the buckets are.  (One slot
+// after another at up to half load, a warp's 32 lookups waited for the longest
+// of their probe sequences: 7,000 cycles in the readout of a large position.)
 struct alignas(32) SegSlot {
   unsigned long long key, at;
   int4 arc;
 };
 constexpr unsigned long long SPILLED = 1ull << 63;
+static_assert(sizeof(SegSlot) * SEG_BUCKET_SLOTS == SEG_BUCKET_BYTES, "a bucket is two slots");
 
 struct Layout {
   int64_t P = 0;         // padded arcs = nwin * WIN

@@ -408,7 +408,9 @@ int build_store(fst_s* f, const int32_t* d_src, const int32_t* d_dst, const int3
   // kernels find a live state's arcs on a symbol with about one probe
   {
     Layout& L = f->bwd;
-    L.buckets = std::min<int64_t>(1 + 3 * std::max<int64_t>(L.nseg, 1) / 2, ((int64_t)1 << 31) - 1);  // (32-bit slots)
+    size_t free_bytes = 0, total_bytes = 0;
+    FST_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
+    L.buckets = seg_buckets(L.nseg, (int64_t)free_bytes);
     if ((rc = dalloc(&L.seg_hash, 2 * L.buckets)) || (rc = dalloc(&L.seg_slot, L.nseg))) return rc;
     k_hash_clear<<<(unsigned)std::min<int64_t>(blocks_for(2 * L.buckets), 152 * 16), TB, 0, s>>>(L.seg_hash, 2 * L.buckets);
     if (L.nseg > 0)
