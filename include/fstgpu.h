@@ -288,9 +288,9 @@ FST_API int fst_set_batch_budget(fst_t* fst, int64_t mem_budget_bytes);
 /* Plans of fst_viterbi_batch and fst_forward_backward_batch: parts_viterbi
  * and parts_fb stream-parallel parts (FST_PLAN_PARTS; 0 = one part: the
  * string kernels fill the device with one) and the layout that the plan's
- * per-position kernels would take (-1 = dense when the dense accumulators
- * and the live pool fit the batch budget in one wave, else compact; 0 =
- * compact; 1 = FST_PLAN_DENSE_ACC), and whether
+ * per-position kernels would take (-1 and 0 = compact; 1 =
+ * FST_PLAN_DENSE_ACC, which also cuts the batch into waves by that layout's
+ * size), and whether
  * the run's launches are recorded into a CUDA graph that is then launched
  * (graph: 0 = no, 1 = yes, never on the legacy default stream or inside a
  * capture the caller began; -1 = the default, no).  The default is 0, 0,
@@ -315,7 +315,8 @@ FST_API int fst_set_batch_plan(fst_t* fst, int32_t parts_viterbi, int32_t parts_
  * holds more live states than a table fits ends the run with FST_ERR_OOM,
  * like a full pool, and leaves the plan usable.  FST_PLAN_DENSE_ACC gives
  * each string a dense accumulator of 2 Q slots instead (no such limit;
- * 16 to 48 bytes a state a string, which bounds the wave size).  Once created,
+ * 16 to 48 bytes a state a string, which bounds the wave size whichever
+ * kernels run).  Once created,
  * the run calls below allocate
  * nothing, so a sequence of them can be captured into a CUDA graph and
  * replayed.  A Viterbi-only plan and a forward-backward-only plan of the
