@@ -64,10 +64,11 @@ PERSIST_NAMES = {"vit": "k_vit_persist", "fwd": "k_fwd_persist", "bwd": "k_bwd_p
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 # the files that decide what the step kernels read and write
 KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "store.cu", "fst_internal.cuh", "strings.cu", "frontier.cuh",
-                  "fixmath.cuh")  # the device code of the batched passes
+                  "fixmath.cuh", "seg_table.cuh")  # the device code of the batched passes
 PASS_KERNELS = {"vit": ("vit_first", "vit_step"), "fwd": ("fwd_first", "fwd_sum", "fwd_step"),
                 "bwd": ("bwd_step",)}
 STRING_NAMES = {"vit": "k_str_forward", "fwd": "k_str_forward", "bwd": "k_str_backward"}  # one launch a pass
+STRING_TRAFFIC = {"vit": "k_str_forward<1>", "fwd": "k_str_forward<0>", "bwd": "k_str_backward"}
 KERNEL_NAMES = {"vit_first": "k_vit_first", "vit_step": "k_vit_step", "fwd_first": "k_fwd_first",
                 "fwd_sum": "k_fwd_sum", "fwd_step": "k_fwd_step", "bwd_step": "k_bwd_step",
                 "vit_final": "k_vit_final", "backtrace": "k_backtrace", "fb_final": "k_fb_final",
@@ -437,6 +438,8 @@ def ingest_traffic(csv_path, line_path):
         if not m:
             continue
         name = m.group(1)
+        if name == "k_str_forward":  # one kernel for both forward recursions, by its template argument
+            name += "<1>" if re.search(r"k_str_forward<(\(bool\))?(1|true)>", d["Kernel Name"]) else "<0>"
         if d["Metric Name"] in ("dram__bytes_read.sum", "dram__bytes_write.sum"):
             v = float(d["Metric Value"].replace(",", ""))
             unit = d.get("Metric Unit", "byte").lower()
@@ -448,7 +451,8 @@ def ingest_traffic(csv_path, line_path):
     alg = live_bytes(live["entries"], live["arcs"])
     passes = {}
     for p, ks in PASS_KERNELS.items():
-        tot = sum(by_kernel.get(KERNEL_NAMES[k], 0.0) for k in ks) + by_kernel.get(PERSIST_NAMES[p], 0.0)
+        tot = sum(by_kernel.get(k, 0.0)
+                  for k in [KERNEL_NAMES[k] for k in ks] + [PERSIST_NAMES[p], STRING_TRAFFIC[p]])
         if tot > 0:
             passes[p] = {"dram_bytes": int(tot), "algorithmic_bytes": int(alg[p]),
                          "dram_per_algorithmic_byte": tot / alg[p]}

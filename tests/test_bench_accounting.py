@@ -242,3 +242,22 @@ def test_reference_arm_line(capsys):
     assert line["e2e"]["h2d_bytes_per_step"] == 0 and line["e2e"]["d2h_bytes_per_step"] == 0
     assert line["e2e"]["value"] == line["value"] and line["e2e"]["unit"] == line["unit"]
     assert line["config"]["workload"].startswith("c1")
+
+
+def test_traffic_of_the_string_kernels(tmp_path, monkeypatch):
+    # one launch a pass; the two forward recursions are one kernel's two
+    # instances, however the list spells the template argument
+    import json
+    monkeypatch.setattr(bench, "TRAFFIC_FILE", str(tmp_path / "traffic.json"))
+    rows = [("void fstgpu::<unnamed>::k_str_forward<1>(fstgpu::LayoutView)", "dram__bytes_read.sum", "Mbyte", "3"),
+            ("void fstgpu::<unnamed>::k_str_forward<(bool)1>(fstgpu::LayoutView)", "dram__bytes_write.sum", "Mbyte", "1"),
+            ("void fstgpu::<unnamed>::k_str_forward<0>(fstgpu::LayoutView)", "dram__bytes_read.sum", "Mbyte", "5"),
+            ("void fstgpu::<unnamed>::k_str_forward<(bool)0>(fstgpu::LayoutView)", "dram__bytes_write.sum", "byte", "7"),
+            ("fstgpu::<unnamed>::k_str_backward(fstgpu::LayoutView)", "dram__bytes_read.sum", "Kbyte", "9")]
+    _ncu_csv(tmp_path / "l.csv", rows)
+    line = {"live_work": {"entries": 10, "arcs": 20}, "config": {"workload": "w", "strings": 2, "accumulators": "dense"}}
+    (tmp_path / "b.json").write_text(json.dumps(line) + "\n")
+    bench.ingest_traffic(str(tmp_path / "l.csv"), str(tmp_path / "b.json"))
+    p = bench.load_traffic("dense")["passes"]
+    assert p["vit"]["dram_bytes"] == 4_000_000 and p["fwd"]["dram_bytes"] == 5_000_007
+    assert p["bwd"]["dram_bytes"] == 9_000
