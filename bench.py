@@ -284,7 +284,9 @@ def roofline(prof, live, peak, peak_src, traffic, stats=None, ids=None, persiste
          "frac": round(achieved / peak, 5), "traffic": None if tr is None else int(tr),
          "per": f"{dom} pass (all its launches)",
          "kernel": (PERSIST_NAMES[dom] if dom in persistent
-                    else STRING_NAMES[dom] if "fwd_sum" in prof and not prof["fwd_sum"][1]
+                    # (single strings may take either; the sums are launches per position only)
+                    else STRING_NAMES[dom] if "fwd_sum" in prof and (not prof["fwd_sum"][1]
+                                                                     or 2 * prof["fwd_sum"][1] < prof["fwd_step"][1])
                     else " + ".join(KERNEL_NAMES[x] for x in PASS_KERNELS[dom])),
          "launches": sum(prof[x][1] for x in PASS_KERNELS[dom]), "pass_ms": round(pass_ms[dom], 3),
          "algorithmic_bytes": int(alg[dom]),
@@ -806,7 +808,9 @@ def plain_launches(f, strs, stats, coef) -> int:
 def string_launches(f, strs, stats, coef) -> int:
     """The same where the handle's driver is the launch driver and its method
     not the one-block kernels: the string kernels, Viterbi as forward +
-    final + trace, forward-backward as forward + final + backward + counts."""
+    final + trace, forward-backward as forward + final + backward + counts
+    (a string whose frontier is expected to stay wide takes launches per
+    position: profiled_launches counts those)."""
     from paper_1701_03038_gb300 import _lib
     pm = f.plain_method()
     if pm["method"] == _lib.PLAIN_BLOCK or pm["driver"] == _lib.DRIVER_PERSISTENT:
@@ -820,6 +824,16 @@ def string_launches(f, strs, stats, coef) -> int:
             pm["method"] == _lib.PLAIN_AUTO and coef[2] + coef[3] * n + coef[4] * arcs < coef[0] + coef[1] * n)
         total += 4 + (int((stats[0][x] > 0).sum()) + 1 + (n > 0) if slice_vit else 3)
     return total
+
+
+def profiled_launches(f, strs, prof, on_slice) -> int | None:
+    """The same from the launches of a profiled step of the frontier kernels,
+    when every string takes those (None: some other kernel does)."""
+    from paper_1701_03038_gb300 import _lib
+    pm = f.plain_method()
+    if on_slice or pm["method"] in (_lib.PLAIN_BLOCK, _lib.PLAIN_SLICE):
+        return None
+    return int(sum(n for _, n in prof.values()))
 
 
 def bench_plain(args, rank, world, dev, fa, strs, f, stats):
@@ -878,6 +892,9 @@ def bench_plain(args, rank, world, dev, fa, strs, f, stats):
     prof = f.profile_read()
     f.profile(False)
     f.set_plain_method(_lib.PLAIN_AUTO)
+    counted = profiled_launches(f, strs, prof, sum(sl))
+    if counted is not None:
+        out["gpu_launches"] = args.steps * counted
     live = {"entries": entries, "arcs": arcs}
     peak, peak_src = load_peak()
     rl, passes = roofline(prof, live, peak, peak_src, None, stats, strs.ids)

@@ -261,3 +261,35 @@ def test_traffic_of_the_string_kernels(tmp_path, monkeypatch):
     p = bench.load_traffic("dense")["passes"]
     assert p["vit"]["dram_bytes"] == 4_000_000 and p["fwd"]["dram_bytes"] == 5_000_007
     assert p["bwd"]["dram_bytes"] == 9_000
+
+
+def test_launches_counted_from_a_profiled_step():
+    # strings on either way of the frontier kernels: what the profile counted;
+    # not where another method's kernels run
+    from paper_1701_03038_gb300 import _lib
+    prof = {"vit_step": (1.0, 1 + 20), "vit_first": (0.1, 1), "vit_final": (0.1, 2), "counts": (0.1, 2), "fwd_sum": (0.0, 0)}
+
+    class Handle:
+        method = _lib.PLAIN_AUTO
+
+        def plain_method(self):
+            return {"method": self.method, "driver": _lib.DRIVER_LAUNCH, "grid_blocks": 0}
+
+    h = Handle()
+    assert bench.profiled_launches(h, None, prof, 0) == 26
+    assert bench.profiled_launches(h, None, prof, 1) is None
+    for m in (_lib.PLAIN_BLOCK, _lib.PLAIN_SLICE):
+        h.method = m
+        assert bench.profiled_launches(h, None, prof, 0) is None
+
+
+def test_kernel_of_a_mixed_profile():
+    # single strings of both ways: the pass is named by the kernel of most strings
+    E, P = 1000, 2000
+    kinds = {k: (0.0, 0) for k in ("vit_first", "vit_step", "fwd_first", "fwd_sum", "fwd_step", "bwd_step")}
+    r, _ = bench.roofline(dict(kinds, bwd_step=(5.0, 119), fwd_step=(1.0, 119), fwd_sum=(0.1, 20)),
+                          {"entries": E, "arcs": P}, 1000.0, "src", None)
+    assert r["kernel"] == "k_str_backward"
+    r, _ = bench.roofline(dict(kinds, bwd_step=(5.0, 100), fwd_step=(1.0, 100), fwd_sum=(0.1, 100)),
+                          {"entries": E, "arcs": P}, 1000.0, "src", None)
+    assert r["kernel"] == "k_bwd_step"
