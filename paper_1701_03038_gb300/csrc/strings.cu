@@ -1868,12 +1868,16 @@ struct Backward {
     // A string by itself: positions that use the same arc add to it one after
     // the other, so that its counts are the same bits every time (everywhere
     // else an arc has one writer a position, and barriers between positions).
-    const uint32_t same = K.strings == 1 ? __match_any_sync(FULL, on ? arc.z : -1 - lane) : 1u << lane;
-    const int rank = __popc(same & lanes_below());
-    const int ranks = (int)__reduce_max_sync(FULL, (unsigned)rank);
-    for (int r = 0; r <= ranks; ++r) {
-      if (on && rank == r) add_count(C, arc.z, g);
-      __syncwarp();
+    if (K.strings == 1) {
+      const uint32_t same = __match_any_sync(FULL, on ? arc.z : -1 - lane);
+      const int rank = __popc(same & lanes_below());
+      const int ranks = (int)__reduce_max_sync(FULL, (unsigned)rank);
+      for (int r = 0; r <= ranks; ++r) {
+        if (on && rank == r) add_count(C, arc.z, g);
+        __syncwarp();
+      }
+    } else if (on) {
+      add_count(C, arc.z, g);
     }
     // the table: the values of position P.t out, the last one in
     empty(P, lane, 32);
