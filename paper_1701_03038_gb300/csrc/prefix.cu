@@ -449,8 +449,9 @@ extern "C" int fst_prefix_log_z(fst_t* f, const int32_t* ids, int32_t n, double*
   if (n == 0) {
     if ((rc = mem.take(f, Scratch::piece(sizeof(Out))))) return rc;
     Out* d_out = mem.get<Out>(1);
-    if ((rc = launch_after(k_close, dim3(1), s, (const float*)nullptr, (const float*)nullptr, f->Q,
-                           (const float*)f->theta_s, (const float*)f->theta_f, d_out)))
+    FST_CUDA(cudaMemsetAsync(&d_out->done, 0, sizeof(d_out->done), s));
+    if ((rc = launch_after(k_close, dim3((unsigned)std::min<int64_t>((Q + 7) / 8, CLOSE_BLOCKS)), s, (const float*)nullptr,
+                           (const float*)nullptr, f->Q, (const float*)f->theta_s, (const float*)f->theta_f, d_out)))
       return rc;
     FST_CUDA(cudaMemcpy(&h, d_out, sizeof(h), cudaMemcpyDeviceToHost));
   } else {
