@@ -309,6 +309,7 @@ struct StringQueue {
   int32_t chunk;
   uint64_t limit_ns;
   double* spoiled;  // backward: CountView::spoiled
+  uint32_t polls;   // a waiting worker looks at the end's marks every so many polls
 };
 // Arcs out of a position's live states up to which a heavy block takes its
 // table in shared memory, half of the table's slots.

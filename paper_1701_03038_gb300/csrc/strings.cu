@@ -283,7 +283,7 @@ __device__ __forceinline__ int32_t next_light(const StringQueue& K) {
       Patience w;
       w.start(K);
       for (uint32_t i = 1; (b = queue_poll(K, QL, ticket)) < 0; ++i) {
-        if (i % 8u == 0u && (all_done(K) || w.over(K))) break;
+        if (i % K.polls == 0u && (all_done(K) || w.over(K))) break;
         __nanosleep(1000);
       }
     }
@@ -463,7 +463,7 @@ struct HeavyPick {
       // else a job to help with, unless there was none to be had the last time
       if (b == PICK_NONE && !idle && peek(K.ctl + CTL_OPEN) != 0u) b = PICK_HELP;
       idle = b == PICK_HELP;
-      if (b == PICK_NONE && (!waiting || ++polls % 8u == 0u)) {
+      if (b == PICK_NONE && (!waiting || ++polls % K.polls == 0u)) {
         if (all_done(K)) {
           b = PICK_LEAVE;
         } else if (!waiting) {
@@ -2195,6 +2195,11 @@ StringQueue string_queue(const StringWork& W, int blocks, int32_t* grid) {
   K.chunk = W.chunk;
   K.limit_ns = W.limit_ns;
   K.spoiled = nullptr;
+  // (waiting workers of few strings look at every poll, a microsecond: a kept
+  // plan of one string of 3 symbols took 45 us for Viterbi and 85 for forward-
+  // backward with a look at every eighth, 33 and 61 so; launches per position
+  // 38 and 64)
+  K.polls = W.Bw <= 64 ? 1u : 8u;
   // (heavy blocks come first, so that they are resident first)
   const int all = (W.Bw + WARPS - 1) / WARPS;
   const int want = all <= blocks / 2 ? std::max(all, blocks / 4) : blocks / 4;
