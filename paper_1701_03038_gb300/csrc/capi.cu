@@ -396,7 +396,7 @@ int plain_string(fst_s* f, bool viterbi, StringWork* K) {
   }
   if (viterbi && !w->str_dense_v) {
     dfree(w->str_fe);
-    if ((rc = dalloc(&w->str_fe, Q + string_light_entries(f->num_sms))) || (rc = dalloc(&w->str_dense_v, Q))) return rc;
+    if ((rc = dalloc(&w->str_fe, Q + string_light_entries(f->num_sms, 1))) || (rc = dalloc(&w->str_dense_v, Q))) return rc;
     FST_CUDA(cudaMemset(w->str_dense_v, 0, (size_t)Q * 8));
   }
   if (!viterbi && !w->str_dense_f) {

@@ -318,7 +318,7 @@ constexpr int32_t STRING_TABLE_ARCS = 1024;
 // pool is handed out range by range, so that the cap counts live entries.
 constexpr int32_t POOL_CHUNK = 64;
 int64_t string_ctl_words(int32_t Bw, int32_t groups2);
-int64_t string_light_entries(int num_sms);
+int64_t string_light_entries(int num_sms, int64_t Bw);
 int32_t string_kept_values();
 // The forward recursion of every string: S.flags and S.pool_top point into
 // W.ctl, which is cleared first.  Fills the pool and the per-token ranges

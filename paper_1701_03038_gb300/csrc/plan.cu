@@ -1122,7 +1122,7 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
     const int64_t per_group = (int64_t)f->Q * ((P->want_vit ? 16 : 0) + (P->want_fb ? 32 : 0) + 4);
     const int32_t groups2 = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(std::min<int64_t>(P->max_bw, 2 * f->num_sms), budget / 4 / per_group));
-    const int64_t fe = P->want_vit ? (int64_t)groups2 * f->Q + string_light_entries(f->num_sms) : 0;
+    const int64_t fe = P->want_vit ? (int64_t)groups2 * f->Q + string_light_entries(f->num_sms, P->max_bw) : 0;
     fst_plan_s* d = donor_owner.get();
     if (d && d->fst == f && d->want_fb == P->want_fb && d->want_vit == P->want_vit && d->cap_bw >= P->max_bw &&
         d->cap_nt >= P->max_ntok && d->pool_cap >= P->pool_cap && d->cap_B >= B && d->cap_fe >= fe &&

@@ -2234,7 +2234,10 @@ int64_t string_ctl_words(int32_t Bw, int32_t groups2) {
   return CTL_WORDS + (int64_t)groups2 * (int64_t)(sizeof(StringJob) / 4) + 2 * ring +
          (int64_t)Bw * (int64_t)(sizeof(StringPark) / 4) + 2;
 }
-int64_t string_light_entries(int num_sms) { return (int64_t)num_sms * 4 * (NT1 / 32) * (HS0 / 2); }
+int64_t string_light_entries(int num_sms, int64_t Bw) {
+  // (at most one light block a string, and half of what is resident)
+  return std::min<int64_t>((int64_t)num_sms * 4, std::max<int64_t>(Bw, 1)) * WARPS * (HS0 / 2);
+}
 int32_t string_kept_values() { return LIGHT_CAP; }
 
 int launch_string_forward(bool viterbi, const LayoutView& L, const int32_t* sym, const FrontierState& S,
