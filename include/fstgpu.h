@@ -308,8 +308,9 @@ FST_API int fst_set_batch_plan(fst_t* fst, int32_t parts_viterbi, int32_t parts_
  * budget).  What only the per-position kernels need (the token lists of
  * every position, their accumulators) is allocated by the call that first
  * asks for them: fst_plan_set_driver (persistent), fst_plan_set_pull,
- * fst_plan_limit_table, fst_plan_table_slots, fst_plan_autotune; those
- * calls then synchronise.  These accumulators are hash tables keyed by (string,
+ * fst_plan_limit_table, fst_plan_table_slots, fst_plan_autotune (those
+ * calls then synchronise), and by fst_plan_create where launches per
+ * position will run the plan.  These accumulators are hash tables keyed by (string,
  * state), sized for 128 live states per token of the busiest position (at
  * most the symbols' destination counts) at half load; a position that
  * holds more live states than a table fits ends the run with FST_ERR_OOM,
@@ -544,7 +545,9 @@ FST_API int fst_plan_live_work(fst_plan_t* plan, int64_t* entries, int64_t* arcs
  *                          current limit, 2 s by default) ends the run with
  *                          FST_ERR_TIMEOUT in the status of every string of
  *                          its wave, and the next run starts clean.  With
- *                          the direction switch or a
+ *                          the direction switch, or where the symbols'
+ *                          slices let expect that most frontiers stay wide
+ *                          (plans of fst_plan_create), or a
  *                          table limit one launch per position and kernel
  *                          kind instead.  Either run can be captured into a
  *                          CUDA graph and replayed.

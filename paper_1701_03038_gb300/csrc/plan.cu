@@ -47,6 +47,7 @@ constexpr int64_t LIVE_FLOOR = (int64_t)1 << 18;
 // internal plan flag: a part of a plan of several parts (the parent owns
 // the count accumulators)
 constexpr int32_t PLAN_PART = 1 << 16;
+constexpr int32_t PLAN_BATCH = 1 << 17;  // of a batch call: built for one run
 
 // *sum += the non-negative values of v[0..n).
 __global__ void k_sum_i32(const int32_t* __restrict__ v, int64_t n, unsigned long long* __restrict__ sum) {
@@ -174,6 +175,7 @@ struct fst_plan_s {
   int32_t str_groups2 = 0;
   int64_t cap_fe = 0;
   bool str_last = false;  // the last forward (or Viterbi) run took the string kernels
+  bool by_launches = false;  // wide frontiers are expected: launches per position are faster
   bool forward_done = false;
   // optional per-launch CUDA events (fst_plan_profile)
   LaunchProfile prof;
@@ -244,25 +246,48 @@ int alloc_store(fst_plan_s* P, T** p, int64_t n) {
 
 // Per string: the arcs its symbols' slices hold and the destinations they
 // can reach, its symbols copied into the plan; *bad is set where a symbol is
-// outside [0, m).  A warp per string.
+// outside [0, m).  est: over all strings, the positions expected to have more
+// than STRING_TABLE_ARCS arcs out of live states, the live states before them
+// and their arcs (live states have their slice's average arcs, which hit its
+// destinations at random).  A warp per string.
 __global__ void k_string_stats(const int32_t* __restrict__ ids, const int64_t* __restrict__ off, int32_t B, int32_t m,
                                const int64_t* __restrict__ sym_arc, const int64_t* __restrict__ sym_seg,
                                int32_t* __restrict__ sym, int64_t* __restrict__ arcs, int64_t* __restrict__ dsts,
-                               int64_t* __restrict__ bad) {
+                               int64_t* __restrict__ bad, float Q, float starts, double* __restrict__ est) {
   const int lane = threadIdx.x & 31;
   const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (b >= B) return;
   const int64_t lo = off[b], hi = off[b + 1];
   long long na = 0, nd = 0;
   bool wrong = false;
-  for (int64_t i = lo + lane; i < hi; i += 32) {
-    const int32_t a = ids[i];
-    sym[i] = a;
-    if (a < 0 || a >= m) {
-      wrong = true;
-    } else {
-      na += sym_arc[a + 1] - sym_arc[a];
-      nd += sym_seg[a + 1] - sym_seg[a];
+  float live = starts, large = 0.f;
+  double from = 0.0, wide = 0.0;
+  for (int64_t i0 = lo; i0 < hi; i0 += 32) {
+    const int64_t i = i0 + lane;
+    float A = 0.f, D = 0.f;
+    if (i < hi) {
+      const int32_t a = ids[i];
+      sym[i] = a;
+      if (a < 0 || a >= m) {
+        wrong = true;
+      } else {
+        const int64_t ca = sym_arc[a + 1] - sym_arc[a], cd = sym_seg[a + 1] - sym_seg[a];
+        na += ca;
+        nd += cd;
+        A = (float)ca;
+        D = (float)cd;
+      }
+    }
+    const int n = (int)min((long long)32, (long long)(hi - i0));
+    for (int k = 0; k < n && live > 0.f; ++k) {
+      const float a = __shfl_sync(0xffffffffu, A, k), d = __shfl_sync(0xffffffffu, D, k);
+      const float x = fminf(live / Q, 1.f) * a;
+      if (x > (float)STRING_TABLE_ARCS) {
+        large += 1.f;
+        from += (double)live;
+        wide += (double)x;
+      }
+      live = a <= 0.f ? 0.f : fmaxf(1.f, x < d * 0.05f ? x : d * (1.f - powf(fmaxf(0.f, 1.f - x / a), a / d)));
     }
   }
 #pragma unroll
@@ -273,6 +298,11 @@ __global__ void k_string_stats(const int32_t* __restrict__ ids, const int64_t* _
   if (lane == 0) {
     arcs[b] = na;
     dsts[b] = nd;
+    if (large > 0.f) {
+      atomicAdd(est, (double)large);
+      atomicAdd(est + 1, from);
+      atomicAdd(est + 2, wide);
+    }
   }
   if (wrong) *bad = 1;
 }
@@ -526,9 +556,10 @@ FrontierState wave_state(fst_plan_s* P, const Wave& W, const float* gweight) {
 }
 
 // Whether a run takes the string kernels: the launch driver without the
-// settings that only the per-position kernels have.
+// settings that only the per-position kernels have, and frontiers that are not
+// expected to stay wide.
 bool string_path(const fst_plan_s* P) {
-  return P->driver == FST_DRIVER_LAUNCH && P->pull_min == 0 && P->table_limit == 0;
+  return P->driver == FST_DRIVER_LAUNCH && P->pull_min == 0 && P->table_limit == 0 && !P->by_launches;
 }
 
 StringWork string_work(fst_plan_s* P, const Wave& W, bool viterbi) {
@@ -854,7 +885,7 @@ static int plan_create_parts(fst_t* f, const int32_t* d_ids, const int64_t* d_of
       continue;
     }
     rc = plan_build(f, d_ids, d_offsets + bs[i], h_off + bs[i], bs[i + 1] - bs[i], part_budget,
-                    (flags & 0xff) | PLAN_PART, s, pd[i], &sub[i]);
+                    (flags & (0xff | PLAN_BATCH)) | PLAN_PART, s, pd[i], &sub[i]);
   }
   if (rc) {
     for (fst_plan_t* q : sub) delete q;
@@ -1043,7 +1074,7 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
     }
     // the strings' lengths and offsets inside their wave, the sums over
     // their symbols, and the symbols
-    const int64_t words = 2 * ((int64_t)B * 3 + 1) + B + 1;  // 4-byte words before the symbols
+    const int64_t words = 2 * ((int64_t)B * 3 + 4) + B + 1;  // 4-byte words before the symbols
     const int64_t arena = (words + N + 4) * 4;
     if (donor_owner && donor_owner->cap_tok >= arena) {
       std::swap(P->tok_arena, donor_owner->tok_arena);
@@ -1058,7 +1089,8 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
     int64_t* a_arcs = a_off + B;
     int64_t* a_dsts = a_arcs + B;
     int64_t* a_bad = a_dsts + B;
-    int32_t* a_n = (int32_t*)(a_bad + 1);
+    double* a_est = (double*)(a_bad + 1);
+    int32_t* a_n = (int32_t*)(a_est + 3);
     int32_t* a_sym = a_n + B + 1;
     std::vector<unsigned char> head((size_t)(words * 4), 0);
     int64_t* h_boff = (int64_t*)head.data();
@@ -1073,11 +1105,12 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
       w.bw_n = a_n + w.b0;
       w.tok_sym = a_sym + w.tok0;
     }
-    std::vector<int64_t> sums((size_t)2 * B + 1, 0);
+    std::vector<int64_t> sums((size_t)2 * B + 4, 0);
     cudaError_t e = cudaMemcpyAsync(P->tok_arena, head.data(), head.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && B > 0) {
       k_string_stats<<<(unsigned)((B + 7) / 8), 256, 0, s>>>(d_ids, d_offsets, B, f->m, f->sym_arc, f->fwd.sym_seg,
-                                                            a_sym - h_off[0], a_arcs, a_dsts, a_bad);
+                                                            a_sym - h_off[0], a_arcs, a_dsts, a_bad, (float)f->Q,
+                                                            (float)f->nstart, a_est);
       e = cudaGetLastError();
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(sums.data(), a_arcs, sums.size() * 8, cudaMemcpyDeviceToHost, s);
@@ -1113,6 +1146,22 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
       // pool entries are named by int32 indices
       P->pool_cap = std::max(P->pool_cap, std::min(std::min(w.pool_bound, want), (int64_t)INT32_MAX));
     }
+    // Whether launches per position run the batch faster than the string
+    // kernels, as for a single string (plain_by_launches in capi.cu): when a
+    // third of its positions are expected to have more arcs than a heavy
+    // block's table holds, and not so many that the launches' atomics collide
+    // -- by destination or, beyond four million arcs a position of all
+    // strings, by number.  (3,000 states of 3.3 arcs a state and symbol, kept
+    // plans, Viterbi and forward-backward, by launches and by string kernels: 1
+    // string of 100 symbols 918 and 2,149 us, 2,663 and 6,187; 16 of 15 to 30
+    // 523 and 954, 1,428 and 2,702; 300 of 10 to 20 1,270 and 1,506, 7,844 and
+    // 4,725.)  A batch call, whose plan runs once, keeps the string kernels:
+    // the step lists and accumulators take longer to lay down than they save.
+    double est[3];
+    memcpy(est, sums.data() + 2 * (size_t)B + 1, sizeof(est));
+    P->by_launches = !(flags & PLAN_BATCH) && est[0] * 3.0 > (double)N &&
+                     (est[2] <= 12.0 * est[1] || est[2] >= 5e5 * est[0]) &&
+                     (double)P->max_bw * est[2] <= 4e6 * est[0];
     // what the string kernels' chunks may leave unused
     P->pool_cap = std::min<int64_t>(P->pool_cap + P->pool_cap / 3 + 3 * POOL_CHUNK * std::min<int64_t>(P->max_bw, 64 * f->num_sms),
                                     (int64_t)INT32_MAX);
@@ -1186,13 +1235,15 @@ static int plan_build(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, 
     delete P;
     return rc;
   }
+  // (what the launches' accumulators may not hold stays with the string kernels)
+  if (P->by_launches && (plan_steps(P) || (P->compact && P->hslots < 2 * P->max_stage))) P->by_launches = false;
   *out = P;
   return FST_OK;
 }
 
 extern "C" int fst_plan_create(fst_t* f, const int32_t* d_ids, const int64_t* d_offsets, int32_t B,
                                int64_t mem_budget_bytes, int32_t flags, void* stream, fst_plan_t** out) {
-  return plan_create(f, d_ids, d_offsets, B, mem_budget_bytes, flags & ~PLAN_PART, stream, nullptr, out);
+  return plan_create(f, d_ids, d_offsets, B, mem_budget_bytes, flags & ~(PLAN_PART | PLAN_BATCH), stream, nullptr, out);
 }
 
 extern "C" int fst_plan_destroy(fst_plan_t* P) {
@@ -1416,7 +1467,7 @@ static void put_cached(fst_t* f, int kind, fst_plan_s* p) {
 // accumulators, which lay down nothing until the per-position kernels are
 // asked for; the handle's setting (fst_set_batch_plan) overrides both.
 static int32_t batch_flags(const fst_t* f, int kind) {
-  int32_t fl = kind == 0 ? FST_PLAN_NO_FB : FST_PLAN_NO_VITERBI;
+  int32_t fl = (kind == 0 ? FST_PLAN_NO_FB : FST_PLAN_NO_VITERBI) | PLAN_BATCH;
   if (f->batch_parts[kind] > 1) fl |= FST_PLAN_PARTS(f->batch_parts[kind]);
   if (f->batch_layout == 1) fl |= FST_PLAN_DENSE_ACC;
   return fl;

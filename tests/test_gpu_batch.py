@@ -457,3 +457,49 @@ def test_forward_pull_matches_push(c2s, parts):
             for a, b in ((cnt, ref[1]), (st, ref[2]), (fi, ref[3])):
                 assert np.allclose(a.cpu().numpy(), b.cpu().numpy(), rtol=1e-9, atol=1e-12), name
     check_batch_fb(o, strs, res["pull"][1][0], res["pull"][1][1][:o.A])
+
+
+@pytest.mark.parametrize("flags,parts", [(0, 1), (0, 3), ("dense", 1), ("dense", 3)])
+@pytest.mark.parametrize("growth,count,launches", [(0.6, 12, False), (3.3, 1, True), (3.3, 12, True), (3.3, 150, None),
+                                                   (20.0, 12, False)])
+def test_plans_of_wide_frontiers(growth, count, launches, flags, parts):
+    # kept plans whose frontiers are expected to stay wide take launches per
+    # position where their tables hold them, others and batch calls the string
+    # kernels; the results are the oracle's either way
+    import torch
+    from paper_1701_03038_gb300 import _lib
+    from paper_1701_03038_gb300.fst import Fst
+    rng = np.random.default_rng(int(10 * growth) + count)
+    Q, V = 3000, 6
+    A = int(Q * V * growth)
+    src, dst, lab = (rng.integers(0, k, A).astype(np.int32) for k in (Q, Q, V))
+    start = np.full(Q, np.inf, np.float32)
+    start[:20] = 0.5
+    fa = synth.FstArrays(Q, V, V, src, dst, lab, lab, rng.uniform(0.1, 3.0, A).astype(np.float32), start,
+                         rng.uniform(0.0, 1.0, Q).astype(np.float32))
+    f, o = Fst.from_arrays(fa), oracle.Fst(fa)
+    lens = rng.integers(8, 16, count)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    strs = synth.Strings(rng.integers(0, V, off[-1]).astype(np.int32), off)
+    ids, doff = torch.from_numpy(strs.ids).cuda(), torch.from_numpy(strs.offsets).cuda()
+    p = f.plan(ids, doff, flags=_lib.PLAN_DENSE_ACC if flags else 0, parts=min(parts, count))
+    p.profile(True)
+    w = torch.rand(count, device="cuda")
+    for _ in range(2):
+        p.viterbi()
+        p.forward_backward(weights=w)
+    torch.cuda.synchronize()
+    steps = p.profile_read()["vit_step"][1]
+    n = min(parts, count)
+    if launches is not None:
+        assert (steps > 4 * n) == launches, steps  # (two runs; a string kernel is one launch)
+    vb = f.viterbi_batch(ids, doff)
+    ofb = o.fb_batch(strs.ids, strs.offsets, weights=w.cpu().numpy().astype(np.float64), nthreads=8)
+    for b in list(range(min(count, 12))) + [count - 1]:
+        lo, hi = off[b], off[b + 1]
+        ov = o.viterbi(strs.get(b))
+        assert_viterbi_equal(p.scores[b].item(), p.paths[lo:hi].cpu().numpy(), p.olabels[lo:hi].cpu().numpy(),
+                             p.status[b].item(), ov)
+        assert_viterbi_equal(vb["scores"][b].item(), vb["paths"][lo:hi].cpu().numpy(), None, vb["status"][b].item(), ov)
+        assert_logz_close(p.logz[b].item(), ofb["logz"][b])
+    assert_counts_close(p.counts.cpu().numpy(), ofb["counts"], batch=True)
